@@ -20,6 +20,7 @@
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that makes every
 // later wait return at once, and the CTA still drains its copies, frees TMEM and exits.
 #include <algorithm>
+#include <numeric>
 
 #include "pc_tc.cuh"
 
@@ -644,6 +645,28 @@ int choose_splits(int n_items, int n_kv_tiles, int sm_count) {
     return best;
 }
 
+// Number of persistent CTAs.  CTAs that start at the same place inside their items run through the same key tiles at the
+// same time: of n CTAs over `items` equal items there are n / gcd(n, items) different starting places, and every one of
+// them is a stream of K and V of its own through L2.  With a cache larger than L2 the many streams of one CTA per SM read
+// everything again for each item (47 whole frames, 96 items on 148 SMs: 37 streams per KV head, 2.36 GB from DRAM for
+// 203 MB of K and V); 144 CTAs have three, and their runs are two thirds of an item, so no item is cut into more than two
+// parts.  So up to 1/32 of the SMs is given up for the fewest starting places, as long as the longest run grows by no more
+// than that (a run counts whole steps).  Measured, one CTA per SM against this rule: attention over 47 whole frames 725 ->
+// 628 us a call, five passes over 7,184 keys 519 -> 513, the step at 47 frames 170.7 -> 169.9, 4,032-token frames (384
+// items, K and V inside L2) 666 -> 667.
+int choose_ctas(int n_items, long long steps, int most) {
+    int best = most, best_starts = most / std::gcd(most, n_items);
+    const long long longest = (steps + most - 1) / most;
+    for (int n = most - 1; n >= most - most / 32; --n) {
+        const int starts = n / std::gcd(n, n_items);
+        if (starts < best_starts && 32 * ((steps + n - 1) / n) <= 33 * longest) {
+            best = n;
+            best_starts = starts;
+        }
+    }
+    return best;
+}
+
 }  // namespace
 
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
@@ -719,12 +742,12 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     P.status = ctx->status;
     P.wait_us = ctx->wait_limit_us;
     P.extra_tx = ctx->test_extra_tx;
-    // Persistent form unless the caller fixed the number of key ranges or asked for the cluster merge: one CTA per SM, but
+    // Persistent form unless the caller fixed the number of key ranges or asked for the cluster merge: one CTA per SM or a few less, but
     // never so many that an item is cut into more than MAX_SPLITS parts (a CTA's run is at least a third of an item).
     const long long T = (long long)n_items * tiles;
     P.persistent = (ctx->kv_splits == 0 && !ctx->cluster_merge) ? 1 : 0;
     if (P.persistent) {
-        P.n_cta = (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T);
+        P.n_cta = choose_ctas(n_items, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
         int most = 1;
         for (int i = 0; i < n_items; ++i) {        // the kernel's own rule (cta_of_step), evaluated for every item
             const long long x0 = (long long)i * tiles, x1 = x0 + tiles - 1;
