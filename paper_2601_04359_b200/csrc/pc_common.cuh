@@ -100,20 +100,25 @@ __device__ __forceinline__ void pc_flag(int32_t *status, int code, int where) {
     if (atomicCAS(status, 0, code) == 0) status[1] = where;
 }
 
-// (cos, sin) for pair i of a head at position p[0..2]; flags and clamps a position outside the table.
-__device__ __forceinline__ float2 pc_rope_cs(const pc_rope_dev &r, int pair, int pt, int ph, int pw, int32_t *status,
-                                             int where) {
+// (cos, sin) for pair i of a head at position p[0..2]; a position outside the table is clamped and noted in `bad`.  No branch
+// and no memory but the one read: look-ups of several tokens can be in flight together.
+__device__ __forceinline__ float2 pc_rope_cs_clamped(const pc_rope_dev &r, int pair, int pt, int ph, int pw, bool &bad) {
     const int a = pair % 3, m = pair / 3;
     // the axis picks its coordinate and table by selects on fixed fields (no indexed access to the parameter block)
     int pa = a == 0 ? pt : (a == 1 ? ph : pw);
     const int mx = a == 0 ? r.max_pos[0] : (a == 1 ? r.max_pos[1] : r.max_pos[2]);
     const int off = a == 0 ? r.off[0] : (a == 1 ? r.off[1] : r.off[2]);
     const int na = a == 0 ? r.n_axis[0] : (a == 1 ? r.n_axis[1] : r.n_axis[2]);
-    if (pa < 0 || pa >= mx) {
-        pc_flag(status, PC_ERR_INVALID_ARG, where);
-        pa = pa < 0 ? 0 : mx - 1;
-    }
+    bad |= pa < 0 || pa >= mx;
+    pa = min(max(pa, 0), mx - 1);
     return __ldg(r.tab + off + (size_t)pa * na + m);
+}
+// the same, with the event recorded at once
+__device__ __forceinline__ float2 pc_rope_cs(const pc_rope_dev &r, int pair, int pt, int ph, int pw, int32_t *status, int where) {
+    bool bad = false;
+    const float2 cs = pc_rope_cs_clamped(r, pair, pt, ph, pw, bad);
+    if (bad) pc_flag(status, PC_ERR_INVALID_ARG, where);
+    return cs;
 }
 
 // One rotary pair turned by (cos, sin), with the roundings spelt out: every kernel that rotates (query pass, key
