@@ -86,6 +86,21 @@ class PackCacheError(RuntimeError):
 
 
 _lib = None
+_native_module = None
+
+
+def _native():
+    """The native side of this binding (csrc/pc_python.cpp): the calls of a generation loop go through it, because building
+    the same structs through ctypes takes longer than the calls themselves.  Loaded with the library, built if absent."""
+    global _native_module
+    if _native_module is None:
+        if not os.path.exists(_build.PYLIB):
+            _build.build(force=True)
+        load()
+        from . import _packcache_py
+        _packcache_py.set_i32_converter(_i32)
+        _native_module = _packcache_py
+    return _native_module
 
 
 def load() -> C.CDLL:
@@ -161,7 +176,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -234,8 +249,7 @@ def pc_plan_budget(kind: int, param: float, total: int, keep_full: int, avail: S
                    min_quota: int = 0) -> np.ndarray:
     avail = _i32(avail)
     out = np.zeros(len(avail), dtype=np.int32)
-    p = pc_budget_params(kind, param, total, keep_full, min_quota)
-    _check(load().pc_plan_budget(C.byref(p), len(avail), _i32p(avail), _i32p(out)), "pc_plan_budget")
+    _check(_native().plan_budget(kind, param, total, keep_full, min_quota, avail, out), "pc_plan_budget")
     return out
 
 
@@ -244,24 +258,22 @@ def pc_score(ctx: Context, src: Cache, q: Optional[torch.Tensor], q_pos: Optiona
              scores: Optional[torch.Tensor] = None, sel_idx: Optional[torch.Tensor] = None, stream=None):
     """Returns (scores [n_src] fp32, sel_idx [sum(budget)] int32), both on the device."""
     budget = _i32(budget)
-    dev = src.history.k.device if src.history.k is not None else torch.device("cuda")
-    if scores is None and scores_override is None:
-        scores = torch.empty(max(src.history.n_tokens, 1), dtype=torch.float32, device=dev)
-    if sel_idx is None:
-        sel_idx = torch.empty(max(int(budget.sum()), 1), dtype=torch.int32, device=dev)
-    n_q = 0 if q is None else q.shape[0]
-    c = src.c()
-    _check(load().pc_score(ctx.handle, C.byref(c), _ptr(q), _ptr(q_pos), n_q, _i32p(budget), _ptr(valid),
-                           _ptr(scores_override), _ptr(scores), _ptr(sel_idx), _stream(stream)), "pc_score")
+    n = _native()
+    if sel_idx is None or (scores is None and scores_override is None):
+        dev = src.history.k.device if src.history.k is not None else torch.device("cuda")
+        if scores is None and scores_override is None:
+            scores = torch.empty(max(src.history.n_tokens, 1), dtype=torch.float32, device=dev)
+        if sel_idx is None:
+            sel_idx = torch.empty(max(n.total(budget), 1), dtype=torch.int32, device=dev)
+    _check(n.score(ctx.handle, src, q, q_pos, budget, valid, scores_override, scores, sel_idx, _stream(stream)), "pc_score")
     return scores, sel_idx
 
 
 def pc_compact(ctx: Context, src: Cache, sel_idx: torch.Tensor, budget, delta_t: int, dst: Cache, stream=None) -> None:
     budget = _i32(budget)
-    cs, cd = src.c(), dst.c()
-    _check(load().pc_compact(ctx.handle, C.byref(cs), _ptr(sel_idx), _i32p(budget), delta_t, C.byref(cd),
-                             _stream(stream)), "pc_compact")
-    dst.history.n_tokens = int(budget.sum())
+    n = _native()
+    _check(n.compact(ctx.handle, src, sel_idx, budget, delta_t, dst, _stream(stream)), "pc_compact")
+    dst.history.n_tokens = n.total(budget)
     dst.frame_count = budget.copy()
 
 
@@ -272,10 +284,7 @@ def pc_attend_frame(ctx: Context, cache: Cache, current: Optional[Segment], q: t
         out = torch.empty_like(q)
     if lse is None and want_lse:
         lse = torch.empty(q.shape[0], q.shape[1], dtype=torch.float32, device=q.device)
-    c = cache.c()
-    cur = current.c() if current is not None else None
-    _check(load().pc_attend_frame(ctx.handle, C.byref(c), C.byref(cur) if cur is not None else None, _ptr(q),
-                                  _ptr(q_pos), q.shape[0], _ptr(out), _ptr(lse), _stream(stream)), "pc_attend_frame")
+    _check(_native().attend_frame(ctx.handle, cache, current, q, q_pos, out, lse, _stream(stream)), "pc_attend_frame")
     return (out, lse) if want_lse else out
 
 
@@ -292,10 +301,9 @@ def pc_frame_step(ctx: Context, src: Cache, budget, delta_t: int, dst: Cache, q:
         out = torch.empty_like(q)
     if lse is None and want_lse:
         lse = torch.empty(q.shape[0], q.shape[1], dtype=torch.float32, device=q.device)
-    cs, cd = src.c(), dst.c()
-    _check(load().pc_frame_step(ctx.handle, C.byref(cs), _i32p(budget), delta_t, C.byref(cd), _ptr(q), _ptr(q_pos), q.shape[0],
-                                _ptr(scores), _ptr(sel_idx), _ptr(out), _ptr(lse), _stream(stream)), "pc_frame_step")
-    dst.history.n_tokens = int(budget.sum())
+    n = _native()
+    _check(n.frame_step(ctx.handle, src, budget, delta_t, dst, q, q_pos, scores, sel_idx, out, lse, _stream(stream)), "pc_frame_step")
+    dst.history.n_tokens = n.total(budget)
     dst.frame_count = budget.copy()
     return (out, scores, sel_idx, lse) if want_lse else (out, scores, sel_idx)
 
@@ -313,10 +321,7 @@ def pc_test_expect_extra_bytes(ctx: Context, n_bytes: int) -> None:
 
 
 def pc_attend_prepare(ctx: Context, cache: Cache, current: Optional[Segment] = None, stream=None) -> None:
-    c = cache.c()
-    cur = current.c() if current is not None else None
-    _check(load().pc_attend_prepare(ctx.handle, C.byref(c), C.byref(cur) if cur is not None else None, _stream(stream)),
-           "pc_attend_prepare")
+    _check(_native().attend_prepare(ctx.handle, cache, current, _stream(stream)), "pc_attend_prepare")
 
 
 def pc_attend_prepared(ctx: Context, q: torch.Tensor, q_pos: torch.Tensor, out: Optional[torch.Tensor] = None,
@@ -325,8 +330,7 @@ def pc_attend_prepared(ctx: Context, q: torch.Tensor, q_pos: torch.Tensor, out: 
         out = torch.empty_like(q)
     if lse is None and want_lse:
         lse = torch.empty(q.shape[0], q.shape[1], dtype=torch.float32, device=q.device)
-    _check(load().pc_attend_prepared(ctx.handle, _ptr(q), _ptr(q_pos), q.shape[0], _ptr(out), _ptr(lse), _stream(stream)),
-           "pc_attend_prepared")
+    _check(_native().attend_prepared(ctx.handle, q, q_pos, out, lse, _stream(stream)), "pc_attend_prepared")
     return (out, lse) if want_lse else out
 
 
@@ -334,7 +338,7 @@ def pc_attend_mass(ctx: Context, lse: torch.Tensor, n_keys: int, mass: Optional[
     """Attention mass of every key of the most recent attention call on ctx (lse = what that call wrote)."""
     if mass is None:
         mass = torch.empty(n_keys, dtype=torch.float32, device=lse.device)
-    _check(load().pc_attend_mass(ctx.handle, _ptr(lse), _ptr(mass), n_keys, _stream(stream)), "pc_attend_mass")
+    _check(_native().attend_mass(ctx.handle, lse, mass, n_keys, _stream(stream)), "pc_attend_mass")
     return mass
 
 
@@ -458,8 +462,7 @@ class Window:
         self.handle = h
 
     def append(self, frame: Segment, stream=None) -> None:
-        f = frame.c()
-        _check(load().pc_window_append(self.handle, C.byref(f), _stream(stream)), "pc_window_append")
+        _check(_native().window_append(self.handle, frame, _stream(stream)), "pc_window_append")
 
     def append_masked(self, frame: Segment, valid: torch.Tensor, n_valid: int, stream=None) -> None:
         f = frame.c()
@@ -478,10 +481,9 @@ class Window:
         """Update and attention in one call; returns (regime, out)."""
         if out is None:
             out = torch.empty_like(q)
-        regime = C.c_int32(-1)
-        _check(load().pc_window_step(self.handle, _ptr(q), _ptr(q_pos), q.shape[0], _ptr(out), _ptr(lse), C.byref(regime),
-                                     _stream(stream)), "pc_window_step")
-        return regime.value, out
+        status, regime = _native().window_step(self.handle, q, q_pos, out, lse, _stream(stream))
+        _check(status, "pc_window_step")
+        return regime, out
 
     def step_host(self, frame: Optional[dict], q: torch.Tensor, q_pos: torch.Tensor, out: torch.Tensor, ws: dict,
                   stream=None) -> int:

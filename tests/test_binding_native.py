@@ -1,0 +1,39 @@
+"""The binding's native side, without a GPU: host arrays of any integer kind, tensors that are not contiguous, a closed
+context."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_04359_b200 import binding as pc
+
+
+@pytest.mark.parametrize("make", [list, tuple, lambda a: np.array(a, np.int64), lambda a: np.array(a, np.int32),
+                                  lambda a: np.array(a, np.int32).repeat(2)[::2], lambda a: torch.tensor(a, dtype=torch.int32)])
+def test_host_arrays_of_any_integer_kind(make):
+    avail = [40, 7, 100, 0, 64]
+    want = pc.pc_plan_budget(pc.PC_LINEAR, 0.0, 90, 0, np.array(avail, np.int32))
+    got = pc.pc_plan_budget(pc.PC_LINEAR, 0, np.int64(90), np.int32(0), make(avail))
+    assert got.dtype == np.int32 and got.tolist() == want.tolist() and want.sum() == 90
+
+
+def _segment(n):
+    return pc.Segment(torch.zeros(n, 2, 8), torch.zeros(n, 2, 8), torch.zeros(n, 4, dtype=torch.int32), n)
+
+
+class _Closed:
+    handle = None
+
+
+def test_errors_reach_the_caller():
+    q, q_pos = torch.zeros(4, 2, 8), torch.zeros(4, 4, dtype=torch.int32)
+    cache = pc.Cache(pc.Segment.empty(), _segment(6), [2, 4])
+    with pytest.raises(pc.PackCacheError) as e:                        # the library refuses a null context before it reads anything
+        pc.pc_attend_frame(_Closed, cache, None, q, q_pos, stream=0)
+    assert e.value.status == pc.PC_ERR_INVALID_ARG
+    with pytest.raises(AssertionError, match="contiguous"):
+        pc.pc_attend_frame(_Closed, cache, None, q.transpose(0, 1), q_pos, out=q, stream=0)
+    with pytest.raises(ValueError):
+        pc.pc_compact(_Closed, cache, q_pos, ["x"], 0, cache, stream=0)
+    assert cache.history.n_tokens == 6                                 # a refused call leaves the destination's count alone
