@@ -34,7 +34,6 @@ enum {
 };
 
 constexpr int PC_MAX_SEGMENTS = 3;
-constexpr int PC_FX_REPLICAS = 8;             // copies of the pooled-query accumulator (see pc_score.cu)
 constexpr int PC_MAX_DEVICES = 64;            // per-device launch state is kept in arrays of this size
 
 // Rotary tables: for axis a (t, h, w) a [max_pos[a]][n_axis[a]] array of (cos, sin) of pos * base^(-m/n_axis[a]).
@@ -57,12 +56,10 @@ struct pc_ctx {
     float2 *rope_tab;          // owned
     int32_t *status;           // device [2]: code, where
     int32_t *host_status;      // pinned [2]
-    // Pooled query of the scoring pass as fixed-point sums (units of 2^-32): PC_FX_REPLICAS copies of Hkv*d 64-bit
-    // integers (the blocks of the query pass spread over the copies; integer addition: the result does not depend on the
-    // order of the blocks) and one ticket word.  The last block of the query pass adds the copies into `qpool` (fp32) and
-    // clears the accumulator, so it is zero between calls.
-    long long *qpool_fx;       // device [PC_FX_REPLICAS * Hkv*d + 1]
-    float *qpool;              // device [Hkv*d]
+    // Pooled query of the scoring pass as fixed-point sums (units of 2^-32): Hkv*d 64-bit integers (integer addition: the
+    // result does not depend on the order of the blocks) and one ticket word.  The scoring kernel reads it and clears it, so
+    // it is zero between calls.
+    long long *qpool_fx;       // device [Hkv*d + 1]
     int qpool_dirty;           // 1: a call failed between the two kernels; the array is cleared before the next use
     // attention scratch (tensor-core path)
     void *k_rot;               // rotated keys, bf16 [rows][Hkv][d]

@@ -37,15 +37,22 @@ template <> struct Elem<__nv_bfloat16> {
 //   q~[g] = (1/n_q) sum_i sum_{h in g} R(p_i) q_ih
 // and, for the tensor-core attention kernel, the rotated bf16 queries with log2(e)/sqrt(d) folded in (q_rot).
 // A few warps share one query token: lane l of a warp reads the 16-byte chunks l, l + 32, ... of the warp's part of the
-// row (all in flight at once); 32 chunks span a multiple of d, so all of a lane's chunks hold the same rotary pairs and
-// the lane needs PER/2 table entries.  The rotated row also goes to a per-token slab in shared memory; after a block
-// barrier the threads add, in a fixed order, the slabs' entries of each pooled element (tokens, then heads), turn the sum
-// into a 64-bit fixed-point number (units of 2^-32) and add it to the global accumulator with an integer atomic:
-// integer addition is associative, so the pooled query does not depend on the order in which blocks arrive.
+// row; 32 chunks span a multiple of d, so all of a lane's chunks hold the same rotary pairs and the lane needs PER/2 table
+// entries.  A block keeps four tokens in work (as far as the row's parts leave it) and walks the tokens with a stride, the
+// next token's row and position requested before the current one is turned; every thread sums its own elements over its
+// tokens in registers.  At the end the sums go to one slab per token slot in shared memory, the threads add, in a fixed
+// order, the slots and then the heads of each pooled element, turn the sum into a 64-bit fixed-point number (units of 2^-32)
+// and add it to the global accumulator with an integer atomic: integer addition is associative, so the pooled query does not
+// depend on the order in which blocks arrive.  The scoring kernel reads the accumulator as it is; nobody waits for a last
+// block to turn it into floats.
+// The kernel is bound by latency: a launch, one round trip for positions and rows, one for table entries, the sums, the
+// atomics.  One block per two tokens (504 at 1,008 queries, each adding all pooled elements) and a last block that converted
+// and cleared the accumulator took, with a scoring kernel of eight tokens behind it, 11.2 us at 1,008 queries of 24 heads
+// (now 7.8), 23.6 at 4,032 (13.2), 9.0 at 135 (6.8), 6.1 at 64 fp32 queries of 4 heads (4.1).  Eight warps a block instead of
+// sixteen 9.0 / 14.6 / 7.8; two or four copies of the accumulator 7.8 to 8.4 at 1,008.
 // ---------------------------------------------------------------------------------------------------------
-constexpr int QPREP_WARPS = 8;                      // warps per block when the parts of a token divide it
+constexpr int QPREP_WARPS = 16;                     // most warps per block, unless one token needs more
 constexpr float FX_ONE = 4294967296.0f;             // 2^32
-constexpr int FX_REPLICAS = PC_FX_REPLICAS;         // copies of the accumulator the blocks of the query pass spread over
 
 template <typename T> __device__ __forceinline__ uint4 pack_row(const float *f);
 template <> __device__ __forceinline__ uint4 pack_row<float>(const float *f) {
@@ -55,104 +62,83 @@ template <> __device__ __forceinline__ uint4 pack_row<__nv_bfloat16>(const float
     return make_uint4(pc_pack_bf16(f[0], f[1]), pc_pack_bf16(f[2], f[3]), pc_pack_bf16(f[4], f[5]), pc_pack_bf16(f[6], f[7]));
 }
 
-// A query row is cut into `parts` runs of CPW x 32 chunks, one warp each (short instruction streams on many warps: the
-// kernel is bound by latency, not by bytes); a block holds `tokens_per_block` tokens.
-template <typename T, int CPW /* chunks per lane of one warp's part of a query row */>
-__global__ void __launch_bounds__(1024) k_qprep(const T *__restrict__ q, const int32_t *__restrict__ q_pos, int n_q,
+// A query row is cut into `parts` runs of CPW x 32 chunks, one warp each; a block holds `slots` tokens at a time.
+template <typename T, int CPW /* chunks per lane of one warp's part of a query row */, int MAX_THREADS>
+__global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, const int32_t *__restrict__ q_pos, int n_q,
                                                 int n_q_heads, int group, int d, int parts, pc_rope_dev rope,
-                                                float out_scale, T *__restrict__ q_rot,
-                                                unsigned long long *fx, double fx_scale, float *__restrict__ pooled,
+                                                float out_scale, T *__restrict__ q_rot, unsigned long long *fx,
                                                 int32_t *status) {
     pc_grid_dep_launch();
     pc_grid_dep_wait();
     constexpr int PER = Elem<T>::PER16, NP = PER / 2;
-    extern __shared__ __align__(16) float slab[];                     // [tokens_per_block][Hq*d]
+    extern __shared__ __align__(16) float slab[];                     // [slots][Hq*d]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tokens_per_block = (blockDim.x >> 5) / parts;
-    const int row_len = n_q_heads * d;
-    const int tok = warp / parts, part = warp - tok * parts;
-    const int i = blockIdx.x * tokens_per_block + tok;
-    if (i < n_q) {
-        const int4 pp = __ldg(reinterpret_cast<const int4 *>(q_pos) + i);
-        const size_t at = (size_t)i * (row_len / PER) + (size_t)part * CPW * 32 + lane;     // in 16-byte chunks
-        const uint4 *src = reinterpret_cast<const uint4 *>(q) + at;
-        uint4 raw[CPW];
+    const int slots = (blockDim.x >> 5) / parts;
+    const int row_len = n_q_heads * d, row_chunks = row_len / PER;
+    const int slot = warp / parts, part = warp - slot * parts;
+    const int chunk0 = part * CPW * 32 + lane, pair0 = ((lane * PER) % d) / 2, stride = gridDim.x * slots;
+    const uint4 *src = reinterpret_cast<const uint4 *>(q) + chunk0;
+    uint4 *dst = q_rot ? reinterpret_cast<uint4 *>(q_rot) + chunk0 : nullptr;
+    int i = blockIdx.x * slots + slot;
+    int4 pp = make_int4(0, 0, 0, 0);
+    uint4 raw[CPW];
+    auto request = [&]() {
+        pp = __ldg(reinterpret_cast<const int4 *>(q_pos) + i);
 #pragma unroll
-        for (int c = 0; c < CPW; ++c) raw[c] = pc_ldg_stream(src + c * 32);
-        const int pair0 = ((lane * PER) % d) / 2;
+        for (int c = 0; c < CPW; ++c) raw[c] = pc_ldg_stream(src + (size_t)i * row_chunks + c * 32);
+    };
+    float acc[CPW][PER];
+#pragma unroll
+    for (int c = 0; c < CPW; ++c)
+#pragma unroll
+        for (int k = 0; k < PER; ++k) acc[c][k] = 0.f;
+    if (i < n_q) request();
+    while (i < n_q) {
+        const int at = i;
         float2 cs[NP];
 #pragma unroll
         for (int u = 0; u < NP; ++u) cs[u] = pc_rope_cs(rope, pair0 + u, pp.x, pp.y, pp.z, status, PC_WHERE_QPOOL_POS);
-        float *mine = slab + (size_t)tok * row_len + ((size_t)part * CPW * 32 + lane) * PER;
-        uint4 *dst = q_rot ? reinterpret_cast<uint4 *>(q_rot) + at : nullptr;
+        uint4 cur[CPW];
+#pragma unroll
+        for (int c = 0; c < CPW; ++c) cur[c] = raw[c];
+        i += stride;
+        if (i < n_q) request();
 #pragma unroll
         for (int c = 0; c < CPW; ++c) {
             float x[PER], r[PER];
-            Elem<T>::unpack(raw[c], x);
+            Elem<T>::unpack(cur[c], x);
 #pragma unroll
             for (int u = 0; u < NP; ++u) {
                 const float2 y = pc_rotate(x[2 * u], x[2 * u + 1], cs[u]);
                 r[2 * u] = y.x;
                 r[2 * u + 1] = y.y;
             }
-            float4 *s4 = reinterpret_cast<float4 *>(mine + (size_t)c * 32 * PER);
 #pragma unroll
-            for (int k = 0; k < PER / 4; ++k) s4[k] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
+            for (int k = 0; k < PER; ++k) acc[c][k] += r[k];
             if (dst) {                                                  // the attention kernel's queries carry its scale
 #pragma unroll
                 for (int k = 0; k < PER; ++k) r[k] = __fmul_rn(r[k], out_scale);
-                dst[c * 32] = pack_row<T>(r);
+                dst[(size_t)at * row_chunks + c * 32] = pack_row<T>(r);
             }
         }
     }
+    float *mine = slab + (size_t)slot * row_len + (size_t)chunk0 * PER;
+#pragma unroll
+    for (int c = 0; c < CPW; ++c) {
+        float4 *s4 = reinterpret_cast<float4 *>(mine + (size_t)c * 32 * PER);
+#pragma unroll
+        for (int k = 0; k < PER / 4; ++k) s4[k] = make_float4(acc[c][4 * k], acc[c][4 * k + 1], acc[c][4 * k + 2], acc[c][4 * k + 3]);
+    }
     __syncthreads();
-    const int n_tokens_used = min(tokens_per_block, n_q - blockIdx.x * tokens_per_block);
     const int n_out = (n_q_heads / group) * d;
-    // blocks spread over FX_REPLICAS copies of the accumulator: fewer atomics queue up on each cache line
-    unsigned long long *mine_fx = fx + (size_t)(blockIdx.x % FX_REPLICAS) * n_out;
-    // four pooled elements per thread at a time, so that four independent sums are in flight; the order of the additions
-    // of each sum is fixed (tokens ascending, heads of the group ascending)
-    for (int e0 = threadIdx.x; e0 < n_out; e0 += 4 * blockDim.x) {
-        const float *s[4];
-        float sum[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int e = min(e0 + k * (int)blockDim.x, n_out - 1), g = e / d, x = e - g * d;
-            s[k] = slab + (size_t)g * group * d + x;
-        }
-        for (int w = 0; w < n_tokens_used; ++w)
-            for (int h = 0; h < group; ++h) {
-                const int off = w * row_len + h * d;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) sum[k] += s[k][off];
-            }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int e = e0 + k * (int)blockDim.x;
-            if (e < n_out) atomicAdd(mine_fx + e, (unsigned long long)__float2ll_rn(sum[k] * FX_ONE));
-        }
-    }
-    // The block that finishes last (a ticket in the word after the last copy; nobody waits for anybody) adds the copies,
-    // writes the pooled query as fp32 and clears the accumulator and the ticket for the next call.  Nothing of this lives
-    // on the host, so a captured graph replays it unchanged.
-    __shared__ int is_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        is_last = atomicAdd(fx + (size_t)FX_REPLICAS * n_out, 1ull) == (unsigned long long)(gridDim.x - 1);
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
     for (int e = threadIdx.x; e < n_out; e += blockDim.x) {
-        long long w = 0;
-#pragma unroll
-        for (int rep = 0; rep < FX_REPLICAS; ++rep) {                     // integer sums: any order gives the same bits
-            w += (long long)__ldcg(fx + (size_t)rep * n_out + e);
-            fx[(size_t)rep * n_out + e] = 0;
-        }
-        pooled[e] = (float)((double)w * fx_scale);
+        const int g = e / d;
+        const float *s = slab + (size_t)g * group * d + (e - g * d);
+        float sum = 0.f;
+        for (int h = 0; h < group; ++h)
+            for (int w = 0; w < slots; ++w) sum += s[w * row_len + h * d];
+        atomicAdd(fx + e, (unsigned long long)__float2ll_rn(sum * FX_ONE));
     }
-    if (threadIdx.x == 0) fx[(size_t)FX_REPLICAS * n_out] = 0;
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -172,7 +158,7 @@ constexpr int SCORE_THREADS = SCORE_WARPS * 32;
 template <typename T, int CPL /* chunks per lane */>
 __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score(const T *__restrict__ k, const int32_t *__restrict__ k_pos,
                                                             const uint8_t *__restrict__ valid, int n_src, int d, float scale,
-                                                            pc_rope_dev rope, const float *__restrict__ pooled,
+                                                            pc_rope_dev rope, unsigned long long *fx, double fx_scale,
                                                             float *__restrict__ scores, int32_t *status) {
     pc_grid_dep_launch();
     constexpr int PER = Elem<T>::PER16, NP = PER / 2;
@@ -198,12 +184,20 @@ __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score(const T *__restrict_
     };
     if (tp < n_pairs) request(tp);
 
+    // the pooled query: the accumulator, scaled
+    constexpr int N_OUT = CPL * 32 * PER;
     for (int idx = threadIdx.x; idx < CPL * NP * 32; idx += SCORE_THREADS) {
         const int l = idx & 31, u = (idx >> 5) % NP, c = idx / (32 * NP);
-        const float2 w = __ldcg(reinterpret_cast<const float2 *>(pooled + (size_t)(c * 32 + l) * PER + 2 * u));
-        qs[idx] = make_float4(w.x, w.y, w.y, -w.x);
+        const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(fx + (size_t)(c * 32 + l) * PER + 2 * u));
+        const float a = (float)((double)w.x * fx_scale), b = (float)((double)w.y * fx_scale);
+        qs[idx] = make_float4(a, b, b, -a);
     }
     __syncthreads();
+    // Every block takes a ticket once it has read the accumulator; whoever finds that all others have read it, too, clears
+    // it for the next call when its tokens are done.  Nobody waits for anybody, and nothing of this lives on the host, so a
+    // captured graph replays it unchanged.
+    unsigned long long ticket = 0;
+    if (threadIdx.x == 0) ticket = atomicAdd(fx + N_OUT, 1ull);
 
     // table slots of this lane's pairs: entry = tbase + coordinate(axis) * stride
     const int pair0 = ((lane * PER) % d) / 2;
@@ -278,6 +272,10 @@ __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score(const T *__restrict_
             }
         }
     }
+    if (warp == 0 && __shfl_sync(0xffffffffu, ticket, 0) == (unsigned long long)(gridDim.x - 1)) {
+        for (int e = lane; e < N_OUT; e += 32) fx[e] = 0;
+        if (lane == 0) fx[N_OUT] = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -298,12 +296,11 @@ __global__ void __launch_bounds__(SEL_THREADS) k_select(const float *__restrict_
 }
 
 // Enqueue the query pass and the scoring kernel on caller-given scratch (a context's, or the library's fixed array).
-// fx: the fixed-point accumulator (PC_FX_REPLICAS copies of Hkv*d sums and one ticket word), all zero on entry and zero
-// again when the query pass has run; pooled: Hkv*d floats, written by the query pass and read by the scoring kernel;
+// fx: the fixed-point accumulator (Hkv*d sums and one ticket word), all zero on entry, filled by the
+// query pass, read by the scoring kernel and zero again when that has run;
 // q_rot / q_scale: where the rotated queries go as well and the factor folded into them.
 template <typename T>
-pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev &rope, long long *fx, float *pooled,
-                        int32_t *status, const void *hist_k, const int32_t *hist_pos, int n_src, const void *q,
+pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev &rope, long long *fx, int32_t *status, const void *hist_k, const int32_t *hist_pos, int n_src, const void *q,
                         const int32_t *q_pos, int32_t n_q, const uint8_t *valid, float *scores, void *q_rot, float q_scale,
                         cudaStream_t stream, pc_ctx *marks) {
     constexpr int PER = Elem<T>::PER16;
@@ -318,25 +315,36 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     const int cpw = qcpl % 3 == 0 ? 3 : (qcpl % 4 == 0 ? 4 : (qcpl % 2 == 0 ? 2 : 1));
     const int parts = qcpl / cpw;
     if (parts > 32) return PC_ERR_UNSUPPORTED;
-    int tokens_per_block = std::max(1, QPREP_WARPS / parts);
-    tokens_per_block = std::max(1, std::min<int>(tokens_per_block, (int)((200u * 1024u) / ((size_t)q_row * sizeof(float)))));
-    const int q_smem = tokens_per_block * q_row * (int)sizeof(float);
-    const int q_blocks = (n_q + tokens_per_block - 1) / tokens_per_block;
+    int slots = std::max(1, QPREP_WARPS / parts);
+    slots = std::max(1, std::min<int>(slots, (int)((200u * 1024u) / ((size_t)q_row * sizeof(float)))));
+    const int q_smem = slots * q_row * (int)sizeof(float);
+    const int q_threads = slots * parts * 32;
     int dev_id = 0;
     PC_CUDA_TRY(cudaGetDevice(&dev_id));
     if (dev_id < 0 || dev_id >= PC_MAX_DEVICES) return PC_ERR_UNSUPPORTED;
     if (marks) pc_mark(marks, PC_MARK_SCORE0, stream);
-#define PC_QPREP_CASE(CPW)                                                                                           \
+#define PC_QPREP_LAUNCH(CPW, MAX_THREADS)                                                                            \
     {                                                                                                               \
-        static int smem_of[PC_MAX_DEVICES] = {};                      /* largest dynamic size allowed so far */      \
+        /* largest dynamic size allowed so far, and resident blocks per SM at the size they were looked up for */   \
+        static int smem_of[PC_MAX_DEVICES] = {}, occ_of[PC_MAX_DEVICES] = {}, occ_at[PC_MAX_DEVICES] = {};          \
         if (q_smem + 1024 > 48 * 1024 && smem_of[dev_id] < q_smem) {   /* the block's static words count, too */    \
-            PC_CUDA_TRY(cudaFuncSetAttribute(k_qprep<T, CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, q_smem)); \
+            PC_CUDA_TRY(cudaFuncSetAttribute(k_qprep<T, CPW, MAX_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, q_smem)); \
             smem_of[dev_id] = q_smem;                                                                               \
         }                                                                                                           \
-        PC_LAUNCH((k_qprep<T, CPW>), dim3(q_blocks), dim3(tokens_per_block * parts * 32), q_smem, stream,           \
+        int occ = occ_at[dev_id] == q_smem + q_threads ? occ_of[dev_id] : 0;                                        \
+        if (occ == 0) {                                                                                             \
+            PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qprep<T, CPW, MAX_THREADS>, q_threads, q_smem)); \
+            occ = std::max(1, occ);                                                                                 \
+            occ_of[dev_id] = occ;                                                                                   \
+            occ_at[dev_id] = q_smem + q_threads;                                                                    \
+        }                                                                                                           \
+        const int q_blocks = std::min((n_q + slots - 1) / slots, sm_count * occ);                                   \
+        PC_LAUNCH((k_qprep<T, CPW, MAX_THREADS>), dim3(q_blocks), dim3(q_threads), q_smem, stream,                  \
                   static_cast<const T *>(q), q_pos, n_q, D.n_q_heads, group, D.head_dim, parts, rope, q_scale,      \
-                  static_cast<T *>(q_rot), reinterpret_cast<unsigned long long *>(fx), fx_scale, pooled, status);   \
+                  static_cast<T *>(q_rot), reinterpret_cast<unsigned long long *>(fx), status);                     \
     }
+#define PC_QPREP_CASE(CPW)                                                                                           \
+    if (q_threads <= 512) PC_QPREP_LAUNCH(CPW, 512) else PC_QPREP_LAUNCH(CPW, 1024)
     switch (cpw) {
     case 3: PC_QPREP_CASE(3) break;        // 24 query heads x 128 bf16: four warps per token
     case 4: PC_QPREP_CASE(4) break;
@@ -344,6 +352,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     default: PC_QPREP_CASE(1) break;
     }
 #undef PC_QPREP_CASE
+#undef PC_QPREP_LAUNCH
     PC_CUDA_TRY(cudaGetLastError());
     if (marks) pc_mark(marks, PC_MARK_QPOOL, stream);
     const float scale = (float)(1.0 / ((double)D.n_q_heads * std::sqrt((double)D.head_dim)));
@@ -360,7 +369,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
         }                                                                                                           \
         const int blocks = std::max(1, std::min((n_pairs + SCORE_WARPS - 1) / SCORE_WARPS, sm_count * per_sm_of[dev_id])); \
         PC_LAUNCH((k_score<T, CPL>), dim3(blocks), dim3(SCORE_THREADS), 0, stream, k, hist_pos, valid, n_src, D.head_dim, scale, rope, \
-                  pooled, scores, status);                                                                          \
+                  reinterpret_cast<unsigned long long *>(fx), fx_scale, scores, status);                             \
     } break;
     switch (chunks / 32) {
         PC_SCORE_CASE(1) PC_SCORE_CASE(2) PC_SCORE_CASE(3) PC_SCORE_CASE(4) PC_SCORE_CASE(6) PC_SCORE_CASE(8)
@@ -418,15 +427,15 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
             if (!pc_score_supports(ctx->desc)) return PC_ERR_UNSUPPORTED;      // before anything is enqueued
             const size_t row = (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim;
             if (ctx->qpool_dirty) {          // an earlier call stopped between the query pass and the scoring kernel
-                PC_CUDA_TRY(cudaMemsetAsync(ctx->qpool_fx, 0, (PC_FX_REPLICAS * row + 1) * sizeof(long long), stream));
+                PC_CUDA_TRY(cudaMemsetAsync(ctx->qpool_fx, 0, (row + 1) * sizeof(long long), stream));
                 ctx->qpool_dirty = 0;
             }
             ctx->qpool_dirty = 1;
             const float q_scale = pc_q_rot_scale(ctx->desc.head_dim);
             st = ctx->desc.dtype == PC_BF16
-                     ? enqueue_score<__nv_bfloat16>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->qpool, ctx->status, src->history.k,
+                     ? enqueue_score<__nv_bfloat16>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->status, src->history.k,
                                                     src->history.pos, n_src, q, q_pos, n_q, valid, scores, q_rot_out, q_scale, stream, ctx)
-                     : enqueue_score<float>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->qpool, ctx->status, src->history.k,
+                     : enqueue_score<float>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->status, src->history.k,
                                             src->history.pos, n_src, q, q_pos, n_q, valid, scores, nullptr, 1.0f, stream, ctx);
             if (st != PC_OK) return st;
             ctx->qpool_dirty = 0;
@@ -459,7 +468,7 @@ extern "C" pc_status pc_score(pc_ctx *ctx, const pc_cache *src, const void *q, c
 // was handed to its own arena at start-up and whose policy forbids driver allocations afterwards, or a
 // latency-critical thread that cannot take the device-wide synchronisation a cudaMalloc / cudaFree implies.  Such
 // callers cannot create a pc_ctx (pc_create allocates), so everything a context would hold for scoring — the rotary
-// table, the fixed-point accumulator of the pooled query and the pooled query itself — lives in one file-scope device array of fixed size
+// table and the fixed-point accumulator of the pooled query — lives in one file-scope device array of fixed size
 // that every GPU loading this library carries until the process exits.
 //
 // In host code the array's name is only a handle; the device address is obtained once per device with
@@ -472,10 +481,9 @@ constexpr int STATIC_MAX_ROPE = 32768;        // rotary table entries: sum over 
 constexpr int STATIC_MAX_QROW = 12288;        // n_q_heads * head_dim: one row of the query pass's shared-memory slab
 constexpr int STATIC_MAX_DEVICES = PC_MAX_DEVICES;
 
-constexpr size_t STATIC_OFF_FX = 256;  /* first 256 bytes unused */       // long long [PC_FX_REPLICAS * STATIC_MAX_ROW + 1 counter word]
-constexpr size_t STATIC_OFF_POOLED = STATIC_OFF_FX + (size_t)PC_FX_REPLICAS * STATIC_MAX_ROW * sizeof(long long) + 256;   // float [STATIC_MAX_ROW]
-constexpr size_t STATIC_OFF_ROPE = STATIC_OFF_POOLED + STATIC_MAX_ROW * sizeof(float);          // float2 [STATIC_MAX_ROPE]
-constexpr size_t STATIC_BYTES = STATIC_OFF_ROPE + (size_t)STATIC_MAX_ROPE * sizeof(float2);    // 332,288 bytes
+constexpr size_t STATIC_OFF_FX = 256;  /* first 256 bytes unused */       // long long [STATIC_MAX_ROW + 1 counter word]
+constexpr size_t STATIC_OFF_ROPE = STATIC_OFF_FX + (size_t)STATIC_MAX_ROW * sizeof(long long) + 256;   // float2 [STATIC_MAX_ROPE]
+constexpr size_t STATIC_BYTES = STATIC_OFF_ROPE + (size_t)STATIC_MAX_ROPE * sizeof(float2);    // 270,848 bytes
 
 static __device__ __align__(256) unsigned char g_static_scratch[STATIC_BYTES];
 
@@ -518,7 +526,6 @@ pc_status launch_score_static(const pc_layer_desc &D, unsigned char *base, const
                               int32_t n_src, const void *q, const int32_t *q_pos, int32_t n_q, const uint8_t *valid,
                               float *scores, int32_t *status, cudaStream_t stream) {
     long long *fx = reinterpret_cast<long long *>(base + STATIC_OFF_FX);
-    float *pooled = reinterpret_cast<float *>(base + STATIC_OFF_POOLED);
     float2 *tab = reinterpret_cast<float2 *>(base + STATIC_OFF_ROPE);
 
     pc_rope_dev rope;
@@ -533,7 +540,7 @@ pc_status launch_score_static(const pc_layer_desc &D, unsigned char *base, const
     // the array keeps whatever the last call left: the table is rewritten before it is read, and the accumulator of the
     // pooled query, which must start at zero, is cleared by the same kernel
     const int row = D.n_kv_heads * D.head_dim;
-    const int fx_words = PC_FX_REPLICAS * row + 1;
+    const int fx_words = row + 1;
     PC_LAUNCH(k_rope_table, dim3((std::max(total, fx_words) + 255) / 256), dim3(256), 0, stream, tab, rope, D.rope_base, total, fx,
               fx_words);
     PC_CUDA_TRY(cudaGetLastError());
@@ -541,7 +548,7 @@ pc_status launch_score_static(const pc_layer_desc &D, unsigned char *base, const
     int sm_count = 0, dev = 0;
     PC_CUDA_TRY(cudaGetDevice(&dev));
     PC_CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
-    return enqueue_score<T>(D, sm_count, rope, fx, pooled, status, hist_k, hist_pos, n_src, q, q_pos, n_q, valid, scores, nullptr,
+    return enqueue_score<T>(D, sm_count, rope, fx, status, hist_k, hist_pos, n_src, q, q_pos, n_q, valid, scores, nullptr,
                             1.0f, stream, nullptr);
 }
 
