@@ -32,25 +32,56 @@ bool tensor_core_path(const pc_ctx *ctx) {
     return ctx->attend_impl != 1 && pc_tensor_core_shape(ctx);
 }
 
+// Tensor-core attention of all n_q rows, the output in parts if somebody waits for them.  `what` holds what is still to be rotated.
+pc_status attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos, int32_t n_q, void *out,
+                    float *lse, cudaStream_t stream, int what, const pc_step_hooks *hooks) {
+    const int part = hooks ? pc_attend_part_rows(ctx, n_q) : n_q;
+    if (part >= n_q) {
+        const pc_status st = pc_launch_attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, what);
+        return st == PC_OK && hooks ? hooks->part_done(hooks->self, 0, n_q, stream) : st;
+    }
+    pc_status st = pc_launch_attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, what & ~PC_TC_ATTEND);
+    const size_t row_bytes = (size_t)ctx->desc.n_q_heads * ctx->desc.head_dim * ctx->elem_size;
+    for (int r = 0; r < n_q && st == PC_OK; r += part) {
+        const int n = part < n_q - r ? part : n_q - r;
+        st = pc_launch_attend_tc(ctx, n_seg, segs, nullptr, nullptr, n, static_cast<char *>(out) + r * row_bytes,
+                                 lse ? lse + (size_t)r * ctx->desc.n_q_heads : nullptr, stream, PC_TC_ATTEND, r);
+        if (st == PC_OK) st = hooks->part_done(hooks->self, r, n, stream);
+    }
+    if (st == PC_OK) ctx->last_n_q = n_q;
+    return st;
+}
+
+pc_status attend_simt(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos, int32_t n_q, void *out,
+                      float *lse, cudaStream_t stream, const pc_step_hooks *hooks) {
+    const pc_status st = pc_launch_attend_simt(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream);
+    return st == PC_OK && hooks ? hooks->part_done(hooks->self, 0, n_q, stream) : st;
+}
+
 }  // namespace
 
-extern "C" pc_status pc_attend_frame(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q,
-                                     const int32_t *q_pos, int32_t n_q, void *out, float *lse, void *stream_) {
+pc_status pc_attend_frame_impl(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
+                               int32_t n_q, void *out, float *lse, cudaStream_t stream, const pc_step_hooks *hooks) {
     if (!ctx || !cache) return PC_ERR_INVALID_ARG;
     pc_status st = check_queries(ctx, q, q_pos, n_q, out, lse);
     if (st != PC_OK) return st;
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     pc_segment segs[PC_MAX_SEGMENTS];
     int n_seg = 0;
     st = gather_segments(ctx, cache, current, segs, &n_seg);
     if (st != PC_OK) return st;
+    if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
     ctx->last_n_q = 0;
     if (tensor_core_path(ctx)) {
         ctx->prepared_n_seg = 0;                       // the rotated-key scratch is about to be overwritten
         ctx->anchor_rot_n = 0;
-        return pc_launch_attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, PC_TC_ALL);
+        return attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, PC_TC_ALL, hooks);
     }
-    return pc_launch_attend_simt(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream);
+    return attend_simt(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, hooks);
+}
+
+extern "C" pc_status pc_attend_frame(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q,
+                                     const int32_t *q_pos, int32_t n_q, void *out, float *lse, void *stream) {
+    return pc_attend_frame_impl(ctx, cache, current, q, q_pos, n_q, out, lse, static_cast<cudaStream_t>(stream), nullptr);
 }
 
 extern "C" pc_status pc_attend_prepare(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, void *stream_) {
@@ -90,14 +121,13 @@ extern "C" pc_status pc_attend_prepared(pc_ctx *ctx, const void *q, const int32_
 // tensor-core path the intermediate passes of the separate calls disappear: the query pass that pools for the scores also
 // leaves the rotated queries, the pack kernel also leaves the rotated keys of what it packs, and the anchors' rotated
 // keys stay in the scratch from the first step that saw them, so attention starts without a rotary pre-pass.
-extern "C" pc_status pc_frame_step(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, int32_t delta_t, pc_cache *dst,
-                                   const void *q, const int32_t *q_pos, int32_t n_q, float *scores, int32_t *sel_idx, void *out,
-                                   float *lse, void *stream_) {
+pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, int32_t delta_t, pc_cache *dst, const void *q,
+                             const int32_t *q_pos, int32_t n_q, float *scores, int32_t *sel_idx, void *out, float *lse,
+                             cudaStream_t stream, const pc_step_hooks *hooks) {
     if (!ctx || !src || !dst || !budget) return PC_ERR_INVALID_ARG;
     pc_status st = check_queries(ctx, q, q_pos, n_q, out, lse);
     if (st != PC_OK) return st;
     if (src->n_frames < 0 || (src->n_frames > 0 && !src->frame_count)) return PC_ERR_INVALID_ARG;
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     int64_t n_sel = 0;
     for (int f = 0; f < src->n_frames; ++f) {
         if (budget[f] < 0) return PC_ERR_INVALID_ARG;
@@ -127,6 +157,7 @@ extern "C" pc_status pc_frame_step(pc_ctx *ctx, const pc_cache *src, const int32
     ctx->q_rot_n = 0;
     st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream);
     if (st != PC_OK) return st;
+    if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
     st = pc_compact_impl(ctx, src, sel_idx, budget, delta_t, dst, k_rot_dst, stream);
     if (st != PC_OK) return st;
     dst->history.n_tokens = (int32_t)n_sel;
@@ -136,14 +167,14 @@ extern "C" pc_status pc_frame_step(pc_ctx *ctx, const pc_cache *src, const int32
     int n_seg = 0;
     if (n_anchor > 0) segs[n_seg++] = src->anchors;
     if (n_sel > 0) segs[n_seg++] = dst->history;
-    if (!tc) return pc_launch_attend_simt(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream);
+    if (!tc) return attend_simt(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, hooks);
     int what = PC_TC_ATTEND;
     if (ctx->q_rot_n != n_q) what |= PC_TC_ROPE_Q;    // nothing was scored, so no query pass ran: rotate the queries now
     const bool anchors_cached = n_anchor > 0 && ctx->anchor_rot_n == n_anchor && ctx->anchor_rot_k == src->anchors.k &&
                                 ctx->anchor_rot_pos == src->anchors.pos;
     if (n_anchor > 0 && !anchors_cached) what |= PC_TC_ROPE_K0;
     ctx->anchor_rot_n = 0;
-    st = pc_launch_attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, what);
+    st = attend_tc(ctx, n_seg, segs, q, q_pos, n_q, out, lse, stream, what, hooks);
     if (st != PC_OK) return st;
     if (n_anchor > 0) {
         ctx->anchor_rot_k = src->anchors.k;
@@ -151,4 +182,11 @@ extern "C" pc_status pc_frame_step(pc_ctx *ctx, const pc_cache *src, const int32
         ctx->anchor_rot_n = n_anchor;
     }
     return PC_OK;
+}
+
+extern "C" pc_status pc_frame_step(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, int32_t delta_t, pc_cache *dst,
+                                   const void *q, const int32_t *q_pos, int32_t n_q, float *scores, int32_t *sel_idx, void *out,
+                                   float *lse, void *stream) {
+    return pc_frame_step_impl(ctx, src, budget, delta_t, dst, q, q_pos, n_q, scores, sel_idx, out, lse, static_cast<cudaStream_t>(stream),
+                              nullptr);
 }

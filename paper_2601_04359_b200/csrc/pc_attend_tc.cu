@@ -681,10 +681,20 @@ pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_r
     return PC_OK;
 }
 
+// A part has enough row tiles for a CTA on (nearly) every SM: an item is cut into at most MAX_SPLITS parts, so fewer items
+// would leave SMs idle.  At most four parts: each costs a launch, a prologue and an epilogue of its own.
+int pc_attend_part_rows(const pc_ctx *ctx, int n_q) {
+    const int tiles = div_up(n_q, TILE);
+    int least = 1;
+    while (least < tiles && ctx->desc.n_kv_heads * div_up(ctx->group * least, 2) * (MAX_SPLITS - 1) < ctx->sm_count - ctx->sm_count / 32) ++least;
+    const int parts = std::max(1, std::min(4, tiles / least));
+    return div_up(tiles, parts) * TILE;
+}
+
 // what: PC_TC_ROPE_K rotates the segments' keys into the context scratch, PC_TC_ROPE_Q rotates the queries,
 // PC_TC_ATTEND runs attention (and the merge) on the rotated data.
 pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos,
-                              int32_t n_q, void *out, float *lse, cudaStream_t stream, int what) {
+                              int32_t n_q, void *out, float *lse, cudaStream_t stream, int what, int q_row0) {
     const pc_layer_desc &D = ctx->desc;
     if (D.head_dim != TILE || D.dtype != PC_BF16) return PC_ERR_UNSUPPORTED;
     const int row_elems = D.n_kv_heads * D.head_dim;
@@ -767,7 +777,7 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     if (P.part_stride > 1 && !P.cluster && (size_t)n_items * P.part_stride * 2 * TILE * TILE > ctx->part_o_floats) return PC_ERR_CAPACITY;
 
     CUtensorMap mq, mk, mv[PC_MAX_SEGMENTS];
-    bool ok = make_map(&mq, q_rot, (uint64_t)n_q, (uint64_t)D.n_q_heads * D.head_dim) &&
+    bool ok = make_map(&mq, q_rot + (size_t)q_row0 * D.n_q_heads * D.head_dim, (uint64_t)n_q, (uint64_t)D.n_q_heads * D.head_dim) &&
               make_map(&mk, k_rot, (uint64_t)tiles * TILE, (uint64_t)row_elems);
     for (int s = 0; s < PC_MAX_SEGMENTS; ++s) {
         const pc_segment &sg = segs[s < n_seg ? s : 0];

@@ -271,7 +271,22 @@ pc_status pc_launch_attend_simt(pc_ctx *ctx, int n_seg, const pc_segment *segs, 
                                 int32_t n_q, void *out, float *lse, cudaStream_t stream);
 // PC_TC_ROPE_K0: rotate the keys of the first segment only (the anchors of a fused frame step)
 enum { PC_TC_ROPE_K = 1, PC_TC_ROPE_Q = 2, PC_TC_ATTEND = 4, PC_TC_ALL = 7, PC_TC_ROPE_K0 = 8 };
+// q_row0: first row of the rotated-query scratch that PC_TC_ATTEND reads (q, out and lse are the caller's, already offset)
 pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos,
-                              int32_t n_q, void *out, float *lse, cudaStream_t stream, int what);
+                              int32_t n_q, void *out, float *lse, cudaStream_t stream, int what, int q_row0 = 0);
+// query rows of one part of a frame's attention when its output is to leave in parts: enough row tiles per part to fill the GPU
+int pc_attend_part_rows(const pc_ctx *ctx, int n_q);
+// What a frame step driven from host memory adds to pc_frame_step / pc_attend_frame: an event the stream waits for before V or
+// the packed positions are first read, and a call after each part of the output has been enqueued (rows [row0, row0 + n)).
+struct pc_step_hooks {
+    cudaEvent_t kv_ready;
+    pc_status (*part_done)(void *self, int row0, int n, cudaStream_t stream);
+    void *self;
+};
+pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, int32_t delta_t, pc_cache *dst, const void *q,
+                             const int32_t *q_pos, int32_t n_q, float *scores, int32_t *sel_idx, void *out, float *lse,
+                             cudaStream_t stream, const pc_step_hooks *hooks);
+pc_status pc_attend_frame_impl(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
+                               int32_t n_q, void *out, float *lse, cudaStream_t stream, const pc_step_hooks *hooks);
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
                                size_t *part_ml_floats);
