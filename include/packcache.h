@@ -333,7 +333,7 @@ pc_status pc_window_step(pc_window *w, const void *q, const int32_t *q_pos, int3
  * bounded): copies the frame that was just finished (its K, V, positions; n_frame may be 0) to the end of the active
  * history buffer and the new frame's queries and positions into the workspace, runs pc_window_step, copies the
  * output back and waits for the stream.  The frame's values and the output travel on a stream of the window's own, beside
- * the kernels; from 1,024 query rows or so (as many as fill the GPU twice) attention runs in parts of the rows so that the
+ * the kernels; from 512 query rows or so (as many as fill the GPU twice) attention runs in parts of the rows so that the
  * output leaves part by part, and then agrees with pc_window_step up to fp32 rounding order (fewer rows: bit for bit).
  * Pinned host memory keeps the copies asynchronous.  All arguments are checked
  * before anything is enqueued.  Errors: as pc_window_append and pc_window_step. */

@@ -30,7 +30,8 @@ using namespace pc_tc;
 
 constexpr int TC_THREADS = 384;
 constexpr int KV_STAGES = 2;
-constexpr int MAX_SPLITS = 4;
+constexpr int MAX_SPLITS = 8;             // most parts of an item
+constexpr int MAX_FIXED_SPLITS = 4;       // most key ranges a caller can fix, and most of the cluster merge
 constexpr float RESCALE_THRESHOLD = 8.0f;
 
 // shared memory map (dynamic, 1024-byte aligned)
@@ -572,8 +573,8 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 
 // ------------------------------------------------------------------------------------------------ combine
 // Merge of the KV ranges' partials.  One block per (query tile of one head, 32-row quadrant); its eight warps take four
-// 16-byte column units each, lanes are consecutive rows, so every load of the partial tiles is a 512-byte run.  Every
-// load of a thread is issued before any is used.
+// 16-byte column units each, lanes are consecutive rows, so every load of the partial tiles is a 512-byte run.  Up to four
+// parts' loads of a thread are issued before any is used.
 __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
     pc_grid_dep_launch();
     pc_grid_dep_wait();
@@ -588,16 +589,22 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
     item_parts(P, item, 0, part0, n_parts);
     if (n_parts < 2) return;                      // the one CTA that had the whole item wrote its output itself
     float2 ml[MAX_SPLITS];
-    float4 o[MAX_SPLITS][4];
+    float4 o[4][4];
+    const float2 *pml = reinterpret_cast<const float2 *>(P.part_ml);
+    const float4 *po = reinterpret_cast<const float4 *>(P.part_o);
+    auto load4 = [&](int s0) {                     // the O units of parts s0 .. s0 + 3
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+            if (s0 + s < n_parts) {
+                const float4 *pt = po + (((size_t)item * P.part_stride + s0 + s) * 2 + t) * (TILE * TILE / 4) + r;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) o[s][u] = __ldcg(pt + (cg * 4 + u) * TILE);
+            }
+    };
 #pragma unroll
     for (int s = 0; s < MAX_SPLITS; ++s)
-        if (s < n_parts) {
-            const size_t tile_slot = ((size_t)item * P.part_stride + s) * 2 + t;
-            ml[s] = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + tile_slot * TILE + r);
-            const float4 *pt = reinterpret_cast<const float4 *>(P.part_o) + tile_slot * (TILE * TILE / 4) + r;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) o[s][u] = __ldcg(pt + (cg * 4 + u) * TILE);
-        }
+        if (s < n_parts) ml[s] = __ldcg(pml + (((size_t)item * P.part_stride + s) * 2 + t) * TILE + r);
+    load4(0);
     float m = -INFINITY;
 #pragma unroll
     for (int s = 0; s < MAX_SPLITS; ++s)
@@ -607,16 +614,18 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int s = 0; s < MAX_SPLITS; ++s)
+    for (int s = 0; s < MAX_SPLITS; ++s) {
+        if (s == 4 && n_parts > 4) load4(4);
         if (s < n_parts) {
             const float sc = exp2f(ml[s].x - m);
             l = fmaf(ml[s].y, sc, l);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                acc[u].x = fmaf(o[s][u].x, sc, acc[u].x); acc[u].y = fmaf(o[s][u].y, sc, acc[u].y);
-                acc[u].z = fmaf(o[s][u].z, sc, acc[u].z); acc[u].w = fmaf(o[s][u].w, sc, acc[u].w);
+                acc[u].x = fmaf(o[s & 3][u].x, sc, acc[u].x); acc[u].y = fmaf(o[s & 3][u].y, sc, acc[u].y);
+                acc[u].z = fmaf(o[s & 3][u].z, sc, acc[u].z); acc[u].w = fmaf(o[s & 3][u].w, sc, acc[u].w);
             }
         }
+    }
     const float inv = 1.f / l;
     // this thread's 16 columns of its row: 32 contiguous bytes
     uint4 w0, w1;
@@ -633,11 +642,11 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
 // ------------------------------------------------------------------------------------------------ host side
 int div_up(int a, int b) { return (a + b - 1) / b; }
 
-// number of KV ranges: fewest waves of CTAs, a fixed cost per CTA standing in for prologue and epilogue
+// number of KV ranges of the cluster merge: fewest waves of CTAs, a fixed cost per CTA standing in for prologue and epilogue
 int choose_splits(int n_items, int n_kv_tiles, int sm_count) {
     int best = 1;
     long best_cost = -1;
-    for (int s = 1; s <= MAX_SPLITS && s <= n_kv_tiles; ++s) {
+    for (int s = 1; s <= MAX_FIXED_SPLITS && s <= n_kv_tiles; ++s) {
         const long waves = div_up(n_items * s, sm_count);
         const long cost = waves * (div_up(n_kv_tiles, s) + 3) + (s > 1 ? 2 : 0);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
@@ -667,17 +676,60 @@ int choose_ctas(int n_items, long long steps, int most) {
     return best;
 }
 
+// Divides the line of (item, key tile) steps over CTAs: fills P.persistent, n_cta, n_splits, part_stride.
+//
+// What a division costs, in quarters of a step (a step is about 1.6 us): its longest run, 14 for a CTA that crosses from one
+// item into the next (the unit boundary), 7 for a merge.  The persistent form takes an even share of the line per CTA; the
+// split form cuts every item into s equal ranges, one CTA each, as long as all are resident at once: no boundary, and with one
+// range no merge.  Measured on rotated keys (query rotation + attention + merge), the persistent form against the one chosen
+// here: 8 / 8 heads, 144 queries x 2,000 keys 22.3 -> 15.9 us, 700 x 3,000 29.8 -> 21.6; 24 / 8 heads,
+// 135 x 472 17.7 -> 14.8, 135 x 1,500 21.0 -> 17.9, 400 x 4,000 36.5 -> 33.7, 700 x 3,000 43.8 -> 39.0; 32 / 16 heads, 500 x
+// 2,000 36.3 -> 31.1.  (Three ranges at most before; merging the ranges of an item in a cluster instead was slower throughout:
+// 20.2 to 22.0 us at 135 x 472.)
+void choose_division(const pc_ctx *ctx, int n_items, int tiles, TcParams &P) {
+    const long long T = (long long)n_items * tiles;
+    P.persistent = 0;
+    if (ctx->kv_splits > 0 || ctx->cluster_merge) {
+        P.n_splits = ctx->kv_splits > 0 ? std::min(ctx->kv_splits, tiles) : choose_splits(n_items, tiles, ctx->sm_count);
+    } else {
+        const int n = choose_ctas(n_items, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
+        int most = 1;
+        for (int i = 0; i < n_items / std::gcd(n, n_items); ++i) {      // the kernel's own rule (cta_of_step); the cuts repeat
+            const long long x0 = (long long)i * tiles, x1 = x0 + tiles - 1;
+            const int first = (int)(((x0 + 1) * n + T - 1) / T) - 1, last = (int)(((x1 + 1) * n + T - 1) / T) - 1;
+            most = std::max(most, last - first + 1);
+        }
+        long long best = 4 * ((T + n - 1) / n) + (n % n_items ? 14 : 0) + (most > 1 ? 7 : 0);
+        P.persistent = 1;
+        P.n_cta = n;
+        P.n_splits = P.part_stride = most;
+        for (int s = 1; s <= MAX_SPLITS && s <= tiles && n_items * s <= ctx->sm_count; ++s) {
+            const long long cost = 4 * div_up(tiles, s) + (s > 1 ? 7 : 0);
+            if (cost < best) {
+                best = cost;
+                P.persistent = 0;
+                P.n_splits = s;
+            }
+        }
+        if (P.persistent) return;
+    }
+    P.n_cta = n_items * P.n_splits;
+    P.part_stride = P.n_splits;
+}
+
 }  // namespace
 
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
                                size_t *part_ml_floats) {
-    (void)sm_count;
     // every segment starts on a tile boundary; the query rows follow the keys in the same scratch
     *k_rot_rows = (size_t)(div_up(d->max_keys, TILE) + PC_MAX_SEGMENTS) * TILE;
     const int group = d->n_q_heads / d->n_kv_heads;
     const int n_items = d->n_kv_heads * div_up(group * div_up(d->max_q, TILE), 2);
-    *part_o_floats = (size_t)n_items * MAX_SPLITS * 2 * TILE * TILE;
-    *part_ml_floats = (size_t)n_items * MAX_SPLITS * 2 * TILE * 2;
+    // slots: a fixed number of ranges per item, or the parts of the persistent form (every CTA and every item boundary makes
+    // one at most, and an item has room for its longest row of them)
+    const size_t slots = std::max((size_t)n_items * MAX_FIXED_SPLITS, (size_t)sm_count + 2 * (size_t)n_items);
+    *part_o_floats = slots * 2 * TILE * TILE;
+    *part_ml_floats = slots * 2 * TILE * 2;
     return PC_OK;
 }
 
@@ -752,27 +804,7 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     P.status = ctx->status;
     P.wait_us = ctx->wait_limit_us;
     P.extra_tx = ctx->test_extra_tx;
-    // Persistent form unless the caller fixed the number of key ranges or asked for the cluster merge: one CTA per SM or a few less, but
-    // never so many that an item is cut into more than MAX_SPLITS parts (a CTA's run is at least a third of an item).
-    const long long T = (long long)n_items * tiles;
-    P.persistent = (ctx->kv_splits == 0 && !ctx->cluster_merge) ? 1 : 0;
-    if (P.persistent) {
-        P.n_cta = choose_ctas(n_items, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
-        int most = 1;
-        for (int i = 0; i < n_items; ++i) {        // the kernel's own rule (cta_of_step), evaluated for every item
-            const long long x0 = (long long)i * tiles, x1 = x0 + tiles - 1;
-            const int first = (int)(((x0 + 1) * P.n_cta + T - 1) / T) - 1, last = (int)(((x1 + 1) * P.n_cta + T - 1) / T) - 1;
-            most = std::max(most, last - first + 1);
-        }
-        if (most > MAX_SPLITS) P.persistent = 0;
-        P.part_stride = most;
-        P.n_splits = most;
-    }
-    if (!P.persistent) {
-        P.n_splits = ctx->kv_splits > 0 ? std::min(ctx->kv_splits, tiles) : choose_splits(n_items, tiles, ctx->sm_count);
-        P.n_cta = n_items * P.n_splits;
-        P.part_stride = P.n_splits;
-    }
+    choose_division(ctx, n_items, tiles, P);
     P.cluster = (!P.persistent && P.n_splits > 1 && ctx->cluster_merge) ? 1 : 0;
     if (P.part_stride > 1 && !P.cluster && (size_t)n_items * P.part_stride * 2 * TILE * TILE > ctx->part_o_floats) return PC_ERR_CAPACITY;
 

@@ -19,7 +19,7 @@ from .test_gpu_parity import bf16_ulp
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("grid", [(7, 9), (20, 26), (24, 42), (33, 40), (40, 64)])
+@pytest.mark.parametrize("grid", [(7, 9), (16, 16), (20, 26), (24, 42), (33, 40), (40, 64)])
 def test_host_step_in_parts(grid):
     cfg = wl.small_bf16(n_frames=3, grid=grid, n_text=37, total=int(1.3 * grid[0] * grid[1]), kind=wl.LINEAR, param=0.0, keep_full=0, seed=7)
     n, W, total = cfg.frame_tokens, 2, cfg.budget.total
@@ -46,7 +46,7 @@ def test_host_step_in_parts(grid):
         assert m == b.n_tokens and all(torch.equal(x[:m], y[:m]) for x, y in ((a.k, b.k), (a.v, b.v), (a.pos, b.pos)))
         got, want = out_host.float().numpy(), out.float().cpu().numpy()
         assert (np.abs(got - want) <= bf16_ulp(want) + 2e-3).all()
-        if n <= 520:                                       # one part
+        if n <= 256:                                       # one part
             assert torch.equal(out_host, out.cpu())
     for w in wins:
         w.close()
