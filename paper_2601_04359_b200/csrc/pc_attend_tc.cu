@@ -31,6 +31,7 @@ using namespace pc_tc;
 constexpr int TC_THREADS = 384;
 constexpr int KV_STAGES = 2;
 constexpr int MAX_SPLITS = 8;             // most parts of an item
+constexpr int BOUNDARY_STEPS = 2;         // what a CTA's crossing into the next item costs, in steps
 constexpr int MAX_FIXED_SPLITS = 4;       // most key ranges a caller can fix, and most of the cluster merge
 constexpr float RESCALE_THRESHOLD = 8.0f;
 
@@ -51,6 +52,7 @@ struct TcParams {
     int n_items;      // (KV head, pair of query tiles)
     int persistent;   // 1: n_cta CTAs share the line of (item, key tile) steps evenly; 0: CTA (item, s) takes one of n_splits ranges
     int n_cta;
+    int gap;          // steps an item boundary is reckoned as when the line is shared out (persistent form)
     int part_stride;  // partial slots reserved per item (most parts any item has)
     int n_seg;
     int cluster;      // 1: the KV ranges of one item form a thread-block cluster and merge through shared memory
@@ -156,27 +158,36 @@ __device__ __forceinline__ void kv_tile_info(const TcParams &P, int jt, int &seg
 // queries and first keys arrive under the current item's last steps, and all SMs finish together.  Split form: CTA
 // (item, s) takes the s-th of n_splits equal ranges of one item (used when the caller fixes the number of key ranges, and
 // by the cluster merge).  The part of an item one CTA works on is a "unit"; an item's units are numbered by "part".
+//
+// A CTA that crosses from one item into the next spends the time of two to three steps on the boundary (the last PV drains, O
+// is read out, the tensor core waits for the next item's first probabilities).  So the line is shared out with `gap` further
+// places behind every item, on which no step lies.
+__host__ __device__ __forceinline__ long long line_length(const TcParams &P) { return (long long)P.n_items * (P.n_kv_tiles + P.gap); }
+__device__ __forceinline__ long long line_cut(const TcParams &P, int c) {        // first step of CTA c (persistent form)
+    const int pitch = P.n_kv_tiles + P.gap;
+    const long long v = line_length(P) * c / P.n_cta, item = v / pitch;
+    return item * P.n_kv_tiles + min((int)(v - item * pitch), P.n_kv_tiles);
+}
 __device__ __forceinline__ void cta_run(const TcParams &P, int c, long long &g0, long long &g1) {
     if (P.persistent) {
-        const long long T = (long long)P.n_items * P.n_kv_tiles;
-        g0 = T * c / P.n_cta;
-        g1 = T * (c + 1) / P.n_cta;
+        g0 = line_cut(P, c);
+        g1 = line_cut(P, c + 1);
     } else {
         const int item = c / P.n_splits, s = c % P.n_splits;
         g0 = (long long)item * P.n_kv_tiles + (long long)P.n_kv_tiles * s / P.n_splits;
         g1 = (long long)item * P.n_kv_tiles + (long long)P.n_kv_tiles * (s + 1) / P.n_splits;
     }
 }
-// persistent form: the CTA whose run holds step x
-__device__ __forceinline__ int cta_of_step(const TcParams &P, long long x) {
-    const long long T = (long long)P.n_items * P.n_kv_tiles;
-    return (int)(((x + 1) * P.n_cta + T - 1) / T) - 1;
+// persistent form: the CTA whose run holds key tile j of an item
+__host__ __device__ __forceinline__ int cta_of_step(const TcParams &P, int item, int j) {
+    const long long L = line_length(P), v = (long long)item * (P.n_kv_tiles + P.gap) + j;
+    return (int)(((v + 1) * P.n_cta + L - 1) / L) - 1;
 }
 // number of parts of an item, and the part the unit of CTA c is
 __device__ __forceinline__ void item_parts(const TcParams &P, int item, int c, int &part, int &parts) {
     if (P.persistent) {
-        const int first = cta_of_step(P, (long long)item * P.n_kv_tiles);
-        const int last = cta_of_step(P, (long long)item * P.n_kv_tiles + P.n_kv_tiles - 1);
+        const int first = cta_of_step(P, item, 0);
+        const int last = cta_of_step(P, item, P.n_kv_tiles - 1);
         part = c - first;
         parts = last - first + 1;
     } else {
@@ -678,8 +689,8 @@ int choose_ctas(int n_items, long long steps, int most) {
 
 // Divides the line of (item, key tile) steps over CTAs: fills P.persistent, n_cta, n_splits, part_stride.
 //
-// What a division costs, in quarters of a step (a step is about 1.6 us): its longest run, 14 for a CTA that crosses from one
-// item into the next (the unit boundary), 7 for a merge.  The persistent form takes an even share of the line per CTA; the
+// What a division costs, in quarters of a step (a step is about 1.6 us): its longest run (boundaries reckoned in, or 14 for
+// them where runs are too short or too long for that), 7 for a merge.  The persistent form takes an even share of the line per CTA; the
 // split form cuts every item into s equal ranges, one CTA each, as long as all are resident at once: no boundary, and with one
 // range no merge.  Measured on rotated keys (query rotation + attention + merge), the persistent form against the one chosen
 // here: 8 / 8 heads, 144 queries x 2,000 keys 22.3 -> 15.9 us, 700 x 3,000 29.8 -> 21.6; 24 / 8 heads,
@@ -693,15 +704,18 @@ void choose_division(const pc_ctx *ctx, int n_items, int tiles, TcParams &P) {
         P.n_splits = ctx->kv_splits > 0 ? std::min(ctx->kv_splits, tiles) : choose_splits(n_items, tiles, ctx->sm_count);
     } else {
         const int n = choose_ctas(n_items, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
-        int most = 1;
-        for (int i = 0; i < n_items / std::gcd(n, n_items); ++i) {      // the kernel's own rule (cta_of_step); the cuts repeat
-            const long long x0 = (long long)i * tiles, x1 = x0 + tiles - 1;
-            const int first = (int)(((x0 + 1) * n + T - 1) / T) - 1, last = (int)(((x1 + 1) * n + T - 1) / T) - 1;
-            most = std::max(most, last - first + 1);
-        }
-        long long best = 4 * ((T + n - 1) / n) + (n % n_items ? 14 : 0) + (most > 1 ? 7 : 0);
-        P.persistent = 1;
+        const bool crossing = n % n_items != 0;
         P.n_cta = n;
+        // Shorter runs than six times the boundary could end up empty; in longer ones than 64 steps it does not show any more.
+        // Boundaries reckoned in against an even share of the steps: the step at 12 frames (runs of 22) 89.7 -> 88.4 us,
+        // passes over 7,184 keys (38) 517.1 -> 514.7, 47 frames (48) 167.9 -> 167.5; in runs of 259 and 267 steps 620.4 -> 624.7
+        // (47 whole frames) and 649.8 -> 655.6 (4,032-token frames).
+        P.gap = crossing && T >= 6LL * BOUNDARY_STEPS * n && T <= 64LL * n ? BOUNDARY_STEPS : 0;
+        int most = 1;
+        for (int i = 0; i < n_items / std::gcd(n, n_items); ++i)        // the cuts repeat
+            most = std::max(most, cta_of_step(P, i, tiles - 1) - cta_of_step(P, i, 0) + 1);
+        long long best = 4 * ((line_length(P) + n - 1) / n) + (crossing && P.gap == 0 ? 14 : 0) + (most > 1 ? 7 : 0);
+        P.persistent = 1;
         P.n_splits = P.part_stride = most;
         for (int s = 1; s <= MAX_SPLITS && s <= tiles && n_items * s <= ctx->sm_count; ++s) {
             const long long cost = 4 * div_up(tiles, s) + (s > 1 ? 7 : 0);
