@@ -34,6 +34,7 @@ enum {
 };
 
 constexpr int PC_MAX_SEGMENTS = 3;
+constexpr int PC_MASS_PARTS = 4;              // pieces the attention mass of a pair of key tiles may come in
 constexpr int PC_MAX_DEVICES = 64;            // per-device launch state is kept in arrays of this size
 
 // Rotary tables: for axis a (t, h, w) a [max_pos[a]][n_axis[a]] array of (cos, sin) of pos * base^(-m/n_axis[a]).
@@ -81,7 +82,7 @@ struct pc_ctx {
     // (read by pc_attend_mass); last_n_q = 0 when there is none
     int last_n_q, last_n_seg;
     int last_seg_n[PC_MAX_SEGMENTS];
-    float *mass_part;          // attention mass: partial sums per KV head and column half, [Hkv][2][k_rot_rows]
+    float *mass_part;          // attention mass: partial sums per piece, KV head and column half, [PC_MASS_PARTS][Hkv][2][k_rot_rows]
     float *mass_norm;          // attention mass: negated base-2 normalisers, [Hq][max_q rounded up to 128]
     // optional per-kernel timing (benchmarks): events at the boundaries of the kernels of each call
     int timing_on;

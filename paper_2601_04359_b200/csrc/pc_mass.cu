@@ -8,9 +8,14 @@
 //
 //   k_mass_norm    writes minus the base-2 normaliser of every query row, transposed to [head][row] and padded with
 //                  -inf to whole tiles, so that one step's 128 values are one contiguous 512-byte run.
-//   k_mass_tc      one CTA = two 128-key tiles of one KV head, which stay in shared memory; the query tiles of the
-//                  head's group stream through a four-stage TMA ring, each stage feeding both key tiles (a CTA per
-//                  single key tile reads every query tile twice as often from L2 for no gain).  The step's
+//   k_mass_tc      a unit = two 128-key tiles of one KV head, which stay in shared memory while the query tiles of the
+//                  head's group stream through a four-stage TMA ring, each stage feeding both key tiles (a unit of a
+//                  single key tile reads every query tile twice as often from L2 for no gain).  Persistent CTAs, one per
+//                  SM, share the line of (unit, query tile) steps evenly: a CTA's run usually crosses from one unit into
+//                  the next, and a unit's sums come in up to MASS_PARTS pieces.  (A CTA per unit left SMs idle in its last
+//                  wave, as many as 38 %: 1,008 queries x 24 heads x
+//                  5,168 keys 70.3 us against 44.9, 9,200 72.7 / 71.2, 12,980 105.7 / 98.2; 300 x 16 x 1,200 20.3 / 11.6;
+//                  1,500 x 8 x 4,000, a unit per CTA either way, 21.5 / 22.5.)  The step's
 //                  normalisers ride along as a bulk copy into an eight-slot ring.  S^T = K Q^T (keys on the TMEM lanes,
 //                  queries on the columns) goes to one of two TMEM buffers per key tile.  Sixteen warps turn scores
 //                  into sums: per key tile and column half one warp per TMEM lane quadrant, one key per thread, 64
@@ -18,15 +23,18 @@
 //                  the waits of one hide behind the exponentials of the others; with two warps per scheduler (128
 //                  columns per thread) and a per-step meeting of the warps to stage the normalisers, a third of
 //                  every step was dead time.  The kernel is bound by the exponentials.
-//   k_mass_reduce  adds the partial sums of the KV heads and column halves in a fixed order, divides by n_q Hq and drops the padding rows
+//   k_mass_reduce  adds the partial sums of the KV heads, column halves and pieces in a fixed order, divides by n_q Hq and drops the padding rows
 //                  between segments.
 // Every wait is bounded as in the attention kernel.
+#include <algorithm>
+
 #include "pc_tc.cuh"
 
 namespace {
 
 using namespace pc_tc;
 
+constexpr int MASS_PARTS = PC_MASS_PARTS;   // most pieces of a unit
 constexpr int MASS_THREADS = 640;          // warp 0 TMA + TMEM owner, warp 1 MMA issuer, warps 4-19 column sums
 constexpr int Q_STAGES = 4;
 constexpr int L_SLOTS = 8;                 // normaliser ring: deeper than query stages + score buffers, see the producer
@@ -39,16 +47,25 @@ constexpr int SM_TOTAL = SM_LSE + L_SLOTS * TILE * 4;
 constexpr int SM_ALLOC = SM_TOTAL + 1024;
 
 enum { BAR_K = 0, BAR_QFULL = 1, BAR_QEMPTY = BAR_QFULL + Q_STAGES, BAR_SFULL = BAR_QEMPTY + Q_STAGES /* [tile][buffer] */,
-       BAR_SEMPTY = BAR_SFULL + 4, BAR_LFULL = BAR_SEMPTY + 4, BAR_DONE = BAR_LFULL + L_SLOTS, N_BARS = BAR_DONE + 1 };
+       BAR_SEMPTY = BAR_SFULL + 4, BAR_LFULL = BAR_SEMPTY + 4, BAR_DONE = BAR_LFULL + L_SLOTS,
+       BAR_KFREE = BAR_DONE + 1, N_BARS = BAR_KFREE + 1 };
 static_assert(N_BARS * 8 + 16 <= 256, "barrier area");
 
 struct MassParams {
     int n_q, n_q_heads, group, n_tb, n_kv_tiles, pairs;    // pairs = key-tile pairs per KV head
     const float *lse;      // [n_q][Hq] natural log
     float *norm;           // [Hq][n_tb * 128]: -log2(e) * lse, -inf past n_q
-    float *part;           // [Hkv][2 column halves][n_kv_tiles * 128]
+    float *part;           // [piece][Hkv][2 column halves][n_kv_tiles * 128]
     int32_t *status;
+    int n_cta, n_steps;    // persistent CTAs; steps (query tiles of the head's group) of a unit
+    int run, longer;       // steps of a CTA's run; the first `longer` CTAs take one more
 };
+__host__ __device__ __forceinline__ int run_start(const MassParams &P, int c) { return c * P.run + min(c, P.longer); }
+// the CTA whose run holds step x
+__host__ __device__ __forceinline__ int cta_of_step(const MassParams &P, int x) {
+    const int head = P.longer * (P.run + 1);
+    return x < head ? x / (P.run + 1) : P.longer + (x - head) / P.run;
+}
 
 __global__ void __launch_bounds__(256) k_mass_norm(const __grid_constant__ MassParams P) {
     pc_grid_dep_launch();
@@ -73,9 +90,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     auto bar = [&](int i) { return bar0 + 8u * i; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = blockIdx.x / P.pairs, jt0 = 2 * (blockIdx.x % P.pairs);
-    const int n_t = min(2, P.n_kv_tiles - jt0);           // 1 when the tile count is odd
-    const int n_steps = P.group * P.n_tb;                 // query tiles of this KV head's group
+    const int G0 = run_start(P, blockIdx.x), G1 = run_start(P, blockIdx.x + 1);     // never empty
 
     if (threadIdx.x == 0) {
         mbar_init(bar(BAR_K), 1);
@@ -89,6 +104,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         }
         for (int i = 0; i < L_SLOTS; ++i) mbar_init(bar(BAR_LFULL + i), 1);
         mbar_init(bar(BAR_DONE), 1);
+        mbar_init(bar(BAR_KFREE), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -105,27 +121,38 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
+        // ring stages, score buffers and normaliser slots follow the step count of the whole run (gs)
         if (lane == 0) {
-            mbar_expect_tx(bar(BAR_K), n_t * TILE_BYTES);
-            for (int t = 0; t < n_t; ++t) {
-                tma_load_2d(base + SM_K + t * TILE_BYTES, &map_k, g * TILE, (jt0 + t) * TILE, bar(BAR_K));
-                tma_load_2d(base + SM_K + t * TILE_BYTES + HALF_BYTES, &map_k, g * TILE + 64, (jt0 + t) * TILE, bar(BAR_K));
-            }
             bool alive = true;
-            for (int s = 0; s < n_steps && alive; ++s) {
-                const int st = s % Q_STAGES, use = s / Q_STAGES;
-                if (use > 0) alive = mbar_wait(bar(BAR_QEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+            int gs = 0, un = 0;
+            for (int x = G0; x < G1 && alive; ++un) {
+                const int unit = x / P.n_steps, s0 = x - unit * P.n_steps;
+                const int n = min(P.n_steps - s0, G1 - x);
+                const int g = unit / P.pairs, jt0 = 2 * (unit % P.pairs);
+                x += n;
+                if (un > 0) alive = mbar_wait(bar(BAR_KFREE), (un - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
                 if (!alive) break;
-                const int tb = s / P.group, h = g * P.group + s % P.group;
-                mbar_expect_tx(bar(BAR_QFULL + st), TILE_BYTES);
-                tma_load_2d(base + SM_Q + st * TILE_BYTES, &map_q, h * TILE, tb * TILE, bar(BAR_QFULL + st));
-                tma_load_2d(base + SM_Q + st * TILE_BYTES + HALF_BYTES, &map_q, h * TILE + 64, tb * TILE, bar(BAR_QFULL + st));
-                // The step's normalisers go to slot s mod 8.  Its previous tenant, step s - 8, is out of use: this point
-                // is reached after the products of step s - 4 completed, those needed the score buffers of step s - 6
-                // released, and a buffer is released only after the step before it was summed up.
-                const int slot = s % L_SLOTS;
-                mbar_expect_tx(bar(BAR_LFULL + slot), TILE * 4);
-                pc_bulk_g2s(base + SM_LSE + slot * TILE * 4, P.norm + ((size_t)h * P.n_tb + tb) * TILE, TILE * 4, bar(BAR_LFULL + slot));
+                mbar_expect_tx(bar(BAR_K), 2 * TILE_BYTES);
+                for (int t = 0; t < 2; ++t) {
+                    const int jt = min(jt0 + t, P.n_kv_tiles - 1);       // an odd tile count: the last tile twice, one copy dropped
+                    tma_load_2d(base + SM_K + t * TILE_BYTES, &map_k, g * TILE, jt * TILE, bar(BAR_K));
+                    tma_load_2d(base + SM_K + t * TILE_BYTES + HALF_BYTES, &map_k, g * TILE + 64, jt * TILE, bar(BAR_K));
+                }
+                for (int s = s0; s < s0 + n && alive; ++s, ++gs) {
+                    const int st = gs % Q_STAGES, use = gs / Q_STAGES;
+                    if (use > 0) alive = mbar_wait(bar(BAR_QEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                    if (!alive) break;
+                    const int tb = s / P.group, h = g * P.group + s % P.group;
+                    mbar_expect_tx(bar(BAR_QFULL + st), TILE_BYTES);
+                    tma_load_2d(base + SM_Q + st * TILE_BYTES, &map_q, h * TILE, tb * TILE, bar(BAR_QFULL + st));
+                    tma_load_2d(base + SM_Q + st * TILE_BYTES + HALF_BYTES, &map_q, h * TILE + 64, tb * TILE, bar(BAR_QFULL + st));
+                    // The step's normalisers go to slot gs mod 8.  Its previous tenant, step gs - 8, is out of use: this point
+                    // is reached after the products of step gs - 4 completed, those needed the score buffers of step gs - 6
+                    // released, and a buffer is released only after the step before it was summed up.
+                    const int slot = gs % L_SLOTS;
+                    mbar_expect_tx(bar(BAR_LFULL + slot), TILE * 4);
+                    pc_bulk_g2s(base + SM_LSE + slot * TILE * 4, P.norm + ((size_t)h * P.n_tb + tb) * TILE, TILE * 4, bar(BAR_LFULL + slot));
+                }
             }
             if (*abort_flag) {
                 // give the copies already issued a bounded chance to land before the CTA's shared memory goes away
@@ -137,29 +164,36 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         // ---------------------------------------------------------------- MMA issuer (converged warp, one elected lane)
         const bool lead = elect_one();
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        bool alive = mbar_wait(bar(BAR_K), 0, abort_flag, P.status, PC_WHERE_MASS_WAIT);
-        for (int s = 0; s < n_steps && alive; ++s) {
-            const int st = s % Q_STAGES, quse = s / Q_STAGES, b = s & 1, use = s >> 1;
-            alive = mbar_wait(bar(BAR_QFULL + st), quse & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
-            for (int t = 0; t < n_t && alive; ++t) {
-                if (use > 0) alive = mbar_wait(bar(BAR_SEMPTY + 2 * t + b), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
-                if (!alive) break;
-                tc_fence_after();
-                const uint32_t ka = base + SM_K + t * TILE_BYTES, qa = base + SM_Q + st * TILE_BYTES;
+        bool alive = true;
+        int gs = 0, un = 0;
+        for (int x = G0; x < G1 && alive; ++un) {
+            const int n = min(P.n_steps - x % P.n_steps, G1 - x);
+            x += n;
+            alive = mbar_wait(bar(BAR_K), un & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+            for (int s = 0; s < n && alive; ++s, ++gs) {
+                const int st = gs % Q_STAGES, quse = gs / Q_STAGES, b = gs & 1, use = gs >> 1;
+                alive = mbar_wait(bar(BAR_QFULL + st), quse & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                for (int t = 0; t < 2 && alive; ++t) {
+                    if (use > 0) alive = mbar_wait(bar(BAR_SEMPTY + 2 * t + b), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                    if (!alive) break;
+                    tc_fence_after();
+                    const uint32_t ka = base + SM_K + t * TILE_BYTES, qa = base + SM_Q + st * TILE_BYTES;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t off = (ks >> 2) * HALF_BYTES + (ks & 3) * 32;
-                    if (lead) mma_ss(tm + (2 * t + b) * TILE, desc_kmajor(ka + off), desc_kmajor(qa + off), IDESC_QK, ks > 0);
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint32_t off = (ks >> 2) * HALF_BYTES + (ks & 3) * 32;
+                        if (lead) mma_ss(tm + (2 * t + b) * TILE, desc_kmajor(ka + off), desc_kmajor(qa + off), IDESC_QK, ks > 0);
+                    }
+                    if (lead) tc_commit(bar(BAR_SFULL + 2 * t + b));
                 }
-                if (lead) tc_commit(bar(BAR_SFULL + 2 * t + b));
+                if (alive && lead) tc_commit(bar(BAR_QEMPTY + st));
             }
-            if (alive && lead) tc_commit(bar(BAR_QEMPTY + st));
+            if (alive && lead) tc_commit(bar(BAR_KFREE));       // the unit's key tiles may be overwritten
         }
         // nothing of ours may still be running on the tensor core when TMEM is freed
         if (lead) tc_commit(bar(BAR_DONE));
         __syncwarp();
         mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_MASS_WAIT);
-    } else if (warp >= 4 && (warp - 4) >> 3 < n_t) {
+    } else if (warp >= 4) {
         // ---------------------------------------------------------------- column sums: one key and 64 query columns per thread
         const int cw = warp - 4;
         const int t = cw >> 3, hf = (cw >> 2) & 1;        // key tile and column half of this warp
@@ -169,7 +203,9 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         const float *lse_s = reinterpret_cast<const float *>(gen + SM_LSE) + hf * 64;
         float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
         bool alive = true;
-        for (int s = 0; s < n_steps && alive; ++s) {
+        int unit = G0 / P.n_steps;
+        int unit_left = min((unit + 1) * P.n_steps, G1) - G0;    // steps of the run that are left in the unit
+        for (int s = 0; s < G1 - G0 && alive; ++s) {
             const int b = s & 1, use = s >> 1, slot = s % L_SLOTS;
             alive = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SFULL + 2 * t + b), use & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT) &&
                                                 mbar_wait(bar(BAR_LFULL + slot), (s / L_SLOTS) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT));
@@ -193,8 +229,16 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
                 acc0 = add2(acc0, x);
                 acc1 = add2(acc1, y);
             }
+            if (--unit_left == 0) {                          // the unit, or this CTA's piece of it, is done
+                const int g = unit / P.pairs, jt = 2 * (unit % P.pairs) + t;
+                const int piece = (int)blockIdx.x - cta_of_step(P, unit * P.n_steps);
+                if (jt < P.n_kv_tiles)
+                    P.part[((((size_t)piece * (P.n_q_heads / P.group) + g) * 2 + hf) * P.n_kv_tiles + jt) * TILE + r] = (acc0.x + acc0.y) + (acc1.x + acc1.y);
+                acc0 = acc1 = make_float2(0.f, 0.f);
+                ++unit;
+                unit_left = min(P.n_steps, G1 - unit * P.n_steps);
+            }
         }
-        if (alive) P.part[(((size_t)g * 2 + hf) * P.n_kv_tiles + jt0 + t) * TILE + r] = (acc0.x + acc0.y) + (acc1.x + acc1.y);
     }
     tc_fence_before();
     __syncthreads();
@@ -211,18 +255,60 @@ struct ReduceParams {
     float inv_rows;                         // 1 / (n_q Hq)
 };
 
-__global__ void __launch_bounds__(256) k_mass_reduce(const __grid_constant__ ReduceParams R, const float *__restrict__ part,
-                                                     float *__restrict__ mass) {
+// One block per key tile, a thread per key and MASS_ROWS rows of threads that share out the KV heads, so that the pieces of
+// different heads are read at the same time; the rows' sums are added in a fixed order.
+constexpr int MASS_ROWS = 8;
+
+__global__ void __launch_bounds__(TILE * MASS_ROWS) k_mass_reduce(const __grid_constant__ ReduceParams R, const __grid_constant__ MassParams P,
+                                                                  float *__restrict__ mass) {
+    __shared__ float rows[MASS_ROWS][TILE];
     pc_grid_dep_launch();
-    pc_grid_dep_wait();
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= R.seg_first[R.n_seg]) return;
+    const int jt = blockIdx.x, key = threadIdx.x % TILE, y = threadIdx.x / TILE;
+    const size_t row = (size_t)jt * TILE + key, stride = (size_t)P.n_kv_tiles * TILE;
     int s = 0;
-    while (s + 1 < R.n_seg && j >= R.seg_first[s + 1]) ++s;
-    const size_t row = (size_t)R.seg_tile0[s] * TILE + (j - R.seg_first[s]);
+    while (s + 1 < R.n_seg && jt >= R.seg_tile0[s + 1]) ++s;
+    const int j = R.seg_first[s] + (jt - R.seg_tile0[s]) * TILE + key;             // key number; past the segment: padding rows
+    pc_grid_dep_wait();
     float sum = 0.f;
-    for (int g = 0; g < 2 * R.n_kv_heads; ++g) sum += part[(size_t)g * R.n_kv_tiles * TILE + row];   // [head][column half]
+    for (int g = y; g < R.n_kv_heads; g += MASS_ROWS) {
+        const float *p = P.part + (size_t)g * 2 * stride + row;
+        float a = __ldcg(p), b = __ldcg(p + stride);                   // the first piece's two column halves
+        const int x = (g * P.pairs + jt / 2) * P.n_steps;
+        const int pieces = cta_of_step(P, x + P.n_steps - 1) - cta_of_step(P, x) + 1;
+        for (int piece = 1; piece < pieces; ++piece) {
+            p += (size_t)R.n_kv_heads * 2 * stride;
+            a += __ldcg(p);
+            b += __ldcg(p + stride);
+        }
+        sum += a + b;
+    }
+    rows[y][key] = sum;
+    __syncthreads();
+    if (y > 0 || j >= R.seg_first[s + 1]) return;
+#pragma unroll
+    for (int k = 1; k < MASS_ROWS; ++k) sum += rows[k][key];
     mass[j] = sum * R.inv_rows;
+}
+
+// Number of persistent CTAs: the fewest steps of the longest run, a change of unit reckoned as three of them (the products and
+// sums drain, the next key tiles load).  One CTA per SM, or a number that gives every CTA whole units or cuts every unit
+// into equal pieces.  The shortest run is at least a unit's steps over MASS_PARTS - 1, so no unit has more than MASS_PARTS pieces.
+int choose_mass_ctas(int units, int n_steps, int sm_count) {
+    const int steps = units * n_steps, shortest = (n_steps + MASS_PARTS - 2) / (MASS_PARTS - 1);
+    const int most = std::min(sm_count, steps / shortest);
+    int best = most;
+    long long best_cost = -1;
+    for (int n = most; n >= 1 && n >= most / 2; --n) {
+        const bool even = units % n == 0 || (n % units == 0 && n_steps % (n / units) == 0);
+        if (!even && n != most) continue;
+        const long long run = (steps + n - 1) / n;
+        const long long cost = run + 3 * (even ? std::max(units / n, 1) - 1 : (run - 1) / n_steps + 1);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = n;
+        }
+    }
+    return best;
 }
 
 }  // namespace
@@ -257,6 +343,12 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
     P.n_tb = (P.n_q + TILE - 1) / TILE;
     P.n_kv_tiles = tiles;
     P.pairs = (tiles + 1) / 2;
+    P.n_steps = P.group * P.n_tb;
+    const int units = D.n_kv_heads * P.pairs;
+    if ((long long)units * P.n_steps > INT32_MAX) return PC_ERR_CAPACITY;
+    P.n_cta = choose_mass_ctas(units, P.n_steps, ctx->sm_count);
+    P.run = units * P.n_steps / P.n_cta;
+    P.longer = units * P.n_steps % P.n_cta;
     P.lse = lse;
     P.part = ctx->mass_part;
     P.norm = ctx->mass_norm;
@@ -277,9 +369,9 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
     pc_mark(ctx, PC_MARK_MASS0, stream);
     PC_LAUNCH(k_mass_norm, dim3((P.n_tb * TILE * D.n_q_heads + 255) / 256), dim3(256), 0, stream, P);
     PC_CUDA_TRY(cudaGetLastError());
-    PC_LAUNCH(k_mass_tc, dim3(D.n_kv_heads * P.pairs), dim3(MASS_THREADS), SM_ALLOC, stream, mq, mk, P);
+    PC_LAUNCH(k_mass_tc, dim3(P.n_cta), dim3(MASS_THREADS), SM_ALLOC, stream, mq, mk, P);
     PC_CUDA_TRY(cudaGetLastError());
-    PC_LAUNCH(k_mass_reduce, dim3((keys + 255) / 256), dim3(256), 0, stream, R, static_cast<const float *>(ctx->mass_part), mass);
+    PC_LAUNCH(k_mass_reduce, dim3(tiles), dim3(TILE * MASS_ROWS), 0, stream, R, P, mass);
     PC_CUDA_TRY(cudaGetLastError());
     pc_mark(ctx, PC_MARK_MASS, stream);
     return PC_OK;
