@@ -81,14 +81,26 @@ struct RopeJobs { RopeJob job[PC_MAX_SEGMENTS + 1]; int n_jobs, total_warps; };
 // One warp per row (a query row wider than a key row is cut into key-row-wide slices, one warp each, so that all warps
 // carry the same load).  32 lanes x 8 elements = 256 is a multiple of d, so all of a lane's chunks (lane, lane + 32, ...)
 // hold the same four rotary pairs: four table entries per lane per row serve every chunk; the output scale (1 for keys)
-// is applied after the rotation, exactly as the query pass of the scoring stage does, so both give the same bits.  All of a row's chunks are loaded before any is used.
+// is applied after the rotation, exactly as the query pass of the scoring stage does, so both give the same bits.  A row's
+// chunks (up to eight at a time) are requested together with its position, before the table entries that wait for it.
+// Bound by memory, so warps in flight count: 64 registers, four blocks per SM.  Measured with the table entries first and 128
+// registers (up to 16 chunks at a time) against this: 50,000 key rows of 2 KB 40.0 -> 36.0 us (5.1 -> 5.7 TB/s), 7,184 7.6 ->
+// 6.5.
 template <int CPL /* chunks per lane */>
-__device__ __forceinline__ void rope_row(const RopeJob &J, int row, int lane, const float2 (&cs)[4], float scale) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(J.src) + (size_t)row * (CPL * 32) + lane;
-    uint4 *dst = reinterpret_cast<uint4 *>(J.dst) + (size_t)row * (CPL * 32) + lane;
+__device__ __forceinline__ void rope_row(const RopeJob &J, int row, int c0, int lane, const pc_rope_dev &rope, int pair0, int32_t *status) {
+    const size_t at = (size_t)row * J.chunks_per_row + c0 * 32 + lane;
+    const uint4 *src = reinterpret_cast<const uint4 *>(J.src) + at;
+    uint4 *dst = reinterpret_cast<uint4 *>(J.dst) + at;
+    const float scale = J.scale;
     uint4 v[CPL];
 #pragma unroll
     for (int c = 0; c < CPL; ++c) v[c] = pc_ldg_stream(src + c * 32);
+    const int4 pp = __ldg(reinterpret_cast<const int4 *>(J.pos) + row / J.rows_per_pos);
+    bool bad = false;
+    float2 cs[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cs[u] = pc_rope_cs_clamped(rope, pair0 + u, pp.x, pp.y, pp.z, bad);
+    if (bad) pc_flag(status, PC_ERR_INVALID_ARG, PC_WHERE_ROPE_POS);
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
         const uint32_t w[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
@@ -102,44 +114,27 @@ __device__ __forceinline__ void rope_row(const RopeJob &J, int row, int lane, co
     }
 }
 
-__global__ void __launch_bounds__(256) k_rope_rows(const __grid_constant__ RopeJobs jobs, pc_rope_dev rope, int d,
+__global__ void __launch_bounds__(256, 4) k_rope_rows(const __grid_constant__ RopeJobs jobs, pc_rope_dev rope, int d,
                                                    int32_t *status) {
     pc_grid_dep_launch();
-    pc_grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp >= jobs.total_warps) return;
     int ji = 0;
     while (ji + 1 < jobs.n_jobs && warp >= jobs.job[ji + 1].first_warp) ++ji;
     const RopeJob &J = jobs.job[ji];
-    const int row = warp - J.first_warp;
-    const int4 pp = __ldg(reinterpret_cast<const int4 *>(J.pos) + row / J.rows_per_pos);
-    const int pair0 = ((lane * 8) % d) / 2;
-    float2 cs[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) cs[u] = pc_rope_cs(rope, pair0 + u, pp.x, pp.y, pp.z, status, PC_WHERE_ROPE_POS);
-    const float scale = J.scale;
-    switch (J.chunks_per_row >> 5) {
-    case 4: rope_row<4>(J, row, lane, cs, scale); break;        // 8 KV heads x 128
-    case 12: rope_row<12>(J, row, lane, cs, scale); break;      // 24 query heads x 128
-    case 1: rope_row<1>(J, row, lane, cs, scale); break;
-    case 2: rope_row<2>(J, row, lane, cs, scale); break;
-    case 8: rope_row<8>(J, row, lane, cs, scale); break;
-    case 16: rope_row<16>(J, row, lane, cs, scale); break;
+    const int row = warp - J.first_warp, pair0 = ((lane * 8) % d) / 2;
+    pc_grid_dep_wait();
+    if (warp >= jobs.total_warps) return;
+    const int n = J.chunks_per_row >> 5;
+    switch (n) {
+    case 4: rope_row<4>(J, row, 0, lane, rope, pair0, status); break;        // 8 KV heads x 128, and a third of 24 query heads
+    case 1: rope_row<1>(J, row, 0, lane, rope, pair0, status); break;
+    case 2: rope_row<2>(J, row, 0, lane, rope, pair0, status); break;
+    case 8: rope_row<8>(J, row, 0, lane, rope, pair0, status); break;
     default:
-        for (int c = 0; c < (J.chunks_per_row >> 5); ++c) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(J.src) + (size_t)row * J.chunks_per_row + c * 32 + lane;
-            uint4 *dst = reinterpret_cast<uint4 *>(J.dst) + (size_t)row * J.chunks_per_row + c * 32 + lane;
-            const uint4 v = pc_ldg_stream(src);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-            uint32_t o[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float2 y = pc_rotate(pc_bf16_lo(w[u]), pc_bf16_hi(w[u]), cs[u]);
-                o[u] = pc_pack_bf16(__fmul_rn(y.x, scale), __fmul_rn(y.y, scale));
-            }
-            *dst = make_uint4(o[0], o[1], o[2], o[3]);
-        }
+        for (int c = 0; c < n; c += n % 4 ? 1 : 4)
+            if (n % 4) rope_row<1>(J, row, c, lane, rope, pair0, status);
+            else rope_row<4>(J, row, c, lane, rope, pair0, status);
     }
 }
 
@@ -605,7 +600,6 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 // parts' loads of a thread are issued before any is used.
 __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
     pc_grid_dep_launch();
-    pc_grid_dep_wait();
     const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5;                   // cg: units 4*cg .. 4*cg+3
     const int quad = blockIdx.x & 3, tile = blockIdx.x >> 2;
     const int h = tile % P.n_q_heads, tb = tile / P.n_q_heads;
@@ -615,6 +609,7 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
     if (row >= P.n_q) return;
     int part0, n_parts;
     item_parts(P, item, 0, part0, n_parts);
+    pc_grid_dep_wait();                           // the divisions above run under the attention kernel's tail
     if (n_parts < 2) return;                      // the one CTA that had the whole item wrote its output itself
     float2 ml[MAX_SPLITS];
     float4 o[4][4];
