@@ -211,6 +211,8 @@ __device__ __forceinline__ void pc_fma2(float2 &d, float2 a, float2 b) {
 // it in the stream is still draining.  A kernel lets its own dependents go at its very start (pc_grid_dep_launch) and
 // must not touch global memory before pc_grid_dep_wait, which returns once the preceding kernel has completed and its
 // writes are visible; only set-up that needs no global data (barrier initialisation, TMEM allocation) goes before it.
+// One exception: the query pass lets the scoring kernel go after its own wait, so that what came before it is complete when
+// the scoring kernel starts, which reads keys and positions ahead of its wait.
 __device__ __forceinline__ void pc_grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pc_grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

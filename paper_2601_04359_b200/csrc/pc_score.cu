@@ -68,8 +68,8 @@ __global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, 
                                                 int n_q_heads, int group, int d, int parts, pc_rope_dev rope,
                                                 float out_scale, T *__restrict__ q_rot, unsigned long long *fx,
                                                 int32_t *status) {
-    pc_grid_dep_launch();
     pc_grid_dep_wait();
+    pc_grid_dep_launch();   // after the wait: the scoring kernel reads keys and positions ahead of its own
     constexpr int PER = Elem<T>::PER16, NP = PER / 2;
     extern __shared__ __align__(16) float slab[];                     // [slots][Hq*d]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -142,53 +142,70 @@ __global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, 
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Score.  One warp takes two history tokens at a time: lane l loads the 16-byte chunks l, l + 32, ... of both rows
-// (streaming loads, all in flight before the first is used: 2 x CPL x 512 bytes per warp) and both position records.
-// 32 chunks span a multiple of d, so all of a lane's chunks cover the same PER/2 rotary pairs (of different heads): the
-// lane sums the two brackets over its chunks and needs PER/2 table look-ups per token.  For a pair (a, b) the two
-// brackets are two-lane products of the pair as it comes out of the unpacking, (k_a, k_b), with (q_a, q_b) and with
-// (q_b, -q_a): two two-lane fp32 multiply-adds per pair, no register shuffling.  The pooled query sits in shared
-// memory in that form; one 16-byte read serves both rows.
-// Blocks are persistent; warps take token pairs round-robin, so the tokens in flight at any time form one contiguous
-// window of the history.
+// Score.  A warp takes a group of consecutive history tokens at a time: LPT lanes share a token's row, 16 bytes at a time,
+// so 32 / LPT tokens lie side by side in the warp, TPL of them one after the other in a lane.  LPT chunks span a multiple of
+// d, so all of a lane's chunks cover the same PER/2 rotary pairs (of different heads): it sums the two brackets over its
+// chunks and needs PER/2 table look-ups per token.  For a pair (a, b) the two brackets are two-lane products of the pair as
+// it comes out of the unpacking, (k_a, k_b), with (q_a, q_b) and with (q_b, -q_a): two two-lane fp32 multiply-adds per pair,
+// no register shuffling.  The pooled query sits in shared memory in that form; one 16-byte read serves a lane's TPL tokens.
+//
+// The rows come by bulk copies (a group's rows are one run of memory) into a ring of stages that belongs to the warp: up to
+// 200 KB an SM in flight while the warps compute.  Rows held in registers (two of a warp, sixteen warps an SM) put 64 KB in
+// flight, and none of it while the row before was worked on.  A warp's first copies go out ahead of its wait for the pooled
+// query: the query pass lets this kernel start only when everything before that pass has completed, so keys and positions
+// are final.  Bound by DRAM at long histories (97 MB at 47 frames), by latency at short ones.  Steps of 24 / 8 heads, rows in
+// registers against this: 12 frames 84.2 -> 81.4 us, 47 frames 150.4 -> 147.2, masked update of 24 frames 141.3 -> 136.5,
+// 135-token frames 28.3 -> 27.4; 32 / 16 heads: 12 frames 115.7 -> 111.6, 47 frames 220.6 -> 209.8.  Eight warps 148.5 at 47
+// frames; warps held to 80 registers and 8 of them, to be resident beside the query pass, 152.0 to 153.8; the look-ups
+// behind the sums instead of in front of them 148.2.
 // ---------------------------------------------------------------------------------------------------------
-constexpr int SCORE_WARPS = 8;
-constexpr int SCORE_THREADS = SCORE_WARPS * 32;
+constexpr int SCORE_WARPS = 12;                      // most warps per block (fewer where two stages of each would not fit)
+constexpr int SCORE_STAGES = 8;                     // most stages of a warp's ring
+constexpr int SCORE_RING = 200 * 1024;              // bytes of a block's rings
 
-template <typename T, int CPL /* chunks per lane */>
-__global__ void __launch_bounds__(SCORE_THREADS, 2) k_score(const T *__restrict__ k, const int32_t *__restrict__ k_pos,
-                                                            const uint8_t *__restrict__ valid, int n_src, int d, float scale,
-                                                            pc_rope_dev rope, unsigned long long *fx, double fx_scale,
-                                                            float *__restrict__ scores, int32_t *status) {
+template <typename T, int LPT /* lanes per token */, int TPL /* tokens per lane */>
+__global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restrict__ k, const int32_t *__restrict__ k_pos,
+                                                               const uint8_t *__restrict__ valid, int n_src, int d, int parts, int stages, float scale,
+                                                               pc_rope_dev rope, unsigned long long *fx, double fx_scale,
+                                                               float *__restrict__ scores, int32_t *status) {
     pc_grid_dep_launch();
-    constexpr int PER = Elem<T>::PER16, NP = PER / 2;
-    __shared__ float4 qs[CPL * NP * 32];                              // (q_a, q_b, q_b, -q_a) of (chunk, pair, lane)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * SCORE_WARPS + warp, n_warps = gridDim.x * SCORE_WARPS;
-    const int n_pairs = (n_src + 1) >> 1;
-    const uint4 *krow = reinterpret_cast<const uint4 *>(k) + lane;
-    pc_grid_dep_wait();   // the pooled query comes from the kernel before
+    constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL;
+    extern __shared__ __align__(128) unsigned char score_smem[];
+    __shared__ __align__(8) unsigned long long bars[SCORE_WARPS * SCORE_STAGES];
+    __shared__ int gave_up;
+    float4 *qs = reinterpret_cast<float4 *>(score_smem);              // (q_a, q_b, q_b, -q_a) of (head, pair, lane of the token)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lt = lane % LPT, side = lane / LPT, n_warps = blockDim.x >> 5;
+    const int row_bytes = parts * LPT * 16, stage_bytes = TOK * row_bytes;
+    const int n_groups = (n_src + TOK - 1) / TOK, step = gridDim.x * n_warps;
+    const uint32_t ring = pc_smem_u32(score_smem) + parts * NP * LPT * 16 + warp * stages * stage_bytes;
+    const uint32_t bar0 = pc_smem_u32(bars) + warp * SCORE_STAGES * 8;
+    int grp = warp * gridDim.x + blockIdx.x;                          // small calls spread over the blocks first
 
-    // this warp's first two rows are requested before the pooled query is staged: both latencies overlap
-    int tp = gw;
-    uint4 raw0[CPL], raw1[CPL];
-    int4 p0 = make_int4(0, 0, 0, 0), p1 = p0;
-    auto request = [&](int pair_idx) {
-        const int j0 = 2 * pair_idx, j1 = min(j0 + 1, n_src - 1);
-        p0 = __ldg(reinterpret_cast<const int4 *>(k_pos) + j0);
-        p1 = __ldg(reinterpret_cast<const int4 *>(k_pos) + j1);
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) raw0[c] = pc_ldg_stream(krow + (size_t)j0 * (CPL * 32) + c * 32);
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) raw1[c] = pc_ldg_stream(krow + (size_t)j1 * (CPL * 32) + c * 32);
+    auto fill = [&](int stage, int group) {                           // one lane
+        const uint32_t bytes = (uint32_t)(min(TOK, n_src - group * TOK) * row_bytes);
+        pc_mbar_expect_tx(bar0 + 8 * stage, bytes);
+        pc_bulk_g2s(ring + stage * stage_bytes, reinterpret_cast<const char *>(k) + (size_t)group * stage_bytes, bytes, bar0 + 8 * stage);
     };
-    if (tp < n_pairs) request(tp);
+    if (lane == 0) {
+        for (int s = 0; s < stages; ++s) pc_mbar_init(bar0 + 8 * s, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int s = 0; s < stages && grp + s * step < n_groups; ++s) fill(s, grp + s * step);
+    }
+    if (threadIdx.x == 0) gave_up = 0;
+    int4 p[TPL];
+    auto positions = [&](int group) {
+#pragma unroll
+        for (int i = 0; i < TPL; ++i) p[i] = __ldcg(reinterpret_cast<const int4 *>(k_pos) + min(group * TOK + i * SIDE + side, n_src - 1));
+    };
+    if (grp < n_groups) positions(grp);
+    pc_grid_dep_wait();                                               // the pooled query comes from the kernel before
 
     // the pooled query: the accumulator, scaled
-    constexpr int N_OUT = CPL * 32 * PER;
-    for (int idx = threadIdx.x; idx < CPL * NP * 32; idx += SCORE_THREADS) {
-        const int l = idx & 31, u = (idx >> 5) % NP, c = idx / (32 * NP);
-        const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(fx + (size_t)(c * 32 + l) * PER + 2 * u));
+    const int n_out = parts * LPT * PER;
+    for (int idx = threadIdx.x; idx < parts * NP * LPT; idx += blockDim.x) {
+        const int l = idx % LPT, u = (idx / LPT) % NP, g = idx / (LPT * NP);
+        const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(fx + (size_t)(g * LPT + l) * PER + 2 * u));
         const float a = (float)((double)w.x * fx_scale), b = (float)((double)w.y * fx_scale);
         qs[idx] = make_float4(a, b, b, -a);
     }
@@ -197,84 +214,101 @@ __global__ void __launch_bounds__(SCORE_THREADS, 2) k_score(const T *__restrict_
     // it for the next call when its tokens are done.  Nobody waits for anybody, and nothing of this lives on the host, so a
     // captured graph replays it unchanged.
     unsigned long long ticket = 0;
-    if (threadIdx.x == 0) ticket = atomicAdd(fx + N_OUT, 1ull);
+    if (threadIdx.x == 0) ticket = atomicAdd(fx + n_out, 1ull);
 
-    // table slots of this lane's pairs: entry = tbase + coordinate(axis) * stride
-    const int pair0 = ((lane * PER) % d) / 2;
-    int tbase[NP], tstride[NP], taxis[NP];
-#pragma unroll
-    for (int u = 0; u < NP; ++u) {
-        const int a = (pair0 + u) % 3;
-        taxis[u] = a;
-        tbase[u] = (a == 0 ? rope.off[0] : (a == 1 ? rope.off[1] : rope.off[2])) + (pair0 + u) / 3;
-        tstride[u] = a == 0 ? rope.n_axis[0] : (a == 1 ? rope.n_axis[1] : rope.n_axis[2]);
-    }
+    // Table entries of this lane's pairs: consecutive pairs take the axes in turn, so pair u's entry is at column m[u] of the
+    // row of coordinate (r + u) mod 3, and the fourth pair's is the one behind the first's.
+    constexpr int AX = NP < 3 ? NP : 3;
+    const int pair0 = ((lt * PER) % d) / 2, r = pair0 % 3;
     const unsigned mt = rope.max_pos[0], mh = rope.max_pos[1], mw = rope.max_pos[2];
-    const float4 *ql = qs + lane;
-
-    auto table = [&](int4 p, float2 (&cs)[NP]) {
-        int pt = p.x, ph = p.y, pw = p.z;
-        if (!((unsigned)pt < mt && (unsigned)ph < mh && (unsigned)pw < mw)) {   // outside the tables: record, clamp
-            pc_flag(status, PC_ERR_INVALID_ARG, PC_WHERE_SCORE_POS);
-            pt = min(max(pt, 0), (int)mt - 1); ph = min(max(ph, 0), (int)mh - 1); pw = min(max(pw, 0), (int)mw - 1);
-        }
+    int first[AX], pitch[AX];
 #pragma unroll
-        for (int u = 0; u < NP; ++u) {
-            const int pa = taxis[u] == 0 ? pt : (taxis[u] == 1 ? ph : pw);
-            cs[u] = __ldg(rope.tab + tbase[u] + pa * tstride[u]);
+    for (int u = 0; u < AX; ++u) {
+        const int a = (pair0 + u) % 3;
+        first[u] = (a == 0 ? rope.off[0] : (a == 1 ? rope.off[1] : rope.off[2])) + (pair0 + u) / 3;
+        pitch[u] = a == 0 ? rope.n_axis[0] : (a == 1 ? rope.n_axis[1] : rope.n_axis[2]);
+    }
+    auto table = [&](int4 q, float2 (&cs)[NP]) {
+        if (!((unsigned)q.x < mt && (unsigned)q.y < mh && (unsigned)q.z < mw)) {   // outside the tables: record, clamp
+            pc_flag(status, PC_ERR_INVALID_ARG, PC_WHERE_SCORE_POS);
+            q.x = min(max(q.x, 0), (int)mt - 1); q.y = min(max(q.y, 0), (int)mh - 1); q.z = min(max(q.z, 0), (int)mw - 1);
         }
+        const int c[3] = {r == 0 ? q.x : (r == 1 ? q.y : q.z), r == 0 ? q.y : (r == 1 ? q.z : q.x), r == 0 ? q.z : (r == 1 ? q.x : q.y)};
+#pragma unroll
+        for (int u = 0; u < NP; ++u) cs[u] = __ldg(rope.tab + (u < AX ? first[u % AX] + c[u % AX] * pitch[u % AX] : first[0] + c[0] * pitch[0] + 1));
     };
 
-    for (; tp < n_pairs; tp += n_warps) {
-        float2 cs0[NP], cs1[NP];
-        table(p0, cs0);
-        table(p1, cs1);
+    int stage = 0, phase = 0;
+    for (; grp < n_groups; grp += step) {
+        float2 cs[TPL][NP];
+#pragma unroll
+        for (int i = 0; i < TPL; ++i) table(p[i], cs[i]);
+        if (grp + step < n_groups) positions(grp + step);
+        if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT))) break;
         // brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair
-        float2 A0[NP], B0[NP], A1[NP], B1[NP];
+        float2 A[TPL][NP], B[TPL][NP];
 #pragma unroll
-        for (int u = 0; u < NP; ++u) A0[u] = B0[u] = A1[u] = B1[u] = make_float2(0.f, 0.f);
+        for (int i = 0; i < TPL; ++i)
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) {
-            float k0[PER], k1[PER];
-            Elem<T>::unpack(raw0[c], k0);
-            Elem<T>::unpack(raw1[c], k1);
+            for (int u = 0; u < NP; ++u) A[i][u] = B[i][u] = make_float2(0.f, 0.f);
+        const uint32_t mine = ring + stage * stage_bytes + side * row_bytes + lt * 16;
+        const float4 *ql = qs + lt;
+#pragma unroll 1
+        for (int g = 0; g < parts; ++g) {
+            float x[TPL][PER];
+#pragma unroll
+            for (int i = 0; i < TPL; ++i) Elem<T>::unpack(pc_lds128(mine + i * SIDE * row_bytes + g * LPT * 16), x[i]);
 #pragma unroll
             for (int u = 0; u < NP; ++u) {
-                const float4 qq = ql[(c * NP + u) * 32];
+                const float4 qq = ql[(g * NP + u) * LPT];
                 const float2 qab = make_float2(qq.x, qq.y), qba = make_float2(qq.z, qq.w);
-                const float2 x0 = make_float2(k0[2 * u], k0[2 * u + 1]), x1 = make_float2(k1[2 * u], k1[2 * u + 1]);
-                A0[u] = __ffma2_rn(qab, x0, A0[u]);
-                B0[u] = __ffma2_rn(qba, x0, B0[u]);
-                A1[u] = __ffma2_rn(qab, x1, A1[u]);
-                B1[u] = __ffma2_rn(qba, x1, B1[u]);
+#pragma unroll
+                for (int i = 0; i < TPL; ++i) {
+                    const float2 kk = make_float2(x[i][2 * u], x[i][2 * u + 1]);
+                    A[i][u] = __ffma2_rn(qab, kk, A[i][u]);
+                    B[i][u] = __ffma2_rn(qba, kk, B[i][u]);
+                }
             }
         }
-        float s0 = 0.f, s1 = 0.f;
+        __syncwarp();                                                 // every lane has read the stage
+        if (lane == 0 && grp + stages * step < n_groups) fill(stage, grp + stages * step);
+        if (++stage == stages) { stage = 0; phase ^= 1; }
+        float s[TPL];
 #pragma unroll
-        for (int u = 0; u < NP; ++u) {
-            s0 = fmaf(cs0[u].x, A0[u].x + A0[u].y, fmaf(cs0[u].y, B0[u].x + B0[u].y, s0));
-            s1 = fmaf(cs1[u].x, A1[u].x + A1[u].y, fmaf(cs1[u].y, B1[u].x + B1[u].y, s1));
+        for (int i = 0; i < TPL; ++i) {
+            s[i] = 0.f;
+#pragma unroll
+            for (int u = 0; u < NP; ++u)
+                s[i] = fmaf(cs[i][u].x, A[i][u].x + A[i][u].y, fmaf(cs[i][u].y, B[i][u].x + B[i][u].y, s[i]));
         }
-        const int j0 = 2 * tp;
-        if (tp + n_warps < n_pairs) request(tp + n_warps);           // the next two rows travel while these are reduced
-        // both sums with six shuffles: after the first exchange the lower half-warp carries token 0, the upper token 1
-        s0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-        float s = lane < 16 ? s0 : s1;
+        // a token's lanes are added up; with two tokens in a lane its lower lanes carry on with the first, the upper ones with the second
+        float sum = s[0];
+        int o = LPT / 2, i_out = 0;
+        if constexpr (TPL == 2) {
+            i_out = lt >= LPT / 2;
+            sum = i_out ? s[1] : s[0];
+            sum += __shfl_xor_sync(0xffffffffu, i_out ? s[0] : s[1], LPT / 2);
+            o = LPT / 4;
+        }
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((lane & 15) == 0) {
-            const int j = j0 + (lane >> 4);
+        for (; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lt % (LPT / TPL) == 0) {
+            const int j = grp * TOK + i_out * SIDE + side;
             if (j < n_src) {
-                float r = s * scale;
+                float r = sum * scale;
                 if (valid && !valid[j]) r = -INFINITY;
                 scores[j] = r;
             }
         }
     }
+    if (grp < n_groups && lane == 0) {
+        // a wait ran out: the copies already issued get a bounded chance to land before the block's shared memory goes away
+        const uint64_t t0 = pc_global_ns();
+        while (pc_global_ns() - t0 < 2000000ull) {}
+    }
     if (warp == 0 && __shfl_sync(0xffffffffu, ticket, 0) == (unsigned long long)(gridDim.x - 1)) {
-        for (int e = lane; e < N_OUT; e += 32) fx[e] = 0;
-        if (lane == 0) fx[N_OUT] = 0;
+        for (int e = lane; e < n_out; e += 32) fx[e] = 0;
+        if (lane == 0) fx[n_out] = 0;
     }
 }
 
@@ -355,24 +389,34 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     PC_CUDA_TRY(cudaGetLastError());
     if (marks) pc_mark(marks, PC_MARK_QPOOL, stream);
     const float scale = (float)(1.0 / ((double)D.n_q_heads * std::sqrt((double)D.head_dim)));
-    const int n_pairs = (n_src + 1) / 2;
     const T *k = static_cast<const T *>(hist_k);
-#define PC_SCORE_CASE(CPL)                                                                                          \
-    case CPL: {                                                                                                     \
-        /* resident blocks per SM of this instance (the grid is persistent), looked up once per device */          \
-        static int per_sm_of[PC_MAX_DEVICES] = {};                                                                  \
-        if (per_sm_of[dev_id] == 0) {                                                                               \
-            int occ = 0;                                                                                            \
-            PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_score<T, CPL>, SCORE_THREADS, 0));    \
-            per_sm_of[dev_id] = std::max(1, occ);                                                                   \
+    const int lpt = std::max(16, D.head_dim / PER), row_bytes = row * (int)sizeof(T);
+    // Two tokens per lane share each read of the pooled query, where every warp gets two stages of them.  Wider rows leave
+    // fewer warps two stages, which pays once there are groups for all warps: 3 KB rows, 44,000 tokens 38.2 (one token) against
+    // 32.6 us, 675 tokens 7.9 against 9.1; 4 KB rows 46.2 against 43.2, 8.8 against 10.9.
+    const int room = SCORE_RING / (4 * (32 / lpt) * row_bytes);      // warps with two stages of two tokens per lane
+    const bool two = room >= SCORE_WARPS || (room >= SCORE_WARPS / 2 && n_src > sm_count * SCORE_WARPS * (32 / lpt));
+    const int tok = (two ? 2 : 1) * (32 / lpt), stage_bytes = tok * row_bytes, n_groups = (n_src + tok - 1) / tok;
+    const int blocks = std::max(1, std::min(n_groups, sm_count)), need = (n_groups + blocks - 1) / blocks;
+    // Short histories: as many warps as it takes to stage the pooled query quickly, and no more (query pass and scores of 675
+    // tokens, 1,024 pooled elements: 7.4 us with 12 warps, 8.1 with 4; the fp32 step with 128 elements 18.7 with 12, 16.5 with 4).
+    const int warps = std::min({SCORE_WARPS, SCORE_RING / (2 * stage_bytes), std::max({4, need, row / 40})});
+    const int stages = std::max(1, std::min({SCORE_STAGES, SCORE_RING / (warps * stage_bytes), (n_groups + blocks * warps - 1) / (blocks * warps)}));
+    const int smem = row * 8 + warps * stages * stage_bytes;
+#define PC_SCORE_CASE(LPT, TPL)                                                                                      \
+    {                                                                                                               \
+        static bool set[PC_MAX_DEVICES] = {};                                                                       \
+        if (!set[dev_id]) {                                                                                         \
+            PC_CUDA_TRY(cudaFuncSetAttribute(k_score<T, LPT, TPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_RING + 16 * 1024)); \
+            set[dev_id] = true;                                                                                     \
         }                                                                                                           \
-        const int blocks = std::max(1, std::min((n_pairs + SCORE_WARPS - 1) / SCORE_WARPS, sm_count * per_sm_of[dev_id])); \
-        PC_LAUNCH((k_score<T, CPL>), dim3(blocks), dim3(SCORE_THREADS), 0, stream, k, hist_pos, valid, n_src, D.head_dim, scale, rope, \
-                  reinterpret_cast<unsigned long long *>(fx), fx_scale, scores, status);                             \
-    } break;
-    switch (chunks / 32) {
-        PC_SCORE_CASE(1) PC_SCORE_CASE(2) PC_SCORE_CASE(3) PC_SCORE_CASE(4) PC_SCORE_CASE(6) PC_SCORE_CASE(8)
-    default: return PC_ERR_UNSUPPORTED;
+        PC_LAUNCH((k_score<T, LPT, TPL>), dim3(blocks), dim3(warps * 32), smem, stream, k, hist_pos, valid, n_src, D.head_dim, row_bytes / (lpt * 16), stages, scale, \
+                  rope, reinterpret_cast<unsigned long long *>(fx), fx_scale, scores, status);                       \
+    }
+    if (lpt == 16) {
+        if (two) PC_SCORE_CASE(16, 2) else PC_SCORE_CASE(16, 1)
+    } else if constexpr (sizeof(T) == 4) {           // fp32 heads of 128
+        if (two) PC_SCORE_CASE(32, 2) else PC_SCORE_CASE(32, 1)
     }
 #undef PC_SCORE_CASE
     PC_CUDA_TRY(cudaGetLastError());
