@@ -597,8 +597,11 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 // ------------------------------------------------------------------------------------------------ combine
 // Merge of the KV ranges' partials.  One block per (query tile of one head, 32-row quadrant); its eight warps take four
 // 16-byte column units each, lanes are consecutive rows, so every load of the partial tiles is a 512-byte run.  Up to four
-// parts' loads of a thread are issued before any is used.
-__global__ void __launch_bounds__(256) k_combine(const TcParams P) {
+// parts' loads of a thread are issued before any is used.  Bound by L2 and its latency, so loads in flight count: an item of the
+// persistent form has two parts nearly always, and built for those the kernel takes 48 registers instead of 108 and four
+// blocks an SM instead of two.  The step at 12 frames 80.6 -> 79.1 us, 47 frames 147.0 -> 145.4; six blocks an SM 79.9 and 146.0.
+template <int PARTS /* most parts of an item */, int BLOCKS /* resident on an SM */>
+__global__ void __launch_bounds__(256, BLOCKS) k_combine(const TcParams P) {
     pc_grid_dep_launch();
     const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5;                   // cg: units 4*cg .. 4*cg+3
     const int quad = blockIdx.x & 3, tile = blockIdx.x >> 2;
@@ -611,13 +614,14 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
     item_parts(P, item, 0, part0, n_parts);
     pc_grid_dep_wait();                           // the divisions above run under the attention kernel's tail
     if (n_parts < 2) return;                      // the one CTA that had the whole item wrote its output itself
-    float2 ml[MAX_SPLITS];
-    float4 o[4][4];
+    constexpr int WAY = PARTS < 4 ? PARTS : 4;      // parts in flight
+    float2 ml[PARTS];
+    float4 o[WAY][4];
     const float2 *pml = reinterpret_cast<const float2 *>(P.part_ml);
     const float4 *po = reinterpret_cast<const float4 *>(P.part_o);
     auto load4 = [&](int s0) {                     // the O units of parts s0 .. s0 + 3
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+        for (int s = 0; s < WAY; ++s)
             if (s0 + s < n_parts) {
                 const float4 *pt = po + (((size_t)item * P.part_stride + s0 + s) * 2 + t) * (TILE * TILE / 4) + r;
 #pragma unroll
@@ -625,27 +629,27 @@ __global__ void __launch_bounds__(256) k_combine(const TcParams P) {
             }
     };
 #pragma unroll
-    for (int s = 0; s < MAX_SPLITS; ++s)
+    for (int s = 0; s < PARTS; ++s)
         if (s < n_parts) ml[s] = __ldcg(pml + (((size_t)item * P.part_stride + s) * 2 + t) * TILE + r);
     load4(0);
     float m = -INFINITY;
 #pragma unroll
-    for (int s = 0; s < MAX_SPLITS; ++s)
+    for (int s = 0; s < PARTS; ++s)
         if (s < n_parts) m = fmaxf(m, ml[s].x);
     float l = 0.f;
     float4 acc[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int s = 0; s < MAX_SPLITS; ++s) {
-        if (s == 4 && n_parts > 4) load4(4);
+    for (int s = 0; s < PARTS; ++s) {
+        if (PARTS > 4 && s == 4 && n_parts > 4) load4(4);
         if (s < n_parts) {
             const float sc = exp2f(ml[s].x - m);
             l = fmaf(ml[s].y, sc, l);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                acc[u].x = fmaf(o[s & 3][u].x, sc, acc[u].x); acc[u].y = fmaf(o[s & 3][u].y, sc, acc[u].y);
-                acc[u].z = fmaf(o[s & 3][u].z, sc, acc[u].z); acc[u].w = fmaf(o[s & 3][u].w, sc, acc[u].w);
+                acc[u].x = fmaf(o[s % WAY][u].x, sc, acc[u].x); acc[u].y = fmaf(o[s % WAY][u].y, sc, acc[u].y);
+                acc[u].z = fmaf(o[s % WAY][u].z, sc, acc[u].z); acc[u].w = fmaf(o[s % WAY][u].w, sc, acc[u].w);
             }
         }
     }
@@ -871,7 +875,10 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     PC_CUDA_TRY(cudaGetLastError());
     pc_mark(ctx, PC_MARK_ATTEND, stream);
     if (P.part_stride > 1 && !P.cluster) {
-        PC_LAUNCH(k_combine, dim3(P.n_tb * D.n_q_heads * 4), dim3(256), 0, stream, P);
+        const dim3 grid(P.n_tb * D.n_q_heads * 4);
+        if (P.part_stride == 2) PC_LAUNCH((k_combine<2, 4>), grid, dim3(256), 0, stream, P);
+        else if (P.part_stride <= 4) PC_LAUNCH((k_combine<4, 3>), grid, dim3(256), 0, stream, P);
+        else PC_LAUNCH((k_combine<MAX_SPLITS, 2>), grid, dim3(256), 0, stream, P);
         PC_CUDA_TRY(cudaGetLastError());
         pc_mark(ctx, PC_MARK_COMBINE, stream);
     }
