@@ -153,12 +153,15 @@ pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *bu
     // now, before the scoring stage enqueues anything
     st = pc_compact_check(ctx, src, sel_idx, budget, dst, nullptr, nullptr);
     if (st != PC_OK) return st;
+    // (with values still on their way the selection need not wait for them; stage marks tell the two stages apart)
+    const bool one_launch = !hooks && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
     ctx->last_n_q = 0;
     ctx->q_rot_n = 0;
-    st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream);
+    st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream, !one_launch);
     if (st != PC_OK) return st;
     if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
-    st = pc_compact_impl(ctx, src, sel_idx, budget, delta_t, dst, k_rot_dst, stream);
+    st = one_launch ? pc_launch_select_pack(ctx, scores, src, budget, delta_t, &dst->history, sel_idx, k_rot_dst, stream)
+                    : pc_compact_impl(ctx, src, sel_idx, budget, delta_t, dst, k_rot_dst, stream);
     if (st != PC_OK) return st;
     dst->history.n_tokens = (int32_t)n_sel;
     dst->n_frames = src->n_frames;

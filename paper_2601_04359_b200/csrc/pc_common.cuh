@@ -263,7 +263,11 @@ pc_status pc_launch_pack(pc_ctx *ctx, const void *src_k, const void *src_v, cons
 bool pc_score_supports(const pc_layer_desc &D);   // the row widths the query pass and the scoring kernel take
 pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
                         const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
-                        cudaStream_t stream);
+                        cudaStream_t stream, bool select = true);   // select = false: scores only, the caller selects
+// selection and pack in one launch (small frames): whether a call's frames suit it, and the launch (arguments already checked)
+bool pc_select_pack_fits(const pc_ctx *ctx, const pc_cache *src, const int32_t *budget);
+pc_status pc_launch_select_pack(pc_ctx *ctx, const float *scores, const pc_cache *src, const int32_t *budget, int delta_t, const pc_segment *dst,
+                                int32_t *sel_idx, void *k_rot_dst, cudaStream_t stream);
 pc_status pc_compact_check(pc_ctx *ctx, const pc_cache *src, const int32_t *sel_idx, const int32_t *budget, const pc_cache *dst,
                            int64_t *n_sel_out, int64_t *n_src_out);   // every host-side check of pc_compact_impl, nothing enqueued
 pc_status pc_compact_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *sel_idx, const int32_t *budget, int32_t delta_t,

@@ -440,7 +440,7 @@ bool pc_score_supports(const pc_layer_desc &D) {
 
 pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
                         const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
-                        cudaStream_t stream) {
+                        cudaStream_t stream, bool select) {
     if (!ctx || !src || !budget) return PC_ERR_INVALID_ARG;
     const int n_frames = src->n_frames;
     if (n_frames < 0 || (n_frames > 0 && !src->frame_count)) return PC_ERR_INVALID_ARG;
@@ -490,7 +490,7 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
     } else if (reinterpret_cast<uintptr_t>(scores_override) & 3) {      // read element by element: any float address will do
         return PC_ERR_INVALID_ARG;
     }
-    if (n_frames > 0 && out > 0) {
+    if (select && n_frames > 0 && out > 0) {
         if (scores_override) pc_mark(ctx, PC_MARK_SCORE, stream);
         // a thread per key, as far as a block goes: frames of 64 and 135 tokens take 2.4 and 2.5 us with 256
         // threads, 2.7 and 2.8 with 1,024; frames of 1,008 and 4,032 tokens 3.6 and 8.0 with 1,024, 3.8 and 8.9 with 512
