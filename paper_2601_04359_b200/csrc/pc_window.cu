@@ -50,13 +50,17 @@ extern "C" pc_status pc_window_create(pc_ctx *ctx, const pc_window_params *param
     w->scores = scores;
     w->sel_idx = sel_idx;
     w->scratch_capacity = std::min(hist_a->capacity, hist_b->capacity);
+    // The stream and the events belong to the context's device, whichever is current here: the steps' own stream is on it, and an
+    // event is recorded on a stream of its own device only.
     const auto on_device = [&]() -> pc_status {
         PC_CUDA_TRY(cudaStreamCreateWithFlags(&w->side, cudaStreamNonBlocking));
         PC_CUDA_TRY(cudaEventCreateWithFlags(&w->main_ev, cudaEventDisableTiming));
         PC_CUDA_TRY(cudaEventCreateWithFlags(&w->side_ev, cudaEventDisableTiming));
         return PC_OK;
     };
-    st = on_device();
+    int current = ctx->device;
+    st = cudaGetDevice(&current) == cudaSuccess && (current == ctx->device || cudaSetDevice(ctx->device) == cudaSuccess) ? on_device() : PC_ERR_CUDA;
+    if (current != ctx->device && cudaSetDevice(current) != cudaSuccess && st == PC_OK) st = PC_ERR_CUDA;
     if (st != PC_OK) {
         pc_window_destroy(w);
         return st;
