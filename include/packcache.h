@@ -335,8 +335,9 @@ pc_status pc_window_step(pc_window *w, const void *q, const int32_t *q_pos, int3
  * output back and waits for the stream.  The frame's values and the output travel on a stream of the window's own, beside
  * the kernels; from 512 query rows or so (as many as fill the GPU twice) attention runs in parts of the rows so that the
  * output leaves part by part, and then agrees with pc_window_step up to fp32 rounding order (fewer rows: bit for bit).
- * Pinned host memory keeps the copies asynchronous.  All arguments are checked
- * before anything is enqueued.  Errors: as pc_window_append and pc_window_step. */
+ * Pinned host memory keeps the copies asynchronous.  All arguments are checked before anything is enqueued; a call that fails
+ * leaves the window as it was (the frame is not appended) and nothing in flight on either stream.
+ * Errors: as pc_window_append and pc_window_step. */
 typedef struct {
     const void *frame_k, *frame_v; /* host [n_frame][Hkv][d]: the frame to append as the newest history frame */
     const int32_t *frame_pos;      /* host [n_frame][4], in the shifted frame of reference (pc_window_state) */

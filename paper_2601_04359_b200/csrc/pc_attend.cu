@@ -3,6 +3,8 @@
 
 namespace {
 
+constexpr int STEP_TILE = 128;        // rows of the rotated-key scratch start on multiples of this
+
 // anchors ++ history ++ current, empty segments dropped
 pc_status gather_segments(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, pc_segment *segs, int *n_seg) {
     *n_seg = 0;
@@ -21,7 +23,7 @@ pc_status gather_segments(pc_ctx *ctx, const pc_cache *cache, const pc_segment *
     return PC_OK;
 }
 
-pc_status check_queries(pc_ctx *ctx, const void *q, const int32_t *q_pos, int32_t n_q, void *out, float *lse) {
+pc_status check_queries(pc_ctx *ctx, const void *q, const int32_t *q_pos, int32_t n_q, const void *out, const float *lse) {
     if (!q || !q_pos || !out || n_q <= 0) return PC_ERR_INVALID_ARG;
     if (!pc_aligned16(q) || !pc_aligned16(q_pos) || !pc_aligned16(out) || (lse && !pc_aligned16(lse))) return PC_ERR_INVALID_ARG;
     if (n_q > ctx->desc.max_q) return PC_ERR_CAPACITY;
@@ -58,7 +60,49 @@ pc_status attend_simt(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void
     return st == PC_OK && hooks ? hooks->part_done(hooks->self, 0, n_q, stream) : st;
 }
 
+// The checks of a fused step up to the pack stage (scoring has its own): what the pack stage would refuse (a destination that
+// overlaps the source, a misaligned or missing buffer) is refused before the scoring stage enqueues anything.
+pc_status check_frame_step(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, const pc_cache *dst, const void *q, const int32_t *q_pos,
+                           int32_t n_q, const int32_t *sel_idx, const void *out, const float *lse, int64_t *n_sel_out) {
+    if (!ctx || !src || !dst || !budget) return PC_ERR_INVALID_ARG;
+    pc_status st = check_queries(ctx, q, q_pos, n_q, out, lse);
+    if (st != PC_OK) return st;
+    if (src->n_frames < 0 || (src->n_frames > 0 && !src->frame_count)) return PC_ERR_INVALID_ARG;
+    int64_t n_sel = 0;
+    for (int f = 0; f < src->n_frames; ++f) {
+        if (budget[f] < 0) return PC_ERR_INVALID_ARG;
+        n_sel += budget[f];
+    }
+    if (n_sel > dst->history.capacity) return PC_ERR_CAPACITY;
+    st = pc_check_segment(&src->anchors, true);
+    if (st != PC_OK) return st;
+    const int n_anchor = src->anchors.n_tokens;
+    if (n_anchor + n_sel == 0) return PC_ERR_INVALID_ARG;
+    if (n_anchor + n_sel > ctx->desc.max_keys) return PC_ERR_CAPACITY;
+    if (tensor_core_path(ctx) && (size_t)((n_anchor + STEP_TILE - 1) / STEP_TILE + (n_sel + STEP_TILE - 1) / STEP_TILE) * STEP_TILE > ctx->k_rot_rows)
+        return PC_ERR_CAPACITY;
+    *n_sel_out = n_sel;
+    return pc_compact_check(ctx, src, sel_idx, budget, dst, nullptr, nullptr);
+}
+
 }  // namespace
+
+pc_status pc_attend_frame_check(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
+                                int32_t n_q, const void *out, const float *lse) {
+    if (!ctx || !cache) return PC_ERR_INVALID_ARG;
+    const pc_status st = check_queries(ctx, q, q_pos, n_q, out, lse);
+    if (st != PC_OK) return st;
+    pc_segment segs[PC_MAX_SEGMENTS];
+    int n_seg = 0;
+    return gather_segments(ctx, cache, current, segs, &n_seg);
+}
+
+pc_status pc_frame_step_check(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, const pc_cache *dst, const void *q, const int32_t *q_pos,
+                              int32_t n_q, const float *scores, const int32_t *sel_idx, const void *out, const float *lse) {
+    int64_t n_sel = 0;
+    const pc_status st = check_frame_step(ctx, src, budget, dst, q, q_pos, n_q, sel_idx, out, lse, &n_sel);
+    return st != PC_OK ? st : pc_score_check(ctx, src, q, q_pos, n_q, budget, nullptr, scores, sel_idx);
+}
 
 pc_status pc_attend_frame_impl(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
                                int32_t n_q, void *out, float *lse, cudaStream_t stream, const pc_step_hooks *hooks) {
@@ -124,35 +168,17 @@ extern "C" pc_status pc_attend_prepared(pc_ctx *ctx, const void *q, const int32_
 pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, int32_t delta_t, pc_cache *dst, const void *q,
                              const int32_t *q_pos, int32_t n_q, float *scores, int32_t *sel_idx, void *out, float *lse,
                              cudaStream_t stream, const pc_step_hooks *hooks) {
-    if (!ctx || !src || !dst || !budget) return PC_ERR_INVALID_ARG;
-    pc_status st = check_queries(ctx, q, q_pos, n_q, out, lse);
-    if (st != PC_OK) return st;
-    if (src->n_frames < 0 || (src->n_frames > 0 && !src->frame_count)) return PC_ERR_INVALID_ARG;
     int64_t n_sel = 0;
-    for (int f = 0; f < src->n_frames; ++f) {
-        if (budget[f] < 0) return PC_ERR_INVALID_ARG;
-        n_sel += budget[f];
-    }
-    if (n_sel > dst->history.capacity) return PC_ERR_CAPACITY;
-    st = pc_check_segment(&src->anchors, true);
+    pc_status st = check_frame_step(ctx, src, budget, dst, q, q_pos, n_q, sel_idx, out, lse, &n_sel);
     if (st != PC_OK) return st;
     const int n_anchor = src->anchors.n_tokens;
-    if (n_anchor + n_sel == 0) return PC_ERR_INVALID_ARG;
-    if (n_anchor + n_sel > ctx->desc.max_keys) return PC_ERR_CAPACITY;
     const bool tc = tensor_core_path(ctx);
-    const int tile = 128;
-    const int anchor_tiles = (n_anchor + tile - 1) / tile;
     void *k_rot_dst = nullptr;
     if (tc) {
-        if ((size_t)(anchor_tiles + (n_sel + tile - 1) / tile) * tile > ctx->k_rot_rows) return PC_ERR_CAPACITY;
         const size_t row_bytes = (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim * sizeof(__nv_bfloat16);
-        k_rot_dst = static_cast<char *>(ctx->k_rot) + (size_t)anchor_tiles * tile * row_bytes;
+        k_rot_dst = static_cast<char *>(ctx->k_rot) + (size_t)((n_anchor + STEP_TILE - 1) / STEP_TILE) * STEP_TILE * row_bytes;
         ctx->prepared_n_seg = 0;                       // the scratch no longer holds a key set of pc_attend_prepare
     }
-    // what the pack stage would refuse (a destination that overlaps the source, a misaligned or missing buffer) is refused
-    // now, before the scoring stage enqueues anything
-    st = pc_compact_check(ctx, src, sel_idx, budget, dst, nullptr, nullptr);
-    if (st != PC_OK) return st;
     // (with values still on their way the selection need not wait for them; stage marks tell the two stages apart)
     const bool one_launch = !hooks && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
     ctx->last_n_q = 0;

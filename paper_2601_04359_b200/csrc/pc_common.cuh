@@ -261,6 +261,8 @@ pc_status pc_launch_pack(pc_ctx *ctx, const void *src_k, const void *src_v, cons
 // pc_score / pc_compact with the extras of the fused frame step: q_rot_out (NULL or the context's rotated-query scratch,
 // filled by the query pass that also pools), k_rot_dst (as pc_launch_pack)
 bool pc_score_supports(const pc_layer_desc &D);   // the row widths the query pass and the scoring kernel take
+pc_status pc_score_check(const pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
+                         const float *scores_override, const float *scores, const int32_t *sel_idx);   // every host-side check of pc_score_impl, nothing enqueued
 pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
                         const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
                         cudaStream_t stream, bool select = true);   // select = false: scores only, the caller selects
@@ -295,5 +297,10 @@ pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *bu
                              cudaStream_t stream, const pc_step_hooks *hooks);
 pc_status pc_attend_frame_impl(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
                                int32_t n_q, void *out, float *lse, cudaStream_t stream, const pc_step_hooks *hooks);
+// every host-side check of these two, nothing enqueued
+pc_status pc_frame_step_check(pc_ctx *ctx, const pc_cache *src, const int32_t *budget, const pc_cache *dst, const void *q, const int32_t *q_pos,
+                              int32_t n_q, const float *scores, const int32_t *sel_idx, const void *out, const float *lse);
+pc_status pc_attend_frame_check(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
+                                int32_t n_q, const void *out, const float *lse);
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
                                size_t *part_ml_floats);

@@ -438,9 +438,9 @@ bool pc_score_supports(const pc_layer_desc &D) {
     return qcpl / cpw <= 32;
 }
 
-pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
-                        const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
-                        cudaStream_t stream, bool select) {
+// Every host-side check of a scoring call, nothing enqueued.
+pc_status pc_score_check(const pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
+                         const float *scores_override, const float *scores, const int32_t *sel_idx) {
     if (!ctx || !src || !budget) return PC_ERR_INVALID_ARG;
     const int n_frames = src->n_frames;
     if (n_frames < 0 || (n_frames > 0 && !src->frame_count)) return PC_ERR_INVALID_ARG;
@@ -449,27 +449,42 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
     if (st != PC_OK) return st;
     const int n_src = src->history.n_tokens;
     if (n_src > ctx->desc.max_keys) return PC_ERR_CAPACITY;
-    FrameTab tab;
     int64_t first = 0, out = 0;
-    int longest = 0;
     for (int f = 0; f < n_frames; ++f) {
         const int n = src->frame_count[f], b = budget[f];
-        longest = std::max(longest, n);
         if (n < 0 || b < 0) return PC_ERR_INVALID_ARG;
         if (b > n) return PC_ERR_BUDGET;
-        tab.f[f] = make_int4((int)first, n, b, (int)out);
         first += n;
         out += b;
     }
     if (first != n_src) return PC_ERR_INVALID_ARG;
     if (out > 0 && (!sel_idx || !pc_aligned16(sel_idx))) return PC_ERR_INVALID_ARG;
+    if (scores_override) return reinterpret_cast<uintptr_t>(scores_override) & 3 ? PC_ERR_INVALID_ARG : PC_OK;   // read element by element: any float address will do
+    if (n_src == 0) return PC_OK;
+    if (!q || !q_pos || n_q <= 0 || !scores) return PC_ERR_INVALID_ARG;
+    if (!pc_aligned16(q) || !pc_aligned16(q_pos) || !pc_aligned16(scores)) return PC_ERR_INVALID_ARG;
+    if (n_q > ctx->desc.max_q) return PC_ERR_CAPACITY;
+    return pc_score_supports(ctx->desc) ? PC_OK : PC_ERR_UNSUPPORTED;
+}
+
+pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
+                        const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
+                        cudaStream_t stream, bool select) {
+    pc_status st = pc_score_check(ctx, src, q, q_pos, n_q, budget, scores_override, scores, sel_idx);
+    if (st != PC_OK) return st;
+    const int n_frames = src->n_frames, n_src = src->history.n_tokens;
+    FrameTab tab;
+    int first = 0, out = 0, longest = 0;
+    for (int f = 0; f < n_frames; ++f) {
+        const int n = src->frame_count[f], b = budget[f];
+        longest = std::max(longest, n);
+        tab.f[f] = make_int4(first, n, b, out);
+        first += n;
+        out += b;
+    }
     const float *select_on = scores_override;
     if (!scores_override) {
         if (n_src > 0) {
-            if (!q || !q_pos || n_q <= 0 || !scores) return PC_ERR_INVALID_ARG;
-            if (!pc_aligned16(q) || !pc_aligned16(q_pos) || !pc_aligned16(scores)) return PC_ERR_INVALID_ARG;
-            if (n_q > ctx->desc.max_q) return PC_ERR_CAPACITY;
-            if (!pc_score_supports(ctx->desc)) return PC_ERR_UNSUPPORTED;      // before anything is enqueued
             const size_t row = (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim;
             if (ctx->qpool_dirty) {          // an earlier call stopped between the query pass and the scoring kernel
                 PC_CUDA_TRY(cudaMemsetAsync(ctx->qpool_fx, 0, (row + 1) * sizeof(long long), stream));
@@ -487,8 +502,6 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
             if (q_rot_out) ctx->q_rot_n = n_q;
         }
         select_on = scores;
-    } else if (reinterpret_cast<uintptr_t>(scores_override) & 3) {      // read element by element: any float address will do
-        return PC_ERR_INVALID_ARG;
     }
     if (select && n_frames > 0 && out > 0) {
         if (scores_override) pc_mark(ctx, PC_MARK_SCORE, stream);

@@ -294,28 +294,53 @@ extern "C" pc_status pc_window_update(pc_window *w, const void *q, const int32_t
 
 namespace {
 
+// what attention runs over where nothing is packed: the window as it is, or (every frame leaves) none of it
+pc_cache unpacked_cache(const pc_window *w, const WindowPlan &pl) {
+    pc_cache cache;
+    cache.anchors = w->anchors;
+    cache.history = w->buf[w->active];
+    if (!pl.fill) cache.history.n_tokens = 0;
+    cache.n_frames = pl.fill ? (int32_t)w->count.size() : 0;
+    cache.frame_count = w->count.data();
+    return cache;
+}
+pc_cache pack_destination(const pc_window *w, const WindowPlan &pl) {
+    pc_cache dst;
+    dst.anchors = w->anchors;
+    dst.history = w->buf[w->active ^ 1];
+    dst.n_frames = pl.stay;
+    dst.frame_count = pl.budget;
+    return dst;
+}
+
+// The plan and every other host-side check of a step, nothing enqueued.
+pc_status window_step_check(pc_window *w, const void *q, const int32_t *q_pos, int32_t n_q, const void *out) {
+    WindowPlan pl;
+    const pc_status st = window_plan(w, nullptr, &pl);
+    if (st != PC_OK) return st;
+    if (pl.fill || pl.stay == 0) {
+        const pc_cache cache = unpacked_cache(w, pl);
+        return pc_attend_frame_check(w->ctx, &cache, nullptr, q, q_pos, n_q, out, nullptr);
+    }
+    const pc_cache dst = pack_destination(w, pl);
+    return pc_frame_step_check(w->ctx, &pl.src, pl.budget, &dst, q, q_pos, n_q, w->scores, w->sel_idx, out, nullptr);
+}
+
+// A step that fails leaves the window as it was.
 pc_status window_step(pc_window *w, const void *q, const int32_t *q_pos, int32_t n_q, void *out, float *lse, int32_t *regime,
                       cudaStream_t stream, const pc_step_hooks *hooks) {
     WindowPlan pl;
     pc_status st = window_plan(w, nullptr, &pl);
     if (st != PC_OK) return st;
     if (pl.fill || pl.stay == 0) {
-        if (!pl.fill) window_commit(w, pl);
-        pc_cache cache;
-        cache.anchors = w->anchors;
-        cache.history = w->buf[w->active];
-        cache.n_frames = (int32_t)w->count.size();
-        cache.frame_count = w->count.data();
+        const pc_cache cache = unpacked_cache(w, pl);
         st = pc_attend_frame_impl(w->ctx, &cache, nullptr, q, q_pos, n_q, out, lse, stream, hooks);
         if (st != PC_OK) return st;
+        if (!pl.fill) window_commit(w, pl);
         if (regime) *regime = pl.fill ? PC_WINDOW_FILL : (pl.left ? PC_WINDOW_SLIDE : PC_WINDOW_PACK);
         return PC_OK;
     }
-    pc_cache dst;
-    dst.anchors = w->anchors;
-    dst.history = w->buf[w->active ^ 1];
-    dst.n_frames = pl.stay;
-    dst.frame_count = pl.budget;
+    pc_cache dst = pack_destination(w, pl);
     st = pc_frame_step_impl(w->ctx, &pl.src, pl.budget, pl.delta_t, &dst, q, q_pos, n_q, w->scores, w->sel_idx, out, lse, stream, hooks);
     if (st != PC_OK) return st;
     window_commit(w, pl);
@@ -364,22 +389,22 @@ extern "C" pc_status pc_window_step_host(pc_window *w, const pc_host_window_step
         if ((int64_t)A.n_tokens + n > A.capacity || (int64_t)A.n_tokens + n > w->scratch_capacity) return PC_ERR_CAPACITY;
         if ((int)w->count.size() + 1 > PC_MAX_FRAMES) return PC_ERR_CAPACITY;
     }
-    // The plan of the step is tried on the window as it will be with the frame appended (host arithmetic only); if it
-    // cannot be made (budget, capacity of the other buffer), the window is left as it was and nothing is enqueued.
+    // The step is planned and checked on the window as it will be with the frame appended (host arithmetic only); if it cannot be
+    // made, the window is left as it was and nothing is enqueued.
     if (n > 0) {
         A.n_tokens += n;
         w->count.push_back(n);
     }
-    {
-        WindowPlan trial;
-        const pc_status st = window_plan(w, nullptr, &trial);
-        if (st != PC_OK) {
-            if (n > 0) {
-                A.n_tokens -= n;
-                w->count.pop_back();
-            }
-            return st;
+    const auto take_back = [&]() {
+        if (n > 0) {
+            A.n_tokens -= n;
+            w->count.pop_back();
         }
+    };
+    pc_status st = window_step_check(w, ws->q, ws->q_pos, in->n_q, ws->out);
+    if (st != PC_OK) {
+        take_back();
+        return st;
     }
     // Every argument is checked: from here on work is enqueued.  What the scores need goes first, on the caller's stream: the
     // queries, then the finished frame's keys and positions, straight to the end of the active history buffer.  Its values
@@ -403,11 +428,15 @@ extern "C" pc_status pc_window_step_host(pc_window *w, const pc_host_window_step
         const pc_step_hooks hooks{w->side_ev, send_home, &trip};
         return window_step(w, ws->q, ws->q_pos, in->n_q, ws->out, nullptr, regime, stream, &hooks);
     };
-    const pc_status st = enqueue();
-    const cudaError_t side = cudaStreamSynchronize(w->side);         // also after an error: nothing of this call stays in flight
-    if (st != PC_OK) return st;
+    st = enqueue();
+    // also after an error: nothing of this call stays in flight, and the frame is not counted as appended
+    const cudaError_t side = cudaStreamSynchronize(w->side), main = cudaStreamSynchronize(stream);
+    if (st != PC_OK) {
+        take_back();
+        return st;
+    }
     PC_CUDA_TRY(side);
-    PC_CUDA_TRY(cudaStreamSynchronize(stream));
+    PC_CUDA_TRY(main);
     return PC_OK;
 }
 

@@ -23,3 +23,62 @@ def test_window_belongs_to_the_device_of_its_context(rt):
     for n in range(1, 4):                                 # fill, then pack
         c.step_host(win)
         assert len(counts(win)) == n
+
+
+def _refused(win, case, log, **kw):
+    before, (_, _, active) = counts(win), win.state()
+    case.rt.reset()
+    with pytest.raises(pc.PackCacheError) as e:
+        case.step_host(win, **kw)
+    assert counts(win) == before and win.state()[2] == active
+    if not log:
+        assert case.rt.log() == []                        # nothing was enqueued
+    return e.value.status
+
+
+def test_host_step_checks_before_it_enqueues(rt):
+    c = Case(rt)
+    win = c.make()
+    skew = torch.zeros(c.ws["q"].numel() + 8, dtype=torch.bfloat16)[1:1 + c.ws["q"].numel()].view_as(c.ws["q"])
+    for f in range(3):                                    # fill, fill to the brim, pack
+        for name in ("q", "out"):
+            assert _refused(win, c, False, **{name: skew}) == pc.PC_ERR_INVALID_ARG
+        c.step_host(win)
+        assert len(counts(win)) == f + 1
+    few = Case(rt, max_keys=200)                          # 37 anchors and 130 tokens fit, two frames (packed to 200 tokens) do not
+    win = few.make()
+    few.step_host(win)
+    assert _refused(win, few, False) == pc.PC_ERR_CAPACITY
+    odd = Case(rt, heads=(10, 5, 128))                    # key rows of 1,280 bytes: attention takes them, scoring does not
+    win = odd.make()
+    odd.step_host(win)
+    assert _refused(win, odd, False) == pc.PC_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("frames", [0, 1, 2])
+def test_host_step_that_fails_leaves_the_window_and_nothing_in_flight(rt, frames):
+    c = Case(rt)
+    win = c.make()
+    for _ in range(frames):
+        c.step_host(win)
+    rt.reset()
+    probe = c.make()
+    for _ in range(frames + 1):
+        rt.reset()
+        c.step_host(probe)
+    calls = [line.split()[0] for line in rt.log()]
+    for name in ("memcpy", "record", "wait", "launch"):
+        for at in range(calls.count(name)):
+            rt.reset()
+            rt.fail(name, at)
+            before, active = counts(win), win.state()[2]
+            with pytest.raises(pc.PackCacheError) as e:
+                c.step_host(win)
+            assert e.value.status == pc.PC_ERR_CUDA
+            assert counts(win) == before and win.state()[2] == active
+            assert sorted(rt.log()[-2:]) == ["synchronize main", "synchronize side"]
+    rt.reset()
+    c.frame.k.fill_(3.0)
+    c.step_host(win)                                      # and the same step still works
+    assert len(counts(win)) == frames + 1
+    assert counts(win) == counts(probe)
