@@ -11,6 +11,7 @@
 // and the angle is the same for every KV head, so the two brackets are summed over heads first and each pair costs
 // one table look-up per token.
 #include <algorithm>
+#include <atomic>
 
 #include "pc_common.cuh"
 #include "pc_select.cuh"
@@ -52,6 +53,7 @@ template <> struct Elem<__nv_bfloat16> {
 // sixteen 9.0 / 14.6 / 7.8; two or four copies of the accumulator 7.8 to 8.4 at 1,008.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int QPREP_WARPS = 16;                     // most warps per block, unless one token needs more
+constexpr int QPREP_SLAB = 200 * 1024;              // most shared memory of a block (one token takes up to 128 KB: 32 parts of 4 x 32 chunks)
 constexpr float FX_ONE = 4294967296.0f;             // 2^32
 
 template <typename T> __device__ __forceinline__ uint4 pack_row(const float *f);
@@ -349,7 +351,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     const int parts = qcpl / cpw;
     if (parts > 32) return PC_ERR_UNSUPPORTED;
     int slots = std::max(1, QPREP_WARPS / parts);
-    slots = std::max(1, std::min<int>(slots, (int)((200u * 1024u) / ((size_t)q_row * sizeof(float)))));
+    slots = std::max(1, std::min<int>(slots, (int)(QPREP_SLAB / ((size_t)q_row * sizeof(float)))));
     const int q_smem = slots * q_row * (int)sizeof(float);
     const int q_threads = slots * parts * 32;
     int dev_id = 0;
@@ -358,18 +360,20 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     if (marks) pc_mark(marks, PC_MARK_SCORE0, stream);
 #define PC_QPREP_LAUNCH(CPW, MAX_THREADS)                                                                            \
     {                                                                                                               \
-        /* largest dynamic size allowed so far, and resident blocks per SM at the size they were looked up for */   \
-        static int smem_of[PC_MAX_DEVICES] = {}, occ_of[PC_MAX_DEVICES] = {}, occ_at[PC_MAX_DEVICES] = {};          \
-        if (q_smem + 1024 > 48 * 1024 && smem_of[dev_id] < q_smem) {   /* the block's static words count, too */    \
-            PC_CUDA_TRY(cudaFuncSetAttribute(k_qprep<T, CPW, MAX_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, q_smem)); \
-            smem_of[dev_id] = q_smem;                                                                               \
+        /* Shared by every context and thread.  The limit on dynamic shared memory is one number of the kernel's, so it is set */ \
+        /* to the most a call can ask for; resident blocks go with their key in one word, so no reader sees half of a pair. */ \
+        static std::atomic<bool> set[PC_MAX_DEVICES];                                                               \
+        static std::atomic<uint64_t> occ_of[PC_MAX_DEVICES];                                                        \
+        if (!set[dev_id]) {                                                                                         \
+            PC_CUDA_TRY(cudaFuncSetAttribute(k_qprep<T, CPW, MAX_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, QPREP_SLAB)); \
+            set[dev_id] = true;                                                                                     \
         }                                                                                                           \
-        int occ = occ_at[dev_id] == q_smem + q_threads ? occ_of[dev_id] : 0;                                        \
+        const uint64_t key = (uint64_t)(q_smem + q_threads) << 32, known = occ_of[dev_id];                          \
+        int occ = (known ^ key) >> 32 ? 0 : (int)known;                                                             \
         if (occ == 0) {                                                                                             \
             PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qprep<T, CPW, MAX_THREADS>, q_threads, q_smem)); \
             occ = std::max(1, occ);                                                                                 \
-            occ_of[dev_id] = occ;                                                                                   \
-            occ_at[dev_id] = q_smem + q_threads;                                                                    \
+            occ_of[dev_id] = key | (uint32_t)occ;                                                                   \
         }                                                                                                           \
         const int q_blocks = std::min((n_q + slots - 1) / slots, sm_count * occ);                                   \
         PC_LAUNCH((k_qprep<T, CPW, MAX_THREADS>), dim3(q_blocks), dim3(q_threads), q_smem, stream,                  \

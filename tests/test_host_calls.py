@@ -82,3 +82,23 @@ def test_host_step_that_fails_leaves_the_window_and_nothing_in_flight(rt, frames
     c.step_host(win)                                      # and the same step still works
     assert len(counts(win)) == frames + 1
     assert counts(win) == counts(probe)
+
+
+def test_two_threads_scoring_rows_of_different_width(rt):
+    """The query pass of 32 heads x 128 takes 64 KB of shared memory a block, that of 40 heads 60 KB, in the same kernel.  The
+    second thread's first call comes while the first one's is between raising the limit and launching."""
+    cases = [Case(rt, heads=(hq, 8, 128), n=8) for hq in (32, 40)]
+    cache, budget = pc.Cache(pc.Segment.empty(), cases[0].frame, np.array([8], np.int32)), (C.c_int32 * 1)(4)
+    scores, sel = torch.zeros(8), torch.zeros(8, dtype=torch.int32)
+    status = []
+
+    def score(c):
+        s = cache.c()
+        status.append(rt.lib.pc_score(c.ctx.handle, C.byref(s), pc._ptr(c.q), pc._ptr(c.q_pos), 8, budget, None, None, pc._ptr(scores), pc._ptr(sel), None))
+
+    other = CALLBACK(lambda: score(cases[1]))
+    rt.lib.rt_on_attribute(other)
+    score(cases[0])
+    score(cases[1])
+    score(cases[0])
+    assert status == [pc.PC_OK] * 4
