@@ -635,8 +635,7 @@ extern "C" pc_status pc_score_tokens_static(const pc_layer_desc *desc, const voi
     if (D.n_q_heads <= 0 || D.n_kv_heads <= 0 || D.n_q_heads % D.n_kv_heads) return PC_ERR_UNSUPPORTED;
     if (!(D.rope_base > 1.0)) return PC_ERR_INVALID_ARG;
     const int row = D.n_kv_heads * D.head_dim;
-    const int per = D.dtype == PC_BF16 ? 8 : 4;
-    if ((row / per) % 32 || (D.n_q_heads * D.head_dim / per) % 32) return PC_ERR_UNSUPPORTED;
+    if (!pc_score_supports(D)) return PC_ERR_UNSUPPORTED;                      // before anything is enqueued
     int64_t rope_entries = 0;
     for (int a = 0; a < 3; ++a) {
         if (D.max_pos[a] <= 0 || D.max_pos[a] > (1 << 20)) return PC_ERR_INVALID_ARG;

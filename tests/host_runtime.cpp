@@ -139,14 +139,8 @@ void **__cudaRegisterFatBinary(void *) { static void *handle; return &handle; }
 void __cudaRegisterFatBinaryEnd(void **) {}
 void __cudaUnregisterFatBinary(void **) {}
 void __cudaRegisterFunction(void **, const char *host, char *, const char *name, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {
-    // the kernel's own name out of the mangled one: a length, then k_...
-    const char *k = strstr(name, "k_");
-    std::string s = k ? k : name;
-    if (k) {
-        const char *d = k;
-        while (d > name && d[-1] >= '0' && d[-1] <= '9') --d;
-        s = s.substr(0, (size_t)atoi(d));
-    }
+    const char *k = strstr(name, "k_");              // the kernel's own name out of the mangled one (small letters and underscores)
+    const std::string s = k ? std::string(k, strspn(k, "abcdefghijklmnopqrstuvwxyz_")) : name;
     g_name[host] = s;
 }
 void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, int) {}

@@ -102,3 +102,13 @@ def test_two_threads_scoring_rows_of_different_width(rt):
     score(cases[1])
     score(cases[0])
     assert status == [pc.PC_OK] * 4
+
+
+@pytest.mark.parametrize("n_kv,status", [(4, pc.PC_OK), (5, pc.PC_ERR_UNSUPPORTED), (6, pc.PC_OK), (7, pc.PC_ERR_UNSUPPORTED), (8, pc.PC_OK)])
+def test_static_scoring_takes_the_row_widths_that_scoring_takes(rt, n_kv, status):
+    """fp32 key rows of n_kv x 512 bytes: 2,560 and 3,584 are refused with nothing enqueued."""
+    desc = pc.pc_layer_desc(n_kv, n_kv, 128, pc.PC_F32, 10000.0, (C.c_int32 * 3)(64, 64, 64), 0, 0)
+    k, pos, out, word = torch.zeros(8, n_kv, 128), torch.zeros(8, 4, dtype=torch.int32), torch.zeros(8), torch.zeros(2, dtype=torch.int32)
+    got = rt.lib.pc_score_tokens_static(C.byref(desc), pc._ptr(k), pc._ptr(pos), 8, pc._ptr(k), pc._ptr(pos), 8, None, pc._ptr(out), pc._ptr(word), None)
+    assert got == status
+    assert [line.split()[1] for line in rt.log()] == (["k_rope_table", "k_qprep", "k_score"] if status == pc.PC_OK else [])
