@@ -384,13 +384,15 @@ pc_status pc_set_kv_splits(pc_ctx *ctx, int32_t n);
  * number of work items fits that; results agree up to fp32 rounding order. */
 pc_status pc_set_cluster_merge(pc_ctx *ctx, int32_t on);
 
-/* Limit of every bounded device-side wait of the context's tensor-core attention kernel, in microseconds (0 = the
- * default of about one second).  A wait that runs out records PC_ERR_TIMEOUT in the status word, the CTA gives up its
- * remaining work, lets its copies land, frees its tensor memory and exits; the context stays usable. */
+/* Limit of every bounded device-side wait of the context's kernels (scoring, tensor-core attention, attention mass), in
+ * microseconds (0 = the default of about one second; pc_score_tokens_static, which has no context, always waits by the
+ * default).  A wait that runs out records PC_ERR_TIMEOUT in the status word, the CTA gives up its remaining work, lets its
+ * copies land, frees its tensor memory and exits; the outputs that depended on it are undefined (scores keep what their buffer
+ * held) and the context stays usable. */
 pc_status pc_set_wait_limit_us(pc_ctx *ctx, uint32_t limit_us);
-/* Test hook for that path: the attention kernel's first barrier of every CTA is told to expect n_bytes more than are
- * ever sent, so its wait runs out after the limit above and pc_poll_status returns PC_ERR_TIMEOUT; the call's output
- * is then undefined.  0 switches the hook off.  Nothing traps and nothing waits without a limit. */
+/* Test hook for that path: the first barrier of every CTA of the attention and mass kernels, and of every warp of the scoring
+ * kernel, is told to expect n_bytes more than are ever sent, so its wait runs out after the limit above and pc_poll_status
+ * returns PC_ERR_TIMEOUT; the call's output is then undefined.  0 switches the hook off.  Nothing traps and nothing waits without a limit. */
 pc_status pc_test_expect_extra_bytes(pc_ctx *ctx, uint32_t n_bytes);
 
 /* Per-kernel timing for benchmarks.  With timing on, each call records CUDA events on its stream at the boundaries

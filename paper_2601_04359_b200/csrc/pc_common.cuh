@@ -69,7 +69,7 @@ struct pc_ctx {
     int kv_splits;             // 0 = chosen per call
     int cluster_merge;         // 1 = KV ranges merge inside the kernel through cluster shared memory (default 0)
     uint32_t wait_limit_us;    // limit of every bounded device-side wait in microseconds; 0 = about one second
-    uint32_t test_extra_tx;    // test hook: bytes the attention kernel's first barrier expects beyond what is sent (0 = off)
+    uint32_t test_extra_tx;    // test hook: bytes the first barrier of the waiting kernels expects beyond what is sent (0 = off)
     // rotated anchor keys kept in k_rot across fused frame steps (anchors never move): the segment they were made from
     const void *anchor_rot_k;
     const int32_t *anchor_rot_pos;

@@ -59,6 +59,8 @@ struct MassParams {
     int32_t *status;
     int n_cta, n_steps;    // persistent CTAs; steps (query tiles of the head's group) of a unit
     int run, longer;       // steps of a CTA's run; the first `longer` CTAs take one more
+    uint32_t wait_us;      // limit of every bounded wait in microseconds (0 = about one second)
+    uint32_t extra_tx;     // test hook: bytes the first barrier expects beyond what is sent (0 = off)
 };
 __host__ __device__ __forceinline__ int run_start(const MassParams &P, int c) { return c * P.run + min(c, P.longer); }
 // the CTA whose run holds step x
@@ -130,9 +132,9 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
                 const int n = min(P.n_steps - s0, G1 - x);
                 const int g = unit / P.pairs, jt0 = 2 * (unit % P.pairs);
                 x += n;
-                if (un > 0) alive = mbar_wait(bar(BAR_KFREE), (un - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                if (un > 0) alive = mbar_wait(bar(BAR_KFREE), (un - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
                 if (!alive) break;
-                mbar_expect_tx(bar(BAR_K), 2 * TILE_BYTES);
+                mbar_expect_tx(bar(BAR_K), 2 * TILE_BYTES + (un == 0 ? P.extra_tx : 0u));
                 for (int t = 0; t < 2; ++t) {
                     const int jt = min(jt0 + t, P.n_kv_tiles - 1);       // an odd tile count: the last tile twice, one copy dropped
                     tma_load_2d(base + SM_K + t * TILE_BYTES, &map_k, g * TILE, jt * TILE, bar(BAR_K));
@@ -140,7 +142,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
                 }
                 for (int s = s0; s < s0 + n && alive; ++s, ++gs) {
                     const int st = gs % Q_STAGES, use = gs / Q_STAGES;
-                    if (use > 0) alive = mbar_wait(bar(BAR_QEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                    if (use > 0) alive = mbar_wait(bar(BAR_QEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
                     if (!alive) break;
                     const int tb = s / P.group, h = g * P.group + s % P.group;
                     mbar_expect_tx(bar(BAR_QFULL + st), TILE_BYTES);
@@ -169,12 +171,12 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         for (int x = G0; x < G1 && alive; ++un) {
             const int n = min(P.n_steps - x % P.n_steps, G1 - x);
             x += n;
-            alive = mbar_wait(bar(BAR_K), un & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+            alive = mbar_wait(bar(BAR_K), un & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
             for (int s = 0; s < n && alive; ++s, ++gs) {
                 const int st = gs % Q_STAGES, quse = gs / Q_STAGES, b = gs & 1, use = gs >> 1;
-                alive = mbar_wait(bar(BAR_QFULL + st), quse & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                alive = mbar_wait(bar(BAR_QFULL + st), quse & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
                 for (int t = 0; t < 2 && alive; ++t) {
-                    if (use > 0) alive = mbar_wait(bar(BAR_SEMPTY + 2 * t + b), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+                    if (use > 0) alive = mbar_wait(bar(BAR_SEMPTY + 2 * t + b), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
                     if (!alive) break;
                     tc_fence_after();
                     const uint32_t ka = base + SM_K + t * TILE_BYTES, qa = base + SM_Q + st * TILE_BYTES;
@@ -192,7 +194,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         // nothing of ours may still be running on the tensor core when TMEM is freed
         if (lead) tc_commit(bar(BAR_DONE));
         __syncwarp();
-        mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_MASS_WAIT);
+        mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
     } else if (warp >= 4) {
         // ---------------------------------------------------------------- column sums: one key and 64 query columns per thread
         const int cw = warp - 4;
@@ -207,8 +209,8 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         int unit_left = min((unit + 1) * P.n_steps, G1) - G0;    // steps of the run that are left in the unit
         for (int s = 0; s < G1 - G0 && alive; ++s) {
             const int b = s & 1, use = s >> 1, slot = s % L_SLOTS;
-            alive = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SFULL + 2 * t + b), use & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT) &&
-                                                mbar_wait(bar(BAR_LFULL + slot), (s / L_SLOTS) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT));
+            alive = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SFULL + 2 * t + b), use & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us) &&
+                                                mbar_wait(bar(BAR_LFULL + slot), (s / L_SLOTS) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us));
             if (!alive) break;
             tc_fence_after();
             uint32_t sv[64];
@@ -353,6 +355,8 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
     P.part = ctx->mass_part;
     P.norm = ctx->mass_norm;
     P.status = ctx->status;
+    P.wait_us = ctx->wait_limit_us;
+    P.extra_tx = ctx->test_extra_tx;
 
     CUtensorMap mq, mk;
     if (!make_map(&mq, ctx->q_rot, (uint64_t)P.n_q, (uint64_t)D.n_q_heads * D.head_dim) ||

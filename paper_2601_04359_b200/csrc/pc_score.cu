@@ -169,7 +169,7 @@ template <typename T, int LPT /* lanes per token */, int TPL /* tokens per lane 
 __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restrict__ k, const int32_t *__restrict__ k_pos,
                                                                const uint8_t *__restrict__ valid, int n_src, int d, int parts, int stages, float scale,
                                                                pc_rope_dev rope, unsigned long long *fx, double fx_scale,
-                                                               float *__restrict__ scores, int32_t *status) {
+                                                               float *__restrict__ scores, int32_t *status, uint32_t wait_us, uint32_t extra_tx) {
     pc_grid_dep_launch();
     constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL;
     extern __shared__ __align__(128) unsigned char score_smem[];
@@ -183,16 +183,16 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
     const uint32_t bar0 = pc_smem_u32(bars) + warp * SCORE_STAGES * 8;
     int grp = warp * gridDim.x + blockIdx.x;                          // small calls spread over the blocks first
 
-    auto fill = [&](int stage, int group) {                           // one lane
+    auto fill = [&](int stage, int group, uint32_t extra = 0) {       // one lane
         const uint32_t bytes = (uint32_t)(min(TOK, n_src - group * TOK) * row_bytes);
-        pc_mbar_expect_tx(bar0 + 8 * stage, bytes);
+        pc_mbar_expect_tx(bar0 + 8 * stage, bytes + extra);
         pc_bulk_g2s(ring + stage * stage_bytes, reinterpret_cast<const char *>(k) + (size_t)group * stage_bytes, bytes, bar0 + 8 * stage);
     };
     if (lane == 0) {
         for (int s = 0; s < stages; ++s) pc_mbar_init(bar0 + 8 * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int s = 0; s < stages && grp + s * step < n_groups; ++s) fill(s, grp + s * step);
+        for (int s = 0; s < stages && grp + s * step < n_groups; ++s) fill(s, grp + s * step, s == 0 ? extra_tx : 0u);
     }
     if (threadIdx.x == 0) gave_up = 0;
     int4 p[TPL];
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
 #pragma unroll
         for (int i = 0; i < TPL; ++i) table(p[i], cs[i]);
         if (grp + step < n_groups) positions(grp + step);
-        if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT))) break;
+        if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT, wait_us))) break;
         // brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair
         float2 A[TPL][NP], B[TPL][NP];
 #pragma unroll
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(THREADS) k_select(const float *__restrict__ sc
 template <typename T>
 pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev &rope, long long *fx, int32_t *status, const void *hist_k, const int32_t *hist_pos, int n_src, const void *q,
                         const int32_t *q_pos, int32_t n_q, const uint8_t *valid, float *scores, void *q_rot, float q_scale,
-                        cudaStream_t stream, pc_ctx *marks) {
+                        cudaStream_t stream, pc_ctx *ctx /* whose marks and wait limit; NULL: none */) {
     constexpr int PER = Elem<T>::PER16;
     const int row = D.n_kv_heads * D.head_dim;
     const int group = D.n_q_heads / D.n_kv_heads;
@@ -357,7 +357,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     int dev_id = 0;
     PC_CUDA_TRY(cudaGetDevice(&dev_id));
     if (dev_id < 0 || dev_id >= PC_MAX_DEVICES) return PC_ERR_UNSUPPORTED;
-    if (marks) pc_mark(marks, PC_MARK_SCORE0, stream);
+    if (ctx) pc_mark(ctx, PC_MARK_SCORE0, stream);
 #define PC_QPREP_LAUNCH(CPW, MAX_THREADS)                                                                            \
     {                                                                                                               \
         /* Shared by every context and thread.  The limit on dynamic shared memory is one number of the kernel's, so it is set */ \
@@ -391,7 +391,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
 #undef PC_QPREP_CASE
 #undef PC_QPREP_LAUNCH
     PC_CUDA_TRY(cudaGetLastError());
-    if (marks) pc_mark(marks, PC_MARK_QPOOL, stream);
+    if (ctx) pc_mark(ctx, PC_MARK_QPOOL, stream);
     const float scale = (float)(1.0 / ((double)D.n_q_heads * std::sqrt((double)D.head_dim)));
     const T *k = static_cast<const T *>(hist_k);
     const int lpt = std::max(16, D.head_dim / PER), row_bytes = row * (int)sizeof(T);
@@ -415,7 +415,8 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
             set[dev_id] = true;                                                                                     \
         }                                                                                                           \
         PC_LAUNCH((k_score<T, LPT, TPL>), dim3(blocks), dim3(warps * 32), smem, stream, k, hist_pos, valid, n_src, D.head_dim, row_bytes / (lpt * 16), stages, scale, \
-                  rope, reinterpret_cast<unsigned long long *>(fx), fx_scale, scores, status);                       \
+                  rope, reinterpret_cast<unsigned long long *>(fx), fx_scale, scores, status,                        \
+                  ctx ? ctx->wait_limit_us : 0u, ctx ? ctx->test_extra_tx : 0u);                            \
     }
     if (lpt == 16) {
         if (two) PC_SCORE_CASE(16, 2) else PC_SCORE_CASE(16, 1)
@@ -424,7 +425,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     }
 #undef PC_SCORE_CASE
     PC_CUDA_TRY(cudaGetLastError());
-    if (marks) pc_mark(marks, PC_MARK_SCORE, stream);
+    if (ctx) pc_mark(ctx, PC_MARK_SCORE, stream);
     return PC_OK;
 }
 

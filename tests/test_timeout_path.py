@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2601_04359_b200 import binding as pc
@@ -41,4 +42,50 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_survives():
     assert (again.view(dtype=good.dtype) == good).all()
     want = oracle.attend(L.q, L.q_pos, [(L.anchor_k, L.anchor_v, L.anchor_pos), (L.hist_k, L.hist_v, L.hist_pos)], cfg.rope_base)
     check_bf16_attention(host(again).astype(np.float64), want)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_frames,grid", [(2, (8, 9)), (9, (24, 42))])        # one group a warp, and a ring that goes round
+def test_a_scoring_wait_that_runs_out(n_frames, grid):
+    """The scoring kernel gives up, its last block still clears the pooled query's accumulator and ticket, and the next
+    call's scores are the ones of a fresh context."""
+    cfg = wl.small_bf16(n_frames=n_frames, grid=grid, seed=61)
+    D = DeviceLayer(wl.make_layer(cfg))
+    ctx = make_ctx(cfg)
+    budget = np.full(n_frames, 7, np.int32)
+    good, good_sel = pc.pc_score(ctx, D.cache, D.q, D.q_pos, budget)
+    assert pc.pc_poll_status(ctx) == pc.PC_OK
+
+    pc.pc_set_wait_limit_us(ctx, 2000)
+    pc.pc_test_expect_extra_bytes(ctx, 16)
+    pc.pc_score(ctx, D.cache, D.q, D.q_pos, budget)
+    assert pc.pc_poll_status(ctx) == pc.PC_ERR_TIMEOUT
+    assert pc.pc_poll_status(ctx) == pc.PC_OK
+
+    pc.pc_test_expect_extra_bytes(ctx, 0)
+    pc.pc_set_wait_limit_us(ctx, 0)
+    again, again_sel = pc.pc_score(ctx, D.cache, D.q, D.q_pos, budget)
+    assert pc.pc_poll_status(ctx) == pc.PC_OK
+    assert torch.equal(again, good) and torch.equal(again_sel, good_sel)
+    ctx.close()
+
+
+def test_a_mass_wait_that_runs_out():
+    cfg = wl.small_bf16(n_frames=2, grid=(8, 9), seed=62)
+    D = DeviceLayer(wl.make_layer(cfg))
+    ctx = make_ctx(cfg)
+    n_keys = cfg.n_anchor + cfg.n_src
+    _, lse = pc.pc_attend_frame(ctx, D.cache, None, D.q, D.q_pos, want_lse=True)
+    good = pc.pc_attend_mass(ctx, lse, n_keys)
+    assert pc.pc_poll_status(ctx) == pc.PC_OK
+
+    pc.pc_set_wait_limit_us(ctx, 2000)
+    pc.pc_test_expect_extra_bytes(ctx, 16)
+    pc.pc_attend_mass(ctx, lse, n_keys)
+    assert pc.pc_poll_status(ctx) == pc.PC_ERR_TIMEOUT
+
+    pc.pc_test_expect_extra_bytes(ctx, 0)
+    pc.pc_set_wait_limit_us(ctx, 0)
+    again = pc.pc_attend_mass(ctx, lse, n_keys)
+    assert pc.pc_poll_status(ctx) == pc.PC_OK and torch.equal(again, good)
     ctx.close()
