@@ -76,11 +76,12 @@ void *handle_of(PyObject *h) {                        // a ctypes c_void_p, or N
 
 void *stream_of(PyObject *s) { return PyLong_AsVoidPtr(s); }
 
-// A host array of int32, held for the duration of a call.
+// A host array of int32 with any number of dimensions, held for the duration of a call.
 struct Ints {
     Py_buffer view{};
     const int32_t *p = nullptr;
-    int32_t n = 0;
+    int32_t n = 0;            // its length (first extent)
+    int64_t size = 0;         // elements in all
     bool take(PyObject *o) {
         if (!as_is(o)) {
             PyObject *a = PyObject_CallOneArg(g_as_i32, o);
@@ -101,13 +102,14 @@ struct Ints {
             return false;
         }
         const char *f = view.format ? view.format : "B";
-        if (view.itemsize != 4 || view.ndim != 1 || f[1] != '\0' || (f[0] != 'i' && f[0] != 'l')) {
+        if (view.itemsize != 4 || view.ndim < 1 || f[1] != '\0' || (f[0] != 'i' && f[0] != 'l')) {
             PyBuffer_Release(&view);
             view = Py_buffer{};
             return false;
         }
         p = static_cast<const int32_t *>(view.buf);
         n = (int32_t)view.shape[0];
+        size = view.len / 4;
         return true;
     }
     ~Ints() {
@@ -199,7 +201,7 @@ PyObject *total(PyObject *, PyObject *const *a, Py_ssize_t n) {             // s
     Ints v;
     if (!v.take(a[0])) return nullptr;
     int64_t s = 0;
-    for (int32_t i = 0; i < v.n; ++i) s += v.p[i];
+    for (int64_t i = 0; i < v.size; ++i) s += v.p[i];
     return PyLong_FromLongLong(s);
 }
 

@@ -10,7 +10,8 @@ from paper_2601_04359_b200 import binding as pc
 
 
 @pytest.mark.parametrize("make", [list, tuple, lambda a: np.array(a, np.int64), lambda a: np.array(a, np.int32),
-                                  lambda a: np.array(a, np.int32).repeat(2)[::2], lambda a: torch.tensor(a, dtype=torch.int32)])
+                                  lambda a: np.array(a, np.int32).repeat(2)[::2], lambda a: torch.tensor(a, dtype=torch.int32),
+                                  lambda a: np.array(a, np.int32)[:, None]])
 def test_host_arrays_of_any_integer_kind(make):
     avail = [40, 7, 100, 0, 64]
     want = pc.pc_plan_budget(pc.PC_LINEAR, 0.0, 90, 0, np.array(avail, np.int32))
