@@ -112,6 +112,12 @@ struct Ints {
         size = view.len / 4;
         return true;
     }
+    // the library reads (or writes) this many entries: a shorter array is an error
+    bool holds(int32_t want, const char *what) const {
+        if (size >= want) return true;
+        PyErr_Format(PyExc_ValueError, "%s has %lld entries, %d are needed", what, (long long)size, (int)want);
+        return false;
+    }
     ~Ints() {
         if (view.obj) PyBuffer_Release(&view);
     }
@@ -192,7 +198,7 @@ PyObject *plan_budget(PyObject *, PyObject *const *a, Py_ssize_t n) {       // k
     p.keep_full = int_of(a[3]);
     p.min_quota = int_of(a[4]);
     Ints avail, out;
-    if (failed() || !avail.take(a[5]) || !out.take(a[6])) return nullptr;
+    if (failed() || !avail.take(a[5]) || !out.take(a[6]) || !out.holds(avail.n, "the budget array")) return nullptr;
     return PyLong_FromLong((long)pc_plan_budget(&p, avail.n, avail.p, const_cast<int32_t *>(out.p)));
 }
 
@@ -212,7 +218,7 @@ PyObject *score(PyObject *, PyObject *const *a, Py_ssize_t n) {             // c
     Tensors<2> q;
     Tensors<4> t;
     void *ctx = handle_of(a[0]), *stream = stream_of(a[9]);
-    if (failed() || !src.take(a[1]) || !q.take(a + 2) || !budget.take(a[4]) || !t.take(a + 5)) return nullptr;
+    if (failed() || !src.take(a[1]) || !q.take(a + 2) || !budget.take(a[4]) || !budget.holds(src.c.n_frames, "budget") || !t.take(a + 5)) return nullptr;
     const int32_t n_q = a[2] == Py_None ? 0 : rows_of(a[2]);
     if (failed()) return nullptr;
     return call([&] {
@@ -229,7 +235,7 @@ PyObject *compact(PyObject *, PyObject *const *a, Py_ssize_t n) {           // c
     Tensors<1> sel;
     void *ctx = handle_of(a[0]), *stream = stream_of(a[6]);
     const int32_t delta_t = int_of(a[4]);
-    if (failed() || !src.take(a[1]) || !sel.take(a + 2) || !budget.take(a[3]) || !dst.take(a[5])) return nullptr;
+    if (failed() || !src.take(a[1]) || !sel.take(a + 2) || !budget.take(a[3]) || !budget.holds(src.c.n_frames, "budget") || !dst.take(a[5])) return nullptr;
     return call([&] { return pc_compact(static_cast<pc_ctx *>(ctx), &src.c, static_cast<int32_t *>(sel.p[0]), budget.p, delta_t, &dst.c, stream); });
 }
 
@@ -285,7 +291,7 @@ PyObject *frame_step(PyObject *, PyObject *const *a, Py_ssize_t n) {        // c
     Tensors<6> t;
     void *ctx = handle_of(a[0]), *stream = stream_of(a[11]);
     const int32_t delta_t = int_of(a[3]);
-    if (failed() || !src.take(a[1]) || !budget.take(a[2]) || !dst.take(a[4]) || !t.take(a + 5)) return nullptr;
+    if (failed() || !src.take(a[1]) || !budget.take(a[2]) || !budget.holds(src.c.n_frames, "budget") || !dst.take(a[4]) || !t.take(a + 5)) return nullptr;
     const int32_t n_q = rows_of(a[5]);
     if (failed()) return nullptr;
     return call([&] {

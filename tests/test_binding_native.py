@@ -38,3 +38,19 @@ def test_errors_reach_the_caller():
     with pytest.raises(ValueError):
         pc.pc_compact(_Closed, cache, q_pos, ["x"], 0, cache, stream=0)
     assert cache.history.n_tokens == 6                                 # a refused call leaves the destination's count alone
+
+
+def test_a_budget_shorter_than_the_frames_is_refused():
+    q, q_pos = torch.zeros(4, 2, 8), torch.zeros(4, 4, dtype=torch.int32)
+    cache, sel = pc.Cache(pc.Segment.empty(), _segment(6), [2, 4]), torch.zeros(6, dtype=torch.int32)
+    calls = [lambda b: pc.pc_score(_Closed, cache, q, q_pos, b, scores=q, sel_idx=sel, stream=0),
+             lambda b: pc.pc_compact(_Closed, cache, sel, b, 0, cache, stream=0),
+             lambda b: pc.pc_frame_step(_Closed, cache, b, 0, cache, q, q_pos, scores=q, sel_idx=sel, out=q, stream=0)]
+    for call in calls:
+        with pytest.raises(ValueError, match="budget has 1 entries, 2 are needed"):
+            call([1])
+        for enough in ([1, 1], [1, 1, 1], [[1], [1]]):                 # the null context is what is refused here
+            with pytest.raises(pc.PackCacheError):
+                call(enough)
+    with pytest.raises(ValueError):
+        pc._native().plan_budget(pc.PC_LINEAR, 0.0, 1, 0, 0, np.array([5, 5], np.int32), np.zeros(1, np.int32))
