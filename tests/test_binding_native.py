@@ -54,3 +54,10 @@ def test_a_budget_shorter_than_the_frames_is_refused():
                 call(enough)
     with pytest.raises(ValueError):
         pc._native().plan_budget(pc.PC_LINEAR, 0.0, 1, 0, 0, np.array([5, 5], np.int32), np.zeros(1, np.int32))
+
+
+def test_current_stream_without_torchs_private_call(monkeypatch):
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 7}))
+    assert pc._stream(None) == 7 and pc._stream(5) == 5
