@@ -2,11 +2,14 @@
 context."""
 from __future__ import annotations
 
+import importlib.machinery
+
 import numpy as np
 import pytest
 import torch
 
 from paper_2601_04359_b200 import binding as pc
+from paper_2601_04359_b200 import build
 
 
 @pytest.mark.parametrize("make", [list, tuple, lambda a: np.array(a, np.int64), lambda a: np.array(a, np.int32),
@@ -61,3 +64,8 @@ def test_current_stream_without_torchs_private_call(monkeypatch):
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("S", (), {"cuda_stream": 7}))
     assert pc._stream(None) == 7 and pc._stream(5) == 5
+
+
+def test_native_module_is_the_one_of_this_interpreter():
+    """Another interpreter's build is not importable here, nor this one there."""
+    assert build.PYLIB.endswith(importlib.machinery.EXTENSION_SUFFIXES[0]) and pc._native().__file__ == build.PYLIB
