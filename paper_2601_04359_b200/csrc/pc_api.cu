@@ -74,7 +74,7 @@ static pc_status create_on_device(pc_ctx *c) {
         PC_CUDA_TRY(cudaMalloc(&c->q_rot, (size_t)desc->max_q * desc->n_q_heads * desc->head_dim * sizeof(__nv_bfloat16)));
         PC_CUDA_TRY(cudaMalloc(&c->part_o, std::max<size_t>(c->part_o_floats, 1) * sizeof(float)));
         PC_CUDA_TRY(cudaMalloc(&c->part_ml, std::max<size_t>(c->part_ml_floats, 1) * sizeof(float)));
-        PC_CUDA_TRY(cudaMalloc(&c->mass_part, c->k_rot_rows * desc->n_kv_heads * 2 * PC_MASS_PARTS * sizeof(float)));
+        PC_CUDA_TRY(cudaMalloc(&c->mass_part, pc_mass_part_floats(desc, c->sm_count, c->k_rot_rows) * sizeof(float)));
         PC_CUDA_TRY(cudaMalloc(&c->mass_norm, (size_t)((desc->max_q + 127) / 128) * 128 * desc->n_q_heads * sizeof(float)));
     }
     return PC_OK;

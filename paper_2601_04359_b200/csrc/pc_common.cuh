@@ -34,7 +34,6 @@ enum {
 };
 
 constexpr int PC_MAX_SEGMENTS = 3;
-constexpr int PC_MASS_PARTS = 4;              // pieces the attention mass of a pair of key tiles may come in
 constexpr int PC_MAX_DEVICES = 64;            // per-device launch state is kept in arrays of this size
 
 // Rotary tables: for axis a (t, h, w) a [max_pos[a]][n_axis[a]] array of (cos, sin) of pos * base^(-m/n_axis[a]).
@@ -82,7 +81,7 @@ struct pc_ctx {
     // (read by pc_attend_mass); last_n_q = 0 when there is none
     int last_n_q, last_n_seg;
     int last_seg_n[PC_MAX_SEGMENTS];
-    float *mass_part;          // attention mass: partial sums per piece, KV head and column half, [PC_MASS_PARTS][Hkv][2][k_rot_rows]
+    float *mass_part;          // attention mass: partial sums of the pieces of (KV head, pair of key tiles)
     float *mass_norm;          // attention mass: negated base-2 normalisers, [Hq][max_q rounded up to 128]
     // optional per-kernel timing (benchmarks): events at the boundaries of the kernels of each call
     int timing_on;
@@ -302,5 +301,6 @@ pc_status pc_frame_step_check(pc_ctx *ctx, const pc_cache *src, const int32_t *b
                               int32_t n_q, const float *scores, const int32_t *sel_idx, const void *out, const float *lse);
 pc_status pc_attend_frame_check(pc_ctx *ctx, const pc_cache *cache, const pc_segment *current, const void *q, const int32_t *q_pos,
                                 int32_t n_q, const void *out, const float *lse);
+size_t pc_mass_part_floats(const pc_layer_desc *d, int sm_count, size_t k_rot_rows);      // size of mass_part
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
                                size_t *part_ml_floats);

@@ -34,7 +34,7 @@ namespace {
 
 using namespace pc_tc;
 
-constexpr int MASS_PARTS = PC_MASS_PARTS;   // most pieces of a unit
+constexpr int MASS_PARTS = 4;              // most pieces of a unit
 constexpr int MASS_THREADS = 640;          // warp 0 TMA + TMEM owner, warp 1 MMA issuer, warps 4-19 column sums
 constexpr int Q_STAGES = 4;
 constexpr int L_SLOTS = 8;                 // normaliser ring: deeper than query stages + score buffers, see the producer
@@ -55,7 +55,9 @@ struct MassParams {
     int n_q, n_q_heads, group, n_tb, n_kv_tiles, pairs;    // pairs = key-tile pairs per KV head
     const float *lse;      // [n_q][Hq] natural log
     float *norm;           // [Hq][n_tb * 128]: -log2(e) * lse, -inf past n_q
-    float *part;           // [piece][Hkv][2 column halves][n_kv_tiles * 128]
+    // Partial sums, [slot][2 key tiles][2 column halves][128].  A piece's slot is its unit's number plus its CTA's: along the line of
+    // steps one or both of them grow at every change, so no two pieces share a slot and there are at most units + n_cta of them.
+    float *part;
     int32_t *status;
     int n_cta, n_steps;    // persistent CTAs; steps (query tiles of the head's group) of a unit
     int run, longer;       // steps of a CTA's run; the first `longer` CTAs take one more
@@ -232,10 +234,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
                 acc1 = add2(acc1, y);
             }
             if (--unit_left == 0) {                          // the unit, or this CTA's piece of it, is done
-                const int g = unit / P.pairs, jt = 2 * (unit % P.pairs) + t;
-                const int piece = (int)blockIdx.x - cta_of_step(P, unit * P.n_steps);
-                if (jt < P.n_kv_tiles)
-                    P.part[((((size_t)piece * (P.n_q_heads / P.group) + g) * 2 + hf) * P.n_kv_tiles + jt) * TILE + r] = (acc0.x + acc0.y) + (acc1.x + acc1.y);
+                P.part[(((size_t)unit + blockIdx.x) * 4 + 2 * t + hf) * TILE + r] = (acc0.x + acc0.y) + (acc1.x + acc1.y);
                 acc0 = acc1 = make_float2(0.f, 0.f);
                 ++unit;
                 unit_left = min(P.n_steps, G1 - unit * P.n_steps);
@@ -251,7 +250,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
 }
 
 struct ReduceParams {
-    int n_seg, n_kv_heads, n_kv_tiles;
+    int n_seg, n_kv_heads;
     int seg_first[PC_MAX_SEGMENTS + 1];     // first key of each segment in the output order; [n_seg] = all keys
     int seg_tile0[PC_MAX_SEGMENTS];         // first tile of each segment in the rotated-key scratch
     float inv_rows;                         // 1 / (n_q Hq)
@@ -266,21 +265,20 @@ __global__ void __launch_bounds__(TILE * MASS_ROWS) k_mass_reduce(const __grid_c
     __shared__ float rows[MASS_ROWS][TILE];
     pc_grid_dep_launch();
     const int jt = blockIdx.x, key = threadIdx.x % TILE, y = threadIdx.x / TILE;
-    const size_t row = (size_t)jt * TILE + key, stride = (size_t)P.n_kv_tiles * TILE;
     int s = 0;
     while (s + 1 < R.n_seg && jt >= R.seg_tile0[s + 1]) ++s;
     const int j = R.seg_first[s] + (jt - R.seg_tile0[s]) * TILE + key;             // key number; past the segment: padding rows
     pc_grid_dep_wait();
     float sum = 0.f;
     for (int g = y; g < R.n_kv_heads; g += MASS_ROWS) {
-        const float *p = P.part + (size_t)g * 2 * stride + row;
-        float a = __ldcg(p), b = __ldcg(p + stride);                   // the first piece's two column halves
-        const int x = (g * P.pairs + jt / 2) * P.n_steps;
-        const int pieces = cta_of_step(P, x + P.n_steps - 1) - cta_of_step(P, x) + 1;
+        const int unit = g * P.pairs + jt / 2, x = unit * P.n_steps, first = cta_of_step(P, x);
+        const int pieces = cta_of_step(P, x + P.n_steps - 1) - first + 1;
+        const float *p = P.part + (((size_t)unit + first) * 4 + 2 * (jt & 1)) * TILE + key;
+        float a = __ldcg(p), b = __ldcg(p + TILE);                     // the first piece's two column halves
         for (int piece = 1; piece < pieces; ++piece) {
-            p += (size_t)R.n_kv_heads * 2 * stride;
+            p += 4 * TILE;
             a += __ldcg(p);
-            b += __ldcg(p + stride);
+            b += __ldcg(p + TILE);
         }
         sum += a + b;
     }
@@ -315,6 +313,11 @@ int choose_mass_ctas(int units, int n_steps, int sm_count) {
 
 }  // namespace
 
+size_t pc_mass_part_floats(const pc_layer_desc *d, int sm_count, size_t k_rot_rows) {
+    const size_t units = (size_t)d->n_kv_heads * ((k_rot_rows / TILE + 1) / 2);
+    return (units + sm_count) * 4 * TILE;
+}
+
 extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, int32_t n_keys, void *stream_) {
     if (!ctx || !lse || !mass) return PC_ERR_INVALID_ARG;
     if (!pc_aligned16(lse) || !pc_aligned16(mass)) return PC_ERR_INVALID_ARG;
@@ -337,7 +340,6 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
     if ((size_t)tiles * TILE > ctx->k_rot_rows) return PC_ERR_CAPACITY;
     R.n_seg = ctx->last_n_seg;
     R.n_kv_heads = D.n_kv_heads;
-    R.n_kv_tiles = tiles;
     R.inv_rows = (float)(1.0 / ((double)ctx->last_n_q * D.n_q_heads));
     P.n_q = ctx->last_n_q;
     P.n_q_heads = D.n_q_heads;

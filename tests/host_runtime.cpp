@@ -69,6 +69,7 @@ cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 148; retu
 cudaError_t cudaGetLastError() { const cudaError_t e = t_last; t_last = cudaSuccess; return e; }
 const char *cudaGetErrorString(cudaError_t) { return "an error of the host runtime"; }
 cudaError_t cudaMalloc(void **p, size_t n) {
+    enter("malloc", std::to_string(n));
     *p = aligned_alloc(256, (n + 255) / 256 * 256);
     rt_memory(*p, n, cudaMemoryTypeDevice, t_device);
     return cudaSuccess;

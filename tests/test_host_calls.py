@@ -112,3 +112,13 @@ def test_static_scoring_takes_the_row_widths_that_scoring_takes(rt, n_kv, status
     got = rt.lib.pc_score_tokens_static(C.byref(desc), pc._ptr(k), pc._ptr(pos), 8, pc._ptr(k), pc._ptr(pos), 8, None, pc._ptr(out), pc._ptr(word), None)
     assert got == status
     assert [line.split()[1] for line in rt.log()] == (["k_rope_table", "k_qprep", "k_score"] if status == pc.PC_OK else [])
+
+
+def test_scratch_of_a_context_per_key(rt):
+    """A key costs its rotated row (8 x 128 bf16) and, for the attention mass, one fp32 sum per KV head and column half."""
+    size = []
+    for keys in (50_000, 250_000):
+        rt.reset()
+        pc.Context(24, 8, 128, pc.PC_BF16, 10000.0, (64, 64, 64), 1008, keys).close()
+        size.append(sum(int(line.split()[1]) for line in rt.log() if line.startswith("malloc")))
+    assert (size[1] - size[0]) / 200_000 <= 8 * 128 * 2 + 8 * 2 * 4 + 1
