@@ -47,7 +47,7 @@ pc_status attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *
     for (int r = 0; r < n_q && st == PC_OK; r += part) {
         const int n = part < n_q - r ? part : n_q - r;
         st = pc_launch_attend_tc(ctx, n_seg, segs, nullptr, nullptr, n, static_cast<char *>(out) + r * row_bytes,
-                                 lse ? lse + (size_t)r * ctx->desc.n_q_heads : nullptr, stream, PC_TC_ATTEND, r);
+                                 lse ? lse + (size_t)r * ctx->desc.n_q_heads : nullptr, stream, PC_TC_ATTEND | PC_TC_GOES_ON, r);
         if (st == PC_OK) st = hooks->part_done(hooks->self, r, n, stream);
     }
     if (st == PC_OK) ctx->last_n_q = n_q;

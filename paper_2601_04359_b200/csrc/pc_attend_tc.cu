@@ -808,8 +808,10 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     }
     jobs.n_jobs = n_jobs;
     jobs.total_warps = warps;
-    ctx->ev_mask &= ~((1u << PC_MARK_ATT0) | (1u << PC_MARK_ROPE) | (1u << PC_MARK_ATTEND) | (1u << PC_MARK_COMBINE));
-    pc_mark(ctx, PC_MARK_ATT0, stream);
+    if (!(what & PC_TC_GOES_ON)) {
+        ctx->ev_mask &= ~((1u << PC_MARK_ATT0) | (1u << PC_MARK_ROPE) | (1u << PC_MARK_ATTEND) | (1u << PC_MARK_COMBINE));
+        pc_mark(ctx, PC_MARK_ATT0, stream);
+    }
     if (n_jobs > 0) {
         PC_LAUNCH(k_rope_rows, dim3(div_up(warps, 8)), dim3(256), 0, stream, jobs, ctx->rope, D.head_dim, ctx->status);
         PC_CUDA_TRY(cudaGetLastError());

@@ -278,7 +278,8 @@ inline float pc_q_rot_scale(int head_dim) { return (float)(1.4426950408889634 / 
 pc_status pc_launch_attend_simt(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos,
                                 int32_t n_q, void *out, float *lse, cudaStream_t stream);
 // PC_TC_ROPE_K0: rotate the keys of the first segment only (the anchors of a fused frame step)
-enum { PC_TC_ROPE_K = 1, PC_TC_ROPE_Q = 2, PC_TC_ATTEND = 4, PC_TC_ALL = 7, PC_TC_ROPE_K0 = 8 };
+// PC_TC_GOES_ON: a further part of a call whose timing marks have begun (the last part's end marks stand)
+enum { PC_TC_ROPE_K = 1, PC_TC_ROPE_Q = 2, PC_TC_ATTEND = 4, PC_TC_ALL = 7, PC_TC_ROPE_K0 = 8, PC_TC_GOES_ON = 16 };
 // q_row0: first row of the rotated-query scratch that PC_TC_ATTEND reads (q, out and lse are the caller's, already offset)
 pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, const void *q, const int32_t *q_pos,
                               int32_t n_q, void *out, float *lse, cudaStream_t stream, int what, int q_row0 = 0);

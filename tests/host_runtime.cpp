@@ -12,12 +12,13 @@
 
 namespace {
 
-struct Thing { int device; };                     // a stream or an event
+struct Thing { int device; int at; };             // a stream, or an event and how many launches came before it
 struct Range { size_t bytes; int kind, device; };
 
 thread_local int t_device = 0;
 thread_local cudaError_t t_last = cudaSuccess;
 std::string g_log;
+int g_launches = 0;
 std::map<std::string, int> g_fail;                // calls of this name left until one fails
 std::map<const void *, std::string> g_name;       // kernels
 std::map<const void *, int> g_smem;               // their dynamic shared-memory limits
@@ -44,6 +45,7 @@ cudaError_t launch(const void *f, size_t smem, const void *stream) {
     const cudaError_t e = enter("launch", g_name[f] + " " + on(stream));
     if (e != cudaSuccess) return e;
     const auto limit = g_smem.find(f);
+    ++g_launches;
     if (smem > (size_t)(limit == g_smem.end() ? 48 * 1024 : limit->second) || device_of(stream) != t_device) return done(cudaErrorInvalidValue);
     return cudaSuccess;
 }
@@ -99,20 +101,24 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
     }
     return cudaSuccess;
 }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = reinterpret_cast<cudaStream_t>(new Thing{t_device}); return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = reinterpret_cast<cudaStream_t>(new Thing{t_device, 0}); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { delete reinterpret_cast<Thing *>(s); return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { return enter("synchronize", on(s)); }
-cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = reinterpret_cast<cudaEvent_t>(new Thing{t_device}); return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = reinterpret_cast<cudaEvent_t>(new Thing{t_device, 0}); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete reinterpret_cast<Thing *>(e); return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
     const cudaError_t r = enter("record", on(s));
     if (r != cudaSuccess) return r;
+    reinterpret_cast<Thing *>(e)->at = g_launches;
     return device_of(s) == reinterpret_cast<Thing *>(e)->device ? cudaSuccess : done(cudaErrorInvalidResourceHandle);
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned) { return enter("wait", on(s)); }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b) {       // in launches
+    *ms = (float)(reinterpret_cast<Thing *>(b)->at - reinterpret_cast<Thing *>(a)->at);
+    return cudaSuccess;
+}
 cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v) {
     g_smem[f] = v;
     if (auto call = g_on_attribute) {

@@ -122,3 +122,18 @@ def test_scratch_of_a_context_per_key(rt):
         pc.Context(24, 8, 128, pc.PC_BF16, 10000.0, (64, 64, 64), 1008, keys).close()
         size.append(sum(int(line.split()[1]) for line in rt.log() if line.startswith("malloc")))
     assert (size[1] - size[0]) / 200_000 <= 8 * 128 * 2 + 8 * 2 * 4 + 1
+
+
+def test_stage_times_of_a_step_in_parts(rt):
+    """520 rows of 24 / 8 heads leave in two parts: the stages cover both, and the rotary pre-pass ahead of them."""
+    c = Case(rt, n=520, total=600)
+    win = c.make()
+    pc.pc_set_timing(c.ctx, True)
+    for f in range(2):                                    # fill: everything is rotated; pack: query pass, scores, selection, pack, the anchors' keys
+        rt.reset()
+        c.step_host(win)
+        log = [line.split()[1] for line in rt.log() if line.startswith("launch")]
+        assert log.count("k_attend_tc") == 2 and log.count("k_rope_rows") == 1
+        t = pc.pc_get_timing(c.ctx)
+        assert t["rope"] == 1 and t["rope"] + t["attend"] + max(t["combine"], 0) == len(log) - (4 if f else 0)
+        assert t["attend"] == len(log) - 1 - log[::-1].index("k_attend_tc") - log.index("k_rope_rows")
