@@ -333,8 +333,12 @@ pc_status pc_window_step(pc_window *w, const void *q, const int32_t *q_pos, int3
  * bounded): copies the frame that was just finished (its K, V, positions; n_frame may be 0) to the end of the active
  * history buffer and the new frame's queries and positions into the workspace, runs pc_window_step, copies the
  * output back and waits for the stream.  The frame's values and the output travel on a stream of the window's own, beside
- * the kernels; from 512 query rows or so (as many as fill the GPU twice) attention runs in parts of the rows so that the
- * output leaves part by part, and then agrees with pc_window_step up to fp32 rounding order (fewer rows: bit for bit).
+ * the kernels.  On the tensor-core path attention runs in parts of the query rows where there are enough rows for two or more
+ * parts that each keep the GPU busy, so that the output leaves part by part: with G = Hq / Hkv and L the fewest 128-row tiles
+ * for which 7 * Hkv * ceil(G * L / 2) reaches 31/32 of the SMs, from 128 * (2 L - 1) + 1 rows on.  On 148 SMs that is from 385
+ * rows for 24/8, 32/8, 24/12 and 32/16 heads, 641 for 16/4, 1,153 for 8/8, 129 for 64/8, 32/32 and 24/24.  Fewer rows give
+ * pc_window_step's output bit for bit.  In parts the keys are cut in other places, which moves the reference that a row's
+ * probabilities are rounded to bf16 against: each probability may differ by that rounding (2^-9 relative on either side).
  * Pinned host memory keeps the copies asynchronous.  All arguments are checked before anything is enqueued; a call that fails
  * leaves the window as it was (the frame is not appended) and nothing in flight on either stream.
  * Errors: as pc_window_append and pc_window_step. */

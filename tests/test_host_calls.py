@@ -137,3 +137,14 @@ def test_stage_times_of_a_step_in_parts(rt):
         t = pc.pc_get_timing(c.ctx)
         assert t["rope"] == 1 and t["rope"] + t["attend"] + max(t["combine"], 0) == len(log) - (4 if f else 0)
         assert t["attend"] == len(log) - 1 - log[::-1].index("k_attend_tc") - log.index("k_rope_rows")
+
+
+@pytest.mark.parametrize("heads,rows", [((24, 8), 385), ((32, 8), 385), ((24, 12), 385), ((32, 16), 385), ((16, 4), 641), ((8, 8), 1153),
+                                        ((64, 8), 129), ((32, 32), 129), ((24, 24), 129)])
+def test_rows_from_which_a_step_runs_in_parts(rt, heads, rows):
+    """The numbers that the header states, for 148 SMs."""
+    for n, parts in ((rows - 1, 1), (rows, 2)):
+        c = Case(rt, heads=heads + (128,), n=n, total=n)
+        rt.reset()
+        c.step_host(c.make())
+        assert sum("k_attend_tc" in line for line in rt.log()) == parts
