@@ -106,6 +106,16 @@ __global__ void __launch_bounds__(APPEND_THREADS) k_append(const uint4 *__restri
     }
 }
 
+// Memory that a kernel on the context's device reads as it is.
+bool on_device(const pc_ctx *ctx, const void *p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == ctx->device;
+}
+
 }  // namespace
 
 extern "C" pc_status pc_window_append(pc_window *w, const pc_segment *frame, void *stream_) {
@@ -119,12 +129,20 @@ extern "C" pc_status pc_window_append(pc_window *w, const pc_segment *frame, voi
     if ((int)w->count.size() + 1 > PC_MAX_FRAMES) return PC_ERR_CAPACITY;
     const size_t row = (size_t)w->ctx->desc.n_kv_heads * w->ctx->desc.head_dim * w->ctx->elem_size;
     const size_t at = (size_t)A.n_tokens * row;
-    const long long n_kv = (long long)(n * row / 16), chunks = 2 * n_kv + n, per_block = APPEND_THREADS * APPEND_CHUNKS;   // rows are multiples of 16 bytes
-    PC_LAUNCH(k_append, dim3((unsigned)((chunks + per_block - 1) / per_block)), dim3(APPEND_THREADS), 0, stream,
-              static_cast<const uint4 *>(frame->k), static_cast<const uint4 *>(frame->v), reinterpret_cast<const uint4 *>(frame->pos),
-              reinterpret_cast<uint4 *>(static_cast<char *>(A.k) + at), reinterpret_cast<uint4 *>(static_cast<char *>(A.v) + at),
-              reinterpret_cast<uint4 *>(A.pos) + A.n_tokens, n_kv, n);
-    PC_CUDA_TRY(cudaGetLastError());
+    char *k = static_cast<char *>(A.k) + at, *v = static_cast<char *>(A.v) + at;
+    int32_t *pos = A.pos + 4 * (size_t)A.n_tokens;
+    if (on_device(w->ctx, frame->k) && on_device(w->ctx, frame->v) && on_device(w->ctx, frame->pos)) {
+        const long long n_kv = (long long)(n * row / 16), chunks = 2 * n_kv + n, per_block = APPEND_THREADS * APPEND_CHUNKS;   // rows are multiples of 16 bytes
+        PC_LAUNCH(k_append, dim3((unsigned)((chunks + per_block - 1) / per_block)), dim3(APPEND_THREADS), 0, stream,
+                  static_cast<const uint4 *>(frame->k), static_cast<const uint4 *>(frame->v), reinterpret_cast<const uint4 *>(frame->pos),
+                  reinterpret_cast<uint4 *>(k), reinterpret_cast<uint4 *>(v), reinterpret_cast<uint4 *>(pos), n_kv, n);
+        PC_CUDA_TRY(cudaGetLastError());
+    } else {
+        // a frame on another GPU, in host memory, or nowhere the driver knows of: the runtime's copies reach the former and refuse the rest
+        PC_CUDA_TRY(cudaMemcpyAsync(k, frame->k, (size_t)n * row, cudaMemcpyDeviceToDevice, stream));
+        PC_CUDA_TRY(cudaMemcpyAsync(v, frame->v, (size_t)n * row, cudaMemcpyDeviceToDevice, stream));
+        PC_CUDA_TRY(cudaMemcpyAsync(pos, frame->pos, (size_t)n * 16, cudaMemcpyDeviceToDevice, stream));
+    }
     A.n_tokens += n;
     w->count.push_back(n);
     return PC_OK;

@@ -9,7 +9,7 @@ import torch
 
 from paper_2601_04359_b200 import binding as pc
 
-from .host_runtime import CALLBACK, Case, _library, counts, rt  # noqa: F401
+from .host_runtime import CALLBACK, DEVICE, PINNED, Case, _library, counts, rt  # noqa: F401
 
 
 def test_window_belongs_to_the_device_of_its_context(rt):
@@ -148,3 +148,21 @@ def test_rows_from_which_a_step_runs_in_parts(rt, heads, rows):
         rt.reset()
         c.step_host(c.make())
         assert sum("k_attend_tc" in line for line in rt.log()) == parts
+
+
+@pytest.mark.parametrize("kind,device,route", [(DEVICE, 0, ["launch k_append main"]), (DEVICE, 1, ["memcpy main"] * 3), (PINNED, 0, ["memcpy main"] * 3),
+                                               (0, 0, ["memcpy main"] * 3)])
+@pytest.mark.parametrize("which", ["k", "v", "pos"])
+def test_append_reads_only_its_own_device_with_a_kernel(rt, kind, device, route, which):
+    """A frame on another GPU, in pinned memory, or in memory the driver does not know goes by the runtime's copies, which
+    reach it or refuse it; a kernel would fault."""
+    c = Case(rt)
+    win = c.make()
+    c.frame.k.normal_()
+    rt.memory(getattr(c.frame, which), kind=kind, device=device)
+    rt.reset()
+    f = c.frame.c()
+    assert rt.lib.pc_window_append(win.handle, C.byref(f), None) == pc.PC_OK
+    assert rt.log() == route and counts(win) == [c.n]
+    if len(route) == 3:
+        assert torch.equal(c.bufs[0].k[:c.n], c.frame.k)

@@ -59,7 +59,7 @@ def _check(grid, heads, one_part, bound):
         m = a.n_tokens
         assert m == b.n_tokens and all(torch.equal(x[:m], y[:m]) for x, y in ((a.k, b.k), (a.v, b.v), (a.pos, b.pos)))
         got, want = out_host.float().numpy(), out.float().cpu().numpy()
-        assert (np.abs(got - want) <= bf16_ulp(want) + (bound or 2.0 ** -8 * float(a.v[:m].float().abs().max()))).all()
+        assert (np.abs(got - want) <= bf16_ulp(want) + (bound or 2.0 ** -8 * float(torch.cat([D.cache.anchors.v, a.v[:m]]).float().abs().max()))).all()
         if one_part:
             assert torch.equal(out_host, out.cpu())
     for w in wins:
