@@ -12,6 +12,7 @@
 // one table look-up per token.
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "pc_common.cuh"
 #include "pc_select.cuh"
@@ -41,11 +42,14 @@ template <> struct Elem<__nv_bfloat16> {
 // row; 32 chunks span a multiple of d, so all of a lane's chunks hold the same rotary pairs and the lane needs PER/2 table
 // entries.  A block keeps four tokens in work (as far as the row's parts leave it) and walks the tokens with a stride, the
 // next token's row and position requested before the current one is turned; every thread sums its own elements over its
-// tokens in registers.  At the end the sums go to one slab per token slot in shared memory, the threads add, in a fixed
-// order, the slots and then the heads of each pooled element, turn the sum into a 64-bit fixed-point number (units of 2^-32)
-// and add it to the global accumulator with an integer atomic: integer addition is associative, so the pooled query does not
-// depend on the order in which blocks arrive.  The scoring kernel reads the accumulator as it is; nobody waits for a last
-// block to turn it into floats.
+// tokens in registers.  At the end the sums go to one slab per token slot in shared memory; for each pooled element the threads
+// add, in a fixed order, the heads and slots of QPREP_SUM_WARPS / parts tokens in fp32, turn that into a 64-bit fixed-point
+// number (units of 2^-32), and go on in integers, up to the global accumulator with an integer atomic: integer addition is
+// associative, so the pooled query does not depend on the order in which blocks arrive, and no fp32 sum has more terms than
+// those tokens give it, however many a block works on: a thread that walks several tokens adds fewer slots, or, where it walks
+// more than those tokens, keeps its own sums' roundings (all slots of a block in one fp32 sum and a thread's tokens as they
+// come: scores 4 to 14 % further from a 64-bit evaluation).  The scoring kernel reads the accumulator as it is;
+// nobody waits for a last block to turn it into floats.
 // The kernel is bound by latency: a launch, one round trip for positions and rows, one for table entries, the sums, the
 // atomics.  One block per two tokens (504 at 1,008 queries, each adding all pooled elements) and a last block that converted
 // and cleared the accumulator took, with a scoring kernel of eight tokens behind it, 11.2 us at 1,008 queries of 24 heads
@@ -53,6 +57,7 @@ template <> struct Elem<__nv_bfloat16> {
 // sixteen 9.0 / 14.6 / 7.8; two or four copies of the accumulator 7.8 to 8.4 at 1,008.
 // ---------------------------------------------------------------------------------------------------------
 constexpr int QPREP_WARPS = 16;                     // most warps per block, unless one token needs more
+constexpr int QPREP_SUM_WARPS = 8;                  // tokens whose elements are added in fp32, in warps
 constexpr int QPREP_SLAB = 200 * 1024;              // most shared memory of a block (one token takes up to 128 KB: 32 parts of 4 x 32 chunks)
 constexpr float FX_ONE = 4294967296.0f;             // 2^32
 
@@ -64,10 +69,12 @@ template <> __device__ __forceinline__ uint4 pack_row<__nv_bfloat16>(const float
     return make_uint4(pc_pack_bf16(f[0], f[1]), pc_pack_bf16(f[2], f[3]), pc_pack_bf16(f[4], f[5]), pc_pack_bf16(f[6], f[7]));
 }
 
-// A query row is cut into `parts` runs of CPW x 32 chunks, one warp each; a block holds `slots` tokens at a time.
-template <typename T, int CPW /* chunks per lane of one warp's part of a query row */, int MAX_THREADS>
-__global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, const int32_t *__restrict__ q_pos, int n_q,
-                                                int n_q_heads, int group, int d, int parts, pc_rope_dev rope,
+// A query row is cut into `parts` runs of CPW x 32 chunks, one warp each; a block holds `slots` tokens at a time, `run` of which
+// go into one fp32 sum.
+// KEEP: a thread's sums over its tokens carry what each addition rounds off into the next one (Kahan), two elements at a time.
+template <typename T, int CPW /* chunks per lane of one warp's part of a query row */, int MAX_THREADS, bool KEEP>
+__global__ void __launch_bounds__(MAX_THREADS, MAX_THREADS == 512 && !KEEP && CPW <= (sizeof(T) == 4 ? 3 : 2) ? 2 : 1) k_qprep(const T *__restrict__ q, const int32_t *__restrict__ q_pos, int n_q,
+                                                int n_q_heads, int group, int d, int parts, int run, pc_rope_dev rope,
                                                 float out_scale, T *__restrict__ q_rot, unsigned long long *fx,
                                                 int32_t *status) {
     pc_grid_dep_wait();
@@ -84,31 +91,33 @@ __global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, 
     int i = blockIdx.x * slots + slot;
     int4 pp = make_int4(0, 0, 0, 0);
     uint4 raw[CPW];
-    auto request = [&]() {
-        pp = __ldg(reinterpret_cast<const int4 *>(q_pos) + i);
-#pragma unroll
-        for (int c = 0; c < CPW; ++c) raw[c] = pc_ldg_stream(src + (size_t)i * row_chunks + c * 32);
-    };
-    float acc[CPW][PER];
+    float2 acc[CPW][NP], off[KEEP ? CPW : 1][KEEP ? NP : 1];
 #pragma unroll
     for (int c = 0; c < CPW; ++c)
 #pragma unroll
-        for (int k = 0; k < PER; ++k) acc[c][k] = 0.f;
-    if (i < n_q) request();
+        for (int u = 0; u < NP; ++u) {
+            acc[c][u] = make_float2(0.f, 0.f);
+            if constexpr (KEEP) off[c][u] = make_float2(0.f, 0.f);
+        }
+    if (i < n_q) {
+        pp = __ldg(reinterpret_cast<const int4 *>(q_pos) + i);
+#pragma unroll
+        for (int c = 0; c < CPW; ++c) raw[c] = pc_ldg_stream(src + (size_t)i * row_chunks + c * 32);
+    }
     while (i < n_q) {
         const int at = i;
         float2 cs[NP];
 #pragma unroll
         for (int u = 0; u < NP; ++u) cs[u] = pc_rope_cs(rope, pair0 + u, pp.x, pp.y, pp.z, status, PC_WHERE_QPOOL_POS);
-        uint4 cur[CPW];
-#pragma unroll
-        for (int c = 0; c < CPW; ++c) cur[c] = raw[c];
         i += stride;
-        if (i < n_q) request();
+        const bool more = i < n_q;
+        if (more) pp = __ldg(reinterpret_cast<const int4 *>(q_pos) + i);
 #pragma unroll
         for (int c = 0; c < CPW; ++c) {
+            const uint4 cur = raw[c];
+            if (more) raw[c] = pc_ldg_stream(src + (size_t)i * row_chunks + c * 32);
             float x[PER], r[PER];
-            Elem<T>::unpack(cur[c], x);
+            Elem<T>::unpack(cur, x);
 #pragma unroll
             for (int u = 0; u < NP; ++u) {
                 const float2 y = pc_rotate(x[2 * u], x[2 * u + 1], cs[u]);
@@ -116,7 +125,17 @@ __global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, 
                 r[2 * u + 1] = y.y;
             }
 #pragma unroll
-            for (int k = 0; k < PER; ++k) acc[c][k] += r[k];
+            for (int u = 0; u < NP; ++u) {
+                const float2 y = make_float2(r[2 * u], r[2 * u + 1]);
+                if constexpr (KEEP) {
+                    const float2 m1 = make_float2(-1.f, -1.f);
+                    const float2 z = __ffma2_rn(off[c][u], m1, y), t = __fadd2_rn(acc[c][u], z);
+                    off[c][u] = __ffma2_rn(z, m1, __ffma2_rn(acc[c][u], m1, t));
+                    acc[c][u] = t;
+                } else {
+                    acc[c][u] = __fadd2_rn(acc[c][u], y);
+                }
+            }
             if (dst) {                                                  // the attention kernel's queries carry its scale
 #pragma unroll
                 for (int k = 0; k < PER; ++k) r[k] = __fmul_rn(r[k], out_scale);
@@ -124,22 +143,58 @@ __global__ void __launch_bounds__(MAX_THREADS) k_qprep(const T *__restrict__ q, 
             }
         }
     }
+    if constexpr (KEEP)
+#pragma unroll
+        for (int c = 0; c < CPW; ++c)
+#pragma unroll
+            for (int u = 0; u < NP; ++u) acc[c][u] = __ffma2_rn(off[c][u], make_float2(-1.f, -1.f), acc[c][u]);
     float *mine = slab + (size_t)slot * row_len + (size_t)chunk0 * PER;
 #pragma unroll
     for (int c = 0; c < CPW; ++c) {
         float4 *s4 = reinterpret_cast<float4 *>(mine + (size_t)c * 32 * PER);
 #pragma unroll
-        for (int k = 0; k < PER / 4; ++k) s4[k] = make_float4(acc[c][4 * k], acc[c][4 * k + 1], acc[c][4 * k + 2], acc[c][4 * k + 3]);
+        for (int k = 0; k < PER / 4; ++k) s4[k] = make_float4(acc[c][2 * k].x, acc[c][2 * k].y, acc[c][2 * k + 1].x, acc[c][2 * k + 1].y);
     }
     __syncthreads();
     const int n_out = (n_q_heads / group) * d;
-    for (int e = threadIdx.x; e < n_out; e += blockDim.x) {
-        const int g = e / d;
-        const float *s = slab + (size_t)g * group * d + (e - g * d);
-        float sum = 0.f;
-        for (int h = 0; h < group; ++h)
-            for (int w = 0; w < slots; ++w) sum += s[w * row_len + h * d];
-        atomicAdd(fx + e, (unsigned long long)__float2ll_rn(sum * FX_ONE));
+    const int used = min(slots, n_q - (int)blockIdx.x * slots);        // slots that had a token
+    // the sums of N elements over the slots w0 .. w0 + run - 1, token by token, head by head: chains of reads and additions, so
+    // two elements go side by side where a thread has more than one
+    auto add_up = [&](auto n, const float *const (&s)[2], int w0, long long (&total)[2]) {
+        constexpr int N = decltype(n)::value;
+        int at = w0 * row_len;
+        float sum[2] = {0.f, 0.f};
+        for (int left = (min(w0 + run, used) - w0) * group, h = group; left > 0; left -= 4) {
+            float x[2][4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int i = 0; i < N; ++i) x[i][k] = k < left ? s[i][at] : 0.f;
+                at += d;
+                if (--h == 0) { h = group; at += row_len - group * d; }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < N; ++i) sum[i] += x[i][k];
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) total[i] += __float2ll_rn(sum[i] * FX_ONE);
+    };
+    auto at_element = [&](int e) { return slab + (size_t)(e / d) * group * d + e % d; };
+    int e = threadIdx.x;
+    for (; e + (int)blockDim.x < n_out; e += 2 * blockDim.x) {
+        const float *const s[2] = {at_element(e), at_element(e + blockDim.x)};
+        long long total[2] = {0, 0};
+        for (int w0 = 0; w0 < used; w0 += run) add_up(std::integral_constant<int, 2>{}, s, w0, total);
+        atomicAdd(fx + e, (unsigned long long)total[0]);
+        atomicAdd(fx + e + blockDim.x, (unsigned long long)total[1]);
+    }
+    if (e < n_out) {
+        const float *const s[2] = {at_element(e), nullptr};
+        long long total[2] = {0, 0};
+        for (int w0 = 0; w0 < used; w0 += run) add_up(std::integral_constant<int, 1>{}, s, w0, total);
+        atomicAdd(fx + e, (unsigned long long)total[0]);
     }
 }
 
@@ -347,46 +402,65 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     const double fx_scale = 1.0 / (4294967296.0 * (double)n_q);
     // a row's chunk rows are dealt to `parts` warps of 1-4 chunk rows each
     const int qcpl = q_chunks / 32;
-    const int cpw = qcpl % 3 == 0 ? 3 : (qcpl % 4 == 0 ? 4 : (qcpl % 2 == 0 ? 2 : 1));
-    const int parts = qcpl / cpw;
+    int cpw = 0, parts = 0, slots = 0, summed = 0, q_smem = 0, q_threads = 0;
+    const auto cut = [&](int chunk_rows) {
+        cpw = chunk_rows;
+        parts = qcpl / cpw;
+        slots = std::max(1, QPREP_WARPS / parts);
+        slots = std::max(1, std::min<int>(slots, (int)(QPREP_SLAB / ((size_t)q_row * sizeof(float)))));
+        summed = std::min(slots, std::max(1, QPREP_SUM_WARPS / parts));
+        q_smem = slots * q_row * (int)sizeof(float);
+        q_threads = slots * parts * 32;
+    };
+    cut(qcpl % 3 == 0 ? 3 : (qcpl % 4 == 0 ? 4 : (qcpl % 2 == 0 ? 2 : 1)));
     if (parts > 32) return PC_ERR_UNSUPPORTED;
-    int slots = std::max(1, QPREP_WARPS / parts);
-    slots = std::max(1, std::min<int>(slots, (int)(QPREP_SLAB / ((size_t)q_row * sizeof(float)))));
-    const int q_smem = slots * q_row * (int)sizeof(float);
-    const int q_threads = slots * parts * 32;
     int dev_id = 0;
     PC_CUDA_TRY(cudaGetDevice(&dev_id));
     if (dev_id < 0 || dev_id >= PC_MAX_DEVICES) return PC_ERR_UNSUPPORTED;
     if (ctx) pc_mark(ctx, PC_MARK_SCORE0, stream);
-#define PC_QPREP_LAUNCH(CPW, MAX_THREADS)                                                                            \
+    // Blocks: as many as are resident at once, each walking over its share of the tokens.  Where a thread then adds up more tokens
+    // than QPREP_SUM_WARPS gives one fp32 sum, it keeps the roundings (blocks of more than 512 threads have no registers for that
+    // and come in more rounds instead).
+    int q_blocks = 0, walked = 0;
+#define PC_QPREP_LAUNCH(KERNEL, RUN)                                                                                 \
     {                                                                                                               \
-        /* Shared by every context and thread.  The limit on dynamic shared memory is one number of the kernel's, so it is set */ \
-        /* to the most a call can ask for; resident blocks go with their key in one word, so no reader sees half of a pair. */ \
+        /* one limit for all sizes: the attribute is the kernel's, whichever thread and context calls */            \
         static std::atomic<bool> set[PC_MAX_DEVICES];                                                               \
-        static std::atomic<uint64_t> occ_of[PC_MAX_DEVICES];                                                        \
         if (!set[dev_id]) {                                                                                         \
-            PC_CUDA_TRY(cudaFuncSetAttribute(k_qprep<T, CPW, MAX_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, QPREP_SLAB)); \
+            PC_CUDA_TRY(cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, QPREP_SLAB));     \
             set[dev_id] = true;                                                                                     \
         }                                                                                                           \
+        PC_LAUNCH((KERNEL), dim3(q_blocks), dim3(q_threads), q_smem, stream, static_cast<const T *>(q), q_pos, n_q, D.n_q_heads, group, \
+                  D.head_dim, parts, RUN, rope, q_scale, static_cast<T *>(q_rot), reinterpret_cast<unsigned long long *>(fx), status); \
+    }
+#define PC_QPREP_CASE(CPW)                                                                                           \
+    {                                                                                                               \
+        /* resident blocks and the size they were looked up for, in one word: no reader sees half of a pair */      \
+        static std::atomic<uint64_t> occ_of[PC_MAX_DEVICES];                                                        \
         const uint64_t key = (uint64_t)(q_smem + q_threads) << 32, known = occ_of[dev_id];                          \
         int occ = (known ^ key) >> 32 ? 0 : (int)known;                                                             \
         if (occ == 0) {                                                                                             \
-            PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qprep<T, CPW, MAX_THREADS>, q_threads, q_smem)); \
+            PC_CUDA_TRY(q_threads <= 512 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qprep<T, CPW, 512, false>, q_threads, q_smem) \
+                                         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qprep<T, CPW, 1024, false>, q_threads, q_smem)); \
             occ = std::max(1, occ);                                                                                 \
             occ_of[dev_id] = key | (uint32_t)occ;                                                                   \
         }                                                                                                           \
-        const int q_blocks = std::min((n_q + slots - 1) / slots, sm_count * occ);                                   \
-        PC_LAUNCH((k_qprep<T, CPW, MAX_THREADS>), dim3(q_blocks), dim3(q_threads), q_smem, stream,                  \
-                  static_cast<const T *>(q), q_pos, n_q, D.n_q_heads, group, D.head_dim, parts, rope, q_scale,      \
-                  static_cast<T *>(q_rot), reinterpret_cast<unsigned long long *>(fx), status);                     \
+        q_blocks = std::min((n_q + slots - 1) / slots, sm_count * occ);                                             \
+        if (q_threads > 512) q_blocks = std::max(q_blocks, (n_q + slots * summed - 1) / (slots * summed));          \
+        walked = (n_q + q_blocks * slots - 1) / (q_blocks * slots);                                                 \
+        if (q_threads > 512) PC_QPREP_LAUNCH((k_qprep<T, CPW, 1024, false>), std::max(1, summed / walked))          \
+        else if (walked <= summed) PC_QPREP_LAUNCH((k_qprep<T, CPW, 512, false>), summed / walked)                  \
+        else if (CPW == 4) { cut(2); continue; }                    /* no registers for both */                    \
+        else PC_QPREP_LAUNCH((k_qprep<T, CPW == 4 ? 3 : CPW, 512, true>), std::max(1, summed / 2))                  \
     }
-#define PC_QPREP_CASE(CPW)                                                                                           \
-    if (q_threads <= 512) PC_QPREP_LAUNCH(CPW, 512) else PC_QPREP_LAUNCH(CPW, 1024)
-    switch (cpw) {
-    case 3: PC_QPREP_CASE(3) break;        // 24 query heads x 128 bf16: four warps per token
-    case 4: PC_QPREP_CASE(4) break;
-    case 2: PC_QPREP_CASE(2) break;
-    default: PC_QPREP_CASE(1) break;
+    for (;;) {
+        switch (cpw) {
+        case 3: PC_QPREP_CASE(3) break;        // 24 query heads x 128 bf16: four warps per token
+        case 4: PC_QPREP_CASE(4) break;
+        case 2: PC_QPREP_CASE(2) break;
+        default: PC_QPREP_CASE(1) break;
+        }
+        break;
     }
 #undef PC_QPREP_CASE
 #undef PC_QPREP_LAUNCH
