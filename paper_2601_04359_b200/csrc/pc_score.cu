@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
                                                                pc_rope_dev rope, unsigned long long *fx, double fx_scale,
                                                                float *__restrict__ scores, int32_t *status, uint32_t wait_us, uint32_t extra_tx) {
     pc_grid_dep_launch();
-    constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL;
+    constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL, CH = 32 / LPT /* chains */;
     extern __shared__ __align__(128) unsigned char score_smem[];
     __shared__ __align__(8) unsigned long long bars[SCORE_WARPS * SCORE_STAGES];
     __shared__ int gave_up;
@@ -302,28 +302,37 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
         for (int i = 0; i < TPL; ++i) table(p[i], cs[i]);
         if (grp + step < n_groups) positions(grp + step);
         if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT, wait_us))) break;
-        // brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair
-        float2 A[TPL][NP], B[TPL][NP];
+        // Brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair.
+        // A lane that shares its token with 15 others has twice as many chunks as one of 32 would: it keeps two chains, chunks
+        // of even and of odd number, and adds their results (one chain: scores up to 10 % further from a 64-bit evaluation; one
+        // chain after the other: 0.3 to 0.8 us more for short histories).
+        float2 A[CH][TPL][NP], B[CH][TPL][NP];
 #pragma unroll
-        for (int i = 0; i < TPL; ++i)
+        for (int c = 0; c < CH; ++c)
 #pragma unroll
-            for (int u = 0; u < NP; ++u) A[i][u] = B[i][u] = make_float2(0.f, 0.f);
+            for (int i = 0; i < TPL; ++i)
+#pragma unroll
+                for (int u = 0; u < NP; ++u) A[c][i][u] = B[c][i][u] = make_float2(0.f, 0.f);
         const uint32_t mine = ring + stage * stage_bytes + side * row_bytes + lt * 16;
         const float4 *ql = qs + lt;
 #pragma unroll 1
-        for (int g = 0; g < parts; ++g) {
-            float x[TPL][PER];
+        for (int g0 = 0; g0 < parts; g0 += CH) {
 #pragma unroll
-            for (int i = 0; i < TPL; ++i) Elem<T>::unpack(pc_lds128(mine + i * SIDE * row_bytes + g * LPT * 16), x[i]);
+            for (int c = 0; c < CH; ++c) {
+                const int g = g0 + c;
+                float x[TPL][PER];
 #pragma unroll
-            for (int u = 0; u < NP; ++u) {
-                const float4 qq = ql[(g * NP + u) * LPT];
-                const float2 qab = make_float2(qq.x, qq.y), qba = make_float2(qq.z, qq.w);
+                for (int i = 0; i < TPL; ++i) Elem<T>::unpack(pc_lds128(mine + i * SIDE * row_bytes + g * LPT * 16), x[i]);
 #pragma unroll
-                for (int i = 0; i < TPL; ++i) {
-                    const float2 kk = make_float2(x[i][2 * u], x[i][2 * u + 1]);
-                    A[i][u] = __ffma2_rn(qab, kk, A[i][u]);
-                    B[i][u] = __ffma2_rn(qba, kk, B[i][u]);
+                for (int u = 0; u < NP; ++u) {
+                    const float4 qq = ql[(g * NP + u) * LPT];
+                    const float2 qab = make_float2(qq.x, qq.y), qba = make_float2(qq.z, qq.w);
+#pragma unroll
+                    for (int i = 0; i < TPL; ++i) {
+                        const float2 kk = make_float2(x[i][2 * u], x[i][2 * u + 1]);
+                        A[c][i][u] = __ffma2_rn(qab, kk, A[c][i][u]);
+                        B[c][i][u] = __ffma2_rn(qba, kk, B[c][i][u]);
+                    }
                 }
             }
         }
@@ -333,10 +342,15 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
         float s[TPL];
 #pragma unroll
         for (int i = 0; i < TPL; ++i) {
-            s[i] = 0.f;
+            float r[CH];
 #pragma unroll
-            for (int u = 0; u < NP; ++u)
-                s[i] = fmaf(cs[i][u].x, A[i][u].x + A[i][u].y, fmaf(cs[i][u].y, B[i][u].x + B[i][u].y, s[i]));
+            for (int c = 0; c < CH; ++c) {
+                r[c] = 0.f;
+#pragma unroll
+                for (int u = 0; u < NP; ++u)
+                    r[c] = fmaf(cs[i][u].x, A[c][i][u].x + A[c][i][u].y, fmaf(cs[i][u].y, B[c][i][u].x + B[c][i][u].y, r[c]));
+            }
+            s[i] = CH == 2 ? r[0] + r[CH - 1] : r[0];
         }
         // a token's lanes are added up; with two tokens in a lane its lower lanes carry on with the first, the upper ones with the second
         float sum = s[0];

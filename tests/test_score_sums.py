@@ -66,3 +66,27 @@ def test_pooled_query_keeps_small_terms_beside_a_large_one(heads, dtype):
     exact = (hq // hk) * (2.0 ** 24 + n_q - 1)
     got = _scores(q, k, hk).astype(np.float64) * hq * np.sqrt(float(d)) * n_q
     assert np.abs(got - exact).max() <= 16 + 3 * (hq // hk)
+
+
+@pytest.mark.parametrize("n_kv,d,dtype", [(4, 128, torch.bfloat16), (8, 128, torch.bfloat16), (16, 128, torch.bfloat16), (2, 64, torch.float32),
+                                          (8, 64, torch.float32), (4, 128, torch.float32), (8, 128, torch.float32)])
+@pytest.mark.parametrize("n", [61, 4099])
+def test_a_key_is_summed_in_short_chains(n_kv, d, dtype, n):
+    q, k = _inputs((1, n_kv, d), dtype, 2), _inputs((n, n_kv, d), dtype, 3)
+    per = 8 if dtype == torch.bfloat16 else 4                          # elements of a 16-byte chunk
+    lanes = max(16, d // per)                                          # lanes that share a key
+    chains = 32 // lanes
+    p = _pooled(q.float().numpy().reshape(1, -1), 1).reshape(-1, chains, lanes, per)
+    x = k.float().numpy().reshape(n, -1, chains, lanes, per)
+    a = np.zeros(x.shape[:1] + x.shape[2:], F)
+    for g in range(x.shape[1]):                                        # one rounding per multiply-add: 48 + 24 bits fit a long double closely enough
+        a = (p[g].astype(np.longdouble) * x[:, g].astype(np.longdouble) + a.astype(np.longdouble)).astype(F)
+    r = np.zeros((n, chains, lanes), F)
+    for u in range(per // 2):
+        r = (a[..., 2 * u] + a[..., 2 * u + 1]) + r
+    s = r[:, 0] + r[:, 1] if chains == 2 else r[:, 0]
+    o = lanes // 2
+    while o:
+        s = s + s[:, np.arange(lanes) ^ o]
+        o //= 2
+    assert np.array_equal(_scores(q, k, n_kv), s[:, 0] * F(1.0 / (n_kv * np.sqrt(float(d)))))
