@@ -72,30 +72,41 @@ struct RopeJob {
     const __nv_bfloat16 *src;
     const int32_t *pos;
     __nv_bfloat16 *dst;
-    int n_rows, chunks_per_row /* 16-byte chunks, a multiple of 32 */, first_warp;
-    int rows_per_pos;      // consecutive rows that share one position record (a wide query row is cut into slices)
+    int first_warp;    // one warp per slice
+    int slices;        // consecutive slices that make a row and share its position record
     float scale;
 };
 struct RopeJobs { RopeJob job[PC_MAX_SEGMENTS + 1]; int n_jobs, total_warps; };
 
-// One warp per row (a query row wider than a key row is cut into key-row-wide slices, one warp each, so that all warps
-// carry the same load).  32 lanes x 8 elements = 256 is a multiple of d, so all of a lane's chunks (lane, lane + 32, ...)
-// hold the same four rotary pairs: four table entries per lane per row serve every chunk; the output scale (1 for keys)
-// is applied after the rotation, exactly as the query pass of the scoring stage does, so both give the same bits.  A row's
-// chunks (up to eight at a time) are requested together with its position, before the table entries that wait for it.
-// Bound by memory, so warps in flight count: 64 registers, four blocks per SM.  Measured with the table entries first and 128
-// registers (up to 16 chunks at a time) against this: 50,000 key rows of 2 KB 40.0 -> 36.0 us (5.1 -> 5.7 TB/s), 7,184 7.6 ->
-// 6.5.
+// One warp per slice of CPL x 32 16-byte chunks; key and query rows are cut into slices of one width (a query row is a whole number
+// of key rows), so all warps of a launch carry the same load.  32 lanes x 8 elements = 256 is a multiple of d, so all of a lane's
+// chunks (lane, lane + 32, ...) hold the same four rotary pairs: four table entries per lane serve them; the output scale (1
+// for keys) is applied after the rotation, exactly as the query pass of the scoring stage does, so both give the same bits.  A
+// slice's chunks are requested together with its position, before the table entries that wait for it.
+// Bound by memory, so warps in flight count: a kernel per width, with the registers that this width needs (40 up to three
+// chunks a lane, six blocks an SM).  One kernel for every width (64 registers, four blocks), rows of 3, 5, 6 and 7 chunks a lane
+// taken chunk by chunk, against this, 7,184 keys: 8 KV heads 5.5 -> 5.6 us, 4 4.6 -> 4.4, 6 8.3 -> 4.9, 10 13.3 -> 6.2, 12 15.2 ->
+// 7.7, 14 18.7 -> 7.9, 16 9.0 -> 9.0; 48,000 keys: 8 34.9 -> 33.3 (5.9 TB/s), 4 22.0 -> 17.9, 6 50.6 -> 23.6, 12 93 -> 47.
+constexpr int rope_blocks(int cpl) { return cpl <= 3 ? 6 : (cpl <= 7 ? 4 : 2); }
 template <int CPL /* chunks per lane */>
-__device__ __forceinline__ void rope_row(const RopeJob &J, int row, int c0, int lane, const pc_rope_dev &rope, int pair0, int32_t *status) {
-    const size_t at = (size_t)row * J.chunks_per_row + c0 * 32 + lane;
+__global__ void __launch_bounds__(256, rope_blocks(CPL)) k_rope_rows(const __grid_constant__ RopeJobs jobs, pc_rope_dev rope, int d, int32_t *status) {
+    pc_grid_dep_launch();
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    int ji = 0;
+    while (ji + 1 < jobs.n_jobs && warp >= jobs.job[ji + 1].first_warp) ++ji;
+    const RopeJob &J = jobs.job[ji];
+    const int slice = warp - J.first_warp, pair0 = ((lane * 8) % d) / 2;
+    pc_grid_dep_wait();
+    if (warp >= jobs.total_warps) return;
+    const size_t at = (size_t)slice * (CPL * 32) + lane;
     const uint4 *src = reinterpret_cast<const uint4 *>(J.src) + at;
     uint4 *dst = reinterpret_cast<uint4 *>(J.dst) + at;
     const float scale = J.scale;
     uint4 v[CPL];
 #pragma unroll
     for (int c = 0; c < CPL; ++c) v[c] = pc_ldg_stream(src + c * 32);
-    const int4 pp = __ldg(reinterpret_cast<const int4 *>(J.pos) + row / J.rows_per_pos);
+    const int4 pp = __ldg(reinterpret_cast<const int4 *>(J.pos) + slice / J.slices);
     bool bad = false;
     float2 cs[4];
 #pragma unroll
@@ -111,30 +122,6 @@ __device__ __forceinline__ void rope_row(const RopeJob &J, int row, int c0, int 
             o[u] = pc_pack_bf16(__fmul_rn(y.x, scale), __fmul_rn(y.y, scale));
         }
         dst[c * 32] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
-}
-
-__global__ void __launch_bounds__(256, 4) k_rope_rows(const __grid_constant__ RopeJobs jobs, pc_rope_dev rope, int d,
-                                                   int32_t *status) {
-    pc_grid_dep_launch();
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int ji = 0;
-    while (ji + 1 < jobs.n_jobs && warp >= jobs.job[ji + 1].first_warp) ++ji;
-    const RopeJob &J = jobs.job[ji];
-    const int row = warp - J.first_warp, pair0 = ((lane * 8) % d) / 2;
-    pc_grid_dep_wait();
-    if (warp >= jobs.total_warps) return;
-    const int n = J.chunks_per_row >> 5;
-    switch (n) {
-    case 4: rope_row<4>(J, row, 0, lane, rope, pair0, status); break;        // 8 KV heads x 128, and a third of 24 query heads
-    case 1: rope_row<1>(J, row, 0, lane, rope, pair0, status); break;
-    case 2: rope_row<2>(J, row, 0, lane, rope, pair0, status); break;
-    case 8: rope_row<8>(J, row, 0, lane, rope, pair0, status); break;
-    default:
-        for (int c = 0; c < n; c += n % 4 ? 1 : 4)
-            if (n % 4) rope_row<1>(J, row, c, lane, rope, pair0, status);
-            else rope_row<4>(J, row, c, lane, rope, pair0, status);
     }
 }
 
@@ -786,26 +773,27 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     RopeJobs jobs{};
     const int k_chunks = row_elems / 8, q_chunks = D.n_q_heads * D.head_dim / 8;
     if (k_chunks % 32 || q_chunks % 32) return PC_ERR_UNSUPPORTED;
+    // chunks per lane: the widest of these that key rows (and with them query rows) are a multiple of; rows have at most 16
+    const int k_cpl = k_chunks / 32;
+    int cpl = 1;
+    for (int m : {2, 13, 11, 7, 5, 3, 4})
+        if (k_cpl % m == 0) cpl = m;
     int tiles = 0, warps = 0, n_jobs = 0;
+    const auto add_job = [&](const void *src, const int32_t *pos, __nv_bfloat16 *dst, int rows, int chunks, float scale) {
+        const int slices = chunks / 32 / cpl;
+        jobs.job[n_jobs++] = RopeJob{static_cast<const __nv_bfloat16 *>(src), pos, dst, warps, slices, scale};
+        warps += rows * slices;
+    };
     for (int s = 0; s < n_seg; ++s) {
-        if ((what & PC_TC_ROPE_K) || (s == 0 && (what & PC_TC_ROPE_K0))) {
-            jobs.job[n_jobs++] = RopeJob{static_cast<const __nv_bfloat16 *>(segs[s].k), segs[s].pos,
-                                         k_rot + (size_t)tiles * TILE * row_elems, segs[s].n_tokens, k_chunks, warps, 1, 1.0f};
-            warps += segs[s].n_tokens;
-        }
+        if ((what & PC_TC_ROPE_K) || (s == 0 && (what & PC_TC_ROPE_K0)))
+            add_job(segs[s].k, segs[s].pos, k_rot + (size_t)tiles * TILE * row_elems, segs[s].n_tokens, k_chunks, 1.0f);
         tiles += div_up(segs[s].n_tokens, TILE);
         P.seg_tile_end[s] = tiles;
         P.seg_n[s] = segs[s].n_tokens;
     }
     if ((size_t)tiles * TILE > ctx->k_rot_rows) return PC_ERR_CAPACITY;
     __nv_bfloat16 *q_rot = static_cast<__nv_bfloat16 *>(ctx->q_rot);
-    if (what & PC_TC_ROPE_Q) {
-        // a query row is as many slices as it holds key-row widths when that divides evenly: every warp then has the same job
-        const int slices = (q_chunks % k_chunks == 0) ? q_chunks / k_chunks : 1;
-        jobs.job[n_jobs++] = RopeJob{static_cast<const __nv_bfloat16 *>(q), q_pos, q_rot, n_q * slices, q_chunks / slices, warps, slices,
-                                     pc_q_rot_scale(D.head_dim)};
-        warps += n_q * slices;
-    }
+    if (what & PC_TC_ROPE_Q) add_job(q, q_pos, q_rot, n_q, q_chunks, pc_q_rot_scale(D.head_dim));
     jobs.n_jobs = n_jobs;
     jobs.total_warps = warps;
     if (!(what & PC_TC_GOES_ON)) {
@@ -813,7 +801,12 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
         pc_mark(ctx, PC_MARK_ATT0, stream);
     }
     if (n_jobs > 0) {
-        PC_LAUNCH(k_rope_rows, dim3(div_up(warps, 8)), dim3(256), 0, stream, jobs, ctx->rope, D.head_dim, ctx->status);
+#define PC_ROPE_CASE(CPL)                                                                                              \
+    case CPL: PC_LAUNCH(k_rope_rows<CPL>, dim3(div_up(warps, 8)), dim3(256), 0, stream, jobs, ctx->rope, D.head_dim, ctx->status); break;
+        switch (cpl) {
+            PC_ROPE_CASE(1) PC_ROPE_CASE(2) PC_ROPE_CASE(3) PC_ROPE_CASE(4) PC_ROPE_CASE(5) PC_ROPE_CASE(7) PC_ROPE_CASE(11) PC_ROPE_CASE(13)
+        }
+#undef PC_ROPE_CASE
         PC_CUDA_TRY(cudaGetLastError());
         pc_mark(ctx, PC_MARK_ROPE, stream);          // no pre-pass (a fused frame step with cached anchors): no mark
     }
