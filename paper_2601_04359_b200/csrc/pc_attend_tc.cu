@@ -674,15 +674,20 @@ int choose_splits(int n_items, int n_kv_tiles, int sm_count) {
 // everything again for each item (47 whole frames, 96 items on 148 SMs: 37 streams per KV head, 2.36 GB from DRAM for
 // 203 MB of K and V); 144 CTAs have three, and their runs are two thirds of an item, so no item is cut into more than two
 // parts.  So up to 1/32 of the SMs is given up for the fewest starting places, as long as the longest run grows by no more
-// than that (a run counts whole steps).  Measured, one CTA per SM against this rule: attention over 47 whole frames 725 ->
-// 628 us a call, five passes over 7,184 keys 519 -> 513, the step at 47 frames 170.7 -> 169.9, 4,032-token frames (384
-// items, K and V inside L2) 666 -> 667.
-int choose_ctas(int n_items, long long steps, int most) {
+// than that (a run counts whole steps), where that makes streams that CTAs share: at least two CTAs of a KV head to a starting place,
+// and runs so much shorter than an item (items fewer than 3/4 of the CTAs) that neighbours stay in step.  Measured, one CTA per SM
+// against this rule: attention over 47 whole frames 725 -> 628 us a call, five passes over 7,184 keys 519 -> 513, the step at 47
+// frames 170.7 -> 169.9.  144 CTAs without the two conditions, against 148 (rotated keys, sides in turn): 16 / 16 heads, 1,008
+// queries x 30,000 keys (9 places, 9 CTAs a head) 232 -> 243 us, 32 / 8, 1,008 x 30,000 (128 items) 464 -> 471, 64 / 8, 1,008 x
+// 30,000 (256) 976 -> 999, 24 / 8, 2,000 x 30,000 (192) 691 -> 702, 24 / 8, 4,032 x 7,184 (384) 326 -> 330; where they hold: 8 / 8,
+// 1,008 x 48,000 (32) 189 -> 178, 24 / 12, 1,008 x 30,000 (96) 352 -> 327, 24 / 8, 400 x 30,000 (48) 157 -> 156.
+int choose_ctas(int n_items, int n_kv_heads, long long steps, int most) {
+    if (4 * n_items >= 3 * most) return most;
     int best = most, best_starts = most / std::gcd(most, n_items);
     const long long longest = (steps + most - 1) / most;
     for (int n = most - 1; n >= most - most / 32; --n) {
         const int starts = n / std::gcd(n, n_items);
-        if (starts < best_starts && 32 * ((steps + n - 1) / n) <= 33 * longest) {
+        if (starts < best_starts && 2 * starts * n_kv_heads <= n && 32 * ((steps + n - 1) / n) <= 33 * longest) {
             best = n;
             best_starts = starts;
         }
@@ -706,7 +711,7 @@ void choose_division(const pc_ctx *ctx, int n_items, int tiles, TcParams &P) {
     if (ctx->kv_splits > 0 || ctx->cluster_merge) {
         P.n_splits = ctx->kv_splits > 0 ? std::min(ctx->kv_splits, tiles) : choose_splits(n_items, tiles, ctx->sm_count);
     } else {
-        const int n = choose_ctas(n_items, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
+        const int n = choose_ctas(n_items, ctx->desc.n_kv_heads, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
         const bool crossing = n % n_items != 0;
         P.n_cta = n;
         // Shorter runs than six times the boundary could end up empty; in longer ones than 64 steps it does not show any more.

@@ -19,6 +19,7 @@ thread_local int t_device = 0;
 thread_local cudaError_t t_last = cudaSuccess;
 std::string g_log;
 int g_launches = 0;
+std::map<std::string, unsigned> g_grid;           // blocks of a kernel's last launch
 std::map<std::string, int> g_fail;                // calls of this name left until one fails
 std::map<const void *, std::string> g_name;       // kernels
 std::map<const void *, int> g_smem;               // their dynamic shared-memory limits
@@ -128,7 +129,11 @@ cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v) {
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) { return launch(f, c->dynamicSmemBytes, c->stream); }
+unsigned rt_blocks(const char *name) { return g_grid[name]; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) {
+    g_grid[g_name[f]] = c->gridDim.x * c->gridDim.y * c->gridDim.z;
+    return launch(f, c->dynamicSmemBytes, c->stream);
+}
 cudaError_t cudaLaunchKernel(const void *f, dim3, dim3, void **, size_t smem, cudaStream_t s) { return launch(f, smem, s); }
 cudaError_t cudaGetSymbolAddress(void **p, const void *) {
     static std::vector<char> all(1 << 20);

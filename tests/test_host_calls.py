@@ -166,3 +166,19 @@ def test_append_reads_only_its_own_device_with_a_kernel(rt, kind, device, route,
     assert rt.log() == route and counts(win) == [c.n]
     if len(route) == 3:
         assert torch.equal(c.bufs[0].k[:c.n], c.frame.k)
+
+
+@pytest.mark.parametrize("heads,rows,keys,blocks", [((24, 8), 1008, 48384, 144), ((24, 8), 1008, 9200, 144), ((8, 8), 1008, 48000, 144),
+                                                    ((16, 16), 1008, 30000, 148), ((64, 8), 1008, 24000, 148), ((8, 8), 4032, 24000, 148),
+                                                    ((24, 8), 4032, 9200, 148)])
+def test_attention_gives_up_sms_only_for_shared_streams(rt, heads, rows, keys, blocks):
+    """144 CTAs where a KV head's CTAs then run through the same keys two or more at a time, each over less than an item; every
+    other shape keeps a CTA on each of the 148 SMs."""
+    c = Case(rt, heads=(heads[0], heads[1], 128), n=1, total=1, anchors=1, max_q=rows, max_keys=keys)
+    empty = lambda n: pc.Segment(torch.empty(n, heads[1], 128, dtype=torch.bfloat16), torch.empty(n, heads[1], 128, dtype=torch.bfloat16),
+                                 torch.empty(n, 4, dtype=torch.int32), n)
+    q, out = (torch.empty(rows, heads[0], 128, dtype=torch.bfloat16) for _ in range(2))
+    s = pc.Cache(empty(keys), pc.Segment.empty(), np.zeros(0, np.int32)).c()
+    pos = torch.empty(rows, 4, dtype=torch.int32)
+    assert rt.lib.pc_attend_frame(c.ctx.handle, C.byref(s), None, pc._ptr(q), pc._ptr(pos), rows, pc._ptr(out), None, None) == pc.PC_OK
+    assert rt.lib.rt_blocks(b"k_attend_tc") == blocks
