@@ -490,8 +490,10 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
     const bool two = room >= SCORE_WARPS || (room >= SCORE_WARPS / 2 && n_src > sm_count * SCORE_WARPS * (32 / lpt));
     const int tok = (two ? 2 : 1) * (32 / lpt), stage_bytes = tok * row_bytes, n_groups = (n_src + tok - 1) / tok;
     const int blocks = std::max(1, std::min(n_groups, sm_count)), need = (n_groups + blocks - 1) / blocks;
-    // Short histories: as many warps as it takes to stage the pooled query quickly, and no more (query pass and scores of 675
-    // tokens, 1,024 pooled elements: 7.4 us with 12 warps, 8.1 with 4; the fp32 step with 128 elements 18.7 with 12, 16.5 with 4).
+    // Short histories: as many warps as it takes to stage the pooled query quickly, and no more: one for every 40 of its elements.
+    // Query pass, scores and selection of 675 tokens with 4 / 8 / 12 warps: 128 elements 8.7 / 7.8 / 7.9 us, 256 (bf16) 9.9 / 9.7 /
+    // 9.9, 512 10.4 / 10.1 / 9.7, 1,024 10.9 / 10.2 / 10.0, 2,048 12.3 / 11.8 / 11.3; of 1,500 tokens: 128 elements 7.8 / 7.9 / 9.0,
+    // 256 (fp32, 4 / 6 / 12 warps) 8.6 / 8.5 / 9.5, 1,024 10.6 / 11.0 / 10.9.
     const int warps = std::min({SCORE_WARPS, SCORE_RING / (2 * stage_bytes), std::max({4, need, row / 40})});
     const int stages = std::max(1, std::min({SCORE_STAGES, SCORE_RING / (warps * stage_bytes), (n_groups + blocks * warps - 1) / (blocks * warps)}));
     const int smem = row * 8 + warps * stages * stage_bytes;
