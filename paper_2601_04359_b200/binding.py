@@ -1,4 +1,5 @@
-"""ctypes binding of ``libpackcache.so`` — same names as the C ABI, argument marshalling only.
+"""Binding of ``libpackcache.so`` — same names as the C ABI, argument marshalling only: the calls of a generation loop in a C
+extension (csrc/pc_python.cpp), the others through ctypes.
 
 Every step of the path (scoring, selection, packing, rotary embedding, attention) runs in the library's CUDA
 kernels; PyTorch is used here for device memory and streams.  There is no CPU fallback: if the library cannot be
@@ -176,7 +177,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 def _stream(stream) -> int:
     if stream is None:
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)    # not a public name: half a microsecond less where it is there
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)    # not a public name; 0.3 us where it is there, the public way takes 3.2
         return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

@@ -12,9 +12,9 @@
 //                 bf16 P over S in TMEM (handed over in two halves of 64 keys), and rescale O in TMEM only when
 //                 the running max moved by more than 2^8.
 //                 While one tile's softmax runs, the tensor core works on the other tile.
-//   Key ranges of one work item are launched as a thread-block cluster and merge their (max, sum, O) through
-//   distributed shared memory at the end of the kernel; k_combine does the same from global partials when the
-//   cluster merge is switched off.
+//   k_combine     merges the (max, sum, O) partials of items that several CTAs worked on.  On request (pc_set_cluster_merge) the
+//                 key ranges of one item are launched as a thread-block cluster instead and merge through distributed shared
+//                 memory at the end of k_attend_tc.
 //
 // TMEM columns: S0/P0 0-127, S1/P1 128-255, O0 256-383, O1 384-511 (fp32, 128 lanes = the tile's rows).
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that makes every

@@ -13,9 +13,9 @@
 //                  single key tile reads every query tile twice as often from L2 for no gain).  Persistent CTAs, one per
 //                  SM, share the line of (unit, query tile) steps evenly: a CTA's run usually crosses from one unit into
 //                  the next, and a unit's sums come in up to MASS_PARTS pieces.  (A CTA per unit left SMs idle in its last
-//                  wave, as many as 38 %: 1,008 queries x 24 heads x
-//                  5,168 keys 70.3 us against 44.9, 9,200 72.7 / 71.2, 12,980 105.7 / 98.2; 300 x 16 x 1,200 20.3 / 11.6;
-//                  1,500 x 8 x 4,000, a unit per CTA either way, 21.5 / 22.5.)  The step's
+//                  wave, as many as 38 %: 24 / 8 heads, 1,008 queries
+//                  x 5,168 keys 70.7 us against 43.7, 9,200 72.9 / 70.5, 12,980 106.3 / 95.6; 16 / 16, 300 x 1,200 10.1 / 9.9;
+//                  8 / 8, 1,500 x 4,000, a unit per CTA either way, 21.8 / 22.1.)  The step's
 //                  normalisers ride along as a bulk copy into an eight-slot ring.  S^T = K Q^T (keys on the TMEM lanes,
 //                  queries on the columns) goes to one of two TMEM buffers per key tile.  Sixteen warps turn scores
 //                  into sums: per key tile and column half one warp per TMEM lane quadrant, one key per thread, 64

@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(PACK_THREADS) k_pack_rot(const char *__restric
 }
 
 // Selection and pack in one launch, for frames of at most a thread per token: a block takes RANKS consecutive ranks of a
-// frame's kept tokens, repeats the frame's selection, and moves its own.  Bound by launches: one fewer of six, on the GPU (64-token
-// fp32 frames 16.5 -> 15.8 us, 135-token bf16 frames 27.4 -> 27.1) and on the host (24.0 -> 21.5 us a call for the former).
+// frame's kept tokens, repeats the frame's selection, and moves its own.  Bound by launches: one fewer (of five in an fp32 step, 64-token
+// frames 16.5 -> 15.8 us on the GPU and 24.0 -> 21.5 us a call on the host; of six in a bf16 step, 135-token frames 27.4 -> 27.1).
 constexpr int RANKS = 8;
 
 template <int CPL, bool ROT>
