@@ -303,23 +303,22 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
         if (grp + step < n_groups) positions(grp + step);
         if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT, wait_us))) break;
         // Brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair.
-        // A lane that shares its token with 15 others has twice as many chunks as one of 32 would: it keeps two chains, chunks
-        // of even and of odd number, and adds their results (one chain: scores up to 10 % further from a 64-bit evaluation; one
-        // chain after the other: 0.3 to 0.8 us more for short histories).
-        float2 A[CH][TPL][NP], B[CH][TPL][NP];
+        // A lane that shares its token with 15 others has twice as many chunks as one of 32 would: it takes those of even number,
+        // then those of odd number, and adds the two results (all in one chain: scores up to 10 % further from a 64-bit
+        // evaluation).  Both chains at once take 161 registers instead of 128, and the block of 12 warps then fills the SM's
+        // registers: the next kernel's first blocks no longer start beside it (step of 135-token frames, 24 / 8 heads, 27.5 -> 29.1 us).
+        float s[TPL];
+        const uint32_t mine = ring + stage * stage_bytes + side * row_bytes + lt * 16;
+        const float4 *ql = qs + lt;
 #pragma unroll
-        for (int c = 0; c < CH; ++c)
+        for (int c = 0; c < CH; ++c) {
+            float2 A[TPL][NP], B[TPL][NP];
 #pragma unroll
             for (int i = 0; i < TPL; ++i)
 #pragma unroll
-                for (int u = 0; u < NP; ++u) A[c][i][u] = B[c][i][u] = make_float2(0.f, 0.f);
-        const uint32_t mine = ring + stage * stage_bytes + side * row_bytes + lt * 16;
-        const float4 *ql = qs + lt;
+                for (int u = 0; u < NP; ++u) A[i][u] = B[i][u] = make_float2(0.f, 0.f);
 #pragma unroll 1
-        for (int g0 = 0; g0 < parts; g0 += CH) {
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const int g = g0 + c;
+            for (int g = c; g < parts; g += CH) {
                 float x[TPL][PER];
 #pragma unroll
                 for (int i = 0; i < TPL; ++i) Elem<T>::unpack(pc_lds128(mine + i * SIDE * row_bytes + g * LPT * 16), x[i]);
@@ -330,28 +329,23 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
 #pragma unroll
                     for (int i = 0; i < TPL; ++i) {
                         const float2 kk = make_float2(x[i][2 * u], x[i][2 * u + 1]);
-                        A[c][i][u] = __ffma2_rn(qab, kk, A[c][i][u]);
-                        B[c][i][u] = __ffma2_rn(qba, kk, B[c][i][u]);
+                        A[i][u] = __ffma2_rn(qab, kk, A[i][u]);
+                        B[i][u] = __ffma2_rn(qba, kk, B[i][u]);
                     }
                 }
+            }
+#pragma unroll
+            for (int i = 0; i < TPL; ++i) {
+                float r = 0.f;
+#pragma unroll
+                for (int u = 0; u < NP; ++u)
+                    r = fmaf(cs[i][u].x, A[i][u].x + A[i][u].y, fmaf(cs[i][u].y, B[i][u].x + B[i][u].y, r));
+                s[i] = c == 0 ? r : s[i] + r;
             }
         }
         __syncwarp();                                                 // every lane has read the stage
         if (lane == 0 && grp + stages * step < n_groups) fill(stage, grp + stages * step);
         if (++stage == stages) { stage = 0; phase ^= 1; }
-        float s[TPL];
-#pragma unroll
-        for (int i = 0; i < TPL; ++i) {
-            float r[CH];
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                r[c] = 0.f;
-#pragma unroll
-                for (int u = 0; u < NP; ++u)
-                    r[c] = fmaf(cs[i][u].x, A[c][i][u].x + A[c][i][u].y, fmaf(cs[i][u].y, B[c][i][u].x + B[c][i][u].y, r[c]));
-            }
-            s[i] = CH == 2 ? r[0] + r[CH - 1] : r[0];
-        }
         // a token's lanes are added up; with two tokens in a lane its lower lanes carry on with the first, the upper ones with the second
         float sum = s[0];
         int o = LPT / 2, i_out = 0;
