@@ -21,6 +21,7 @@ DEVICE, PINNED = 2, 1                                     # cudaMemoryType
 class Runtime:
     def __init__(self, path):
         self.lib = C.CDLL(path)
+        self.open = []                                    # contexts and windows, closed while the binding still uses this library
         self.lib.rt_log.restype = C.c_char_p
         self.lib.rt_memory.argtypes = [C.c_void_p, C.c_size_t, C.c_int, C.c_int]
         self.lib.rt_fail.argtypes = [C.c_char_p, C.c_int]
@@ -68,6 +69,8 @@ def rt(_library, monkeypatch):
     r.reset()
     r.device(0)
     yield r
+    for x in reversed(r.open):
+        x.close()
     r.reset()
     r.device(0)
 
@@ -84,10 +87,16 @@ class Case:
         self.anchors, self.bufs, self.frame = seg(anchors, anchors), [seg(total + 2 * n, 0) for _ in range(2)], seg(n, n)
         for s in [self.anchors, self.frame] + self.bufs:
             rt.memory(s.k, s.v, s.pos)
-        self.make = lambda: pc.Window(self.ctx, window, pc.PC_LINEAR, 0.0, total, 0, self.anchors, self.bufs[0], self.bufs[1])
+        self.window = (window, pc.PC_LINEAR, 0.0, total, 0)
+        rt.open.append(self.ctx)
         self.q, self.q_pos = torch.zeros(n, hq, d, dtype=bf), torch.zeros(n, 4, dtype=torch.int32)
         self.out = torch.zeros_like(self.q)
         self.ws = {"q": torch.zeros_like(self.q), "q_pos": torch.zeros_like(self.q_pos), "out": torch.zeros_like(self.q)}
+
+    def make(self):
+        win = pc.Window(self.ctx, *self.window, self.anchors, self.bufs[0], self.bufs[1])
+        self.rt.open.append(win)
+        return win
 
     def step_host(self, win, **kw):
         f = {"k": self.frame.k, "v": self.frame.v, "pos": self.frame.pos}
