@@ -5,18 +5,30 @@
 //                 segments start on 128-row boundaries, and rotates Q with log2(e)/sqrt(d) folded in.
 //   k_attend_tc   persistent CTAs (one per SM) share the line of (item, key tile) steps evenly; an item = two 128-row
 //                 query tiles that share a KV head (grouped-query packing).
-//                 Warp 0 lane 0 drives TMA (K and V tiles, 128B swizzle, two stages each), warp 1 lane 0 issues
-//                 tcgen05.mma: S_t = Q_t K^T (both operands K-major in shared memory) into TMEM, and
-//                 O_t += P_t V with P_t read from TMEM and V MN-major in shared memory.  Warps 4-7 / 8-11 are the
-//                 softmax groups of tile 0 / 1: tcgen05.ld the S row, running max and sum in fp32 (base 2), write
-//                 bf16 P over S in TMEM (handed over in two halves of 64 keys), and rescale O in TMEM only when
+//                 Warp 0 lane 0 drives TMA (K and V tiles, 128B swizzle, two stages each), warps 1 and 2 issue
+//                 tcgen05.mma S = Q_t K^T of tile 0 and 1 (both operands K-major in shared memory) into TMEM, and warp 3
+//                 O_t += P_t V of both with P_t read from TMEM and V MN-major in shared memory.  Warps 4-7 / 8-11 are the
+//                 softmax groups of tile 0 / 1: tcgen05.ld the S row into registers, running max and sum in fp32 (base 2),
+//                 write bf16 P beside it (handed over in two halves of 64 keys), and rescale O in TMEM only when
 //                 the running max moved by more than 2^8.
 //                 While one tile's softmax runs, the tensor core works on the other tile.
 //   k_combine     merges the (max, sum, O) partials of items that several CTAs worked on.  On request (pc_set_cluster_merge) the
 //                 key ranges of one item are launched as a thread-block cluster instead and merge through distributed shared
 //                 memory at the end of k_attend_tc.
 //
-// TMEM columns: S0/P0 0-127, S1/P1 128-255, O0 256-383, O1 384-511 (fp32, 128 lanes = the tile's rows).
+// TMEM columns: S 0-127 (both tiles in turn), P0 128-191, P1 192-255, O0 256-383, O1 384-511 (128 lanes = the tile's rows).
+// A score row stays in TMEM only until it is in its thread's registers, so one S serves both tiles, and P has columns of its own:
+// a tile's next Q K^T waits for the other tile's scores to be read and no longer for its own P V, which wrote P over S and made
+// softmax -> P V -> Q K^T one chain (3,030 cycles per 128 keys of both tiles, of which the tensor core, the exponentials and
+// shared memory need 2,050 each).  What it took to get something from that, all on the critical path before: a wait
+// whose phase is complete costs 75 cycles instead of 155 with the first question outside the bounded loop; one commit behind a
+// group of multiply-adds (a second one in a row waits until the group has run: stages and query tiles are
+// released by the softmax warps); Q K^T and P V from different warps (in one, the tensor core's queue of about two
+// multiply-adds ran dry at every change); Q K^T of the two tiles from warps of two schedulers (the softmax warps beside
+// an issuer of Q K^T take 1,600 instead of 1,400 cycles for a row's exponentials); sums held to their chunk of exponentials; a warp's
+// number that the compiler knows to be uniform.  2,650 cycles before the last of these, bound by the softmax warps (1,024 cycles of exponentials of 16 a clock per row, twice).
+// That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
+// whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452.
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that makes every
 // later wait return at once, and the CTA still drains its copies, frees TMEM and exits.
 #include <algorithm>
@@ -44,8 +56,12 @@ constexpr int SM_ML = SM_BAR + 256;                       // (max, sum) of both 
 constexpr int SM_TOTAL = SM_ML + 2 * TILE * 8;
 constexpr int SM_ALLOC = SM_TOTAL + 1024;                 // slack for manual alignment
 
-enum { BAR_Q = 0, BAR_QFREE = 1, BAR_KEMPTY = 2, BAR_VFULL = 5, BAR_VEMPTY = 7, BAR_SFULL = 9, BAR_PHALF = 11 /* [tile][half] */,
-       BAR_DONE = 15, N_BARS = 16 };
+enum { BAR_Q = 0 /* [tile] */, BAR_QFREE = 2 /* [tile] */, BAR_VFULL = 4 /* [stage] */, BAR_EMPTY = 6 /* [step & 1] */, BAR_SFULL = 8 /* [tile] */,
+       BAR_SFREE = 10 /* [tile] */, BAR_PHALF = 12 /* [tile][half] */, BAR_PVDONE = 16 /* [tile] */, BAR_DONE = 18, N_BARS = 19 };
+static_assert(N_BARS * 8 + 12 <= 256, "barriers, abort flag and TMEM address share 256 bytes");
+
+// TMEM columns
+constexpr int TM_S = 0, TM_P = TILE, TM_O = 2 * TILE;     // scores; P of tile t at TM_P + 64 t; O of tile t at TM_O + 128 t
 
 struct TcParams {
     int n_q, n_q_heads, group, n_tb, tiles_per_g, pairs_per_g, n_splits, n_kv_tiles;
@@ -186,6 +202,17 @@ __device__ __forceinline__ Unit unit_at(const TcParams &P, long long g, long lon
     return u;
 }
 
+// arrival without a branch around it
+__device__ __forceinline__ void arrive_if(bool who, uint32_t bar) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)who) : "memory");
+}
+// Wait of a whole warp.  The first question stands alone: a phase that is complete is seen in 75 to 85 cycles instead of the
+// 155 that the way through the bounded wait's loop takes.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int32_t *status, uint32_t limit_us) {
+    if (__builtin_expect(__all_sync(0xffffffffu, pc_mbar_try(bar, parity)), 1)) return true;
+    return __all_sync(0xffffffffu, pc_mbar_wait(bar, parity, abort_flag, status, PC_WHERE_ATTN_WAIT, limit_us));
+}
+
 __global__ void __launch_bounds__(TC_THREADS, 1)
 k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
             const __grid_constant__ CUtensorMap map_v0, const __grid_constant__ CUtensorMap map_v1,
@@ -199,24 +226,27 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const uint32_t bar0 = base + SM_BAR;
     auto bar = [&](int i) { return bar0 + 8u * i; };
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // from one lane, so that the compiler knows a warp's number, and with it barrier and tensor-memory addresses and descriptors, to be
+    // the same in all lanes and keeps them in uniform registers
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     long long G0, G1;
     cta_run(P, (int)blockIdx.x, G0, G1);           // this CTA's run of steps (never empty: the host sizes the grid so)
 
     if (threadIdx.x == 0) {
-        mbar_init(bar(BAR_Q), 1);
-        mbar_init(bar(BAR_QFREE), 1);
-        mbar_init(bar(BAR_KEMPTY), 1);
         for (int s = 0; s < KV_STAGES; ++s) {
             mbar_init(bar(BAR_VFULL + s), 1);
-            mbar_init(bar(BAR_VEMPTY + s), 1);
+            mbar_init(bar(BAR_EMPTY + s), 4);
         }
         for (int t = 0; t < 2; ++t) {
+            mbar_init(bar(BAR_Q + t), 1);
+            mbar_init(bar(BAR_QFREE + t), 4);
             mbar_init(bar(BAR_SFULL + t), 1);
-            mbar_init(bar(BAR_PHALF + 2 * t), 128);
-            mbar_init(bar(BAR_PHALF + 2 * t + 1), 128);
+            mbar_init(bar(BAR_SFREE + t), 4);
+            mbar_init(bar(BAR_PVDONE + t), 1);
+            mbar_init(bar(BAR_PHALF + 2 * t), 4);
+            mbar_init(bar(BAR_PHALF + 2 * t + 1), 4);
         }
-        mbar_init(bar(BAR_DONE), 1);
+        mbar_init(bar(BAR_DONE), 3);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -239,9 +269,9 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         // ---------------------------------------------------------------- TMA producer
         reg_dealloc<72>();
         if (lane == 0) {
-            // A unit's query tiles arrive on BAR_Q once the last QK^T of the unit before has completed (BAR_QFREE); the
-            // run's first K tile rides with the first queries.  After that V(step) and K(step + 1) always travel together:
-            // they are needed at the same point and their stages are released at the same point, so one full / empty
+            // A unit's query tile t arrives on BAR_Q + t once the tile's last QK^T of the unit before has completed (BAR_QFREE + t);
+            // the run's first K tile rides with tile 0's first queries.  After that V(step) and K(step + 1) always travel together:
+            // they are needed at about the same time and their stages are released together, so one full / empty
             // barrier pair serves both.  K(step + 1) may be the first tile of the next unit.
             bool alive = true;
             int gs = 0, un = 0;
@@ -250,25 +280,27 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 g += U.n_j;
                 const int kvh = U.item / P.pairs_per_g, pair = U.item % P.pairs_per_g;
                 const int n_tiles_q = min(2, P.tiles_per_g - 2 * pair);
-                if (un > 0) alive = mbar_wait(bar(BAR_QFREE), (un - 1) & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
-                if (!alive) break;
-                mbar_expect_tx(bar(BAR_Q), (2 + (un == 0 ? 1 : 0)) * TILE_BYTES + (un == 0 ? P.extra_tx : 0u));
-                for (int t = 0; t < 2; ++t) {
+                for (int t = 0; t < 2 && alive; ++t) {
+                    if (un > 0) alive = mbar_wait(bar(BAR_QFREE + t), (un - 1) & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
+                    if (!alive) break;
+                    const bool first = un == 0 && t == 0;
+                    mbar_expect_tx(bar(BAR_Q + t), (first ? 2 : 1) * TILE_BYTES + (first ? P.extra_tx : 0u));
                     const int T = 2 * pair + min(t, n_tiles_q - 1), tb = T / P.group, h = kvh * P.group + T % P.group;
-                    tma_load_2d(base + SM_Q + t * TILE_BYTES, &map_q, h * TILE, tb * TILE, bar(BAR_Q));
-                    tma_load_2d(base + SM_Q + t * TILE_BYTES + HALF_BYTES, &map_q, h * TILE + 64, tb * TILE, bar(BAR_Q));
+                    tma_load_2d(base + SM_Q + t * TILE_BYTES, &map_q, h * TILE, tb * TILE, bar(BAR_Q + t));
+                    tma_load_2d(base + SM_Q + t * TILE_BYTES + HALF_BYTES, &map_q, h * TILE + 64, tb * TILE, bar(BAR_Q + t));
+                    if (first) {
+                        tma_load_2d(base + SM_K, &map_k, kvh * TILE, U.jb * TILE, bar(BAR_Q));
+                        tma_load_2d(base + SM_K + HALF_BYTES, &map_k, kvh * TILE + 64, U.jb * TILE, bar(BAR_Q));
+                    }
                 }
-                if (un == 0) {
-                    tma_load_2d(base + SM_K, &map_k, kvh * TILE, U.jb * TILE, bar(BAR_Q));
-                    tma_load_2d(base + SM_K + HALF_BYTES, &map_k, kvh * TILE + 64, U.jb * TILE, bar(BAR_Q));
-                }
+                if (!alive) break;
                 for (int j = 0; j < U.n_j && alive; ++j, ++gs) {
-                    const int st = gs % KV_STAGES, use = gs / KV_STAGES, kst = (gs + 1) % KV_STAGES;
+                    const int st = gs % KV_STAGES, kst = (gs + 1) % KV_STAGES;
                     int seg, local, n_valid;
                     kv_tile_info(P, U.jb + j, seg, local, n_valid);
                     const CUtensorMap *mv = seg == 0 ? &map_v0 : (seg == 1 ? &map_v1 : &map_v2);
-                    if (use > 0) alive = mbar_wait(bar(BAR_VEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
-                    else if (gs == 1) alive = mbar_wait(bar(BAR_KEMPTY), 0, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);   // K(2) lands where K(0) was
+                    // PV(step - 2) and QK^T(step - 1) have read what lies where V(step) and K(step + 1) go
+                    if (gs > 0) alive = mbar_wait(bar(BAR_EMPTY + ((gs - 1) & 1)), ((gs - 1) >> 1) & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
                     if (!alive) break;
                     const bool in_unit = j + 1 < U.n_j, more = in_unit || g < G1;
                     mbar_expect_tx(bar(BAR_VFULL + st), (more ? 2 : 1) * TILE_BYTES);
@@ -288,97 +320,110 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 while (global_ns() - t0 < 2000000ull) {}
             }
         }
-    } else if (warp == 1) {
-        // ---------------------------------------------------------------- MMA issuer
-        // The warp stays converged (every lane takes the waits) and only the tcgen05 instructions are predicated on
+    } else if (warp < 4) {
+        // ---------------------------------------------------------------- MMA issuers: warps 1 and 2 S = Q_t K^T, warp 3 O += P V
+        // A warp stays converged (every lane takes the waits) and only the tcgen05 instructions are predicated on
         // one elected lane: issuing a multiply-add then costs about 12 cycles instead of about 60.
         reg_dealloc<72>();
         const bool lead = elect_one();
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        auto issue_qk = [&](int t, int st) {
-            const uint32_t qa = base + SM_Q + t * TILE_BYTES, ka = base + SM_K + st * TILE_BYTES;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const uint32_t off = (ks >> 2) * HALF_BYTES + (ks & 3) * 32;
-                if (lead) mma_ss(tm + t * TILE, desc_kmajor(qa + off), desc_kmajor(ka + off), IDESC_QK, ks > 0);
-            }
-        };
-        bool alive = mbar_wait(bar(BAR_Q), 0, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
-        int gs = 0, un = 0;
-        if (alive) {
+        const int n_steps = (int)(G1 - G0);
+        auto wait = [&](int b, int parity) {
+            const bool ok = warp_wait(bar(b), parity, abort_flag, P.status, P.wait_us);
             tc_fence_after();
-            for (int t = 0; t < 2; ++t) {
-                issue_qk(t, 0);
+            return ok;
+        };
+        bool alive = true;
+        if (warp < 3) {
+            const int t = warp - 1;
+            const uint64_t dq0 = desc_kmajor(base + SM_Q + t * TILE_BYTES), dk0 = desc_kmajor(base + SM_K);
+            long long g = G0;
+            int un = -1, left = 0;                           // this unit, and its steps left
+#pragma unroll 1
+            for (int gs = 0; gs < n_steps; ++gs) {
+                if (left == 0) {
+                    left = unit_at(P, g, G1).n_j;
+                    g += left;
+                    ++un;
+                    alive = wait(BAR_Q + t, un & 1);
+                    if (!alive) break;
+                }
+                --left;
+                if (gs > 0) alive = wait(BAR_VFULL + (gs - 1) % KV_STAGES, ((gs - 1) / KV_STAGES) & 1);      // K(step) came with V(step - 1)
+                if (alive && gs + t > 0) alive = wait(BAR_SFREE + (t ^ 1), (gs + t + 1) & 1);      // the other tile's scores have left the columns
+                if (!alive) break;
+                uint64_t dq = dq0, dk = dk0 + (gs % KV_STAGES) * (TILE_BYTES >> 4);
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4)
+                        if (lead) mma_ss(tm + TM_S, dq + k4 * 2, dk + k4 * 2, IDESC_QK, (half > 0 || k4 > 0));
+                    dq += HALF_BYTES >> 4;
+                    dk += HALF_BYTES >> 4;
+                }
                 if (lead) tc_commit(bar(BAR_SFULL + t));
             }
-            if (lead) tc_commit(bar(BAR_KEMPTY));
-            if (unit_at(P, G0, G1).n_j == 1 && lead) tc_commit(bar(BAR_QFREE));      // that was the first unit's only QK^T
-        }
-        for (long long g = G0; g < G1 && alive; ++un) {
-            const Unit U = unit_at(P, g, G1);
-            g += U.n_j;
-            const int next_n_j = g < G1 ? unit_at(P, g, G1).n_j : 0;
-            for (int j = 0; j < U.n_j && alive; ++j, ++gs) {
-                const int st = gs % KV_STAGES, use = gs / KV_STAGES, nst = (gs + 1) % KV_STAGES;
-                alive = mbar_wait(bar(BAR_VFULL + st), use & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);      // V(step) and K(step + 1)
-                const bool in_unit = j + 1 < U.n_j, more = in_unit || next_n_j > 0;
+        } else {
+            const uint64_t dv0 = desc_mnmajor(base + SM_V);
+            int at = (int)(G0 % P.n_kv_tiles);               // key tile of the step
+#pragma unroll 1
+            for (int gs = 0; gs < n_steps && alive; ++gs) {
+                const int st = gs % KV_STAGES;
+                const bool first = gs == 0 || at == 0;       // of its unit
+                alive = wait(BAR_VFULL + st, (gs / KV_STAGES) & 1);
+                // the cluster merge stages O_0 where both query tiles lie: tile 1's last QK^T has read them before O_0 is final
+                if (P.cluster && gs + 1 == n_steps) alive = alive && wait(BAR_SFULL + 1, gs & 1);
+#pragma unroll 1
                 for (int t = 0; t < 2 && alive; ++t) {
-                    const uint32_t va = base + SM_V + st * TILE_BYTES;
                     // P arrives in two halves of 64 keys: the first PV steps run while the rest is exponentiated
-                    for (int hf = 0; hf < 2 && alive; ++hf) {
-                        alive = mbar_wait(bar(BAR_PHALF + 2 * t + hf), gs & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
+                    uint64_t dv = dv0 + st * (TILE_BYTES >> 4);
+                    uint32_t pa = tm + TM_P + t * (TILE / 2);
+                    const uint32_t oa = tm + TM_O + t * TILE;
+#pragma unroll 1
+                    for (int hf = 0; hf < 2; ++hf) {
+                        alive = wait(BAR_PHALF + 2 * t + hf, gs & 1);
                         if (!alive) break;
-                        tc_fence_after();
 #pragma unroll
-                        for (int k4 = 0; k4 < 4; ++k4) {   // 16 keys per step: P columns advance by 8 (two bf16 per column)
-                            const int ks = hf * 4 + k4;
-                            if (lead)
-                                mma_ts(tm + 256 + t * TILE, tm + t * TILE + ks * 8, desc_mnmajor(va + ks * 2048), IDESC_PV, (j > 0 || ks > 0));
-                        }
+                        for (int k4 = 0; k4 < 4; ++k4)     // 16 keys per step: P columns advance by 8 (two bf16 per column)
+                            if (lead) mma_ts(oa, pa + k4 * 8, dv + k4 * (2048 >> 4), IDESC_PV, (!first || hf > 0 || k4 > 0));
+                        dv += 8192 >> 4;
+                        pa += 32;
                     }
-                    if (!alive) break;
-                    if (more) {
-                        if (!in_unit && t == 0) {           // the next unit's queries must be in before its first QK^T
-                            alive = mbar_wait(bar(BAR_Q), (un + 1) & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
-                            if (!alive) break;
-                            tc_fence_after();
-                        }
-                        issue_qk(t, nst);
-                    }
-                    if (lead) tc_commit(bar(BAR_SFULL + t));          // S_t of the next step ready, and / or O_t of this unit final
+                    if (alive && lead) tc_commit(bar(BAR_PVDONE + t));            // P_t may be overwritten, O_t read
                 }
-                if (alive && lead) {
-                    // the QK^T just issued were the last of their unit: its query tiles may be overwritten
-                    if (more && (in_unit ? j + 2 == U.n_j : next_n_j == 1)) tc_commit(bar(BAR_QFREE));
-                    tc_commit(bar(BAR_VEMPTY + st));        // PV(step) and QK(step + 1) are behind this: V stage st and K stage nst are free
-                }
+                if (++at == P.n_kv_tiles) at = 0;
             }
         }
         // make sure nothing of ours is still running on the tensor core before TMEM is freed
         if (lead) tc_commit(bar(BAR_DONE));
         __syncwarp();
         mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
-    } else if (warp < 4) {
-        reg_dealloc<72>();
     } else {
         // ---------------------------------------------------------------- softmax + correction + epilogue
-        reg_alloc<208>();
+        reg_alloc<216>();
         const int t = (warp - 4) >> 2;
         const int quad = warp & 3;                       // TMEM lane quadrant this warp may touch
         const int r = quad * 32 + lane;                  // row of the tile
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-        const uint32_t s_addr = tmem + lane_addr + t * TILE;
-        const uint32_t o_addr = tmem + lane_addr + 256 + t * TILE;
+        const uint32_t s_addr = tmem + lane_addr + TM_S;
+        const uint32_t p_addr = tmem + lane_addr + TM_P + t * (TILE / 2);
+        const uint32_t o_addr = tmem + lane_addr + TM_O + t * TILE;
         bool alive = true;
+        const bool lead = elect_one();
         const int n_steps = (int)(G1 - G0);
         Unit U = unit_at(P, G0, G1);
         long long g = G0 + U.n_j;                        // end of the unit
         float m_used = -INFINITY, l = 0.f;
         int j = 0;
+        auto next_end = [&](int jt) {                    // last tile of the segment that tile jt is in
+            int seg = 0;
+            while (seg + 1 < P.n_seg && jt >= P.seg_tile_end[seg]) ++seg;
+            return P.seg_tile_end[seg] - 1;
+        };
+        int ragged = next_end(U.jb);
         // One turn per step and one more for the last read-out.  A unit's output leaves O_t in the turn behind its last step,
         // after the next unit's first probabilities are computed and before they are handed over (the first PV of a unit
-        // overwrites O_t): the scores of that turn come with the last PV's completion, and the stores run under the tensor
-        // core's next work.  Reading and storing O_t first left the tensor core idle meanwhile: the step at
+        // overwrites O_t): the stores run under the tensor core's next work.  Reading and storing O_t first left the tensor core idle meanwhile: the step at
         // 12 frames 88.1 against 86.4 us, 47 frames 167.4 against 165.5, 4,032-token frames 663.9 against 656.3.
         for (int gs = 0; alive; ++gs) {
             const bool end = gs == n_steps, flush = end || j == U.n_j;
@@ -390,14 +435,23 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 j = 0;
                 m_used = -INFINITY;
                 l = 0.f;
+                ragged = next_end(0);
             }
-            // scores of this step, and (the same commit) the PV of the step before is done
-            alive = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SFULL + t), gs & 1, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us));
-            if (!alive) break;
             if (!end) {
-                int seg, local, n_valid;
-                kv_tile_info(P, U.jb + j, seg, local, n_valid);
+                alive = warp_wait(bar(BAR_SFULL + t), gs & 1, abort_flag, P.status, P.wait_us);
+                if (!alive) break;
                 tc_fence_after();
+                if (__builtin_expect(U.jb + j == ragged, 0)) {      // last tile of a segment: keys past its end score -inf
+                    int seg, local, n_valid;
+                    kv_tile_info(P, ragged, seg, local, n_valid);
+                    ragged = P.seg_tile_end[min(seg + 1, P.n_seg - 1)] - 1;
+                    int i = n_valid;
+#pragma unroll 1
+                    for (; i & 7; ++i) tmem_st1(s_addr + i, 0xFF800000u);
+#pragma unroll 1
+                    for (; i < TILE; i += 8) tmem_st8(s_addr + i, 0xFF800000u);
+                    tmem_wait_st();
+                }
                 // the whole score row of this thread: one TMEM pass
                 uint32_t sv[128];
                 tmem_ld32(s_addr, sv);
@@ -405,11 +459,12 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 tmem_ld32(s_addr + 64, sv + 64);
                 tmem_ld32(s_addr + 96, sv + 96);
                 tmem_wait_ld();
-                if (n_valid < TILE) {                        // ragged last tile of a segment: keys past its end score -inf
-#pragma unroll
-                    for (int i = 0; i < TILE; ++i)
-                        if (i >= n_valid) sv[i] = 0xFF800000u;
-                }
+                tc_fence_before();
+                __syncwarp();
+                arrive_if(lead, bar(BAR_SFREE + t));         // the columns are the other tile's
+                if (j + 1 == U.n_j) arrive_if(lead, bar(BAR_QFREE + t));      // that was the unit's last QK^T of this tile
+                // the PV of the step before: its P columns are written again below, and O_t may be rescaled
+                const bool pv_done = gs == 0 || pc_mbar_test(bar(BAR_PVDONE + t), (gs - 1) & 1);
                 float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
                 for (int i = 0; i < TILE; i += 4) {
@@ -421,7 +476,14 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
                 // lazy rescale: move the reference maximum only when it grew by more than the threshold
                 const bool grow = mx > m_used + RESCALE_THRESHOLD;
-                if (__any_sync(0xffffffffu, grow)) {
+                if (__builtin_expect(!__all_sync(0xffffffffu, pv_done), 0)) {
+                    alive = warp_wait(bar(BAR_PVDONE + t), (gs - 1) & 1, abort_flag, P.status, P.wait_us);
+                    if (!alive) break;
+                }
+                tc_fence_after();
+                // tile 1 comes last: QK^T(step) and PV(step - 1) have read their keys and values
+                if (t == 1) arrive_if(lead, bar(BAR_EMPTY + (gs & 1)));
+                if (__builtin_expect(__any_sync(0xffffffffu, grow), 0)) {
                     const float m_new = fmaxf(m_used, mx);
                     const float corr = fast_exp2(m_used - m_new);       // 0 on the first tile (m_used = -inf)
                     l *= corr;
@@ -438,7 +500,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                     }
                     m_used = m_new;
                 }
-                // p = 2^(s - m) as bf16 pairs, written over the S columns; the row sum runs on two-lane adds
+                // p = 2^(s - m) as bf16 pairs; the row sum runs on two-lane adds
                 const float2 neg_m = make_float2(-m_used, -m_used);
                 float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
 #pragma unroll
@@ -455,17 +517,24 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                         pk[i] = pc_pack_bf16(x.x, x.y);
                         pk[i + 1] = pc_pack_bf16(y.x, y.y);
                     }
-                    tmem_st16(s_addr + c * 16, pk);
+                    // the sums belong in the gaps of this chunk's exponentials, not behind the hand-over
+                    asm volatile("" : "+f"(la.x), "+f"(la.y), "+f"(lb.x), "+f"(lb.y));
+                    tmem_st16(p_addr + c * 16, pk);
                     if (c & 1) {                               // keys 0-63, then 64-127, handed to the tensor core
                         tmem_wait_st();
                         tc_fence_before();
-                        if (!flush) mbar_arrive(bar(BAR_PHALF + 2 * t + (c >> 1)));
+                        __syncwarp();
+                        arrive_if(lead && !flush, bar(BAR_PHALF + 2 * t + (c >> 1)));
                     }
                 }
                 l += (la.x + la.y) + (lb.x + lb.y);
             }
-            if (flush) {
+            if (end) {
+                alive = warp_wait(bar(BAR_PVDONE + t), (gs - 1) & 1, abort_flag, P.status, P.wait_us);
+                if (!alive) break;
                 tc_fence_after();
+            }
+            if (__builtin_expect(flush, 0)) {
                 // the thread's whole O row leaves TMEM in one pass (four loads in flight, one wait)
                 uint32_t v[128];
                 tmem_ld32(o_addr, v);
@@ -475,8 +544,9 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 tmem_wait_ld();
                 if (!end) {
                     tc_fence_before();
-                    mbar_arrive(bar(BAR_PHALF + 2 * t));
-                    mbar_arrive(bar(BAR_PHALF + 2 * t + 1));
+                    __syncwarp();
+                    arrive_if(lead, bar(BAR_PHALF + 2 * t));
+                    arrive_if(lead, bar(BAR_PHALF + 2 * t + 1));
                 }
                 const int kvh = e_item / P.pairs_per_g, pair = e_item % P.pairs_per_g;
                 const int n_tiles_q = min(2, P.tiles_per_g - 2 * pair);
@@ -504,7 +574,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 } else if (P.cluster) {
                     // (split form, one unit per CTA) Stage O (un-normalised, fp32) and (max, sum) in shared memory that no
                     // multiply-add reads any more: tile 0 over both query tiles (every QK^T has completed once this tile's
-                    // last PV has), tile 1 over the key stages (its own last PV is the last multiply-add of the CTA).
+                    // last PV has, which was issued behind the other tile's last QK^T), tile 1 over the key stages (its own last PV is the last multiply-add of the CTA).
                     const uint32_t stage = base + (t == 0 ? SM_Q : SM_K);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) sts128(stage + stage_off(i, r), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
