@@ -767,7 +767,7 @@ int choose_ctas(int n_items, int n_kv_heads, long long steps, int most) {
 
 // Divides the line of (item, key tile) steps over CTAs: fills P.persistent, n_cta, n_splits, part_stride.
 //
-// What a division costs, in quarters of a step (a step is about 1.6 us): its longest run (boundaries reckoned in, or 14 for
+// What a division costs, in quarters of a step (a step is about 1.4 us): its longest run (boundaries reckoned in, or 14 for
 // them where runs are too short or too long for that), 7 for a merge.  The persistent form takes an even share of the line per CTA; the
 // split form cuts every item into s equal ranges, one CTA each, as long as all are resident at once: no boundary, and with one
 // range no merge.  Measured on rotated keys (query rotation + attention + merge), the persistent form against the one chosen
