@@ -97,7 +97,8 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     const uint32_t bar0 = base + SM_BAR;
     auto bar = [&](int i) { return bar0 + 8u * i; };
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // from one lane: known to be uniform, addresses and descriptors stay in uniform registers (guided step of 12 frames 130.8 -> 130.2 us)
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int G0 = run_start(P, blockIdx.x), G1 = run_start(P, blockIdx.x + 1);     // never empty
     const int unit0 = WHOLE ? (int)blockIdx.x : G0 / P.n_steps, g0 = unit0 / P.pairs, pair0 = unit0 - g0 * P.pairs;
     const int n_t = WHOLE ? min(2, P.n_kv_tiles - 2 * pair0) : 2;
