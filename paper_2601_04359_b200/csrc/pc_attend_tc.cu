@@ -29,8 +29,8 @@
 // number that the compiler knows to be uniform.  2,650 cycles before the last of these, bound by the softmax warps (1,024 cycles of exponentials of 16 a clock per row, twice).
 // That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
 // whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452.
-// Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that makes every
-// later wait return at once, and the CTA still drains its copies, frees TMEM and exits.
+// Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that ends every
+// later wait, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
 #include <algorithm>
 #include <numeric>
 
@@ -314,11 +314,6 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                     }
                 }
             }
-            if (*abort_flag) {
-                // give the copies already issued a bounded chance to land before the CTA's shared memory goes away
-                const uint64_t t0 = global_ns();
-                while (global_ns() - t0 < 2000000ull) {}
-            }
         }
     } else if (warp < 4) {
         // ---------------------------------------------------------------- MMA issuers: warps 1 and 2 S = Q_t K^T, warp 3 O += P V
@@ -397,7 +392,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         // make sure nothing of ours is still running on the tensor core before TMEM is freed
         if (lead) tc_commit(bar(BAR_DONE));
         __syncwarp();
-        mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_ATTN_WAIT, P.wait_us);
+        pc_mbar_drain(bar(BAR_DONE), 0, P.status, PC_WHERE_ATTN_WAIT);
     } else {
         // ---------------------------------------------------------------- softmax + correction + epilogue
         reg_alloc<216>();
@@ -599,6 +594,8 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
+    // every thread has done with its waits: the flag is final, and copies may be in flight that nobody waited for
+    if (threadIdx.x == 0 && *abort_flag) pc_let_copies_land();
     if (P.cluster && P.n_splits > 1) {
         // Merge the KV ranges of this item across the cluster: CTA `rank` finishes every n_splits-th row of the two
         // tiles, reading each peer's staged O and (max, sum) through distributed shared memory.  Sixteen threads share

@@ -195,6 +195,21 @@ __device__ __forceinline__ bool pc_mbar_wait(uint32_t bar, uint32_t parity, vola
         }
     }
 }
+// Wait for work that is under way and needs nothing more to end (multiply-adds that were issued, before their tensor memory is
+// freed): neither a caller's limit nor the abort flag cuts it short; one second bounds it all the same.
+__device__ __forceinline__ void pc_mbar_drain(uint32_t bar, uint32_t parity, int32_t *status, int where) {
+    const uint64_t t0 = pc_global_ns();
+    while (!pc_mbar_try(bar, parity))
+        if (pc_global_ns() - t0 > 1000000000ull) {
+            pc_flag(status, PC_ERR_TIMEOUT, where);
+            break;
+        }
+}
+// The copies a CTA has in flight when it gave up land within this time (one thread, before the shared memory goes away)
+__device__ __forceinline__ void pc_let_copies_land() {
+    const uint64_t t0 = pc_global_ns();
+    while (pc_global_ns() - t0 < 2000000ull) {}
+}
 // global -> shared bulk copy (both 16-byte aligned, size a multiple of 16), completion counted on an mbarrier
 __device__ __forceinline__ void pc_bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"

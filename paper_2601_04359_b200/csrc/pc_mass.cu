@@ -168,11 +168,6 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
                 }
                 if constexpr (WHOLE) break;
             }
-            if (*abort_flag) {
-                // give the copies already issued a bounded chance to land before the CTA's shared memory goes away
-                const uint64_t t0 = global_ns();
-                while (global_ns() - t0 < 2000000ull) {}
-            }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (converged warp, one elected lane)
@@ -207,7 +202,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         // nothing of ours may still be running on the tensor core when TMEM is freed
         if (lead) tc_commit(bar(BAR_DONE));
         __syncwarp();
-        mbar_wait(bar(BAR_DONE), 0, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
+        pc_mbar_drain(bar(BAR_DONE), 0, P.status, PC_WHERE_MASS_WAIT);
     } else if (warp >= 4 && (warp - 4) >> 3 < n_t) {
         // ---------------------------------------------------------------- column sums: one key and 64 query columns per thread
         const int cw = warp - 4;
@@ -260,6 +255,8 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
+    // every thread has done with its waits: the flag is final, and copies may be in flight that nobody waited for
+    if (threadIdx.x == 0 && *abort_flag) pc_let_copies_land();
 }
 
 struct ReduceParams {

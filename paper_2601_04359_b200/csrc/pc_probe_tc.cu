@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(128, 1) k_mma_rate(int form, int rounds, long 
         }
         if (lead) tc_commit(bar0 + 16);                 // everything issued has completed once this phase does
         __syncwarp();
-        mbar_wait(bar0 + 16, 0, abort_flag, status, PC_WHERE_ATTN_WAIT, wait_us);
+        pc_mbar_drain(bar0 + 16, 0, status, PC_WHERE_ATTN_WAIT);
         const long long c1 = clock64();
         const uint64_t n1 = global_ns();
         if (lead) {

@@ -366,11 +366,8 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
             }
         }
     }
-    if (grp < n_groups && lane == 0) {
-        // a wait ran out: the copies already issued get a bounded chance to land before the block's shared memory goes away
-        const uint64_t t0 = pc_global_ns();
-        while (pc_global_ns() - t0 < 2000000ull) {}
-    }
+    // a wait ran out: copies are in flight that this warp no longer waits for
+    if (grp < n_groups && lane == 0) pc_let_copies_land();
     if (warp == 0 && __shfl_sync(0xffffffffu, ticket, 0) == (unsigned long long)(gridDim.x - 1)) {
         for (int e = lane; e < n_out; e += 32) fx[e] = 0;
         if (lane == 0) fx[n_out] = 0;

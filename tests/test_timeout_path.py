@@ -89,3 +89,41 @@ def test_a_mass_wait_that_runs_out():
     again = pc.pc_attend_mass(ctx, lse, n_keys)
     assert pc.pc_poll_status(ctx) == pc.PC_OK and torch.equal(again, good)
     ctx.close()
+
+
+def _calls(ctx, D, cfg):
+    budget = np.full(cfg.n_frames, 7, np.int32)
+    n_keys = cfg.n_anchor + cfg.n_src
+    _, lse = pc.pc_attend_frame(ctx, D.cache, None, D.q, D.q_pos, want_lse=True)
+    calls = {"attend": lambda: pc.pc_attend_frame(ctx, D.cache, None, D.q, D.q_pos),
+             "mass": lambda: pc.pc_attend_mass(ctx, lse, n_keys),
+             "score": lambda: pc.pc_score(ctx, D.cache, D.q, D.q_pos, budget)}
+    for call in calls.values():
+        call()
+    assert pc.pc_poll_status(ctx) == pc.PC_OK
+    return calls
+
+
+def _timed_out_ms(ctx, call, limit_us):
+    pc.pc_set_wait_limit_us(ctx, limit_us)
+    pc.pc_test_expect_extra_bytes(ctx, 16)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record()
+    call()
+    b.record()
+    assert pc.pc_poll_status(ctx) == pc.PC_ERR_TIMEOUT
+    pc.pc_test_expect_extra_bytes(ctx, 0)
+    pc.pc_set_wait_limit_us(ctx, 0)
+    return a.elapsed_time(b)
+
+
+def test_copies_get_time_to_land_whoever_gives_up():
+    """A run of one step or two: the warp that issues the copies is done before another one gives up, and the copies still get
+    their two milliseconds."""
+    cfg = wl.small_bf16(n_frames=2, grid=(8, 9), seed=63)
+    D = DeviceLayer(wl.make_layer(cfg))
+    ctx = make_ctx(cfg)
+    for name, call in _calls(ctx, D, cfg).items():
+        ms = _timed_out_ms(ctx, call, 2000)
+        assert ms >= 2 + 2, f"{name}: {ms:.2f} ms"
+    ctx.close()
