@@ -389,8 +389,8 @@ pc_status pc_set_kv_splits(pc_ctx *ctx, int32_t n);
 pc_status pc_set_cluster_merge(pc_ctx *ctx, int32_t on);
 
 /* Limit of every bounded device-side wait of the context's kernels (scoring, tensor-core attention, attention mass), in
- * microseconds (0 = the default of about one second; pc_score_tokens_static, which has no context, always waits by the
- * default).  A wait that runs out records PC_ERR_TIMEOUT in the status word, the CTA gives up its remaining work, lets its
+ * microseconds, to within some ten (0 = the default of about one second; pc_score_tokens_static, which has no context, always
+ * waits by the default).  A wait that runs out records PC_ERR_TIMEOUT in the status word, the CTA gives up its remaining work, lets its
  * copies land, frees its tensor memory and exits; the outputs that depended on it are undefined (scores keep what their buffer
  * held) and the context stays usable. */
 pc_status pc_set_wait_limit_us(pc_ctx *ctx, uint32_t limit_us);

@@ -29,8 +29,8 @@
 // number that the compiler knows to be uniform.  2,650 cycles before the last of these, bound by the softmax warps (1,024 cycles of exponentials of 16 a clock per row, twice).
 // That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
 // whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452.
-// Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT, raises a CTA-wide abort flag that ends every
-// later wait, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
+// Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT and raises a CTA-wide abort flag; every later wait whose
+// phase is not complete gives up within some ten microseconds, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
 #include <algorithm>
 #include <numeric>
 
@@ -206,8 +206,8 @@ __device__ __forceinline__ Unit unit_at(const TcParams &P, long long g, long lon
 __device__ __forceinline__ void arrive_if(bool who, uint32_t bar) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)who) : "memory");
 }
-// Wait of a whole warp.  The first question stands alone: a phase that is complete is seen in 75 to 85 cycles instead of the
-// 155 that the way through the bounded wait's loop takes.
+// Wait of a whole warp.  The first question stands alone: a phase that is complete is seen in 75 to 85 cycles; through the loop
+// that the bounded wait began with once it took 155.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int32_t *status, uint32_t limit_us) {
     if (__builtin_expect(__all_sync(0xffffffffu, pc_mbar_try(bar, parity)), 1)) return true;
     return __all_sync(0xffffffffu, pc_mbar_wait(bar, parity, abort_flag, status, PC_WHERE_ATTN_WAIT, limit_us));

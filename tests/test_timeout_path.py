@@ -127,3 +127,16 @@ def test_copies_get_time_to_land_whoever_gives_up():
         ms = _timed_out_ms(ctx, call, 2000)
         assert ms >= 2 + 2, f"{name}: {ms:.2f} ms"
     ctx.close()
+
+
+@pytest.mark.parametrize("limit_us", [200, 2000])
+def test_a_wait_gives_up_when_its_limit_is_reached(limit_us):
+    """A call whose first wait runs out takes the limit, the time that copies in flight get to land (2 ms) and a few questions of
+    4 to 10 us each, and no more: 3 ms are left for those and the launches around the kernel."""
+    cfg = wl.small_bf16(n_frames=2, grid=(8, 9), seed=64)
+    D = DeviceLayer(wl.make_layer(cfg))
+    ctx = make_ctx(cfg)
+    for name, call in _calls(ctx, D, cfg).items():
+        ms = _timed_out_ms(ctx, call, limit_us)
+        assert ms <= limit_us / 1000 + 5, f"{name}: {ms:.2f} ms"
+    ctx.close()
