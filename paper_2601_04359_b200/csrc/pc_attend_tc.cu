@@ -41,6 +41,12 @@ namespace {
 using namespace pc_tc;
 
 constexpr int TC_THREADS = 384;
+// Registers a thread: as launched (all that one CTA of this size can have), then of warps 0-3 and of the softmax warps 4-11, which hold
+// a whole score row.  setmaxnreg.inc waits without a limit for registers that are not there, so the split may not exceed what the
+// block was launched with; that the compiler gave it as many is checked before the first launch.
+constexpr int REGS_LAUNCH = 65536 / TC_THREADS / 8 * 8, REGS_ISSUE = 72, REGS_SOFTMAX = 216;
+constexpr int REGS_SPLIT = 128 * REGS_ISSUE + 256 * REGS_SOFTMAX;
+static_assert(REGS_SPLIT <= TC_THREADS * REGS_LAUNCH && REGS_ISSUE % 8 == 0 && REGS_SOFTMAX % 8 == 0, "more registers than the block has");
 constexpr int KV_STAGES = 2;
 constexpr int MAX_SPLITS = 8;             // most parts of an item
 constexpr int BOUNDARY_STEPS = 2;         // what a CTA's crossing into the next item costs, in steps
@@ -264,10 +270,10 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     // Steps are counted through the whole run (gs): ring stages and barrier phases follow gs, so a unit boundary is an
     // ordinary step for the key / value pipeline.  Both query tiles always run; a unit whose head group has an odd tile
     // count loads its one tile twice and the second copy's result is dropped.
-    // the softmax warps hold a whole 128-column score row per thread: registers move from warps 0-3 to warps 4-11
+    // registers move from warps 0-3 to warps 4-11
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        reg_dealloc<72>();
+        reg_dealloc<REGS_ISSUE>();
         if (lane == 0) {
             // A unit's query tile t arrives on BAR_Q + t once the tile's last QK^T of the unit before has completed (BAR_QFREE + t);
             // the run's first K tile rides with tile 0's first queries.  After that V(step) and K(step + 1) always travel together:
@@ -319,7 +325,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         // ---------------------------------------------------------------- MMA issuers: warps 1 and 2 S = Q_t K^T, warp 3 O += P V
         // A warp stays converged (every lane takes the waits) and only the tcgen05 instructions are predicated on
         // one elected lane: issuing a multiply-add then costs about 12 cycles instead of about 60.
-        reg_dealloc<72>();
+        reg_dealloc<REGS_ISSUE>();
         const bool lead = elect_one();
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
         const int n_steps = (int)(G1 - G0);
@@ -395,7 +401,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         pc_mbar_drain(bar(BAR_DONE), 0, P.status, PC_WHERE_ATTN_WAIT);
     } else {
         // ---------------------------------------------------------------- softmax + correction + epilogue
-        reg_alloc<216>();
+        reg_alloc<REGS_SOFTMAX>();
         const int t = (warp - 4) >> 2;
         const int quad = warp & 3;                       // TMEM lane quadrant this warp may touch
         const int r = quad * 32 + lane;                  // row of the tile
@@ -919,6 +925,12 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     static bool attr_set[PC_MAX_DEVICES] = {};      // the attribute belongs to the device, not to the process
     if (ctx->device < 0 || ctx->device >= PC_MAX_DEVICES) return PC_ERR_UNSUPPORTED;
     if (!attr_set[ctx->device]) {
+        cudaFuncAttributes a;
+        PC_CUDA_TRY(cudaFuncGetAttributes(&a, k_attend_tc));
+        if (a.numRegs * TC_THREADS < REGS_SPLIT) {
+            fprintf(stderr, "packcache: attention kernel built with %d registers a thread, its warps would wait for more\n", a.numRegs);
+            return PC_ERR_CUDA;
+        }
         PC_CUDA_TRY(cudaFuncSetAttribute(k_attend_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_ALLOC));
         attr_set[ctx->device] = true;
     }

@@ -24,6 +24,7 @@ std::map<std::string, int> g_fail;                // calls of this name left unt
 std::map<const void *, std::string> g_name;       // kernels
 std::map<const void *, int> g_smem;               // their dynamic shared-memory limits
 std::map<const char *, Range> g_memory;
+int g_registers = 168;                            // what every kernel says it was built with
 void (*g_on_attribute)() = nullptr;               // called once, inside the next cudaFuncSetAttribute, after it took effect
 
 cudaError_t done(cudaError_t e) {
@@ -60,6 +61,7 @@ void rt_reset() {
     g_log.clear();
     g_fail.clear();
     g_on_attribute = nullptr;
+    g_registers = 168;
     t_last = cudaSuccess;
 }
 void rt_fail(const char *name, int after) { g_fail[name] = after; }
@@ -126,6 +128,12 @@ cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v) {
         g_on_attribute = nullptr;
         call();
     }
+    return cudaSuccess;
+}
+void rt_registers(int n) { g_registers = n; }
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes *a, const void *) {
+    memset(a, 0, sizeof *a);
+    a->numRegs = g_registers;
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) { *n = 2; return cudaSuccess; }

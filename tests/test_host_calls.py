@@ -182,3 +182,17 @@ def test_attention_gives_up_sms_only_for_shared_streams(rt, heads, rows, keys, b
     pos = torch.empty(rows, 4, dtype=torch.int32)
     assert rt.lib.pc_attend_frame(c.ctx.handle, C.byref(s), None, pc._ptr(q), pc._ptr(pos), rows, pc._ptr(out), None, None) == pc.PC_OK
     assert rt.lib.rt_blocks(b"k_attend_tc") == blocks
+
+
+def test_attention_is_not_launched_with_fewer_registers_than_its_warps_share_out(rt):
+    """Its softmax warps ask for registers that the block must have been launched with, and wait for them without a limit."""
+    rt.device(2)                                          # a device on which no other test has launched it
+    c = Case(rt)
+    rt.memory(c.q, c.q_pos, c.out, device=2)
+    cache = pc.Cache(c.anchors, c.frame, np.array([c.n], np.int32)).c()
+    attend = lambda: rt.lib.pc_attend_frame(c.ctx.handle, C.byref(cache), None, pc._ptr(c.q), pc._ptr(c.q_pos), c.n, pc._ptr(c.out), None, None)  # noqa: E731
+    launched = lambda: [line for line in rt.log() if line.startswith("launch k_attend")]  # noqa: E731
+    rt.lib.rt_registers(160)
+    assert attend() == pc.PC_ERR_CUDA and not launched()
+    rt.lib.rt_registers(168)
+    assert attend() == pc.PC_OK and len(launched()) == 1
