@@ -749,11 +749,12 @@ int choose_splits(int n_items, int n_kv_tiles, int sm_count) {
 // parts.  So up to 1/32 of the SMs is given up for the fewest starting places, as long as the longest run grows by no more
 // than that (a run counts whole steps), where that makes streams that CTAs share: at least two CTAs of a KV head to a starting place,
 // and runs so much shorter than an item (items fewer than 3/4 of the CTAs) that neighbours stay in step.  Measured, one CTA per SM
-// against this rule: attention over 47 whole frames 725 -> 628 us a call, five passes over 7,184 keys 519 -> 513, the step at 47
-// frames 170.7 -> 169.9.  144 CTAs without the two conditions, against 148 (rotated keys, sides in turn): 16 / 16 heads, 1,008
-// queries x 30,000 keys (9 places, 9 CTAs a head) 232 -> 243 us, 32 / 8, 1,008 x 30,000 (128 items) 464 -> 471, 64 / 8, 1,008 x
-// 30,000 (256) 976 -> 999, 24 / 8, 2,000 x 30,000 (192) 691 -> 702, 24 / 8, 4,032 x 7,184 (384) 326 -> 330; where they hold: 8 / 8,
-// 1,008 x 48,000 (32) 189 -> 178, 24 / 12, 1,008 x 30,000 (96) 352 -> 327, 24 / 8, 400 x 30,000 (48) 157 -> 156.
+// against this rule: attention over 47 whole frames 677 -> 571 us a call, five passes over 7,184 keys 461 -> 452, the step at 47
+// frames 151.0 -> 149.7, at 12 79.5 -> 77.9.  With the loop before this one (probabilities over the scores): 144 CTAs without the two
+// conditions, against 148 (rotated keys, sides in turn): 16 / 16 heads, 1,008 queries x 30,000 keys (9 places, 9 CTAs a head)
+// 232 -> 243 us, 32 / 8, 1,008 x 30,000 (128 items) 464 -> 471, 64 / 8, 1,008 x 30,000 (256) 976 -> 999, 24 / 8, 2,000 x 30,000
+// (192) 691 -> 702, 24 / 8, 4,032 x 7,184 (384) 326 -> 330; where they hold: 8 / 8, 1,008 x 48,000 (32) 189 -> 178, 24 / 12,
+// 1,008 x 30,000 (96) 352 -> 327, 24 / 8, 400 x 30,000 (48) 157 -> 156.
 int choose_ctas(int n_items, int n_kv_heads, long long steps, int most) {
     if (4 * n_items >= 3 * most) return most;
     int best = most, best_starts = most / std::gcd(most, n_items);
@@ -770,14 +771,16 @@ int choose_ctas(int n_items, int n_kv_heads, long long steps, int most) {
 
 // Divides the line of (item, key tile) steps over CTAs: fills P.persistent, n_cta, n_splits, part_stride.
 //
-// What a division costs, in quarters of a step (a step is about 1.4 us): its longest run (boundaries reckoned in, or 14 for
-// them where runs are too short or too long for that), 7 for a merge.  The persistent form takes an even share of the line per CTA; the
+// What a division costs, in quarters of a step (a step is about 1.4 us): its longest run (boundaries reckoned in, or 16 for
+// them where runs are too short or too long for that), 8 for a merge.  The persistent form takes an even share of the line per CTA; the
 // split form cuts every item into s equal ranges, one CTA each, as long as all are resident at once: no boundary, and with one
 // range no merge.  Measured on rotated keys (query rotation + attention + merge), the persistent form against the one chosen
-// here: 8 / 8 heads, 144 queries x 2,000 keys 22.3 -> 15.9 us, 700 x 3,000 29.8 -> 21.6; 24 / 8 heads,
-// 135 x 472 17.7 -> 14.8, 135 x 1,500 21.0 -> 17.9, 400 x 4,000 36.5 -> 33.7, 700 x 3,000 43.8 -> 39.0; 32 / 16 heads, 500 x
-// 2,000 36.3 -> 31.1.  (Three ranges at most before; merging the ranges of an item in a cluster instead was slower throughout:
-// 20.2 to 22.0 us at 135 x 472.)
+// here: 16 / 4 heads, 556 queries x 1,549 keys 29.1 -> 21.9 us, 74 x 4,767 20.9 -> 18.4; 24 / 8, 300 x 305 17.8 -> 17.2 (two ranges,
+// which 7 for a merge took, 18.7), 355 x 2,818 27.5 -> 26.4; 32 / 8, 237 x 1,040 20.3 -> 18.8, 1,040 x 3,629 75.1 -> 65.2; 32 / 16,
+// 500 x 2,000 29.1 -> 28.1.  Over 274 calls of 20 to 2,500 queries and 100 to 14,000 keys (10 to 260 us) the choice takes 2.0 % more
+// than the best form of each, in the geometric mean; most where the reckoning is level, more than four parts are merged and the
+// persistent form stands: 32 / 8, 48 x 1,033 17.2 against 14.7 in five ranges.  (Merging the ranges of an item in a cluster instead:
+// 24 / 8, 135 x 472 in three 24.1 against 15.9, 1,008 x 9,200 in two 143 against 133.)
 void choose_division(const pc_ctx *ctx, int n_items, int tiles, TcParams &P) {
     const long long T = (long long)n_items * tiles;
     P.persistent = 0;
@@ -787,19 +790,19 @@ void choose_division(const pc_ctx *ctx, int n_items, int tiles, TcParams &P) {
         const int n = choose_ctas(n_items, ctx->desc.n_kv_heads, T, (int)std::min<long long>(std::min<long long>(ctx->sm_count, (long long)n_items * (MAX_SPLITS - 1)), T));
         const bool crossing = n % n_items != 0;
         P.n_cta = n;
-        // Shorter runs than six times the boundary could end up empty; in longer ones than 64 steps it does not show any more.
-        // Boundaries reckoned in against an even share of the steps: the step at 12 frames (runs of 22) 89.7 -> 88.4 us,
-        // passes over 7,184 keys (38) 517.1 -> 514.7, 47 frames (48) 167.9 -> 167.5; in runs of 259 and 267 steps 620.4 -> 624.7
-        // (47 whole frames) and 649.8 -> 655.6 (4,032-token frames).
+        // Shorter runs than six times the boundary could end up empty; in longer ones than 64 steps it shows little.
+        // Boundaries reckoned in against an even share of the steps, a pass: 4,160 keys (runs of 22) 56.8 -> 54.6 us, 7,184 (38) 88.7 ->
+        // 85.6, 9,200 (48) 108.1 -> 105.7; in runs of 75 to 127 166.2 -> 165.0, 187.3 -> 181.4, 266.0 -> 263.0, of 131 to 343 within
+        // 1 % either way but for 721.9 -> 736.3 (305), and 154.4 -> 157.8 (69, 71 key tiles an item).
         P.gap = crossing && T >= 6LL * BOUNDARY_STEPS * n && T <= 64LL * n ? BOUNDARY_STEPS : 0;
         int most = 1;
         for (int i = 0; i < n_items / std::gcd(n, n_items); ++i)        // the cuts repeat
             most = std::max(most, cta_of_step(P, i, tiles - 1) - cta_of_step(P, i, 0) + 1);
-        long long best = 4 * ((line_length(P) + n - 1) / n) + (crossing && P.gap == 0 ? 14 : 0) + (most > 1 ? 7 : 0);
+        long long best = 4 * ((line_length(P) + n - 1) / n) + (crossing && P.gap == 0 ? 16 : 0) + (most > 1 ? 8 : 0);
         P.persistent = 1;
         P.n_splits = P.part_stride = most;
         for (int s = 1; s <= MAX_SPLITS && s <= tiles && n_items * s <= ctx->sm_count; ++s) {
-            const long long cost = 4 * div_up(tiles, s) + (s > 1 ? 7 : 0);
+            const long long cost = 4 * div_up(tiles, s) + (s > 1 ? 8 : 0);
             if (cost < best) {
                 best = cost;
                 P.persistent = 0;

@@ -196,3 +196,14 @@ def test_attention_is_not_launched_with_fewer_registers_than_its_warps_share_out
     assert attend() == pc.PC_ERR_CUDA and not launched()
     rt.lib.rt_registers(168)
     assert attend() == pc.PC_OK and len(launched()) == 1
+
+
+def test_a_merge_is_reckoned_as_what_it_takes(rt):
+    """40 items of four key tiles: two ranges each (80 CTAs) save two steps and cost a merge, which is as long; one range, no merge."""
+    c = Case(rt, n=300, anchors=304)
+    one = pc.Segment(c.frame.k, c.frame.v, c.frame.pos, 1)
+    cache = pc.Cache(c.anchors, one, np.array([1], np.int32)).c()
+    rt.lib.rt_blocks.argtypes = [C.c_char_p]
+    assert rt.lib.pc_attend_frame(c.ctx.handle, C.byref(cache), None, pc._ptr(c.q), pc._ptr(c.q_pos), c.n, pc._ptr(c.out), None, None) == pc.PC_OK
+    assert rt.lib.rt_blocks(b"k_attend_tc") == 40
+    assert not [line for line in rt.log() if line.startswith("launch k_combine")]
