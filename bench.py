@@ -351,7 +351,7 @@ def run_cuda(args):
     stream_single_ms = float(np.median(singles))
     stream_b2b_ms = timed(stream_fn, 100)
 
-    # ---- yardstick for the attention kernel: its tensor-core issue stream alone (no loads, no softmax), one CTA per SM, a few
+    # ---- yardstick for the attention kernel: its tensor-core instructions alone (no loads, no softmax), one CTA per SM, a few
     # milliseconds per form: cycles per 128 x 128 x 16 multiply-add and the SM clock under that load
     sm_count = torch.cuda.get_device_properties(local).multi_processor_count
     mma = {form: pc.pc_probe_mma_rate(ctx, form, rounds=2000) for form in ("qk", "pv", "mix")}
@@ -559,9 +559,9 @@ def run_cuda(args):
                          "cycles_per_mma": {k: round(v[0], 2) for k, v in mma.items()}, "sm_ghz_under_load": {k: round(v[1], 3) for k, v in mma.items()},
                          "tflops_mix_never_waiting": 524288.0 * sm_count * mma["mix"][1] * 1e9 / mma["mix"][0] / 1e12,
                          "frac_of_yardstick": achieved / (524288.0 * sm_count * mma["mix"][1] * 1e9 / mma["mix"][0] / 1e12),
-                         "what": "pc_probe_mma_rate: the kernel's own tcgen05.mma stream (Q K^T from shared memory, P V with P in "
-                                 "tensor memory, and both in the kernel's order) issued back to back on every SM with nothing else "
-                                 "running; 524,288 flop per multiply-add x SMs x clock / cycles is what the tensor cores deliver "
+                         "what": "pc_probe_mma_rate: the kernel's tcgen05.mma instructions (Q K^T from shared memory, P V with P in "
+                                 "tensor memory, and both in turn) issued back to back by one warp on every SM with nothing else "
+                                 "running (the kernel issues from three warps, in no fixed order); 524,288 flop per multiply-add x SMs x clock / cycles is what the tensor cores deliver "
                                  "to this instruction mix when they never wait"},
                      "how": "flops / the kernel's mean duration by CUDA events on the launching stream: the event mark in front "
                             "of the kernel left out, span of the pack kernel and this one minus the pack kernel's own span (the "

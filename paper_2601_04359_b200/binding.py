@@ -401,7 +401,7 @@ MMA_FORMS = {"qk": (0, 16), "pv": (1, 16), "mix": (2, 32)}   # form id, multiply
 
 
 def pc_probe_mma_rate(ctx: Context, form: str, rounds: int = 2000, n_cta: int | None = None, stream=None):
-    """The attention kernel's tensor-core issue stream alone (form "qk", "pv" or "mix").  Returns (cycles per multiply-add,
+    """The attention kernel's tensor-core instructions alone (form "qk", "pv" or "mix": both in turn).  Returns (cycles per multiply-add,
     SM clock in GHz), each the median over the CTAs (one per SM unless n_cta says otherwise).  Synchronises."""
     fid, per_round = MMA_FORMS[form]
     if n_cta is None:

@@ -26,9 +26,11 @@
 // released by the softmax warps); Q K^T and P V from different warps (in one, the tensor core's queue of about two
 // multiply-adds ran dry at every change); Q K^T of the two tiles from warps of two schedulers (the softmax warps beside
 // an issuer of Q K^T take 1,600 instead of 1,400 cycles for a row's exponentials); sums held to their chunk of exponentials; a warp's
-// number that the compiler knows to be uniform.  2,650 cycles before the last of these, bound by the softmax warps (1,024 cycles of exponentials of 16 a clock per row, twice).
+// number that the compiler knows to be uniform.  2,560 cycles now, bound by the softmax warps (the exponentials of a tile's 128 rows take
+// 1,024 at 16 a clock, twice).
 // That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
-// whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452.
+// whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452; since the
+// bounded wait lost its loop of questions 77.2, 148.5, 586, 569 and 450.
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT and raises a CTA-wide abort flag; every later wait whose
 // phase is not complete gives up within some ten microseconds, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
 #include <algorithm>

@@ -1,6 +1,7 @@
-// Measurement support: the issue stream of the attention kernel's tensor-core multiply-adds with nothing else going on, as a
-// yardstick for that kernel: how many SM cycles one tcgen05.mma (128 x 128 x 16, bf16, fp32 accumulate) takes back to back,
-// and what the SM clock is meanwhile (cycles against the global timer).
+// Measurement support: the attention kernel's tensor-core multiply-adds issued by one warp with nothing else going on, as a yardstick
+// of what the tensor core delivers to them: how many SM cycles one tcgen05.mma (128 x 128 x 16, bf16, fp32 accumulate) takes
+// back to back, and what the SM clock is meanwhile (cycles against the global timer).  Operands lie as in that kernel; the order
+// is not its own: there three warps issue, into one S for both query tiles, as scores and probabilities come and go.
 #include "pc_tc.cuh"
 
 namespace {
@@ -10,10 +11,11 @@ using namespace pc_tc;
 constexpr int PROBE_SM_BAR = 6 * TILE_BYTES;                    // two query tiles, two K stages, two V stages, as in the attention kernel
 constexpr int PROBE_SM_ALLOC = PROBE_SM_BAR + 256 + 1024;       // barriers etc. + slack for manual alignment
 
-// One CTA per SM (the shared memory sees to that), one issuing warp.  A round is what the attention kernel issues per key
-// tile for both query tiles: form 0 only the QK^T multiply-adds (A and B in shared memory; 16 per round), form 1 only the
-// PV multiply-adds (A in tensor memory; 16 per round), form 2 both in the kernel's order (32 per round).  Two rounds are in
-// flight: round i is issued once round i - 2 has completed.  Operands are pseudo-random bf16; the results are not used.
+// One CTA per SM (the shared memory sees to that), one issuing warp.  A round is as many multiply-adds as the attention kernel issues
+// per key tile for both query tiles: form 0 only Q K^T (A and B in shared memory; 16 per round), form 1 only P V (A in tensor
+// memory; 16 per round), form 2 both in turn, P V and Q K^T of tile 0, then of tile 1 (32 per round), each tile with scores
+// of its own that its P V reads as probabilities.  Two rounds are in flight: round i is issued once round i - 2 has
+// completed.  Operands are pseudo-random bf16; the results are not used.
 __global__ void __launch_bounds__(128, 1) k_mma_rate(int form, int rounds, long long *cycles, long long *nanos, uint32_t wait_us,
                                                       int32_t *status) {
     pc_grid_dep_launch();

@@ -92,17 +92,17 @@ def _lumos(name: str, n_frames: int, budget: Budget, **kw) -> Config:
 
 
 CONFIGS: Dict[str, Config] = {
-    # configs[0]: tiny fp32 correctness case; closed-form half-life-1 allocation (Eq. 7)
+    # tiny fp32 correctness case; closed-form half-life-1 allocation (Eq. 7)
     "tiny": Config(name="tiny", n_q_heads=4, n_kv_heads=2, head_dim=64, dtype=F32,
                    n_text=32, grid=(8, 8), n_frames=6,
                    budget=Budget(CLOSED_HALF, 0.5, 128)),
-    # configs[1]: 12 history frames, 25% of history, linear decay
+    # 12 history frames, 25% of history, linear decay
     "lumos12": _lumos("lumos12", 12, Budget(LINEAR, 0.0, (12 * 1008) // 4)),
-    # configs[2]: 24 history frames, 6048 retained, half-life 4
+    # 24 history frames, 6048 retained, half-life 4
     "lumos24": _lumos("lumos24", 24, Budget(HALFLIFE, 4.0, 6048)),
-    # configs[3]: 47 history frames, newest 2 kept whole, 6048 over the rest at half-life 4
+    # 47 history frames, newest 2 kept whole, 6048 over the rest at half-life 4
     "lumos47": _lumos("lumos47", 47, Budget(HALFLIFE, 4.0, 2 * 1008 + 6048, keep_full=2)),
-    # configs[4]: 28 stacked layers of the lumos shape, sweep driven by the caller
+    # 28 stacked layers of the lumos shape, sweep driven by the caller
     "stack28": _lumos("stack28", 47, Budget(HALFLIFE, 4.0, (47 * 1008) // 4), n_layers=28),
 }
 
