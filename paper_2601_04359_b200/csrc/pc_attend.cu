@@ -183,10 +183,13 @@ pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *bu
     const bool one_launch = !hooks && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
     ctx->last_n_q = 0;
     ctx->q_rot_n = 0;
-    st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream, !one_launch);
+    const pc_front_args args{src, budget, nullptr, scores, sel_idx, delta_t, &dst->history, k_rot_dst};
+    const pc_front_args *front = !hooks && n_sel > 0 && pc_front_fits(ctx, src, true) ? &args : nullptr;
+    st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream, !one_launch, front);
     if (st != PC_OK) return st;
     if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
-    st = one_launch ? pc_launch_select_pack(ctx, scores, src, budget, delta_t, &dst->history, sel_idx, k_rot_dst, stream)
+    if (!front)
+        st = one_launch ? pc_launch_select_pack(ctx, scores, src, budget, delta_t, &dst->history, sel_idx, k_rot_dst, stream)
                     : pc_compact_impl(ctx, src, sel_idx, budget, delta_t, dst, k_rot_dst, stream);
     if (st != PC_OK) return st;
     dst->history.n_tokens = (int32_t)n_sel;

@@ -281,6 +281,20 @@ pc_status pc_check_segment(const pc_segment *s, bool allow_empty);
 pc_status pc_launch_pack(pc_ctx *ctx, const void *src_k, const void *src_v, const int32_t *src_pos, const int32_t *sel_idx,
                          int n_sel, int n_src, int delta_t, void *dst_k, void *dst_v, int32_t *dst_pos, void *k_rot_dst,
                          cudaStream_t stream);
+// Scores, selection and (dst given) pack of a small history in one launch behind the query pass, and whether a call suits it;
+// arguments already checked
+struct pc_front_args {
+    const pc_cache *src;
+    const int32_t *budget;
+    const uint8_t *valid;
+    float *scores;
+    int32_t *sel_idx;
+    int32_t delta_t;
+    const pc_segment *dst;       // NULL: no pack
+    void *k_rot_dst;             // as pc_launch_pack
+};
+bool pc_front_fits(const pc_ctx *ctx, const pc_cache *src, bool pack);
+pc_status pc_launch_front(pc_ctx *ctx, const pc_front_args &args, int32_t n_q, cudaStream_t stream);
 // pc_score / pc_compact with the extras of the fused frame step: q_rot_out (NULL or the context's rotated-query scratch,
 // filled by the query pass that also pools), k_rot_dst (as pc_launch_pack)
 bool pc_score_supports(const pc_layer_desc &D);   // the row widths the query pass and the scoring kernel take
@@ -288,7 +302,7 @@ pc_status pc_score_check(const pc_ctx *ctx, const pc_cache *src, const void *q, 
                          const float *scores_override, const float *scores, const int32_t *sel_idx);   // every host-side check of pc_score_impl, nothing enqueued
 pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
                         const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
-                        cudaStream_t stream, bool select = true);   // select = false: scores only, the caller selects
+                        cudaStream_t stream, bool select = true, const pc_front_args *front = nullptr);   // select = false: scores only, the caller selects; front: selection and pack in one launch with the scores
 // selection and pack in one launch (small frames): whether a call's frames suit it, and the launch (arguments already checked)
 bool pc_select_pack_fits(const pc_ctx *ctx, const pc_cache *src, const int32_t *budget);
 pc_status pc_launch_select_pack(pc_ctx *ctx, const float *scores, const pc_cache *src, const int32_t *budget, int delta_t, const pc_segment *dst,

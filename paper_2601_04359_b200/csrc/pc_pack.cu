@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(PACK_THREADS) k_select_pack(const float *__res
     const int first = blockIdx.x * RANKS, n = min(RANKS, fr.z - first), out0 = fr.w + first;
     pc_grid_dep_wait();
     if (n <= 0) return;
-    frame_select<PACK_THREADS>(scores, fr, sm, status, [&](int at, int idx) {
+    frame_select<PACK_THREADS>(scores + fr.x, fr, sm, status, [&](int at, int idx) {
         if ((unsigned)(at - first) < (unsigned)n) {
             mine[at - first] = idx;
             sel_idx[fr.w + at] = idx;

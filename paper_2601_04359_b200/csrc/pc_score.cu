@@ -14,25 +14,10 @@
 #include <atomic>
 #include <type_traits>
 
-#include "pc_common.cuh"
+#include "pc_rows.cuh"
 #include "pc_select.cuh"
 
 namespace {
-
-template <typename T> struct Elem;
-template <> struct Elem<float> {
-    static constexpr int PER16 = 4;
-    static __device__ __forceinline__ void unpack(const uint4 &v, float *f) {
-        f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
-    }
-};
-template <> struct Elem<__nv_bfloat16> {
-    static constexpr int PER16 = 8;
-    static __device__ __forceinline__ void unpack(const uint4 &v, float *f) {
-        f[0] = pc_bf16_lo(v.x); f[1] = pc_bf16_hi(v.x); f[2] = pc_bf16_lo(v.y); f[3] = pc_bf16_hi(v.y);
-        f[4] = pc_bf16_lo(v.z); f[5] = pc_bf16_hi(v.z); f[6] = pc_bf16_lo(v.w); f[7] = pc_bf16_hi(v.w);
-    }
-};
 
 // ---------------------------------------------------------------------------------------------------------
 // Query pass.  One read of Q serves both consumers of the rotated queries: the pooled query of the scoring pass
@@ -59,16 +44,6 @@ template <> struct Elem<__nv_bfloat16> {
 constexpr int QPREP_WARPS = 16;                     // most warps per block, unless one token needs more
 constexpr int QPREP_SUM_WARPS = 8;                  // tokens whose elements are added in fp32, in warps
 constexpr int QPREP_SLAB = 200 * 1024;              // most shared memory of a block (one token takes up to 128 KB: 32 parts of 4 x 32 chunks)
-constexpr float FX_ONE = 4294967296.0f;             // 2^32
-
-template <typename T> __device__ __forceinline__ uint4 pack_row(const float *f);
-template <> __device__ __forceinline__ uint4 pack_row<float>(const float *f) {
-    return make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
-}
-template <> __device__ __forceinline__ uint4 pack_row<__nv_bfloat16>(const float *f) {
-    return make_uint4(pc_pack_bf16(f[0], f[1]), pc_pack_bf16(f[2], f[3]), pc_pack_bf16(f[4], f[5]), pc_pack_bf16(f[6], f[7]));
-}
-
 // A query row is cut into `parts` runs of CPW x 32 chunks, one warp each; a block holds `slots` tokens at a time, `run` of which
 // go into one fp32 sum.
 // KEEP: a thread's sums over its tokens carry what each addition rounds off into the next one (Kahan), two elements at a time.
@@ -139,7 +114,7 @@ __global__ void __launch_bounds__(MAX_THREADS, MAX_THREADS == 512 && !KEEP && CP
             if (dst) {                                                  // the attention kernel's queries carry its scale
 #pragma unroll
                 for (int k = 0; k < PER; ++k) r[k] = __fmul_rn(r[k], out_scale);
-                dst[(size_t)at * row_chunks + c * 32] = pack_row<T>(r);
+                dst[(size_t)at * row_chunks + c * 32] = Elem<T>::pack(r);
             }
         }
     }
@@ -226,7 +201,7 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
                                                                pc_rope_dev rope, unsigned long long *fx, double fx_scale,
                                                                float *__restrict__ scores, int32_t *status, uint32_t wait_us, uint32_t extra_tx) {
     pc_grid_dep_launch();
-    constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL, CH = 32 / LPT /* chains */;
+    constexpr int PER = Elem<T>::PER16, NP = PER / 2, SIDE = 32 / LPT, TOK = SIDE * TPL;
     extern __shared__ __align__(128) unsigned char score_smem[];
     __shared__ __align__(8) unsigned long long bars[SCORE_WARPS * SCORE_STAGES];
     __shared__ int gave_up;
@@ -273,76 +248,16 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
     unsigned long long ticket = 0;
     if (threadIdx.x == 0) ticket = atomicAdd(fx + n_out, 1ull);
 
-    // Table entries of this lane's pairs: consecutive pairs take the axes in turn, so pair u's entry is at column m[u] of the
-    // row of coordinate (r + u) mod 3, and the fourth pair's is the one behind the first's.
-    constexpr int AX = NP < 3 ? NP : 3;
-    const int pair0 = ((lt * PER) % d) / 2, r = pair0 % 3;
-    const unsigned mt = rope.max_pos[0], mh = rope.max_pos[1], mw = rope.max_pos[2];
-    int first[AX], pitch[AX];
-#pragma unroll
-    for (int u = 0; u < AX; ++u) {
-        const int a = (pair0 + u) % 3;
-        first[u] = (a == 0 ? rope.off[0] : (a == 1 ? rope.off[1] : rope.off[2])) + (pair0 + u) / 3;
-        pitch[u] = a == 0 ? rope.n_axis[0] : (a == 1 ? rope.n_axis[1] : rope.n_axis[2]);
-    }
-    auto table = [&](int4 q, float2 (&cs)[NP]) {
-        if (!((unsigned)q.x < mt && (unsigned)q.y < mh && (unsigned)q.z < mw)) {   // outside the tables: record, clamp
-            pc_flag(status, PC_ERR_INVALID_ARG, PC_WHERE_SCORE_POS);
-            q.x = min(max(q.x, 0), (int)mt - 1); q.y = min(max(q.y, 0), (int)mh - 1); q.z = min(max(q.z, 0), (int)mw - 1);
-        }
-        const int c[3] = {r == 0 ? q.x : (r == 1 ? q.y : q.z), r == 0 ? q.y : (r == 1 ? q.z : q.x), r == 0 ? q.z : (r == 1 ? q.x : q.y)};
-#pragma unroll
-        for (int u = 0; u < NP; ++u) cs[u] = __ldg(rope.tab + (u < AX ? first[u % AX] + c[u % AX] * pitch[u % AX] : first[0] + c[0] * pitch[0] + 1));
-    };
-
+    const ScoreTable<T> table(rope, lt, d);
     int stage = 0, phase = 0;
     for (; grp < n_groups; grp += step) {
         float2 cs[TPL][NP];
 #pragma unroll
-        for (int i = 0; i < TPL; ++i) table(p[i], cs[i]);
+        for (int i = 0; i < TPL; ++i) table.at(rope, p[i], cs[i], status);
         if (grp + step < n_groups) positions(grp + step);
         if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT, wait_us))) break;
-        // Brackets per pair:  A = sum q_a k_a + q_b k_b,  B = sum q_b k_a - q_a k_b, each as the two lanes of one register pair.
-        // A lane that shares its token with 15 others has twice as many chunks as one of 32 would: it takes those of even number,
-        // then those of odd number, and adds the two results (all in one chain: scores up to 10 % further from a 64-bit
-        // evaluation).  Both chains at once take 161 registers instead of 128, and the block of 12 warps then fills the SM's
-        // registers: the next kernel's first blocks no longer start beside it (step of 135-token frames, 24 / 8 heads, 27.5 -> 29.1 us).
         float s[TPL];
-        const uint32_t mine = ring + stage * stage_bytes + side * row_bytes + lt * 16;
-        const float4 *ql = qs + lt;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            float2 A[TPL][NP], B[TPL][NP];
-#pragma unroll
-            for (int i = 0; i < TPL; ++i)
-#pragma unroll
-                for (int u = 0; u < NP; ++u) A[i][u] = B[i][u] = make_float2(0.f, 0.f);
-#pragma unroll 1
-            for (int g = c; g < parts; g += CH) {
-                float x[TPL][PER];
-#pragma unroll
-                for (int i = 0; i < TPL; ++i) Elem<T>::unpack(pc_lds128(mine + i * SIDE * row_bytes + g * LPT * 16), x[i]);
-#pragma unroll
-                for (int u = 0; u < NP; ++u) {
-                    const float4 qq = ql[(g * NP + u) * LPT];
-                    const float2 qab = make_float2(qq.x, qq.y), qba = make_float2(qq.z, qq.w);
-#pragma unroll
-                    for (int i = 0; i < TPL; ++i) {
-                        const float2 kk = make_float2(x[i][2 * u], x[i][2 * u + 1]);
-                        A[i][u] = __ffma2_rn(qab, kk, A[i][u]);
-                        B[i][u] = __ffma2_rn(qba, kk, B[i][u]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < TPL; ++i) {
-                float r = 0.f;
-#pragma unroll
-                for (int u = 0; u < NP; ++u)
-                    r = fmaf(cs[i][u].x, A[i][u].x + A[i][u].y, fmaf(cs[i][u].y, B[i][u].x + B[i][u].y, r));
-                s[i] = c == 0 ? r : s[i] + r;
-            }
-        }
+        score_rows<T, LPT, TPL>(ring + stage * stage_bytes + side * row_bytes + lt * 16, SIDE * row_bytes, parts, qs + lt, cs, s);
         __syncwarp();                                                 // every lane has read the stage
         if (lane == 0 && grp + stages * step < n_groups) fill(stage, grp + stages * step);
         if (++stage == stages) { stage = 0; phase ^= 1; }
@@ -387,7 +302,7 @@ __global__ void __launch_bounds__(THREADS) k_select(const float *__restrict__ sc
     const int4 fr = tab.f[blockIdx.x];
     if (fr.z <= 0 || fr.y <= 0) return;
     const int out0 = fr.w;
-    frame_select<THREADS>(scores, fr, sm, status, [&](int at, int idx) { sel_idx[out0 + at] = idx; });
+    frame_select<THREADS>(scores + fr.x, fr, sm, status, [&](int at, int idx) { sel_idx[out0 + at] = idx; });
 }
 
 // Enqueue the query pass and the scoring kernel on caller-given scratch (a context's, or the library's fixed array).
@@ -397,7 +312,8 @@ __global__ void __launch_bounds__(THREADS) k_select(const float *__restrict__ sc
 template <typename T>
 pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev &rope, long long *fx, int32_t *status, const void *hist_k, const int32_t *hist_pos, int n_src, const void *q,
                         const int32_t *q_pos, int32_t n_q, const uint8_t *valid, float *scores, void *q_rot, float q_scale,
-                        cudaStream_t stream, pc_ctx *ctx /* whose marks and wait limit; NULL: none */) {
+                        cudaStream_t stream, pc_ctx *ctx /* whose marks and wait limit; NULL: none */,
+                        const pc_front_args *front = nullptr /* scores, selection and pack in one launch */) {
     constexpr int PER = Elem<T>::PER16;
     const int row = D.n_kv_heads * D.head_dim;
     const int group = D.n_q_heads / D.n_kv_heads;
@@ -471,6 +387,7 @@ pc_status enqueue_score(const pc_layer_desc &D, int sm_count, const pc_rope_dev 
 #undef PC_QPREP_LAUNCH
     PC_CUDA_TRY(cudaGetLastError());
     if (ctx) pc_mark(ctx, PC_MARK_QPOOL, stream);
+    if (front) return pc_launch_front(ctx, *front, n_q, stream);
     const float scale = (float)(1.0 / ((double)D.n_q_heads * std::sqrt((double)D.head_dim)));
     const T *k = static_cast<const T *>(hist_k);
     const int lpt = std::max(16, D.head_dim / PER), row_bytes = row * (int)sizeof(T);
@@ -555,7 +472,7 @@ pc_status pc_score_check(const pc_ctx *ctx, const pc_cache *src, const void *q, 
 
 pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const int32_t *q_pos, int32_t n_q, const int32_t *budget,
                         const uint8_t *valid, const float *scores_override, float *scores, int32_t *sel_idx, void *q_rot_out,
-                        cudaStream_t stream, bool select) {
+                        cudaStream_t stream, bool select, const pc_front_args *front) {
     pc_status st = pc_score_check(ctx, src, q, q_pos, n_q, budget, scores_override, scores, sel_idx);
     if (st != PC_OK) return st;
     const int n_frames = src->n_frames, n_src = src->history.n_tokens;
@@ -569,6 +486,7 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
         out += b;
     }
     const float *select_on = scores_override;
+    const pc_front_args here{src, budget, valid, scores, sel_idx, 0, nullptr, nullptr};
     if (!scores_override) {
         if (n_src > 0) {
             const size_t row = (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim;
@@ -577,19 +495,20 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
                 ctx->qpool_dirty = 0;
             }
             ctx->qpool_dirty = 1;
+            if (!front && select && out > 0 && pc_front_fits(ctx, src, false)) front = &here;
             const float q_scale = pc_q_rot_scale(ctx->desc.head_dim);
             st = ctx->desc.dtype == PC_BF16
                      ? enqueue_score<__nv_bfloat16>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->status, src->history.k,
-                                                    src->history.pos, n_src, q, q_pos, n_q, valid, scores, q_rot_out, q_scale, stream, ctx)
+                                                    src->history.pos, n_src, q, q_pos, n_q, valid, scores, q_rot_out, q_scale, stream, ctx, front)
                      : enqueue_score<float>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->status, src->history.k,
-                                            src->history.pos, n_src, q, q_pos, n_q, valid, scores, nullptr, 1.0f, stream, ctx);
+                                            src->history.pos, n_src, q, q_pos, n_q, valid, scores, nullptr, 1.0f, stream, ctx, front);
             if (st != PC_OK) return st;
             ctx->qpool_dirty = 0;
             if (q_rot_out) ctx->q_rot_n = n_q;
         }
         select_on = scores;
     }
-    if (select && n_frames > 0 && out > 0) {
+    if (!front && select && n_frames > 0 && out > 0) {
         if (scores_override) pc_mark(ctx, PC_MARK_SCORE, stream);
         // a thread per key, as far as a block goes: frames of 64 and 135 tokens take 2.4 and 2.5 us with 256
         // threads, 2.7 and 2.8 with 1,024; frames of 1,008 and 4,032 tokens 3.6 and 8.0 with 1,024, 3.8 and 8.9 with 512

@@ -33,15 +33,14 @@ template <int THREADS> struct SelectShared {
     int n_bin, want, n_list, want_eq;
 };
 
-// The whole block selects frame `fr` (budget > 0, n > 0); keep(rank, global index) is called once per kept token by the
+// The whole block selects frame `fr` (budget > 0, n > 0), whose scores start at `s`; keep(rank, global index) is called once per kept token by the
 // thread that owns it.  Every thread of the block must call this.
 template <int THREADS, typename Keep>
-__device__ __forceinline__ void frame_select(const float *__restrict__ scores, int4 fr, SelectShared<THREADS> &sm,
+__device__ __forceinline__ void frame_select(const float *__restrict__ s, int4 fr, SelectShared<THREADS> &sm,
                                              int32_t *status, Keep keep) {
     constexpr int WARPS = THREADS / 32, PER = SEL_BINS / THREADS;
     static_assert(WARPS <= 32 && PER >= 1, "a warp reads the warps' totals, a thread owns whole bins");
     const int first = fr.x, n = fr.y, budget = fr.z;
-    const float *s = scores + first;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t below = (1u << lane) - 1u;
 
