@@ -188,8 +188,10 @@ __global__ void __launch_bounds__(MAX_THREADS, MAX_THREADS == 512 && !KEEP && CP
 // are final.  Bound by DRAM at long histories (97 MB at 47 frames), by latency at short ones.  Steps of 24 / 8 heads, rows in
 // registers against this: 12 frames 84.2 -> 81.4 us, 47 frames 150.4 -> 147.2, masked update of 24 frames 141.3 -> 136.5,
 // 135-token frames 28.3 -> 27.4; 32 / 16 heads: 12 frames 115.7 -> 111.6, 47 frames 220.6 -> 209.8.  Eight warps 148.5 at 47
-// frames; warps held to 80 registers and 8 of them, to be resident beside the query pass, 152.0 to 153.8; the look-ups
-// behind the sums instead of in front of them 148.2.
+// frames; warps held to 80 registers and 8 of them, to be resident beside the query pass, 152.0 to 153.8.  A group's table look-ups are
+// made a group ahead, the first ones ahead of the wait for the pooled query, so no sum waits for them: 11 frames of 420 tokens, 24 / 12 heads,
+// 47.7 -> 46.9 us, 7 of 459, 24 / 8, 33.1 -> 32.8, 12 of 1,008 74.5 -> 74.2, longer ones level (both chains side by side in 157
+// registers, or two chunk rows a turn: level as well).
 // ---------------------------------------------------------------------------------------------------------
 constexpr int SCORE_WARPS = 12;                      // most warps per block (fewer where two stages of each would not fit)
 constexpr int SCORE_STAGES = 8;                     // most stages of a warp's ring
@@ -230,7 +232,17 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
 #pragma unroll
         for (int i = 0; i < TPL; ++i) p[i] = __ldcg(reinterpret_cast<const int4 *>(k_pos) + min(group * TOK + i * SIDE + side, n_src - 1));
     };
-    if (grp < n_groups) positions(grp);
+    const ScoreTable<T> table(rope, lt, d);
+    float2 cs[TPL][NP];
+    auto look_up = [&]() {
+#pragma unroll
+        for (int i = 0; i < TPL; ++i) table.at(rope, p[i], cs[i], status);
+    };
+    if (grp < n_groups) {
+        positions(grp);
+        look_up();
+        if (grp + step < n_groups) positions(grp + step);
+    }
     pc_grid_dep_wait();                                               // the pooled query comes from the kernel before
 
     // the pooled query: the accumulator, scaled
@@ -248,18 +260,17 @@ __global__ void __launch_bounds__(SCORE_WARPS * 32, 1) k_score(const T *__restri
     unsigned long long ticket = 0;
     if (threadIdx.x == 0) ticket = atomicAdd(fx + n_out, 1ull);
 
-    const ScoreTable<T> table(rope, lt, d);
     int stage = 0, phase = 0;
     for (; grp < n_groups; grp += step) {
-        float2 cs[TPL][NP];
-#pragma unroll
-        for (int i = 0; i < TPL; ++i) table.at(rope, p[i], cs[i], status);
-        if (grp + step < n_groups) positions(grp + step);
         if (!__all_sync(0xffffffffu, pc_mbar_wait(bar0 + 8 * stage, phase, &gave_up, status, PC_WHERE_SCORE_WAIT, wait_us))) break;
         float s[TPL];
         score_rows<T, LPT, TPL>(ring + stage * stage_bytes + side * row_bytes + lt * 16, SIDE * row_bytes, parts, qs + lt, cs, s);
         __syncwarp();                                                 // every lane has read the stage
         if (lane == 0 && grp + stages * step < n_groups) fill(stage, grp + stages * step);
+        if (grp + step < n_groups) {
+            look_up();
+            if (grp + 2 * step < n_groups) positions(grp + 2 * step);
+        }
         if (++stage == stages) { stage = 0; phase ^= 1; }
         // a token's lanes are added up; with two tokens in a lane its lower lanes carry on with the first, the upper ones with the second
         float sum = s[0];
