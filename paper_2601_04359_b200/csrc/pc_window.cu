@@ -19,7 +19,7 @@ struct pc_window {
     int32_t scratch_capacity;
     // the step from host memory: V and the output travel on a stream of their own, beside the kernels
     cudaStream_t side;
-    cudaEvent_t main_ev, side_ev;
+    cudaEvent_t main_ev, keys_ev, side_ev;
 };
 
 extern "C" pc_status pc_window_create(pc_ctx *ctx, const pc_window_params *params, const pc_segment *anchors,
@@ -55,6 +55,7 @@ extern "C" pc_status pc_window_create(pc_ctx *ctx, const pc_window_params *param
     const auto on_device = [&]() -> pc_status {
         PC_CUDA_TRY(cudaStreamCreateWithFlags(&w->side, cudaStreamNonBlocking));
         PC_CUDA_TRY(cudaEventCreateWithFlags(&w->main_ev, cudaEventDisableTiming));
+        PC_CUDA_TRY(cudaEventCreateWithFlags(&w->keys_ev, cudaEventDisableTiming));
         PC_CUDA_TRY(cudaEventCreateWithFlags(&w->side_ev, cudaEventDisableTiming));
         return PC_OK;
     };
@@ -73,6 +74,7 @@ extern "C" pc_status pc_window_destroy(pc_window *w) {
     if (!w) return PC_ERR_INVALID_ARG;
     if (w->side) cudaStreamDestroy(w->side);
     if (w->main_ev) cudaEventDestroy(w->main_ev);
+    if (w->keys_ev) cudaEventDestroy(w->keys_ev);
     if (w->side_ev) cudaEventDestroy(w->side_ev);
     delete w;
     return PC_OK;
@@ -366,6 +368,69 @@ pc_status window_step(pc_window *w, const void *q, const int32_t *q_pos, int32_t
     return PC_OK;
 }
 
+// A step from host memory goes up and home by a kernel each as long as it moves no more than this in all and its attention is one part.
+// Window of six frames, the runtime's copies on two streams against the kernels, us a call (in brackets MB both ways): 24 / 8 heads, 30 tokens
+// (0.5) 72.7 -> 62.8, 135 (2.2) 133 -> 100, 360 (5.9) 198 -> 179, 486 (8.0) 216 -> 224; 8 / 8 heads, 682 (5.6) 221 -> 176, 988 (8.1)
+// 232 -> 230; 32 / 16, 135 (3.3) 122 -> 124, 247 (6.1) 185 -> 186, 360 (8.8) 230 -> 237.
+constexpr size_t SMALL_STEP = 6 << 20;
+
+// Runs of 16-byte chunks between pinned host memory and the device in one launch.  Bound by the link: 50 GB/s from and to pinned memory
+// where the copy engine does 54, but no start-up of 3 to 9 us for every run, no hand-over from engine to kernel (5 us), and launched like any
+// other kernel of the library.
+constexpr int MOVE_THREADS = 256, MOVE_CHUNKS = 4, MOVE_RUNS = 5;
+struct Runs {
+    int n;
+    const uint4 *src[MOVE_RUNS];
+    uint4 *dst[MOVE_RUNS];
+    long long end[MOVE_RUNS];        // chunks up to the run's end
+};
+__global__ void __launch_bounds__(MOVE_THREADS) k_move(const __grid_constant__ Runs R) {
+    pc_grid_dep_launch();
+    const long long i0 = (long long)blockIdx.x * (MOVE_THREADS * MOVE_CHUNKS) + threadIdx.x;
+    pc_grid_dep_wait();
+    uint4 x[MOVE_CHUNKS];
+    uint4 *to[MOVE_CHUNKS];
+#pragma unroll
+    for (int c = 0; c < MOVE_CHUNKS; ++c) {
+        const long long i = i0 + c * MOVE_THREADS;
+        to[c] = nullptr;
+        long long first = 0;
+        for (int r = 0; r < R.n; ++r) {
+            if (i >= first && i < R.end[r]) {
+                x[c] = pc_ldg_stream(R.src[r] + (i - first));
+                to[c] = R.dst[r] + (i - first);
+            }
+            first = R.end[r];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < MOVE_CHUNKS; ++c)
+        if (to[c]) *to[c] = x[c];
+}
+void add_run(Runs &R, const void *src, void *dst, size_t bytes) {
+    R.src[R.n] = static_cast<const uint4 *>(src);
+    R.dst[R.n] = static_cast<uint4 *>(dst);
+    R.end[R.n] = (R.n ? R.end[R.n - 1] : 0) + (long long)(bytes / 16);
+    ++R.n;
+}
+pc_status launch_move(const Runs &R, cudaStream_t stream) {
+    const long long chunks = R.end[R.n - 1], per_block = MOVE_THREADS * MOVE_CHUNKS;
+    PC_LAUNCH(k_move, dim3((unsigned)((chunks + per_block - 1) / per_block)), dim3(MOVE_THREADS), 0, stream, R);
+    PC_CUDA_TRY(cudaGetLastError());
+    return PC_OK;
+}
+
+// Where a kernel finds `bytes` of pinned host memory; NULL where it cannot (pageable, in part or at all, or not on 16 bytes).
+void *device_view(const void *p, size_t bytes) {
+    cudaPointerAttributes a, z;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&z, static_cast<const char *>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer || !pc_aligned16(a.devicePointer) || !pc_aligned16(p)) return nullptr;
+    return z.devicePointer == static_cast<char *>(a.devicePointer) + bytes - 1 ? a.devicePointer : nullptr;
+}
+
 // A part of the output is enqueued: it goes home on the side stream while the next part is computed.
 struct HomeTrip {
     pc_window *w;
@@ -424,29 +489,58 @@ extern "C" pc_status pc_window_step_host(pc_window *w, const pc_host_window_step
         take_back();
         return st;
     }
-    // Every argument is checked: from here on work is enqueued.  What the scores need goes first, on the caller's stream: the
-    // queries, then the finished frame's keys and positions, straight to the end of the active history buffer.  Its values
-    // follow on the side stream, under the scoring and the selection, and the output leaves there in parts, under the
-    // attention of the next part.  What remains is the upload of queries, keys and values
-    // (10.4 MB for a 1,008-token frame: 270 us from the pinned memory this was measured with), the attention behind it and the
-    // last part's way home: 508 -> 432 us against everything in a row on one stream.
-    const size_t at = (size_t)(A.n_tokens - n);
-    const auto enqueue = [&]() -> pc_status {
-        PC_CUDA_TRY(cudaMemcpyAsync(ws->q, in->q, (size_t)in->n_q * qrow, cudaMemcpyHostToDevice, stream));
-        PC_CUDA_TRY(cudaMemcpyAsync(ws->q_pos, in->q_pos, (size_t)in->n_q * 16, cudaMemcpyHostToDevice, stream));
+    // Every argument is checked: from here on work is enqueued.
+    const size_t at = (size_t)(A.n_tokens - n), q_bytes = (size_t)in->n_q * qrow, kv_bytes = (size_t)n * row, q_pos_bytes = (size_t)in->n_q * 16, pos_bytes = (size_t)n * 16;
+    char *const to_k = static_cast<char *>(A.k) + at * row, *const to_v = static_cast<char *>(A.v) + at * row;
+    int32_t *const to_pos = A.pos + 4 * at;
+    const void *const q_pos = device_view(in->q_pos, q_pos_bytes), *const pos = n > 0 ? device_view(in->frame_pos, pos_bytes) : nullptr;
+    // A small step goes up and home by a kernel each, and runs as a step on the device does in between.
+    const auto enqueue_small = [&](const void *q, const void *k, const void *v, void *out) -> pc_status {
+        Runs up{}, home{};
+        add_run(up, q, ws->q, q_bytes);
+        add_run(up, q_pos, ws->q_pos, q_pos_bytes);
         if (n > 0) {
-            PC_CUDA_TRY(cudaMemcpyAsync(A.pos + 4 * at, in->frame_pos, (size_t)n * 16, cudaMemcpyHostToDevice, stream));
-            PC_CUDA_TRY(cudaMemcpyAsync(static_cast<char *>(A.k) + at * row, in->frame_k, (size_t)n * row, cudaMemcpyHostToDevice, stream));
+            add_run(up, k, to_k, kv_bytes);
+            add_run(up, v, to_v, kv_bytes);
+            add_run(up, pos, to_pos, pos_bytes);
         }
-        PC_CUDA_TRY(cudaEventRecord(w->main_ev, stream));            // whatever used the buffers before is behind this, too
+        pc_status s = launch_move(up, stream);
+        if (s == PC_OK) s = window_step(w, ws->q, ws->q_pos, in->n_q, ws->out, nullptr, regime, stream, nullptr);
+        add_run(home, ws->out, out, q_bytes);
+        return s == PC_OK ? launch_move(home, stream) : s;
+    };
+    // In a larger one what the scores need goes first: the queries, then the finished frame's keys, straight to the end of the active history
+    // buffer, on the side stream; the positions come by a kernel beside them.  The values follow under the scoring and
+    // the selection, and the output leaves in parts, under the attention of the next part.  What remains is the upload of
+    // queries, keys and values (10.4 MB for a 1,008-token frame, 195 us at the copy engine's rate), the attention behind it and the
+    // last part's way home: everything in a row on one stream took 508 us, with the positions as copies of their own and the values behind an event of the keys' stream 411.
+    const auto enqueue = [&]() -> pc_status {
+        PC_CUDA_TRY(cudaEventRecord(w->main_ev, stream));            // whatever used the buffers before
         PC_CUDA_TRY(cudaStreamWaitEvent(w->side, w->main_ev, 0));
-        if (n > 0) PC_CUDA_TRY(cudaMemcpyAsync(static_cast<char *>(A.v) + at * row, in->frame_v, (size_t)n * row, cudaMemcpyHostToDevice, w->side));
+        PC_CUDA_TRY(cudaMemcpyAsync(ws->q, in->q, q_bytes, cudaMemcpyHostToDevice, w->side));
+        Runs small{};
+        if (q_pos) add_run(small, q_pos, ws->q_pos, q_pos_bytes);
+        else PC_CUDA_TRY(cudaMemcpyAsync(ws->q_pos, in->q_pos, q_pos_bytes, cudaMemcpyHostToDevice, w->side));
+        if (pos) add_run(small, pos, to_pos, pos_bytes);
+        else if (n > 0) PC_CUDA_TRY(cudaMemcpyAsync(to_pos, in->frame_pos, pos_bytes, cudaMemcpyHostToDevice, w->side));
+        if (n > 0) PC_CUDA_TRY(cudaMemcpyAsync(to_k, in->frame_k, kv_bytes, cudaMemcpyHostToDevice, w->side));
+        PC_CUDA_TRY(cudaEventRecord(w->keys_ev, w->side));
+        if (n > 0) PC_CUDA_TRY(cudaMemcpyAsync(to_v, in->frame_v, kv_bytes, cudaMemcpyHostToDevice, w->side));
         PC_CUDA_TRY(cudaEventRecord(w->side_ev, w->side));
+        if (small.n > 0) {
+            const pc_status s = launch_move(small, stream);
+            if (s != PC_OK) return s;
+        }
+        PC_CUDA_TRY(cudaStreamWaitEvent(stream, w->keys_ev, 0));
         HomeTrip trip{w, static_cast<const char *>(ws->out), static_cast<char *>(in->out), qrow};
         const pc_step_hooks hooks{w->side_ev, send_home, &trip};
         return window_step(w, ws->q, ws->q_pos, in->n_q, ws->out, nullptr, regime, stream, &hooks);
     };
-    st = enqueue();
+    const bool small = q_pos && (n == 0 || pos) && 2 * q_bytes + 2 * kv_bytes <= SMALL_STEP && pc_attend_part_rows(w->ctx, in->n_q) >= in->n_q;
+    const void *const q = small ? device_view(in->q, q_bytes) : nullptr, *const k = small && n > 0 ? device_view(in->frame_k, kv_bytes) : nullptr;
+    const void *const v = k ? device_view(in->frame_v, kv_bytes) : nullptr;
+    void *const out = q && (n == 0 || v) ? device_view(in->out, q_bytes) : nullptr;
+    st = out ? enqueue_small(q, k, v, out) : enqueue();
     // also after an error: nothing of this call stays in flight, and the frame is not counted as appended
     const cudaError_t side = cudaStreamSynchronize(w->side), main = cudaStreamSynchronize(stream);
     if (st != PC_OK) {
