@@ -67,13 +67,18 @@ static pc_status create_on_device(pc_ctx *c) {
     PC_CUDA_TRY(cudaMalloc(&c->qpool_fx, ((size_t)row + 1) * sizeof(long long)));
     PC_CUDA_TRY(cudaMemset(c->qpool_fx, 0, ((size_t)row + 1) * sizeof(long long)));
     if (desc->dtype == PC_BF16) {
-        pc_status st = pc_attend_tc_scratch(desc, c->sm_count, &c->k_rot_rows, &c->part_o_floats, &c->part_ml_floats);
+        size_t sync_words = 0;
+        pc_status st = pc_attend_tc_scratch(desc, c->sm_count, &c->k_rot_rows, &c->part_o_floats, &c->part_ml_floats, &sync_words);
         if (st != PC_OK) return st;
         PC_CUDA_TRY(cudaMalloc(&c->k_rot, c->k_rot_rows * row * sizeof(__nv_bfloat16)));
         PC_CUDA_TRY(cudaMemset(c->k_rot, 0, c->k_rot_rows * row * sizeof(__nv_bfloat16)));
         PC_CUDA_TRY(cudaMalloc(&c->q_rot, (size_t)desc->max_q * desc->n_q_heads * desc->head_dim * sizeof(__nv_bfloat16)));
         PC_CUDA_TRY(cudaMalloc(&c->part_o, std::max<size_t>(c->part_o_floats, 1) * sizeof(float)));
         PC_CUDA_TRY(cudaMalloc(&c->part_ml, std::max<size_t>(c->part_ml_floats, 1) * sizeof(float)));
+        const uint32_t first_call = 1;
+        PC_CUDA_TRY(cudaMalloc(&c->part_sync, sync_words * sizeof(uint32_t)));
+        PC_CUDA_TRY(cudaMemset(c->part_sync, 0, sync_words * sizeof(uint32_t)));
+        PC_CUDA_TRY(cudaMemcpy(c->part_sync, &first_call, sizeof(first_call), cudaMemcpyHostToDevice));
         PC_CUDA_TRY(cudaMalloc(&c->mass_part, pc_mass_part_floats(desc, c->sm_count, c->k_rot_rows) * sizeof(float)));
         PC_CUDA_TRY(cudaMalloc(&c->mass_norm, (size_t)((desc->max_q + 127) / 128) * 128 * desc->n_q_heads * sizeof(float)));
     }
@@ -118,6 +123,7 @@ extern "C" pc_status pc_destroy(pc_ctx *c) {
     cudaFree(c->q_rot);
     cudaFree(c->part_o);
     cudaFree(c->part_ml);
+    cudaFree(c->part_sync);
     cudaFree(c->mass_part);
     cudaFree(c->mass_norm);
     delete c;

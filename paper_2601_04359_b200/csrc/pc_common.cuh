@@ -90,6 +90,7 @@ struct pc_ctx {
     cudaEvent_t ev[PC_N_MARKS];
     float *part_o;             // split-KV partial outputs
     float *part_ml;            // split-KV partial (max, sum)
+    uint32_t *part_sync;       // number of the call, tickets, and per item the number of the call whose second part lies in part_o; number 1, else zero at first
     size_t part_o_floats, part_ml_floats;
 };
 
@@ -342,4 +343,4 @@ pc_status pc_attend_frame_check(pc_ctx *ctx, const pc_cache *cache, const pc_seg
                                 int32_t n_q, const void *out, const float *lse);
 size_t pc_mass_part_floats(const pc_layer_desc *d, int sm_count, size_t k_rot_rows);      // size of mass_part
 pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_rot_rows, size_t *part_o_floats,
-                               size_t *part_ml_floats);
+                               size_t *part_ml_floats, size_t *part_sync_words);
