@@ -31,10 +31,12 @@ using pc_tc::peer_addr;
 
 constexpr int FRONT_THREADS = 512, FRONT_WARPS = FRONT_THREADS / 32;
 // Clusters of eight CTAs (the portable size), as long as all of them find room beside the query pass's last blocks: with twelve and
-// more the last ones start late (16 to 24 frames 5 to 15 % slower than the separate kernels), and clusters of four are faster.
+// more the last ones start late (16 to 24 frames 5 to 15 % slower than the separate kernels).  Clusters of four from there on: 24 / 8 heads, 30 and
+// 60 tokens, 12 to 24 frames, the separate kernels against eleven clusters that take several frames each, and against clusters of
+// four: 24.9 -> 24.3 and 23.5 us on average; 96 tokens, 20 frames 26.6 -> 27.3 and 24.9.
 constexpr int FRONT_CTAS = 8, FRONT_CLUSTERS = 11, FRONT_CTAS_MANY = 4, FRONT_CLUSTERS_MANY = 32;
 constexpr int FRONT_FRAMES = FRONT_CTAS_MANY * FRONT_CLUSTERS_MANY;
-static_assert(FRONT_CTAS * FRONT_CLUSTERS <= FRONT_FRAMES, "a cluster has at least a CTA for every frame of its own");
+static_assert(FRONT_CLUSTERS <= FRONT_FRAMES, "a cluster has at least a CTA for every frame of its own");
 constexpr int FRONT_SMEM = 220 * 1024;
 
 struct FrontParams {
@@ -254,8 +256,8 @@ bool lay_out(const pc_ctx *ctx, const pc_cache *src, bool pack, FrontParams &P, 
     // Tokens of a CTA: what its warps score at once (32), or somewhat more of short rows.  24 / 8 heads (2 KB), 5 frames: 247 tokens (31 a CTA)
     // 28.3 -> 27.6 us, 330 (42) 32.3 -> 33.8; 16 / 4 heads (1 KB): 330 tokens 29.9 -> 29.2, 486 (61) 32.2 -> 33.7; fp32, 512 bytes: 294 (37) 39.0 -> 38.0.
     const auto suits = [&]() { return cap <= 32 || (cap <= 48 && (long long)cap * D.n_kv_heads * D.head_dim * ctx->elem_size <= 72 * 1024); };
-    if (src->n_frames <= FRONT_CTAS * FRONT_CLUSTERS) cut(FRONT_CTAS, FRONT_CLUSTERS);
-    if (src->n_frames > FRONT_CTAS * FRONT_CLUSTERS || !suits()) cut(FRONT_CTAS_MANY, FRONT_CLUSTERS_MANY);
+    if (src->n_frames <= FRONT_CLUSTERS) cut(FRONT_CTAS, FRONT_CLUSTERS);
+    else cut(FRONT_CTAS_MANY, FRONT_CLUSTERS_MANY);
     if (!suits()) return false;
     const int row = D.n_kv_heads * D.head_dim, row_bytes = row * ctx->elem_size;
     P.row_bytes = row_bytes;
