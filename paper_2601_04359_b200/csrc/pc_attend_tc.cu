@@ -608,7 +608,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
             ++j;
         }
         // ---- the run's last unit.  If it is the first part of an item in two parts, the second one lies in the scratch, stored by the same warp of the
-        // next CTA at the start of its run (split form: just now): it is fetched under the last PV and added here, in the order of the
+        // next CTA at the start of its run: it is fetched under the last PV and added here, in the order of the
         // merge kernel and with its arithmetic.
         const Place p = place_of(U.item);
         const bool head = MERGE && p.parts == 2 && p.part == 0;
@@ -1027,7 +1027,10 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     P.extra_tx = ctx->test_extra_tx;
     choose_division(ctx, n_items, tiles, P);
     P.cluster = (!P.persistent && P.n_splits > 1 && ctx->cluster_merge) ? 1 : 0;
-    const bool merge = !P.cluster && P.part_stride == 2;
+    // Merged in the kernel: items in two parts of which the second is there long before it is asked for, as it is where runs cross items.
+    // Two parts that end together (split form, or two CTAs to an item) would have the one wait for the other's stores: 703 queries of
+    // 24 / 8 heads x 2,689 keys 67.8 (merge kernel) against 71.2 us.
+    const bool merge = P.persistent && P.part_stride == 2 && P.n_cta % n_items != 0;
     P.sync = ctx->part_sync;
     if (P.part_stride > 1 && !P.cluster && (size_t)n_items * P.part_stride * 2 * TILE * TILE > ctx->part_o_floats) return PC_ERR_CAPACITY;
 
@@ -1075,9 +1078,10 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     }
     PC_CUDA_TRY(cudaGetLastError());
     pc_mark(ctx, PC_MARK_ATTEND, stream);
-    if (P.part_stride > 2 && !P.cluster) {
+    if (P.part_stride > 1 && !P.cluster && !merge) {
         const dim3 grid(P.n_tb * D.n_q_heads * 4);
-        if (P.part_stride <= 4) PC_LAUNCH((k_combine<4, 3>), grid, dim3(256), 0, stream, P);
+        if (P.part_stride == 2) PC_LAUNCH((k_combine<2, 4>), grid, dim3(256), 0, stream, P);
+        else if (P.part_stride <= 4) PC_LAUNCH((k_combine<4, 3>), grid, dim3(256), 0, stream, P);
         else PC_LAUNCH((k_combine<MAX_SPLITS, 2>), grid, dim3(256), 0, stream, P);
         PC_CUDA_TRY(cudaGetLastError());
         pc_mark(ctx, PC_MARK_COMBINE, stream);

@@ -1,5 +1,5 @@
 """Items that two CTAs share: the one with the first part adds the second to it at the end of its run.  Whole frames whose runs cross
-items (persistent form), two fixed key ranges (both parts end at the same time), an odd number of query tiles, rows past the last;
+items, two fixed key ranges (which end together and are merged by a kernel of their own), an odd number of query tiles, rows past the last;
 against the oracle, and the same bits again from call to call, from a captured graph, and after a call that gave up."""
 from __future__ import annotations
 
