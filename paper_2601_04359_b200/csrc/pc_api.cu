@@ -80,7 +80,6 @@ static pc_status create_on_device(pc_ctx *c) {
         PC_CUDA_TRY(cudaMemset(c->part_sync, 0, sync_words * sizeof(uint32_t)));
         PC_CUDA_TRY(cudaMemcpy(c->part_sync, &first_call, sizeof(first_call), cudaMemcpyHostToDevice));
         PC_CUDA_TRY(cudaMalloc(&c->mass_part, pc_mass_part_floats(desc, c->sm_count, c->k_rot_rows) * sizeof(float)));
-        PC_CUDA_TRY(cudaMalloc(&c->mass_norm, (size_t)((desc->max_q + 127) / 128) * 128 * desc->n_q_heads * sizeof(float)));
     }
     return PC_OK;
 }
@@ -125,7 +124,6 @@ extern "C" pc_status pc_destroy(pc_ctx *c) {
     cudaFree(c->part_ml);
     cudaFree(c->part_sync);
     cudaFree(c->mass_part);
-    cudaFree(c->mass_norm);
     delete c;
     return PC_OK;
 }

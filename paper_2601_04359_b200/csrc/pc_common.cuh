@@ -82,7 +82,6 @@ struct pc_ctx {
     int last_n_q, last_n_seg;
     int last_seg_n[PC_MAX_SEGMENTS];
     float *mass_part;          // attention mass: partial sums of the pieces of (KV head, pair of key tiles)
-    float *mass_norm;          // attention mass: negated base-2 normalisers, [Hq][max_q rounded up to 128]
     // optional per-kernel timing (benchmarks): events at the boundaries of the kernels of each call
     int timing_on;
     unsigned ev_mask;

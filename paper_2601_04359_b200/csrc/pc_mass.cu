@@ -6,8 +6,6 @@
 // the attention kernel wrote.  With the normaliser of every row known, a key's mass is a plain column sum of
 // 2^(s_ij - lse2_i), so no running maximum and no second operand are needed:
 //
-//   k_mass_norm    writes minus the base-2 normaliser of every query row, transposed to [head][row] and padded with
-//                  -inf to whole tiles, so that one step's 128 values are one contiguous 512-byte run.
 //   k_mass_tc      a unit = two 128-key tiles of one KV head, which stay in shared memory while the query tiles of the
 //                  head's group stream through a four-stage TMA ring, each stage feeding both key tiles (a unit of a
 //                  single key tile reads every query tile twice as often from L2 for no gain).  Persistent CTAs, one per
@@ -16,7 +14,8 @@
 //                  wave, as many as 38 %: 24 / 8 heads, 1,008 queries
 //                  x 5,168 keys 70.7 us against 43.7, 9,200 72.9 / 70.5, 12,980 106.3 / 95.6; 16 / 16, 300 x 1,200 10.1 / 9.9;
 //                  8 / 8, 1,500 x 4,000, a unit per CTA either way, 21.8 / 22.1.)  The step's
-//                  normalisers ride along as a bulk copy into an eight-slot ring.  S^T = K Q^T (keys on the TMEM lanes,
+//                  normalisers go into an eight-slot ring beside it, fetched by the warp that issues the copies (laid out by a kernel of its own for a bulk
+//                  copy first: guided steps of 28 to 294 tokens 4 to 10 % longer, of 1,008 0.7 %).  S^T = K Q^T (keys on the TMEM lanes,
 //                  queries on the columns) goes to one of two TMEM buffers per key tile.  Sixteen warps turn scores
 //                  into sums: per key tile and column half one warp per TMEM lane quadrant, one key per thread, 64
 //                  columns per step: 2^(s + (-lse2)) added up in registers.  Four such warps share each scheduler, so
@@ -54,7 +53,6 @@ static_assert(N_BARS * 8 + 16 <= 256, "barrier area");
 struct MassParams {
     int n_q, n_q_heads, group, n_tb, n_kv_tiles, pairs;    // pairs = key-tile pairs per KV head
     const float *lse;      // [n_q][Hq] natural log
-    float *norm;           // [Hq][n_tb * 128]: -log2(e) * lse, -inf past n_q
     // Partial sums, [slot][2 key tiles][2 column halves][128].  A piece's slot is its unit's number plus its CTA's: along the line of
     // steps one or both of them grow at every change, so no two pieces share a slot and there are at most units + n_cta of them.
     float *part;
@@ -69,16 +67,6 @@ __host__ __device__ __forceinline__ int run_start(const MassParams &P, int c) { 
 __host__ __device__ __forceinline__ int cta_of_step(const MassParams &P, int x) {
     const int head = P.longer * (P.run + 1);
     return x < head ? x / (P.run + 1) : P.longer + (x - head) / P.run;
-}
-
-__global__ void __launch_bounds__(256) k_mass_norm(const __grid_constant__ MassParams P) {
-    pc_grid_dep_launch();
-    pc_grid_dep_wait();
-    const int rows = P.n_tb * TILE;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * P.n_q_heads) return;
-    const int row = idx / P.n_q_heads, h = idx % P.n_q_heads;         // consecutive threads read consecutive floats
-    P.norm[(size_t)h * rows + row] = row < P.n_q ? -1.4426950408889634f * __ldg(P.lse + idx) : -INFINITY;
 }
 
 // WHOLE: every CTA has one unit and all of it (n_cta = units), which needs none of what a change of unit takes in the loops.  The
@@ -132,42 +120,58 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        // ring stages, score buffers and normaliser slots follow the step count of the whole run (gs)
-        if (lane == 0) {
-            bool alive = true;
-            int gs = 0, un = 0, unit = unit0, g = g0, pair = pair0;
-            for (int x = G0; x < G1 && alive; ++un) {
-                if (un > 0) {
-                    ++unit;
-                    if (++pair == P.pairs) { pair = 0; ++g; }
-                }
-                const int s0 = x - unit * P.n_steps, n = min(P.n_steps - s0, G1 - x), jt0 = 2 * pair;
-                x += n;
-                if (!WHOLE && un > 0) alive = mbar_wait(bar(BAR_KFREE), (un - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
-                if (!alive) break;
+        // Ring stages, score buffers and normaliser slots follow the step count of the whole run (gs).  One lane issues the copies; all of them fetch
+        // the step's normalisers (a query's values of all heads lie side by side, so a step's are one word of every row), ahead of the wait
+        // for the stage.
+        bool alive = true;
+        int gs = 0, un = 0, unit = unit0, g = g0, pair = pair0;
+        auto wait = [&](int b, int parity) {
+            return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us));
+        };
+        float *const norms = reinterpret_cast<float *>(gen + SM_LSE);
+        for (int x = G0; x < G1 && alive; ++un) {
+            if (un > 0) {
+                ++unit;
+                if (++pair == P.pairs) { pair = 0; ++g; }
+            }
+            const int s0 = x - unit * P.n_steps, n = min(P.n_steps - s0, G1 - x), jt0 = 2 * pair;
+            x += n;
+            if (!WHOLE && un > 0) alive = wait(BAR_KFREE, (un - 1) & 1);
+            if (!alive) break;
+            if (lane == 0) {
                 mbar_expect_tx(bar(BAR_K), n_t * TILE_BYTES + (un == 0 ? P.extra_tx : 0u));
                 for (int t = 0; t < n_t; ++t) {
                     const int jt = min(jt0 + t, P.n_kv_tiles - 1);       // an odd tile count: the last tile twice, one copy dropped
                     tma_load_2d(base + SM_K + t * TILE_BYTES, &map_k, g * TILE, jt * TILE, bar(BAR_K));
                     tma_load_2d(base + SM_K + t * TILE_BYTES + HALF_BYTES, &map_k, g * TILE + 64, jt * TILE, bar(BAR_K));
                 }
-                for (int s = s0; s < s0 + n && alive; ++s, ++gs) {
-                    const int st = gs % Q_STAGES, use = gs / Q_STAGES;
-                    if (use > 0) alive = mbar_wait(bar(BAR_QEMPTY + st), (use - 1) & 1, abort_flag, P.status, PC_WHERE_MASS_WAIT, P.wait_us);
-                    if (!alive) break;
-                    const int tb = s / P.group, h = g * P.group + s % P.group;
+            }
+            for (int s = s0; s < s0 + n && alive; ++s, ++gs) {
+                const int st = gs % Q_STAGES, use = gs / Q_STAGES;
+                const int tb = s / P.group, h = g * P.group + s % P.group;
+                float lse[TILE / 32];
+#pragma unroll
+                for (int k = 0; k < TILE / 32; ++k) {
+                    const int row = tb * TILE + k * 32 + lane;
+                    lse[k] = row < P.n_q ? -1.4426950408889634f * __ldg(P.lse + (size_t)row * P.n_q_heads + h) : -INFINITY;
+                }
+                if (use > 0) alive = wait(BAR_QEMPTY + st, (use - 1) & 1);
+                if (!alive) break;
+                if (lane == 0) {
                     mbar_expect_tx(bar(BAR_QFULL + st), TILE_BYTES);
                     tma_load_2d(base + SM_Q + st * TILE_BYTES, &map_q, h * TILE, tb * TILE, bar(BAR_QFULL + st));
                     tma_load_2d(base + SM_Q + st * TILE_BYTES + HALF_BYTES, &map_q, h * TILE + 64, tb * TILE, bar(BAR_QFULL + st));
-                    // The step's normalisers go to slot gs mod 8.  Its previous tenant, step gs - 8, is out of use: this point
-                    // is reached after the products of step gs - 4 completed, those needed the score buffers of step gs - 6
-                    // released, and a buffer is released only after the step before it was summed up.
-                    const int slot = gs % L_SLOTS;
-                    mbar_expect_tx(bar(BAR_LFULL + slot), TILE * 4);
-                    pc_bulk_g2s(base + SM_LSE + slot * TILE * 4, P.norm + ((size_t)h * P.n_tb + tb) * TILE, TILE * 4, bar(BAR_LFULL + slot));
                 }
-                if constexpr (WHOLE) break;
+                // The step's normalisers go to slot gs mod 8.  Its previous tenant, step gs - 8, is out of use: this point
+                // is reached after the products of step gs - 4 completed, those needed the score buffers of step gs - 6
+                // released, and a buffer is released only after the step before it was summed up.
+                const int slot = gs % L_SLOTS;
+#pragma unroll
+                for (int k = 0; k < TILE / 32; ++k) norms[slot * TILE + k * 32 + lane] = lse[k];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(BAR_LFULL + slot));
             }
+            if constexpr (WHOLE) break;
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer (converged warp, one elected lane)
@@ -370,7 +374,6 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
     P.longer = units * P.n_steps % P.n_cta;
     P.lse = lse;
     P.part = ctx->mass_part;
-    P.norm = ctx->mass_norm;
     P.status = ctx->status;
     P.wait_us = ctx->wait_limit_us;
     P.extra_tx = ctx->test_extra_tx;
@@ -389,8 +392,6 @@ extern "C" pc_status pc_attend_mass(pc_ctx *ctx, const float *lse, float *mass, 
         attr_set[ctx->device] = true;
     }
     pc_mark(ctx, PC_MARK_MASS0, stream);
-    PC_LAUNCH(k_mass_norm, dim3((P.n_tb * TILE * D.n_q_heads + 255) / 256), dim3(256), 0, stream, P);
-    PC_CUDA_TRY(cudaGetLastError());
     if (P.n_cta == units) PC_LAUNCH(k_mass_tc<true>, dim3(P.n_cta), dim3(MASS_THREADS), SM_ALLOC, stream, mq, mk, P);
     else PC_LAUNCH(k_mass_tc<false>, dim3(P.n_cta), dim3(MASS_THREADS), SM_ALLOC, stream, mq, mk, P);
     PC_CUDA_TRY(cudaGetLastError());
