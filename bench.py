@@ -31,7 +31,7 @@ METRIC = "late_frame_attn_plus_compaction_latency"
 UNIT = "ms/frame"
 WORKLOAD = "lumos47"
 N_LAYERS = 4          # rotated input sets; 4 x ~0.2 GB > L2 (--layers changes it for small profiler captures)
-KERNELS_PER_STEP = 6  # k_qprep, k_score, k_select, k_pack, k_attend_tc, k_combine (anchors' rotated keys are kept per layer)
+KERNELS_PER_STEP = 5  # k_qprep, k_score, k_select, k_pack, k_attend_tc (anchors' rotated keys are kept per layer)
 
 
 def _peaks():
@@ -357,7 +357,7 @@ def run_cuda(args):
     mma = {form: pc.pc_probe_mma_rate(ctx, form, rounds=2000) for form in ("qk", "pv", "mix")}
     assert pc.pc_poll_status(ctx) == pc.PC_OK
 
-    # ---- the same frame through the three separate calls (pc_score, pc_compact, pc_attend_frame: eight launches)
+    # ---- the same frame through the three separate calls (pc_score, pc_compact, pc_attend_frame: six launches)
     for i in range(3):
         step_separate(i)
     sep_ms = timed(step_separate, min(args.steps, 200))
@@ -570,13 +570,13 @@ def run_cuda(args):
         "kernels_ms": stages,
         "kernels_ms_pipelined": {k: (round(v, 5) if v is not None else None) for k, v in pipelined.items()},
         "separate_calls": {"ms_per_frame": sep_ms, "what": "the same frame through pc_score, pc_compact and pc_attend_frame "
-                           "(eight launches: Q read twice, rotary pre-pass over anchors and packed history)"},
+                           "(six launches: Q read twice, rotary pre-pass over anchors and packed history)"},
         "late4": late,
         "extra_pass": {"ms_per_pass": pass_ms, "what": "one more attention pass of the frame over the unchanged packed cache "
                        "(pc_attend_prepared: query rotation, attention, merge; keys were rotated once per frame)"},
         "attention_mass": {"ms": mass_ms, "keys": cfg.n_anchor + n_sel,
                            "what": "pc_attend_mass after an attention pass over the packed cache: K Q^T on tensor cores, "
-                                   "column sums of the normalised probabilities (three launches)"},
+                                   "column sums of the normalised probabilities (two launches)"},
         "incremental": {"ms_per_frame": inc_ms, "source_tokens": inc_src,
                         "mode": "cache window in the Slide regime (pc_window_append + pc_window_step): append the newest frame, "
                                 "drop the oldest, re-plan, score and re-select from packed + new, pack, attend (same keys attended)"},
