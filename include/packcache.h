@@ -339,7 +339,8 @@ pc_status pc_window_step(pc_window *w, const void *q, const int32_t *q_pos, int3
  * rows for 24/8, 32/8, 24/12 and 32/16 heads, 641 for 16/4, 1,153 for 8/8, 129 for 64/8, 32/32 and 24/24.  Fewer rows give
  * pc_window_step's output bit for bit.  In parts the keys are cut in other places, which moves the reference that a row's
  * probabilities are rounded to bf16 against: each probability may differ by that rounding (2^-9 relative on either side).
- * Pinned host memory keeps the copies asynchronous.  All arguments are checked before anything is enqueued; a call that fails
+ * Pinned host memory (in whole, on 16 bytes) keeps the copies asynchronous, and a step that moves up to 6 MB then goes up and home by a
+ * kernel each, which read and write it in place of the copies.  All arguments are checked before anything is enqueued; a call that fails
  * leaves the window as it was (the frame is not appended) and nothing in flight on either stream.
  * Errors: as pc_window_append and pc_window_step. */
 typedef struct {

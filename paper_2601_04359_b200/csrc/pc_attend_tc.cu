@@ -12,7 +12,8 @@
 //                 write bf16 P beside it (handed over in two halves of 64 keys), and rescale O in TMEM only when
 //                 the running max moved by more than 2^8.
 //                 While one tile's softmax runs, the tensor core works on the other tile.
-//   k_combine     merges the (max, sum, O) partials of items that several CTAs worked on.  On request (pc_set_cluster_merge) the
+//                 An item that two CTAs share, as most are where runs cross items, is merged by the one with its first keys, at the end of its run.
+//   k_combine     merges the (max, sum, O) partials of the other items that several CTAs worked on.  On request (pc_set_cluster_merge) the
 //                 key ranges of one item are launched as a thread-block cluster instead and merge through distributed shared
 //                 memory at the end of k_attend_tc.
 //
@@ -30,7 +31,8 @@
 // 1,024 at 16 a clock, twice).
 // That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
 // whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452; since the
-// bounded wait lost its loop of questions 77.2, 148.5, 586, 569 and 450.
+// bounded wait lost its loop of questions 77.2, 148.5, 586, 569 and 450; with the merge in this kernel, both sides in turn on one box, the step at
+// 12 frames 75.5 -> 74.5, at 47 149.0 -> 147.0, of 4,032-token frames 588 -> 579, five passes 452 -> 441, the whole cache 569 -> 565.
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT and raises a CTA-wide abort flag; every later wait whose
 // phase is not complete gives up within some ten microseconds, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
 #include <algorithm>
@@ -771,8 +773,8 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 // ------------------------------------------------------------------------------------------------ combine
 // Merge of the KV ranges' partials.  One block per (query tile of one head, 32-row quadrant); its eight warps take four
 // 16-byte column units each, lanes are consecutive rows, so every load of the partial tiles is a 512-byte run.  Up to four
-// parts' loads of a thread are issued before any is used.  Bound by L2 and its latency, so loads in flight count: an item of the
-// persistent form has two parts nearly always, and built for those the kernel takes 48 registers instead of 108 and four
+// parts' loads of a thread are issued before any is used.  Bound by L2 and its latency, so loads in flight count: for items in
+// two parts (which the attention kernel leaves to this one where they end together) the kernel is built with 48 registers instead of 108 and four
 // blocks an SM instead of two.  The step at 12 frames 80.6 -> 79.1 us, 47 frames 147.0 -> 145.4; six blocks an SM 79.9 and 146.0.
 template <int PARTS /* most parts of an item */, int BLOCKS /* resident on an SM */>
 __global__ void __launch_bounds__(256, BLOCKS) k_combine(const TcParams P) {
