@@ -445,7 +445,9 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         int ragged = next_end(U.jb);
         // A unit's output leaves O_t in the turn behind its last step, after the next unit's first probabilities are computed and before they
         // are handed over (the first PV of a unit overwrites O_t): the stores run under the tensor core's next work.  Reading and storing O_t first left the tensor core idle meanwhile: the step at
-        // 12 frames 88.1 against 86.4 us, 47 frames 167.4 against 165.5, 4,032-token frames 663.9 against 656.3.  The run's last unit leaves behind the loop.
+        // 12 frames 88.1 against 86.4 us, 47 frames 167.4 against 165.5, 4,032-token frames 663.9 against 656.3.  The run's last unit leaves
+        // in one more turn, or behind the loop where that may take a merge.  The kernel without merges has its read-out in the loop and written out
+        // by itself: behind the loop, or through the functions that the other one uses, calls of a few steps took 0.2 to 0.6 us longer.
         const auto read_out = [&](uint32_t (&v)[128]) {  // the thread's whole O row leaves TMEM in one pass (four loads in flight, one wait)
             tmem_ld32(o_addr, v);
             tmem_ld32(o_addr + 32, v + 32);
@@ -488,11 +490,11 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
             for (int i = 0; i < 32; ++i) ptile[i * TILE] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             *reinterpret_cast<float2 *>(P.part_ml + ((size_t)p.slot * TILE + r) * 2) = make_float2(m_e, l_e);
         };
-        for (int gs = 0; gs < n_steps && alive; ++gs) {
-            const bool flush = j == U.n_j;
+        for (int gs = 0; alive && (!MERGE || gs < n_steps); ++gs) {
+            const bool end = !MERGE && gs == n_steps, flush = end || j == U.n_j;
             const int e_item = U.item;                   // the unit to flush
             const float m_e = m_used, l_e = l;
-            if (flush) {
+            if (flush && !end) {
                 U = unit_at(P, g, G1);
                 g += U.n_j;
                 j = 0;
@@ -500,206 +502,264 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                 l = 0.f;
                 ragged = next_end(0);
             }
-            alive = warp_wait(bar(BAR_SFULL + t), gs & 1, abort_flag, P.status, P.wait_us);
-            if (!alive) break;
-            tc_fence_after();
-            if (__builtin_expect(U.jb + j == ragged, 0)) {      // last tile of a segment: keys past its end score -inf
-                int seg, local, n_valid;
-                kv_tile_info(P, ragged, seg, local, n_valid);
-                ragged = P.seg_tile_end[min(seg + 1, P.n_seg - 1)] - 1;
-                int i = n_valid;
-#pragma unroll 1
-                for (; i & 7; ++i) tmem_st1(s_addr + i, 0xFF800000u);
-#pragma unroll 1
-                for (; i < TILE; i += 8) tmem_st8(s_addr + i, 0xFF800000u);
-                tmem_wait_st();
-            }
-            // the whole score row of this thread: one TMEM pass
-            uint32_t sv[128];
-            tmem_ld32(s_addr, sv);
-            tmem_ld32(s_addr + 32, sv + 32);
-            tmem_ld32(s_addr + 64, sv + 64);
-            tmem_ld32(s_addr + 96, sv + 96);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            arrive_if(lead, bar(BAR_SFREE + t));         // the columns are the other tile's
-            if (j + 1 == U.n_j) arrive_if(lead, bar(BAR_QFREE + t));      // that was the unit's last QK^T of this tile
-            // the PV of the step before: its P columns are written again below, and O_t may be rescaled
-            const bool pv_done = gs == 0 || pc_mbar_test(bar(BAR_PVDONE + t), (gs - 1) & 1);
-            float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < TILE; i += 4) {
-                mx0 = fmaxf(mx0, __uint_as_float(sv[i]));
-                mx1 = fmaxf(mx1, __uint_as_float(sv[i + 1]));
-                mx2 = fmaxf(mx2, __uint_as_float(sv[i + 2]));
-                mx3 = fmaxf(mx3, __uint_as_float(sv[i + 3]));
-            }
-            const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-            // lazy rescale: move the reference maximum only when it grew by more than the threshold
-            const bool grow = mx > m_used + RESCALE_THRESHOLD;
-            if (__builtin_expect(!__all_sync(0xffffffffu, pv_done), 0)) {
-                alive = warp_wait(bar(BAR_PVDONE + t), (gs - 1) & 1, abort_flag, P.status, P.wait_us);
+            if (!end) {
+                alive = warp_wait(bar(BAR_SFULL + t), gs & 1, abort_flag, P.status, P.wait_us);
                 if (!alive) break;
-            }
-            tc_fence_after();
-            // tile 1 comes last: QK^T(step) and PV(step - 1) have read their keys and values
-            if (t == 1) arrive_if(lead, bar(BAR_EMPTY + (gs & 1)));
-            if (__builtin_expect(__any_sync(0xffffffffu, grow), 0)) {
-                const float m_new = fmaxf(m_used, mx);
-                const float corr = fast_exp2(m_used - m_new);       // 0 on the first tile (m_used = -inf)
-                l *= corr;
-                if (j > 0) {
-                    uint32_t v[32];
+                tc_fence_after();
+                if (__builtin_expect(U.jb + j == ragged, 0)) {      // last tile of a segment: keys past its end score -inf
+                    int seg, local, n_valid;
+                    kv_tile_info(P, ragged, seg, local, n_valid);
+                    ragged = P.seg_tile_end[min(seg + 1, P.n_seg - 1)] - 1;
+                    int i = n_valid;
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
-                        tmem_ld32(o_addr + c * 32, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * corr);
-                        tmem_st32(o_addr + c * 32, v);
-                    }
-                }
-                m_used = m_new;
-            }
-            // p = 2^(s - m) as bf16 pairs; the row sum runs on two-lane adds
-            const float2 neg_m = make_float2(-m_used, -m_used);
-            float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint32_t pk[16];
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                    float2 x = add2(make_float2(__uint_as_float(sv[c * 32 + 2 * i]), __uint_as_float(sv[c * 32 + 2 * i + 1])), neg_m);
-                    float2 y = add2(make_float2(__uint_as_float(sv[c * 32 + 2 * i + 2]), __uint_as_float(sv[c * 32 + 2 * i + 3])), neg_m);
-                    x.x = fast_exp2(x.x); x.y = fast_exp2(x.y);
-                    y.x = fast_exp2(y.x); y.y = fast_exp2(y.y);
-                    la = add2(la, x);
-                    lb = add2(lb, y);
-                    pk[i] = pc_pack_bf16(x.x, x.y);
-                    pk[i + 1] = pc_pack_bf16(y.x, y.y);
-                }
-                // the sums belong in the gaps of this chunk's exponentials, not behind the hand-over
-                asm volatile("" : "+f"(la.x), "+f"(la.y), "+f"(lb.x), "+f"(lb.y));
-                tmem_st16(p_addr + c * 16, pk);
-                if (c & 1) {                               // keys 0-63, then 64-127, handed to the tensor core
+                    for (; i & 7; ++i) tmem_st1(s_addr + i, 0xFF800000u);
+#pragma unroll 1
+                    for (; i < TILE; i += 8) tmem_st8(s_addr + i, 0xFF800000u);
                     tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    arrive_if(lead && !flush, bar(BAR_PHALF + 2 * t + (c >> 1)));
                 }
-            }
-            l += (la.x + la.y) + (lb.x + lb.y);
-            if (__builtin_expect(flush, 0)) {
-                uint32_t v[128];
-                read_out(v);
+                // the whole score row of this thread: one TMEM pass
+                uint32_t sv[128];
+                tmem_ld32(s_addr, sv);
+                tmem_ld32(s_addr + 32, sv + 32);
+                tmem_ld32(s_addr + 64, sv + 64);
+                tmem_ld32(s_addr + 96, sv + 96);
+                tmem_wait_ld();
                 tc_fence_before();
                 __syncwarp();
-                arrive_if(lead, bar(BAR_PHALF + 2 * t));
-                arrive_if(lead, bar(BAR_PHALF + 2 * t + 1));
-                const Place p = place_of(e_item);
-                if (p.there) {
-                    if (p.parts == 1) write_whole(p, v, m_e, l_e);
-                    else write_part(p, v, m_e, l_e);
+                arrive_if(lead, bar(BAR_SFREE + t));         // the columns are the other tile's
+                if (j + 1 == U.n_j) arrive_if(lead, bar(BAR_QFREE + t));      // that was the unit's last QK^T of this tile
+                // the PV of the step before: its P columns are written again below, and O_t may be rescaled
+                const bool pv_done = gs == 0 || pc_mbar_test(bar(BAR_PVDONE + t), (gs - 1) & 1);
+                float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < TILE; i += 4) {
+                    mx0 = fmaxf(mx0, __uint_as_float(sv[i]));
+                    mx1 = fmaxf(mx1, __uint_as_float(sv[i + 1]));
+                    mx2 = fmaxf(mx2, __uint_as_float(sv[i + 2]));
+                    mx3 = fmaxf(mx3, __uint_as_float(sv[i + 3]));
                 }
-                if (MERGE && p.part == 1) {
+                const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+                // lazy rescale: move the reference maximum only when it grew by more than the threshold
+                const bool grow = mx > m_used + RESCALE_THRESHOLD;
+                if (__builtin_expect(!__all_sync(0xffffffffu, pv_done), 0)) {
+                    alive = warp_wait(bar(BAR_PVDONE + t), (gs - 1) & 1, abort_flag, P.status, P.wait_us);
+                    if (!alive) break;
+                }
+                tc_fence_after();
+                // tile 1 comes last: QK^T(step) and PV(step - 1) have read their keys and values
+                if (t == 1) arrive_if(lead, bar(BAR_EMPTY + (gs & 1)));
+                if (__builtin_expect(__any_sync(0xffffffffu, grow), 0)) {
+                    const float m_new = fmaxf(m_used, mx);
+                    const float corr = fast_exp2(m_used - m_new);       // 0 on the first tile (m_used = -inf)
+                    l *= corr;
+                    if (j > 0) {
+                        uint32_t v[32];
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            tmem_ld32(o_addr + c * 32, v);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * corr);
+                            tmem_st32(o_addr + c * 32, v);
+                        }
+                    }
+                    m_used = m_new;
+                }
+                // p = 2^(s - m) as bf16 pairs; the row sum runs on two-lane adds
+                const float2 neg_m = make_float2(-m_used, -m_used);
+                float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i += 2) {
+                        float2 x = add2(make_float2(__uint_as_float(sv[c * 32 + 2 * i]), __uint_as_float(sv[c * 32 + 2 * i + 1])), neg_m);
+                        float2 y = add2(make_float2(__uint_as_float(sv[c * 32 + 2 * i + 2]), __uint_as_float(sv[c * 32 + 2 * i + 3])), neg_m);
+                        x.x = fast_exp2(x.x); x.y = fast_exp2(x.y);
+                        y.x = fast_exp2(y.x); y.y = fast_exp2(y.y);
+                        la = add2(la, x);
+                        lb = add2(lb, y);
+                        pk[i] = pc_pack_bf16(x.x, x.y);
+                        pk[i + 1] = pc_pack_bf16(y.x, y.y);
+                    }
+                    // the sums belong in the gaps of this chunk's exponentials, not behind the hand-over
+                    asm volatile("" : "+f"(la.x), "+f"(la.y), "+f"(lb.x), "+f"(lb.y));
+                    tmem_st16(p_addr + c * 16, pk);
+                    if (c & 1) {                               // keys 0-63, then 64-127, handed to the tensor core
+                        tmem_wait_st();
+                        tc_fence_before();
+                        __syncwarp();
+                        arrive_if(lead && !flush, bar(BAR_PHALF + 2 * t + (c >> 1)));
+                    }
+                }
+                l += (la.x + la.y) + (lb.x + lb.y);
+            }
+            if (end) {
+                alive = warp_wait(bar(BAR_PVDONE + t), (gs - 1) & 1, abort_flag, P.status, P.wait_us);
+                if (!alive) break;
+                tc_fence_after();
+            }
+            if (__builtin_expect(flush, 0)) {
+                if constexpr (MERGE) {
+                    uint32_t v[128];
+                    read_out(v);
+                    tc_fence_before();
                     __syncwarp();
-                    arrive_if(lead, bar(BAR_PART));
+                    arrive_if(lead, bar(BAR_PHALF + 2 * t));
+                    arrive_if(lead, bar(BAR_PHALF + 2 * t + 1));
+                    const Place p = place_of(e_item);
+                    if (p.there) {
+                        if (p.parts == 1) write_whole(p, v, m_e, l_e);
+                        else write_part(p, v, m_e, l_e);
+                    }
+                    if (p.part == 1) {
+                        __syncwarp();
+                        arrive_if(lead, bar(BAR_PART));
+                    }
+                } else {
+                    // the thread's whole O row leaves TMEM in one pass (four loads in flight, one wait)
+                    uint32_t v[128];
+                    tmem_ld32(o_addr, v);
+                    tmem_ld32(o_addr + 32, v + 32);
+                    tmem_ld32(o_addr + 64, v + 64);
+                    tmem_ld32(o_addr + 96, v + 96);
+                    tmem_wait_ld();
+                    if (!end) {
+                        tc_fence_before();
+                        __syncwarp();
+                        arrive_if(lead, bar(BAR_PHALF + 2 * t));
+                        arrive_if(lead, bar(BAR_PHALF + 2 * t + 1));
+                    }
+                    const int kvh = e_item / P.pairs_per_g, pair = e_item % P.pairs_per_g;
+                    const int n_tiles_q = min(2, P.tiles_per_g - 2 * pair);
+                    int part, parts;
+                    item_parts(P, e_item, (int)blockIdx.x, part, parts);
+                    const int T = 2 * pair + t, tb = T / P.group, h = kvh * P.group + T % P.group;
+                    const int row = tb * TILE + r;
+                    if (t >= n_tiles_q) {
+                        // the second copy of a single query tile: dropped
+                    } else if (parts == 1) {
+                        const float inv = 1.f / l_e;
+                        __nv_bfloat16 *orow = P.out + ((size_t)row * P.n_q_heads + h) * TILE;
+                        if (row < P.n_q) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                uint4 w;
+                                w.x = pc_pack_bf16(__uint_as_float(v[8 * i + 0]) * inv, __uint_as_float(v[8 * i + 1]) * inv);
+                                w.y = pc_pack_bf16(__uint_as_float(v[8 * i + 2]) * inv, __uint_as_float(v[8 * i + 3]) * inv);
+                                w.z = pc_pack_bf16(__uint_as_float(v[8 * i + 4]) * inv, __uint_as_float(v[8 * i + 5]) * inv);
+                                w.w = pc_pack_bf16(__uint_as_float(v[8 * i + 6]) * inv, __uint_as_float(v[8 * i + 7]) * inv);
+                                *reinterpret_cast<uint4 *>(orow + i * 8) = w;
+                            }
+                        }
+                        if (P.lse && row < P.n_q) P.lse[(size_t)row * P.n_q_heads + h] = (m_e + log2f(l_e)) * 0.6931471805599453f;
+                    } else if (P.cluster) {
+                        // (split form, one unit per CTA) Stage O (un-normalised, fp32) and (max, sum) in shared memory that no
+                        // multiply-add reads any more: tile 0 over both query tiles (every QK^T has completed once this tile's
+                        // last PV has, which was issued behind the other tile's last QK^T), tile 1 over the key stages (its own last PV is the last multiply-add of the CTA).
+                        const uint32_t stage = base + (t == 0 ? SM_Q : SM_K);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) sts128(stage + stage_off(i, r), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        *reinterpret_cast<float2 *>(gen + SM_ML + (t * TILE + r) * 8) = make_float2(m_e, l_e);
+                    } else {
+                        // Partial tile layout: 16-byte unit (c4, r) = columns 4*c4..4*c4+3 of row r at unit c4*128 + r, so the 32 rows
+                        // of a warp store 512 contiguous bytes per instruction (a row-major tile would touch 32 lines per store).
+                        const size_t tile_slot = ((size_t)e_item * P.part_stride + part) * 2 + t;
+                        uint4 *ptile = reinterpret_cast<uint4 *>(P.part_o) + tile_slot * (TILE * TILE / 4) + r;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) ptile[i * TILE] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        *reinterpret_cast<float2 *>(P.part_ml + (tile_slot * TILE + r) * 2) = make_float2(m_e, l_e);
+                    }
                 }
             }
+            if (end) break;
             ++j;
         }
         // ---- the run's last unit.  If it is the first part of an item in two parts, the second one lies in the scratch, stored by the same warp of the
         // next CTA at the start of its run: it is fetched under the last PV and added here, in the order of the
         // merge kernel and with its arithmetic.
-        const Place p = place_of(U.item);
-        const bool head = MERGE && p.parts == 2 && p.part == 0;
-        uint4 x[32];
-        float2 ml = make_float2(-INFINITY, 0.f);
-        if (__builtin_expect(head && alive, 0)) {
-            const uint32_t *flag = P.sync + 2 + U.item;
-            const uint32_t call = __ldcg(P.sync);
-            const uint64_t t0 = pc_global_ns(), limit_ns = P.wait_us ? (uint64_t)P.wait_us * 1000ull : 10000000000ull;      // (that CTA may have to wait for an SM that somebody else's kernel holds)
-            for (;;) {
-                uint32_t seen;
-                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-                if (__all_sync(0xffffffffu, seen == call)) break;
-                if (*abort_flag || pc_global_ns() - t0 > limit_ns) {
-                    if (!*abort_flag) pc_flag(P.status, PC_ERR_TIMEOUT, PC_WHERE_ATTN_WAIT);
-                    *abort_flag = 1;
-                    alive = false;
+        if constexpr (MERGE) {
+            const Place p = place_of(U.item);
+            const bool head = p.parts == 2 && p.part == 0;
+            uint4 x[32];
+            float2 ml = make_float2(-INFINITY, 0.f);
+            if (__builtin_expect(head && alive, 0)) {
+                const uint32_t *flag = P.sync + 2 + U.item;
+                const uint32_t call = __ldcg(P.sync);
+                const uint64_t t0 = pc_global_ns(), limit_ns = P.wait_us ? (uint64_t)P.wait_us * 1000ull : 10000000000ull;      // (that CTA may have to wait for an SM that somebody else's kernel holds)
+                for (;;) {
+                    uint32_t seen;
+                    asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
+                    if (__all_sync(0xffffffffu, seen == call)) break;
+                    if (*abort_flag || pc_global_ns() - t0 > limit_ns) {
+                        if (!*abort_flag) pc_flag(P.status, PC_ERR_TIMEOUT, PC_WHERE_ATTN_WAIT);
+                        *abort_flag = 1;
+                        alive = false;
+                    }
+                    alive = __all_sync(0xffffffffu, alive);
+                    if (!alive) break;
                 }
-                alive = __all_sync(0xffffffffu, alive);
-                if (!alive) break;
+                if (alive) {
+                    const size_t slot = p.slot + 2;
+                    const uint4 *ptile = reinterpret_cast<const uint4 *>(P.part_o) + slot * (TILE * TILE / 4) + r;
+                    ml = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + slot * TILE + r);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) x[i] = __ldcg(ptile + i * TILE);
+                }
             }
+            if (alive) alive = warp_wait(bar(BAR_PVDONE + t), (n_steps - 1) & 1, abort_flag, P.status, P.wait_us);
             if (alive) {
-                const size_t slot = p.slot + 2;
-                const uint4 *ptile = reinterpret_cast<const uint4 *>(P.part_o) + slot * (TILE * TILE / 4) + r;
-                ml = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + slot * TILE + r);
+                tc_fence_after();
+                if (!head) {
+                    uint32_t v[128];
+                    read_out(v);
+                    if (p.there) {
+                        if (p.parts == 1) write_whole(p, v, m_used, l); else write_part(p, v, m_used, l);
+                    }
+                    if (p.part == 1) {
+                        __syncwarp();
+                        arrive_if(lead, bar(BAR_PART));
+                    }
+                } else {
+                    // Rows leave through shared memory, over the queries of this tile (its last QK^T has been seen): a warp's store then covers two whole rows
+                    // of 256 bytes instead of 16 bytes of each of 32.  16-byte unit c of row r at r * 256 + (c ^ (r & 15)) * 16: no bank twice.
+                    const float m = fmaxf(m_used, ml.x), sc0 = head ? exp2f(m_used - m) : 1.f, sc1 = exp2f(ml.x - m);
+                    const float lsum = head ? fmaf(ml.y, sc1, l * sc0) : l, inv = 1.f / lsum;
+                    const uint32_t stage = base + SM_Q + t * TILE_BYTES + quad * (32 * 256);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) x[i] = __ldcg(ptile + i * TILE);
-            }
-        }
-        if (alive) alive = warp_wait(bar(BAR_PVDONE + t), (n_steps - 1) & 1, abort_flag, P.status, P.wait_us);
-        if (alive) {
-            tc_fence_after();
-            if (!head) {
-                uint32_t v[128];
-                read_out(v);
-                if (!MERGE && P.cluster) {
-                    // (split form, one unit per CTA) Stage O (un-normalised, fp32) and (max, sum) in shared memory that no
-                    // multiply-add reads any more: tile 0 over both query tiles (every QK^T has completed once this tile's
-                    // last PV has, which was issued behind the other tile's last QK^T), tile 1 over the key stages (its own last PV is the last multiply-add of the CTA).
-                    const uint32_t stage = base + (t == 0 ? SM_Q : SM_K);
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t v[32];
+                        tmem_ld32(o_addr + c * 32, v);
+                        tmem_wait_ld();
+                        if (head) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) sts128(stage + stage_off(i, r), v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                    *reinterpret_cast<float2 *>(gen + SM_ML + (t * TILE + r) * 8) = make_float2(m_used, l);
-                } else if (p.there) {
-                    if (p.parts == 1) write_whole(p, v, m_used, l); else write_part(p, v, m_used, l);
-                }
-                if (MERGE && p.part == 1) {
-                    __syncwarp();
-                    arrive_if(lead, bar(BAR_PART));
-                }
-            } else {
-                // Rows leave through shared memory, over the queries of this tile (its last QK^T has been seen): a warp's store then covers two whole rows
-                // of 256 bytes instead of 16 bytes of each of 32.  16-byte unit c of row r at r * 256 + (c ^ (r & 15)) * 16: no bank twice.
-                const float m = fmaxf(m_used, ml.x), sc0 = head ? exp2f(m_used - m) : 1.f, sc1 = exp2f(ml.x - m);
-                const float lsum = head ? fmaf(ml.y, sc1, l * sc0) : l, inv = 1.f / lsum;
-                const uint32_t stage = base + SM_Q + t * TILE_BYTES + quad * (32 * 256);
+                            for (int i = 0; i < 8; ++i) {
+                                const uint4 y = x[8 * c + i];
+                                v[4 * i + 0] = __float_as_uint(fmaf(__uint_as_float(y.x), sc1, __uint_as_float(v[4 * i + 0]) * sc0));
+                                v[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(y.y), sc1, __uint_as_float(v[4 * i + 1]) * sc0));
+                                v[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(y.z), sc1, __uint_as_float(v[4 * i + 2]) * sc0));
+                                v[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(y.w), sc1, __uint_as_float(v[4 * i + 3]) * sc0));
+                            }
+                        }
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(o_addr + c * 32, v);
-                    tmem_wait_ld();
-                    if (head) {
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t w[4];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const uint4 y = x[8 * c + i];
-                            v[4 * i + 0] = __float_as_uint(fmaf(__uint_as_float(y.x), sc1, __uint_as_float(v[4 * i + 0]) * sc0));
-                            v[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(y.y), sc1, __uint_as_float(v[4 * i + 1]) * sc0));
-                            v[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(y.z), sc1, __uint_as_float(v[4 * i + 2]) * sc0));
-                            v[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(y.w), sc1, __uint_as_float(v[4 * i + 3]) * sc0));
+                            for (int k = 0; k < 4; ++k) w[k] = pc_pack_bf16(__uint_as_float(v[8 * i + 2 * k]) * inv, __uint_as_float(v[8 * i + 2 * k + 1]) * inv);
+                            sts128(stage + lane * 256 + (((4 * c + i) ^ (lane & 15)) << 4), w[0], w[1], w[2], w[3]);
                         }
                     }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) w[k] = pc_pack_bf16(__uint_as_float(v[8 * i + 2 * k]) * inv, __uint_as_float(v[8 * i + 2 * k + 1]) * inv);
-                        sts128(stage + lane * 256 + (((4 * c + i) ^ (lane & 15)) << 4), w[0], w[1], w[2], w[3]);
-                    }
-                }
-                __syncwarp();
-                if (p.there) {
-                    const int row0 = p.row - lane;
+                    __syncwarp();
+                    if (p.there) {
+                        const int row0 = p.row - lane;
 #pragma unroll 4
-                    for (int i = 0; i < 16; ++i) {
-                        const int rr = 2 * i + (lane >> 4), c = lane & 15;
-                        const uint4 w = pc_lds128(stage + rr * 256 + ((c ^ (rr & 15)) << 4));
-                        if (row0 + rr < P.n_q) *reinterpret_cast<uint4 *>(P.out + ((size_t)(row0 + rr) * P.n_q_heads + p.h) * TILE + c * 8) = w;
+                        for (int i = 0; i < 16; ++i) {
+                            const int rr = 2 * i + (lane >> 4), c = lane & 15;
+                            const uint4 w = pc_lds128(stage + rr * 256 + ((c ^ (rr & 15)) << 4));
+                            if (row0 + rr < P.n_q) *reinterpret_cast<uint4 *>(P.out + ((size_t)(row0 + rr) * P.n_q_heads + p.h) * TILE + c * 8) = w;
+                        }
+                        if (P.lse && p.row < P.n_q) P.lse[(size_t)p.row * P.n_q_heads + p.h] = (m + log2f(lsum)) * 0.6931471805599453f;
                     }
-                    if (P.lse && p.row < P.n_q) P.lse[(size_t)p.row * P.n_q_heads + p.h] = (m + log2f(lsum)) * 0.6931471805599453f;
                 }
             }
         }
