@@ -113,7 +113,7 @@ pc_status pc_attend_frame_impl(pc_ctx *ctx, const pc_cache *cache, const pc_segm
     int n_seg = 0;
     st = gather_segments(ctx, cache, current, segs, &n_seg);
     if (st != PC_OK) return st;
-    if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
+    if (hooks && hooks->kv_ready) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
     ctx->last_n_q = 0;
     if (tensor_core_path(ctx)) {
         ctx->prepared_n_seg = 0;                       // the rotated-key scratch is about to be overwritten
@@ -180,14 +180,15 @@ pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *bu
         ctx->prepared_n_seg = 0;                       // the scratch no longer holds a key set of pc_attend_prepare
     }
     // (with values still on their way the selection need not wait for them; stage marks tell the two stages apart)
-    const bool one_launch = !hooks && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
+    const bool on_the_way = hooks && hooks->kv_ready;
+    const bool one_launch = !on_the_way && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
     ctx->last_n_q = 0;
     ctx->q_rot_n = 0;
     const pc_front_args args{src, budget, nullptr, scores, sel_idx, delta_t, &dst->history, k_rot_dst};
-    const pc_front_args *front = !hooks && n_sel > 0 && pc_front_fits(ctx, src, true) ? &args : nullptr;
+    const pc_front_args *front = !on_the_way && n_sel > 0 && pc_front_fits(ctx, src, true) ? &args : nullptr;
     st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream, !one_launch, front);
     if (st != PC_OK) return st;
-    if (hooks) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
+    if (on_the_way) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));
     if (!front)
         st = one_launch ? pc_launch_select_pack(ctx, scores, src, budget, delta_t, &dst->history, sel_idx, k_rot_dst, stream)
                     : pc_compact_impl(ctx, src, sel_idx, budget, delta_t, dst, k_rot_dst, stream);

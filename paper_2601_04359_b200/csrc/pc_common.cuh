@@ -324,7 +324,7 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
 // query rows of one part of a frame's attention when its output is to leave in parts: enough row tiles per part to fill the GPU
 int pc_attend_part_rows(const pc_ctx *ctx, int n_q);
 // What a frame step driven from host memory adds to pc_frame_step / pc_attend_frame: an event the stream waits for before V or
-// the packed positions are first read, and a call after each part of the output has been enqueued (rows [row0, row0 + n)).
+// the packed positions are first read (NULL: they are there), and a call after each part of the output has been enqueued (rows [row0, row0 + n)).
 struct pc_step_hooks {
     cudaEvent_t kv_ready;
     pc_status (*part_done)(void *self, int row0, int n, cudaStream_t stream);

@@ -431,7 +431,8 @@ void *device_view(const void *p, size_t bytes) {
     return z.devicePointer == static_cast<char *>(a.devicePointer) + bytes - 1 ? a.devicePointer : nullptr;
 }
 
-// A part of the output is enqueued: it goes home on the side stream while the next part is computed.
+// A part of the output is enqueued: it goes home on the side stream while the next part is computed, or (a small step, in one part) by a
+// kernel behind it.  Either way ahead of the window's change of state, behind which nothing is enqueued that could fail.
 struct HomeTrip {
     pc_window *w;
     const char *from;
@@ -445,6 +446,12 @@ pc_status send_home(void *self, int row0, int n, cudaStream_t stream) {
     PC_CUDA_TRY(cudaStreamWaitEvent(h.w->side, h.w->main_ev, 0));
     PC_CUDA_TRY(cudaMemcpyAsync(h.to + row0 * h.row_bytes, h.from + row0 * h.row_bytes, n * h.row_bytes, cudaMemcpyDeviceToHost, h.w->side));
     return PC_OK;
+}
+pc_status move_home(void *self, int row0, int n, cudaStream_t stream) {
+    const HomeTrip &h = *static_cast<const HomeTrip *>(self);
+    Runs home{};
+    add_run(home, h.from + row0 * h.row_bytes, h.to + row0 * h.row_bytes, n * h.row_bytes);
+    return launch_move(home, stream);
 }
 
 }  // namespace
@@ -496,7 +503,7 @@ extern "C" pc_status pc_window_step_host(pc_window *w, const pc_host_window_step
     const void *const q_pos = device_view(in->q_pos, q_pos_bytes), *const pos = n > 0 ? device_view(in->frame_pos, pos_bytes) : nullptr;
     // A small step goes up and home by a kernel each, and runs as a step on the device does in between.
     const auto enqueue_small = [&](const void *q, const void *k, const void *v, void *out) -> pc_status {
-        Runs up{}, home{};
+        Runs up{};
         add_run(up, q, ws->q, q_bytes);
         add_run(up, q_pos, ws->q_pos, q_pos_bytes);
         if (n > 0) {
@@ -504,10 +511,10 @@ extern "C" pc_status pc_window_step_host(pc_window *w, const pc_host_window_step
             add_run(up, v, to_v, kv_bytes);
             add_run(up, pos, to_pos, pos_bytes);
         }
-        pc_status s = launch_move(up, stream);
-        if (s == PC_OK) s = window_step(w, ws->q, ws->q_pos, in->n_q, ws->out, nullptr, regime, stream, nullptr);
-        add_run(home, ws->out, out, q_bytes);
-        return s == PC_OK ? launch_move(home, stream) : s;
+        HomeTrip trip{w, static_cast<const char *>(ws->out), static_cast<char *>(out), qrow};
+        const pc_step_hooks hooks{nullptr, move_home, &trip};
+        const pc_status s = launch_move(up, stream);
+        return s == PC_OK ? window_step(w, ws->q, ws->q_pos, in->n_q, ws->out, nullptr, regime, stream, &hooks) : s;
     };
     // In a larger one what the scores need goes first: the queries, then the finished frame's keys, straight to the end of the active history
     // buffer, on the side stream; the positions come by a kernel beside them.  The values follow under the scoring and

@@ -66,7 +66,12 @@ void rt_reset() {
 }
 void rt_fail(const char *name, int after) { g_fail[name] = after; }
 void rt_on_attribute(void (*f)()) { g_on_attribute = f; }
-void rt_memory(const void *p, size_t bytes, int kind, int device) { g_memory[static_cast<const char *>(p)] = Range{bytes, kind, device}; }
+void rt_memory(const void *p_, size_t bytes, int kind, int device) {
+    const char *p = static_cast<const char *>(p_);
+    for (auto r = g_memory.begin(); r != g_memory.end();)       // what lay there before is gone
+        r = r->first < p + bytes && p < r->first + r->second.bytes ? g_memory.erase(r) : std::next(r);
+    g_memory[p] = Range{bytes, kind, device};
+}
 
 cudaError_t cudaGetDevice(int *d) { *d = t_device; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { t_device = d; return cudaSuccess; }
@@ -101,6 +106,7 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
     if (r != g_memory.begin() && c < (--r)->first + r->second.bytes) {
         a->type = static_cast<cudaMemoryType>(r->second.kind);
         a->device = r->second.device;
+        if (a->type == cudaMemoryTypeHost) a->devicePointer = const_cast<void *>(p);
     }
     return cudaSuccess;
 }

@@ -93,6 +93,11 @@ class Case:
         self.out = torch.zeros_like(self.q)
         self.ws = {"q": torch.zeros_like(self.q), "q_pos": torch.zeros_like(self.q_pos), "out": torch.zeros_like(self.q)}
 
+    def pin(self):
+        """What a step takes from host memory and brings back there is pinned."""
+        self.rt.memory(self.frame.k, self.frame.v, self.frame.pos, self.q, self.q_pos, self.out, kind=PINNED)
+        return self
+
     def make(self):
         win = pc.Window(self.ctx, *self.window, self.anchors, self.bufs[0], self.bufs[1])
         self.rt.open.append(win)
