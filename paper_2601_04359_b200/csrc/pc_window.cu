@@ -1,5 +1,7 @@
 // Cache window: the Fill / Pack / Slide regimes (Sec. 3.4, Fig. 6) and the temporal rebase (Eq. 9) as a host-side state
 // machine around pc_plan_budget, pc_score and pc_compact; its one kernel turns a cache mask (Eq. 1) into row indices.
+#include <cuda.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -420,15 +422,29 @@ pc_status launch_move(const Runs &R, cudaStream_t stream) {
     return PC_OK;
 }
 
-// Where a kernel finds `bytes` of pinned host memory; NULL where it cannot (pageable, in part or at all, or not on 16 bytes).
+// Where a kernel finds `bytes` of pinned host memory; NULL where it cannot (pageable, in part or at all, managed, or not on 16 bytes).  The
+// driver says from where to where the allocation or registration around p goes: two pinned ends do not make the middle pinned.
 void *device_view(const void *p, size_t bytes) {
-    cudaPointerAttributes a, z;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&z, static_cast<const char *>(p) + bytes - 1) != cudaSuccess) {
+    typedef CUresult (*AttributesFn)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const AttributesFn attributes = []() -> AttributesFn {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+            return reinterpret_cast<AttributesFn>(f);
         cudaGetLastError();
         return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer || !pc_aligned16(a.devicePointer) || !pc_aligned16(p)) return nullptr;
-    return z.devicePointer == static_cast<char *>(a.devicePointer) + bytes - 1 ? a.devicePointer : nullptr;
+    }();
+    if (!attributes || !pc_aligned16(p)) return nullptr;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr at = 0, first = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &at, &first, &size};
+    const CUdeviceptr host = reinterpret_cast<CUdeviceptr>(p);
+    if (attributes(5, what, to, host) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed) return nullptr;
+    if (at != host || host < first || host - first > size || size - (host - first) < bytes) return nullptr;    // (one address on either side, as unified addressing has it)
+    return const_cast<void *>(p);
 }
 
 // A part of the output is enqueued: it goes home on the side stream while the next part is computed, or (a small step, in one part) by a

@@ -106,7 +106,6 @@ cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
     if (r != g_memory.begin() && c < (--r)->first + r->second.bytes) {
         a->type = static_cast<cudaMemoryType>(r->second.kind);
         a->device = r->second.device;
-        if (a->type == cudaMemoryTypeHost) a->devicePointer = const_cast<void *>(p);
     }
     return cudaSuccess;
 }
@@ -155,8 +154,22 @@ cudaError_t cudaGetSymbolAddress(void **p, const void *) {
     return cudaSuccess;
 }
 static CUresult encode(...) { return CUDA_SUCCESS; }
-cudaError_t cudaGetDriverEntryPoint(const char *, void **p, unsigned long long, cudaDriverEntryPointQueryResult *q) {
-    *p = reinterpret_cast<void *>(encode);
+static CUresult pointer_attributes(unsigned n, CUpointer_attribute *what, void **to, CUdeviceptr p) {
+    const char *c = reinterpret_cast<const char *>(p);
+    auto r = g_memory.upper_bound(c);
+    const bool known = r != g_memory.begin() && c < (--r)->first + r->second.bytes;
+    for (unsigned i = 0; i < n; ++i) switch (what[i]) {
+        case CU_POINTER_ATTRIBUTE_MEMORY_TYPE: *static_cast<unsigned *>(to[i]) = known ? r->second.kind : 0; break;
+        case CU_POINTER_ATTRIBUTE_IS_MANAGED: *static_cast<unsigned *>(to[i]) = 0; break;
+        case CU_POINTER_ATTRIBUTE_DEVICE_POINTER: *static_cast<CUdeviceptr *>(to[i]) = known ? p : 0; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_START_ADDR: *static_cast<CUdeviceptr *>(to[i]) = known ? reinterpret_cast<CUdeviceptr>(r->first) : 0; break;
+        case CU_POINTER_ATTRIBUTE_RANGE_SIZE: *static_cast<size_t *>(to[i]) = known ? r->second.bytes : 0; break;
+        default: return CUDA_ERROR_INVALID_VALUE;
+    }
+    return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPoint(const char *name, void **p, unsigned long long, cudaDriverEntryPointQueryResult *q) {
+    *p = strcmp(name, "cuPointerGetAttributes") ? reinterpret_cast<void *>(encode) : reinterpret_cast<void *>(pointer_attributes);
     *q = cudaDriverEntryPointSuccess;
     return cudaSuccess;
 }

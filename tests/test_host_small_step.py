@@ -8,7 +8,7 @@ import pytest
 
 from paper_2601_04359_b200 import binding as pc
 
-from .host_runtime import Case, _library, counts, rt  # noqa: F401
+from .host_runtime import PINNED, Case, _library, counts, rt  # noqa: F401
 
 
 def launches(rt):
@@ -52,3 +52,21 @@ def test_small_step_that_fails_leaves_the_window(rt, frames, n):
                 assert e.status == pc.PC_ERR_CUDA and state(win) == before
                 assert sorted(rt.log()[-2:]) == ["synchronize main", "synchronize side"]
         assert at > 0 and state(win)[:4] == want          # and the same step still works
+
+
+@pytest.mark.parametrize("which", ["q", "q_pos", "k", "v", "pos", "out"])
+def test_memory_that_is_pinned_at_both_ends_only_goes_by_copies(rt, which):
+    """Two registered ranges with pageable memory in between: a kernel that read it would fault."""
+    c = Case(rt, n=130, total=200).pin()
+    win = c.make()
+    t = {"q": c.q, "q_pos": c.q_pos, "out": c.out, "k": c.frame.k, "v": c.frame.v, "pos": c.frame.pos}[which]
+    rt.memory(t[:40], t[90:], kind=PINNED)
+    rt.reset()
+    c.step_host(win)
+    copies = sum(line.startswith("memcpy") for line in rt.log())
+    # positions by copies as well if they are what is not pinned in whole
+    assert copies == (5 if which in ("q_pos", "pos") else 4) and launches(rt)[-1] != "k_move"
+    rt.memory(t, kind=PINNED)
+    rt.reset()
+    c.step_host(win)
+    assert launches(rt)[0] == launches(rt)[-1] == "k_move" and not any(line.startswith("memcpy") for line in rt.log())
