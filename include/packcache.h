@@ -399,6 +399,10 @@ pc_status pc_set_wait_limit_us(pc_ctx *ctx, uint32_t limit_us);
  * kernel, is told to expect n_bytes more than are ever sent, so its wait runs out after the limit above and pc_poll_status
  * returns PC_ERR_TIMEOUT; the call's output is then undefined.  0 switches the hook off.  Nothing traps and nothing waits without a limit. */
 pc_status pc_test_expect_extra_bytes(pc_ctx *ctx, uint32_t n_bytes);
+/* Test hook for the merge in the attention kernel.  A CTA with the first part of an item that two CTAs share looks for the other's part
+ * for a tenth of a millisecond; if it has not come by then (that CTA may still wait for an SM), the last CTA of the call merges the two.
+ * With the hook on, none looks and all is left to the last one: the same results.  The limit above has no part in this. */
+pc_status pc_test_leave_parts(pc_ctx *ctx, int32_t on);
 
 /* Per-kernel timing for benchmarks.  With timing on, each call records CUDA events on its stream at the boundaries
  * of its kernels (a few microseconds of overhead per call); pc_get_timing waits for the last recorded events and

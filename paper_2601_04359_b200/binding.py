@@ -27,7 +27,7 @@ EXPORTS = ["pc_create", "pc_destroy", "pc_plan_budget", "pc_score", "pc_compact"
            "pc_frame_step_host", "pc_status_string", "pc_score_tokens_static", "pc_set_cluster_merge",
            "pc_window_create", "pc_window_destroy", "pc_window_append", "pc_window_append_masked", "pc_window_update", "pc_window_cache",
            "pc_window_state", "pc_attend_prepare", "pc_attend_prepared", "pc_attend_mass", "pc_frame_step",
-           "pc_forget_anchors", "pc_set_wait_limit_us", "pc_test_expect_extra_bytes", "pc_window_step", "pc_window_step_host", "pc_set_timing_skip",
+           "pc_forget_anchors", "pc_set_wait_limit_us", "pc_test_expect_extra_bytes", "pc_test_leave_parts", "pc_window_step", "pc_window_step_host", "pc_set_timing_skip",
            "pc_get_span", "pc_probe_stream_read", "pc_probe_mma_rate"]
 
 
@@ -146,6 +146,7 @@ def load() -> C.CDLL:
     lib.pc_forget_anchors.argtypes = [C.c_void_p]
     lib.pc_set_wait_limit_us.argtypes = [C.c_void_p, C.c_uint32]
     lib.pc_test_expect_extra_bytes.argtypes = [C.c_void_p, C.c_uint32]
+    lib.pc_test_leave_parts.argtypes = [C.c_void_p, C.c_int32]
     lib.pc_window_create.argtypes = [C.c_void_p, C.POINTER(pc_window_params), C.POINTER(pc_segment), C.POINTER(pc_segment),
                                      C.POINTER(pc_segment), C.c_void_p, C.c_void_p, C.POINTER(C.c_void_p)]
     lib.pc_window_destroy.argtypes = [C.c_void_p]
@@ -320,6 +321,10 @@ def pc_set_wait_limit_us(ctx: Context, limit_us: int) -> None:
 
 def pc_test_expect_extra_bytes(ctx: Context, n_bytes: int) -> None:
     _check(load().pc_test_expect_extra_bytes(ctx.handle, n_bytes), "pc_test_expect_extra_bytes")
+
+
+def pc_test_leave_parts(ctx: Context, on: bool) -> None:
+    _check(load().pc_test_leave_parts(ctx.handle, int(on)), "pc_test_leave_parts")
 
 
 def pc_attend_prepare(ctx: Context, cache: Cache, current: Optional[Segment] = None, stream=None) -> None:

@@ -146,6 +146,12 @@ extern "C" pc_status pc_test_expect_extra_bytes(pc_ctx *c, uint32_t n_bytes) {
     return PC_OK;
 }
 
+extern "C" pc_status pc_test_leave_parts(pc_ctx *c, int32_t on) {
+    if (!c) return PC_ERR_INVALID_ARG;
+    c->test_leave_parts = on != 0;
+    return PC_OK;
+}
+
 extern "C" pc_status pc_forget_anchors(pc_ctx *c) {
     if (!c) return PC_ERR_INVALID_ARG;
     c->anchor_rot_n = 0;

@@ -70,6 +70,10 @@ enum { BAR_Q = 0 /* [tile] */, BAR_QFREE = 2 /* [tile] */, BAR_VFULL = 4 /* [sta
        BAR_SFREE = 10 /* [tile] */, BAR_PHALF = 12 /* [tile][half] */, BAR_PVDONE = 16 /* [tile] */, BAR_DONE = 18, BAR_PART = 19, N_BARS = 20 };
 static_assert(N_BARS * 8 + 12 <= 256, "barriers, abort flag and TMEM address share 256 bytes");
 
+constexpr int SYNC_PARTS = 2, LEFT_PER_ITEM = 8;          // words of TcParams::sync
+// How long a CTA with a first part looks for the second one before it leaves both to the last CTA
+constexpr uint64_t PART_NS = 100000;
+
 // TMEM columns
 constexpr int TM_S = 0, TM_P = TILE, TM_O = 2 * TILE;     // scores; P of tile t at TM_P + 64 t; O of tile t at TM_O + 128 t
 
@@ -90,7 +94,11 @@ struct TcParams {
     float *lse;
     float *part_o;    // [item*S + s][2] tiles of 128 x 128 fp32, 16-byte unit (c4, r) at c4*128 + r
     float *part_ml;   // [item*S + s][2][128][2]
-    uint32_t *sync;   // merge: [0] number of the call, [1] tickets of CTAs that are done, [2 + item] number of the call that left the second part
+    // Merge: [0] number of the call, [1] tickets of CTAs that are done and, in the upper half, how many of them left a merge to the last one;
+    // from SYNC_PARTS on, per item, the number of the call that left the second part; behind those, per item, tile and quarter, that of the
+    // call that left the merge.
+    uint32_t *sync;
+    int leave_parts;  // test hook: every merge is left to the last CTA
     int32_t *status;
 };
 
@@ -224,6 +232,29 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return __all_sync(0xffffffffu, pc_mbar_wait(bar, parity, abort_flag, status, PC_WHERE_ATTN_WAIT, limit_us));
 }
 
+// Merges that were left, a warp of the last CTA per (item, tile, quarter), with the merge kernel's order and arithmetic: 32 rows, one a lane.
+// A function of its own: as part of the kernel's code it made every call 0.3 us longer (the step at 12 frames 70.7 against 71.0 us, 70.5 without it).
+__device__ __noinline__ void merge_left(const TcParams &P, uint32_t call, int w, int lane) {
+    for (int e = w; e < P.n_items * LEFT_PER_ITEM; e += (TC_THREADS - 128) / 32) {
+        if (__ldcg(P.sync + SYNC_PARTS + P.n_items + e) != call) continue;
+        const int item = e / LEFT_PER_ITEM, t = (e >> 2) & 1, r = (e & 3) * 32 + lane;
+        const int T = 2 * (item % P.pairs_per_g) + t, h = item / P.pairs_per_g * P.group + T % P.group, row = T / P.group * TILE + r;
+        if (row >= P.n_q) continue;
+        const size_t slot = (size_t)item * P.part_stride * 2 + t;
+        const float2 a = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + slot * TILE + r), b = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + (slot + 2) * TILE + r);
+        const float m = fmaxf(a.x, b.x), sc0 = exp2f(a.x - m), sc1 = exp2f(b.x - m), l = fmaf(b.y, sc1, a.y * sc0), inv = 1.f / l;
+        const float4 *po = reinterpret_cast<const float4 *>(P.part_o) + slot * (TILE * TILE / 4) + r;
+        uint2 *orow = reinterpret_cast<uint2 *>(P.out + ((size_t)row * P.n_q_heads + h) * TILE);
+#pragma unroll 4
+        for (int c = 0; c < TILE / 4; ++c) {
+            const float4 x = __ldcg(po + c * TILE), y = __ldcg(po + TILE * TILE / 2 + c * TILE);
+            orow[c] = make_uint2(pc_pack_bf16(fmaf(y.x, sc1, x.x * sc0) * inv, fmaf(y.y, sc1, x.y * sc0) * inv),
+                                 pc_pack_bf16(fmaf(y.z, sc1, x.z * sc0) * inv, fmaf(y.w, sc1, x.w * sc0) * inv));
+        }
+        if (P.lse) P.lse[(size_t)row * P.n_q_heads + h] = (m + log2f(l)) * 0.6931471805599453f;
+    }
+}
+
 // MERGE: items in two parts are merged by the CTA that has the first one.  A kernel of its own: with what that takes in its code, calls
 // that merge nothing took 0.3 us longer.
 template <bool MERGE>
@@ -236,6 +267,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + SM_BAR + N_BARS * 8);
+    volatile int *left_here = abort_flag + 1;            // a warp of this CTA left a merge
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(gen + SM_BAR + N_BARS * 8 + 8);
     const uint32_t bar0 = base + SM_BAR;
     auto bar = [&](int i) { return bar0 + 8u * i; };
@@ -263,6 +295,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         mbar_init(bar(BAR_DONE), 3);
         mbar_init(bar(BAR_PART), 8);
         *abort_flag = 0;
+        *left_here = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -297,7 +330,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
             bool owes = MERGE && first_part == 1;
             const auto pass_on = [&]() {
                 __threadfence();
-                asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(P.sync + 2 + (int)(G0 / P.n_kv_tiles)), "r"(__ldcg(P.sync)) : "memory");
+                asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(P.sync + SYNC_PARTS + (int)(G0 / P.n_kv_tiles)), "r"(__ldcg(P.sync)) : "memory");
                 owes = false;
             };
             for (long long g = G0; g < G1 && alive; ++un) {
@@ -677,29 +710,25 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         }
         // ---- the run's last unit.  If it is the first part of an item in two parts, the second one lies in the scratch, stored by the same warp of the
         // next CTA at the start of its run: it is fetched under the last PV and added here, in the order of the
-        // merge kernel and with its arithmetic.
+        // merge kernel and with its arithmetic.  That CTA may not have had an SM yet (somebody else's kernel holds it), and this one's SM may be what it is waiting
+        // for, so a part that does not come is no error: the first one is stored as well, and the last CTA merges them.
         if constexpr (MERGE) {
             const Place p = place_of(U.item);
-            const bool head = p.parts == 2 && p.part == 0;
+            const bool head = p.parts == 2 && p.part == 0 && p.there;
+            bool merge = false;
             uint4 x[32];
             float2 ml = make_float2(-INFINITY, 0.f);
-            if (__builtin_expect(head && alive, 0)) {
-                const uint32_t *flag = P.sync + 2 + U.item;
+            if (__builtin_expect(head && alive && !P.leave_parts, 0)) {
+                const uint32_t *flag = P.sync + SYNC_PARTS + U.item;
                 const uint32_t call = __ldcg(P.sync);
-                const uint64_t t0 = pc_global_ns(), limit_ns = P.wait_us ? (uint64_t)P.wait_us * 1000ull : 10000000000ull;      // (that CTA may have to wait for an SM that somebody else's kernel holds)
+                const uint64_t t0 = pc_global_ns();
                 for (;;) {
                     uint32_t seen;
                     asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-                    if (__all_sync(0xffffffffu, seen == call)) break;
-                    if (*abort_flag || pc_global_ns() - t0 > limit_ns) {
-                        if (!*abort_flag) pc_flag(P.status, PC_ERR_TIMEOUT, PC_WHERE_ATTN_WAIT);
-                        *abort_flag = 1;
-                        alive = false;
-                    }
-                    alive = __all_sync(0xffffffffu, alive);
-                    if (!alive) break;
+                    merge = __all_sync(0xffffffffu, seen == call);
+                    if (merge || __any_sync(0xffffffffu, *abort_flag || pc_global_ns() - t0 > PART_NS)) break;
                 }
-                if (alive) {
+                if (merge) {
                     const size_t slot = p.slot + 2;
                     const uint4 *ptile = reinterpret_cast<const uint4 *>(P.part_o) + slot * (TILE * TILE / 4) + r;
                     ml = __ldcg(reinterpret_cast<const float2 *>(P.part_ml) + slot * TILE + r);
@@ -710,7 +739,7 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
             if (alive) alive = warp_wait(bar(BAR_PVDONE + t), (n_steps - 1) & 1, abort_flag, P.status, P.wait_us);
             if (alive) {
                 tc_fence_after();
-                if (!head) {
+                if (!merge) {
                     uint32_t v[128];
                     read_out(v);
                     if (p.there) {
@@ -719,27 +748,28 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                     if (p.part == 1) {
                         __syncwarp();
                         arrive_if(lead, bar(BAR_PART));
+                    } else if (head && lead) {
+                        P.sync[SYNC_PARTS + P.n_items + U.item * LEFT_PER_ITEM + t * 4 + quad] = __ldcg(P.sync);
+                        *left_here = 1;
                     }
                 } else {
                     // Rows leave through shared memory, over the queries of this tile (its last QK^T has been seen): a warp's store then covers two whole rows
                     // of 256 bytes instead of 16 bytes of each of 32.  16-byte unit c of row r at r * 256 + (c ^ (r & 15)) * 16: no bank twice.
-                    const float m = fmaxf(m_used, ml.x), sc0 = head ? exp2f(m_used - m) : 1.f, sc1 = exp2f(ml.x - m);
-                    const float lsum = head ? fmaf(ml.y, sc1, l * sc0) : l, inv = 1.f / lsum;
+                    const float m = fmaxf(m_used, ml.x), sc0 = exp2f(m_used - m), sc1 = exp2f(ml.x - m);
+                    const float lsum = fmaf(ml.y, sc1, l * sc0), inv = 1.f / lsum;
                     const uint32_t stage = base + SM_Q + t * TILE_BYTES + quad * (32 * 256);
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         uint32_t v[32];
                         tmem_ld32(o_addr + c * 32, v);
                         tmem_wait_ld();
-                        if (head) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const uint4 y = x[8 * c + i];
-                                v[4 * i + 0] = __float_as_uint(fmaf(__uint_as_float(y.x), sc1, __uint_as_float(v[4 * i + 0]) * sc0));
-                                v[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(y.y), sc1, __uint_as_float(v[4 * i + 1]) * sc0));
-                                v[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(y.z), sc1, __uint_as_float(v[4 * i + 2]) * sc0));
-                                v[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(y.w), sc1, __uint_as_float(v[4 * i + 3]) * sc0));
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            const uint4 y = x[8 * c + i];
+                            v[4 * i + 0] = __float_as_uint(fmaf(__uint_as_float(y.x), sc1, __uint_as_float(v[4 * i + 0]) * sc0));
+                            v[4 * i + 1] = __float_as_uint(fmaf(__uint_as_float(y.y), sc1, __uint_as_float(v[4 * i + 1]) * sc0));
+                            v[4 * i + 2] = __float_as_uint(fmaf(__uint_as_float(y.z), sc1, __uint_as_float(v[4 * i + 2]) * sc0));
+                            v[4 * i + 3] = __float_as_uint(fmaf(__uint_as_float(y.w), sc1, __uint_as_float(v[4 * i + 3]) * sc0));
                         }
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -750,16 +780,14 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
                         }
                     }
                     __syncwarp();
-                    if (p.there) {
-                        const int row0 = p.row - lane;
+                    const int row0 = p.row - lane;
 #pragma unroll 4
-                        for (int i = 0; i < 16; ++i) {
-                            const int rr = 2 * i + (lane >> 4), c = lane & 15;
-                            const uint4 w = pc_lds128(stage + rr * 256 + ((c ^ (rr & 15)) << 4));
-                            if (row0 + rr < P.n_q) *reinterpret_cast<uint4 *>(P.out + ((size_t)(row0 + rr) * P.n_q_heads + p.h) * TILE + c * 8) = w;
-                        }
-                        if (P.lse && p.row < P.n_q) P.lse[(size_t)p.row * P.n_q_heads + p.h] = (m + log2f(lsum)) * 0.6931471805599453f;
+                    for (int i = 0; i < 16; ++i) {
+                        const int rr = 2 * i + (lane >> 4), c = lane & 15;
+                        const uint4 w = pc_lds128(stage + rr * 256 + ((c ^ (rr & 15)) << 4));
+                        if (row0 + rr < P.n_q) *reinterpret_cast<uint4 *>(P.out + ((size_t)(row0 + rr) * P.n_q_heads + p.h) * TILE + c * 8) = w;
                     }
+                    if (P.lse && p.row < P.n_q) P.lse[(size_t)p.row * P.n_q_heads + p.h] = (m + log2f(lsum)) * 0.6931471805599453f;
                 }
             }
         }
@@ -772,11 +800,30 @@ k_attend_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     }
     // every thread has done with its waits: the flag is final, and copies may be in flight that nobody waited for
     if (threadIdx.x == 0 && *abort_flag) pc_let_copies_land();
-    // The last CTA to come here moves the call's number on: what this call left in the flags means nothing to the next one, also if
-    // some of it was given up, and a captured call replays unchanged.
-    if (MERGE && threadIdx.x == 0 && atomicAdd(P.sync + 1, 1u) == (uint32_t)gridDim.x - 1) {
-        P.sync[1] = 0;
-        atomicAdd(P.sync, 1u);
+    if constexpr (MERGE) {
+        // The last CTA to come here moves the call's number on: what this call left in the flags means nothing to the next one, also if
+        // some of it was given up, and a captured call replays unchanged.  It also merges what was left: every part of the call is
+        // stored and fenced ahead of its CTA's ticket (a second part by pass_on, which this thread ran).
+        // That something was left travels with the ticket: a look behind it (a fence and a load) made every call 1.2 us longer.
+        volatile uint32_t *last = reinterpret_cast<volatile uint32_t *>(gen + SM_BAR + N_BARS * 8 + 4);   // (left_here and tmem_slot, read already) anything left, number of the call
+        if (threadIdx.x == 0) {
+            const uint32_t mine = *left_here ? 0x10000u : 0u;
+            uint32_t left = 0;
+            if (mine) __threadfence();
+            const uint32_t ticket = atomicAdd(P.sync + 1, 1u + mine);
+            if ((ticket & 0xFFFFu) == (uint32_t)gridDim.x - 1) {
+                left = (ticket >> 16) + mine;
+                if (left) {
+                    __threadfence();
+                    last[1] = __ldcg(P.sync);
+                }
+                P.sync[1] = 0;
+                atomicAdd(P.sync, 1u);
+            }
+            last[0] = left;
+        }
+        __syncthreads();
+        if (__builtin_expect(last[0] != 0 && warp >= 4, 0)) merge_left(P, last[1], warp - 4, lane);
     }
     if (!MERGE && P.cluster && P.n_splits > 1) {
         // Merge the KV ranges of this item across the cluster: CTA `rank` finishes every n_splits-th row of the two
@@ -948,7 +995,7 @@ int choose_ctas(int n_items, int n_kv_heads, long long steps, int most) {
 // Divides the line of (item, key tile) steps over CTAs: fills P.persistent, n_cta, n_splits, part_stride.
 //
 // What a division costs, in quarters of a step (a step is about 1.4 us): its longest run (boundaries reckoned in, or 16 for
-// them where runs are too short or too long for that), 8 for a merge.  The persistent form takes an even share of the line per CTA; the
+// them where runs are too short or too long for that), 8 for a merge (in the attention kernel as well, where it takes less).  The persistent form takes an even share of the line per CTA; the
 // split form cuts every item into s equal ranges, one CTA each, as long as all are resident at once: no boundary, and with one
 // range no merge.  Measured on rotated keys (query rotation + attention + merge), the persistent form against the one chosen
 // here: 16 / 4 heads, 556 queries x 1,549 keys 29.1 -> 21.9 us, 74 x 4,767 20.9 -> 18.4; 24 / 8, 300 x 305 17.8 -> 17.2 (two ranges,
@@ -1004,7 +1051,7 @@ pc_status pc_attend_tc_scratch(const pc_layer_desc *d, int sm_count, size_t *k_r
     const size_t slots = std::max((size_t)n_items * MAX_FIXED_SPLITS, (size_t)sm_count + 2 * (size_t)n_items);
     *part_o_floats = slots * 2 * TILE * TILE;
     *part_ml_floats = slots * 2 * TILE * 2;
-    *part_sync_words = 2 + (size_t)n_items;
+    *part_sync_words = SYNC_PARTS + (size_t)n_items * (1 + LEFT_PER_ITEM);
     return PC_OK;
 }
 
@@ -1089,11 +1136,14 @@ pc_status pc_launch_attend_tc(pc_ctx *ctx, int n_seg, const pc_segment *segs, co
     P.extra_tx = ctx->test_extra_tx;
     choose_division(ctx, n_items, tiles, P);
     P.cluster = (!P.persistent && P.n_splits > 1 && ctx->cluster_merge) ? 1 : 0;
-    // Merged in the kernel: items in two parts of which the second is there long before it is asked for, as it is where runs cross items.
-    // Two parts that end together (split form, or two CTAs to an item) would have the one wait for the other's stores: 703 queries of
-    // 24 / 8 heads x 2,689 keys 67.8 (merge kernel) against 71.2 us.
+    // Merged in the kernel: items in two parts where runs cross items.  The second part of an item is then the first unit of its CTA and lies there long
+    // before it is asked for, or it is that CTA's whole run and ends a step or two ahead of the first (three CTAs to two items, as 96 items on 144 CTAs:
+    // every second item); both kinds together still gain (96 items: the step at 12 frames 75.5 -> 74.5 us).  Where all pairs end together (split form, or
+    // two CTAs to an item) the one only waits for the other's stores: 703 queries of 24 / 8 heads x 2,689 keys 67.8 (merge kernel)
+    // against 71.2 us.
     const bool merge = P.persistent && P.part_stride == 2 && P.n_cta % n_items != 0;
     P.sync = ctx->part_sync;
+    P.leave_parts = ctx->test_leave_parts;
     if (P.part_stride > 1 && !P.cluster && (size_t)n_items * P.part_stride * 2 * TILE * TILE > ctx->part_o_floats) return PC_ERR_CAPACITY;
 
     CUtensorMap mq, mk, mv[PC_MAX_SEGMENTS];

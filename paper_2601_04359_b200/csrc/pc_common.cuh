@@ -68,6 +68,7 @@ struct pc_ctx {
     int kv_splits;             // 0 = chosen per call
     int cluster_merge;         // 1 = KV ranges merge inside the kernel through cluster shared memory (default 0)
     uint32_t wait_limit_us;    // limit of every bounded device-side wait in microseconds; 0 = about one second
+    int32_t test_leave_parts;  // test hook: the attention kernel leaves every merge to its last CTA
     uint32_t test_extra_tx;    // test hook: bytes the first barrier of the waiting kernels expects beyond what is sent (0 = off)
     // rotated anchor keys kept in k_rot across fused frame steps (anchors never move): the segment they were made from
     const void *anchor_rot_k;
@@ -89,7 +90,7 @@ struct pc_ctx {
     cudaEvent_t ev[PC_N_MARKS];
     float *part_o;             // split-KV partial outputs
     float *part_ml;            // split-KV partial (max, sum)
-    uint32_t *part_sync;       // number of the call, tickets, and per item the number of the call whose second part lies in part_o; number 1, else zero at first
+    uint32_t *part_sync;       // state of the merge in the attention kernel (TcParams::sync): number 1, else zero at first
     size_t part_o_floats, part_ml_floats;
 };
 
