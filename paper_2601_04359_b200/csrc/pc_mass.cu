@@ -153,7 +153,7 @@ k_mass_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
 #pragma unroll
                 for (int k = 0; k < TILE / 32; ++k) {
                     const int row = tb * TILE + k * 32 + lane;
-                    lse[k] = row < P.n_q ? -1.4426950408889634f * __ldg(P.lse + (size_t)row * P.n_q_heads + h) : -INFINITY;
+                    lse[k] = row < P.n_q ? -1.4426950408889634f * __ldcg(P.lse + (size_t)row * P.n_q_heads + h) : -INFINITY;
                 }
                 if (use > 0) alive = wait(BAR_QEMPTY + st, (use - 1) & 1);
                 if (!alive) break;

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(MOVE_THREADS) k_move(const __grid_constant__ R
         long long first = 0;
         for (int r = 0; r < R.n; ++r) {
             if (i >= first && i < R.end[r]) {
-                x[c] = pc_ldg_stream(R.src[r] + (i - first));
+                x[c] = __ldcg(R.src[r] + (i - first));         // (not as constant data: a kernel that this one overlaps writes the output)
                 to[c] = R.dst[r] + (i - first);
             }
             first = R.end[r];
