@@ -253,13 +253,26 @@ bool lay_out(const pc_ctx *ctx, const pc_cache *src, bool pack, FrontParams &P, 
                 longest = std::max(longest, n);
             }
     };
-    // Tokens of a CTA: what its warps score at once (32), or somewhat more of short rows.  24 / 8 heads (2 KB), 5 frames: 247 tokens (31 a CTA)
-    // 28.3 -> 27.6 us, 330 (42) 32.3 -> 33.8; 16 / 4 heads (1 KB): 330 tokens 29.9 -> 29.2, 486 (61) 32.2 -> 33.7; fp32, 512 bytes: 294 (37) 39.0 -> 38.0.
-    const auto suits = [&]() { return cap <= 32 || (cap <= 48 && (long long)cap * D.n_kv_heads * D.head_dim * ctx->elem_size <= 72 * 1024); };
+    const int row = D.n_kv_heads * D.head_dim, row_bytes = row * ctx->elem_size;
+    const bool fp32 = D.dtype != PC_BF16;
+    // Tokens of a CTA: what its warps score at once (32), or more of narrow rows, most in clusters of eight.  Steps one after the other, the separate kernels
+    // against this one, us.  Clusters of eight: 2 KB, 5 frames of 257 to 288 tokens (33 to 36 a CTA) 28.9 -> 28.6, 9 frames 30.6 -> 30.2 (captured 28.4 and 28.4,
+    // 29.1 and 29.2), of 296 and more 29.8 -> 30.0; 1.5 KB, 288 to 320 26.0 -> 25.6 and 28.1 -> 27.5, 352 to 384 27.6 -> 27.7 and 29.5 -> 30.3; 1 KB, 288 to 384
+    // 27.5 -> 26.3 and 29.4 -> 29.0; 512 bytes, bf16, 3 and 5 frames 23.9 -> 22.5, 9 frames 24.7 -> 25.6; fp32 35.3 -> 34.0 on average of 5 and 9.
+    // Clusters of four, 16 frames: 2 KB, 132 tokens (33) 26.3 -> 26.0, 144 27.9 -> 28.1; 1.5 KB, 132 to 152 27.8 -> 24.3; 1 KB 26.0 -> 24.1; 512 bytes
+    // bf16 24.8 -> 22.7, fp32 30.0 -> 30.7, its rows of 1 and 1.5 KB 41.1 -> 41.7.
+    const auto most = [&]() {
+        if (P.ctas == FRONT_CTAS_MANY && (fp32 || row_bytes > 1536)) return 32;
+        return row_bytes <= 1024 ? 48 : (row_bytes <= 1536 ? 40 : (row_bytes <= 2048 ? 36 : 32));
+    };
+    // One frame and no pack, more than 256 tokens: 10.1 -> 10.7 us.  fp32 rows of 512 bytes, more than 16 frames: 24 of 100 tokens 28.8 -> 30.6, 32 of 32
+    // 22.0 -> 23.9, 32 of 100 33.9 -> 35.7 (16 of 100 26.2 -> 22.9).
+    const auto suits = [&]() {
+        return cap <= most() && (pack || src->n_frames > 1 || cap <= 32) && (!fp32 || row_bytes > 512 || src->n_frames <= 16);
+    };
     if (src->n_frames <= FRONT_CLUSTERS) cut(FRONT_CTAS, FRONT_CLUSTERS);
     else cut(FRONT_CTAS_MANY, FRONT_CLUSTERS_MANY);
     if (!suits()) return false;
-    const int row = D.n_kv_heads * D.head_dim, row_bytes = row * ctx->elem_size;
     P.row_bytes = row_bytes;
     P.cap = cap;
     long long at = 8LL * row;                       // the pooled query
