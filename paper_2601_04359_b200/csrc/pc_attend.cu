@@ -184,8 +184,8 @@ pc_status pc_frame_step_impl(pc_ctx *ctx, const pc_cache *src, const int32_t *bu
     const bool one_launch = !on_the_way && !ctx->timing_on && pc_select_pack_fits(ctx, src, budget);
     ctx->last_n_q = 0;
     ctx->q_rot_n = 0;
-    const pc_front_args args{src, budget, nullptr, scores, sel_idx, delta_t, &dst->history, k_rot_dst};
-    const pc_front_args *front = !on_the_way && n_sel > 0 && pc_front_fits(ctx, src, true) ? &args : nullptr;
+    pc_front_args args{src, budget, nullptr, scores, sel_idx, delta_t, &dst->history, k_rot_dst, {}};
+    const pc_front_args *front = !on_the_way && n_sel > 0 && pc_front_fits(ctx, src, true, &args.plan) ? &args : nullptr;
     st = pc_score_impl(ctx, src, q, q_pos, n_q, budget, nullptr, nullptr, scores, sel_idx, tc ? ctx->q_rot : nullptr, stream, !one_launch, front);
     if (st != PC_OK) return st;
     if (on_the_way) PC_CUDA_TRY(cudaStreamWaitEvent(stream, hooks->kv_ready, 0));

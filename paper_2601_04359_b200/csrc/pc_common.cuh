@@ -282,8 +282,13 @@ pc_status pc_check_segment(const pc_segment *s, bool allow_empty);
 pc_status pc_launch_pack(pc_ctx *ctx, const void *src_k, const void *src_v, const int32_t *src_pos, const int32_t *sel_idx,
                          int n_sel, int n_src, int delta_t, void *dst_k, void *dst_v, int32_t *dst_pos, void *k_rot_dst,
                          cudaStream_t stream);
-// Scores, selection and (dst given) pack of a small history in one launch behind the query pass, and whether a call suits it;
+// Scores, selection and (dst given) pack of a small history in one launch behind the query pass, and whether and how a call suits it;
 // arguments already checked
+struct pc_front_plan {
+    int ctas, clusters;          // CTAs of a cluster, clusters
+    int cap;                     // most tokens of a CTA
+    int at_keys, at_tok, at_rows, smem;      // places in its shared memory, and how much of that
+};
 struct pc_front_args {
     const pc_cache *src;
     const int32_t *budget;
@@ -293,8 +298,9 @@ struct pc_front_args {
     int32_t delta_t;
     const pc_segment *dst;       // NULL: no pack
     void *k_rot_dst;             // as pc_launch_pack
+    pc_front_plan plan;
 };
-bool pc_front_fits(const pc_ctx *ctx, const pc_cache *src, bool pack);
+bool pc_front_fits(const pc_ctx *ctx, const pc_cache *src, bool pack, pc_front_plan *plan);
 pc_status pc_launch_front(pc_ctx *ctx, const pc_front_args &args, int32_t n_q, cudaStream_t stream);
 // pc_score / pc_compact with the extras of the fused frame step: q_rot_out (NULL or the context's rotated-query scratch,
 // filled by the query pass that also pools), k_rot_dst (as pc_launch_pack)

@@ -37,6 +37,7 @@ constexpr int FRONT_THREADS = 512, FRONT_WARPS = FRONT_THREADS / 32;
 constexpr int FRONT_CTAS = 8, FRONT_CLUSTERS = 11, FRONT_CTAS_MANY = 4, FRONT_CLUSTERS_MANY = 32;
 constexpr int FRONT_FRAMES = FRONT_CTAS_MANY * FRONT_CLUSTERS_MANY;
 static_assert(FRONT_CLUSTERS <= FRONT_FRAMES, "a cluster has at least a CTA for every frame of its own");
+constexpr int FRONT_TOKENS = 48;                    // most tokens of a CTA
 constexpr int FRONT_SMEM = 220 * 1024;
 
 struct FrontParams {
@@ -54,7 +55,7 @@ struct FrontParams {
     int delta_t, n_frames;
     int32_t *status;
     uint32_t wait_us, extra_tx;
-    int ctas, cap, at_keys, at_tok, at_rows;        // CTAs of a cluster; most tokens of a CTA; places in its shared memory
+    int ctas, cap, at_keys, at_tok, at_rows;        // as pc_front_plan
     pc_rope_dev rope;
     int4 f[FRONT_FRAMES];                           // (first token, tokens, budget, output offset)
 };
@@ -236,23 +237,31 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const __grid_constan
     if (tid == 0 && gave_up) pc_let_copies_land();
 }
 
-// How a call is laid out: clusters, and the shared memory of a CTA; false where it does not fit or the separate kernels are faster.
-bool lay_out(const pc_ctx *ctx, const pc_cache *src, bool pack, FrontParams &P, int &clusters, int &smem) {
+// How a call is laid out: clusters, and the shared memory of a CTA; false where it does not fit or the separate kernels are faster.  Every scoring
+// call asks, so a long history is refused at once and the rest takes a division a frame at most (a walk over all CTAs took 0.5 us of host time at
+// 5 frames and 1.6 at 47, twice a call).
+bool lay_out(const pc_ctx *ctx, const pc_cache *src, bool pack, pc_front_plan &L) {
     const pc_layer_desc &D = ctx->desc;
-    if (src->n_frames < 1 || src->n_frames > FRONT_FRAMES || src->history.n_tokens > (1 << 20)) return false;
-    int cap = 1, longest = 1;
-    const auto cut = [&](int ctas, int most) {
-        P.ctas = ctas;
-        clusters = std::min(src->n_frames, most);
+    const int n_frames = src->n_frames;
+    if (n_frames < 1 || n_frames > FRONT_FRAMES || src->history.n_tokens > FRONT_TOKENS * FRONT_FRAMES) return false;
+    const bool many = n_frames > FRONT_CLUSTERS;
+    L.ctas = many ? FRONT_CTAS_MANY : FRONT_CTAS;
+    L.clusters = std::min(n_frames, FRONT_CLUSTERS_MANY);
+    int longest = 1;
+    for (int f = 0; f < n_frames; ++f) longest = std::max(longest, src->frame_count[f]);
+    if (longest > FRONT_TOKENS * L.ctas) return false;
+    int cap = (longest + L.ctas - 1) / L.ctas;      // most tokens of a CTA: a cluster to a frame, or (front_frame) a cluster's CTAs shared out over its frames
+    if (n_frames > L.clusters) {
         cap = 1;
-        for (int c = 0; c < clusters; ++c)
-            for (int r = 0; r < ctas; ++r) {
-                const FrontFrame f = front_frame(src->n_frames, clusters, c, r, ctas);
-                const int n = src->frame_count[f.frame];
-                cap = std::max(cap, share(n, r - f.first + 1, f.n) - share(n, r - f.first, f.n));
-                longest = std::max(longest, n);
+        for (int c = 0; c < L.clusters; ++c) {
+            const int f0 = share(n_frames, c, L.clusters), nf = share(n_frames, c + 1, L.clusters) - f0;
+            for (int j = 0, first = 0; j < nf; ++j) {
+                const int end = ((j + 1) * L.ctas + nf - 1) / nf, n = end - first;
+                cap = std::max(cap, (src->frame_count[f0 + j] + n - 1) / n);
+                first = end;
             }
-    };
+        }
+    }
     const int row = D.n_kv_heads * D.head_dim, row_bytes = row * ctx->elem_size;
     const bool fp32 = D.dtype != PC_BF16;
     // Tokens of a CTA: what its warps score at once (32), or more of narrow rows, most in clusters of eight.  Steps one after the other, the separate kernels
@@ -262,34 +271,28 @@ bool lay_out(const pc_ctx *ctx, const pc_cache *src, bool pack, FrontParams &P, 
     // Clusters of four, 16 frames: 2 KB, 132 tokens (33) 26.3 -> 26.0, 144 27.9 -> 28.1; 1.5 KB, 132 to 152 27.8 -> 24.3; 1 KB 26.0 -> 24.1; 512 bytes
     // bf16 24.8 -> 22.7, fp32 30.0 -> 30.7, its rows of 1 and 1.5 KB 41.1 -> 41.7.
     const auto most = [&]() {
-        if (P.ctas == FRONT_CTAS_MANY && (fp32 || row_bytes > 1536)) return 32;
-        return row_bytes <= 1024 ? 48 : (row_bytes <= 1536 ? 40 : (row_bytes <= 2048 ? 36 : 32));
+        if (many && (fp32 || row_bytes > 1536)) return 32;
+        return row_bytes <= 1024 ? FRONT_TOKENS : (row_bytes <= 1536 ? 40 : (row_bytes <= 2048 ? 36 : 32));
     };
     // One frame and no pack, more than 256 tokens: 10.1 -> 10.7 us.  fp32 rows of 512 bytes, more than 16 frames: 24 of 100 tokens 28.8 -> 30.6, 32 of 32
     // 22.0 -> 23.9, 32 of 100 33.9 -> 35.7 (16 of 100 26.2 -> 22.9).
-    const auto suits = [&]() {
-        return cap <= most() && (pack || src->n_frames > 1 || cap <= 32) && (!fp32 || row_bytes > 512 || src->n_frames <= 16);
-    };
-    if (src->n_frames <= FRONT_CLUSTERS) cut(FRONT_CTAS, FRONT_CLUSTERS);
-    else cut(FRONT_CTAS_MANY, FRONT_CLUSTERS_MANY);
-    if (!suits()) return false;
-    P.row_bytes = row_bytes;
-    P.cap = cap;
+    if (cap > most() || (!pack && n_frames == 1 && cap > 32) || (fp32 && row_bytes <= 512 && n_frames > 16)) return false;
+    L.cap = cap;
     long long at = 8LL * row;                       // the pooled query
     const auto place = [&](int &p, long long bytes) {
         at = (at + 127) / 128 * 128;
         p = (int)std::min<long long>(at, INT32_MAX);
         at += bytes;
     };
-    place(P.at_keys, 4LL * longest);
-    place(P.at_tok, 24LL * cap);
-    place(P.at_rows, (pack ? 2LL : 1LL) * cap * row_bytes);
-    smem = (int)std::min<long long>(at, INT32_MAX);
+    place(L.at_keys, 4LL * longest);
+    place(L.at_tok, 24LL * cap);
+    place(L.at_rows, (pack ? 2LL : 1LL) * cap * row_bytes);
+    L.smem = (int)std::min<long long>(at, INT32_MAX);
     return cap > 1 && at <= FRONT_SMEM;              // (a token each: a history of no more than a CTA's worth, left to the separate kernels)
 }
 
 template <typename T, int LPT, bool PACK>
-pc_status launch(const pc_ctx *ctx, const FrontParams &P, int clusters, int smem, cudaStream_t stream) {
+pc_status launch(const pc_ctx *ctx, const FrontParams &P, const pc_front_plan &L, cudaStream_t stream) {
     static std::atomic<bool> set[PC_MAX_DEVICES];
     if (ctx->device < 0 || ctx->device >= PC_MAX_DEVICES) return PC_ERR_UNSUPPORTED;
     if (!set[ctx->device]) {
@@ -297,15 +300,15 @@ pc_status launch(const pc_ctx *ctx, const FrontParams &P, int clusters, int smem
         set[ctx->device] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * P.ctas);
+    cfg.gridDim = dim3(L.clusters * L.ctas);
     cfg.blockDim = dim3(FRONT_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = L.smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = P.ctas;
+    attr[1].val.clusterDim.x = L.ctas;
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -316,19 +319,22 @@ pc_status launch(const pc_ctx *ctx, const FrontParams &P, int clusters, int smem
 
 }  // namespace
 
-bool pc_front_fits(const pc_ctx *ctx, const pc_cache *src, bool pack) {
-    FrontParams P;
-    int clusters, smem;
-    return !ctx->timing_on && src->history.n_tokens > 0 && lay_out(ctx, src, pack, P, clusters, smem);
+bool pc_front_fits(const pc_ctx *ctx, const pc_cache *src, bool pack, pc_front_plan *plan) {
+    return !ctx->timing_on && src->history.n_tokens > 0 && lay_out(ctx, src, pack, *plan);
 }
 
 pc_status pc_launch_front(pc_ctx *ctx, const pc_front_args &A, int32_t n_q, cudaStream_t stream) {
     const pc_layer_desc &D = ctx->desc;
     const pc_cache *src = A.src;
     const pc_segment *dst = A.dst;
+    const pc_front_plan &L = A.plan;
     FrontParams P;
-    int clusters = 0, smem = 0;
-    if (!lay_out(ctx, src, dst != nullptr, P, clusters, smem)) return PC_ERR_UNSUPPORTED;
+    P.ctas = L.ctas;
+    P.cap = L.cap;
+    P.at_keys = L.at_keys;
+    P.at_tok = L.at_tok;
+    P.at_rows = L.at_rows;
+    P.row_bytes = D.n_kv_heads * D.head_dim * ctx->elem_size;
     P.k = static_cast<const char *>(src->history.k);
     P.v = static_cast<const char *>(src->history.v);
     P.pos = src->history.pos;
@@ -356,7 +362,7 @@ pc_status pc_launch_front(pc_ctx *ctx, const pc_front_args &A, int32_t n_q, cuda
         out += A.budget[f];
     }
     const bool wide = D.head_dim * ctx->elem_size > 256;             // fp32 heads of 128: 32 lanes a token
-    if (D.dtype == PC_BF16) return dst ? launch<__nv_bfloat16, 16, true>(ctx, P, clusters, smem, stream) : launch<__nv_bfloat16, 16, false>(ctx, P, clusters, smem, stream);
-    if (!wide) return dst ? launch<float, 16, true>(ctx, P, clusters, smem, stream) : launch<float, 16, false>(ctx, P, clusters, smem, stream);
-    return dst ? launch<float, 32, true>(ctx, P, clusters, smem, stream) : launch<float, 32, false>(ctx, P, clusters, smem, stream);
+    if (D.dtype == PC_BF16) return dst ? launch<__nv_bfloat16, 16, true>(ctx, P, L, stream) : launch<__nv_bfloat16, 16, false>(ctx, P, L, stream);
+    if (!wide) return dst ? launch<float, 16, true>(ctx, P, L, stream) : launch<float, 16, false>(ctx, P, L, stream);
+    return dst ? launch<float, 32, true>(ctx, P, L, stream) : launch<float, 32, false>(ctx, P, L, stream);
 }

@@ -497,7 +497,7 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
         out += b;
     }
     const float *select_on = scores_override;
-    const pc_front_args here{src, budget, valid, scores, sel_idx, 0, nullptr, nullptr};
+    pc_front_args here{src, budget, valid, scores, sel_idx, 0, nullptr, nullptr, {}};
     if (!scores_override) {
         if (n_src > 0) {
             const size_t row = (size_t)ctx->desc.n_kv_heads * ctx->desc.head_dim;
@@ -506,7 +506,7 @@ pc_status pc_score_impl(pc_ctx *ctx, const pc_cache *src, const void *q, const i
                 ctx->qpool_dirty = 0;
             }
             ctx->qpool_dirty = 1;
-            if (!front && select && out > 0 && pc_front_fits(ctx, src, false)) front = &here;
+            if (!front && select && out > 0 && pc_front_fits(ctx, src, false, &here.plan)) front = &here;
             const float q_scale = pc_q_rot_scale(ctx->desc.head_dim);
             st = ctx->desc.dtype == PC_BF16
                      ? enqueue_score<__nv_bfloat16>(ctx->desc, ctx->sm_count, ctx->rope, ctx->qpool_fx, ctx->status, src->history.k,
