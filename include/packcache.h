@@ -339,8 +339,9 @@ pc_status pc_window_step(pc_window *w, const void *q, const int32_t *q_pos, int3
  * rows for 24/8, 32/8, 24/12 and 32/16 heads, 641 for 16/4, 1,153 for 8/8, 129 for 64/8, 32/32 and 24/24.  Fewer rows give
  * pc_window_step's output bit for bit.  In parts the keys are cut in other places, which moves the reference that a row's
  * probabilities are rounded to bf16 against: each probability may differ by that rounding (2^-9 relative on either side).
- * Pinned host memory (in whole, on 16 bytes) keeps the copies asynchronous, and a step that moves up to 6 MB then goes up and home by a
- * kernel each, which read and write it in place of the copies.  All arguments are checked before anything is enqueued; a call that fails
+ * Pinned host memory (in whole, within one allocation or registration, on 16 bytes) keeps the copies asynchronous, and a step whose attention is one
+ * part and whose queries, output, keys and values together take up to 6 MiB then goes up and home by a kernel each, which read and write
+ * it in place of the copies.  All arguments are checked before anything is enqueued; a call that fails
  * leaves the window as it was (the frame is not appended) and nothing in flight on either stream.
  * Errors: as pc_window_append and pc_window_step. */
 typedef struct {
@@ -405,7 +406,8 @@ pc_status pc_test_expect_extra_bytes(pc_ctx *ctx, uint32_t n_bytes);
 pc_status pc_test_leave_parts(pc_ctx *ctx, int32_t on);
 
 /* Per-kernel timing for benchmarks.  With timing on, each call records CUDA events on its stream at the boundaries
- * of its kernels (a few microseconds of overhead per call); pc_get_timing waits for the last recorded events and
+ * of its kernels (a few microseconds of overhead per call; stages that would share a launch, as scores, selection and pack of a small
+ * history do, get one each then); pc_get_timing waits for the last recorded events and
  * writes the duration in milliseconds of each kernel of the most recent calls, -1 for a kernel that did not run.
  * ms is a host array [PC_N_STAGES]. */
 enum { PC_STAGE_QPOOL = 0 /* the query pass */, PC_STAGE_SCORE = 1, PC_STAGE_SELECT = 2, PC_STAGE_PACK = 3, PC_STAGE_ROPE = 4,

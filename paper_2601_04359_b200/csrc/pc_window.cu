@@ -370,10 +370,12 @@ pc_status window_step(pc_window *w, const void *q, const int32_t *q_pos, int32_t
     return PC_OK;
 }
 
-// A step from host memory goes up and home by a kernel each as long as it moves no more than this in all and its attention is one part.
-// Window of six frames, the runtime's copies on two streams against the kernels, us a call (in brackets MB both ways): 24 / 8 heads, 30 tokens
-// (0.5) 72.7 -> 62.8, 135 (2.2) 133 -> 100, 360 (5.9) 198 -> 179, 486 (8.0) 216 -> 224; 8 / 8 heads, 682 (5.6) 221 -> 176, 988 (8.1)
-// 232 -> 230; 32 / 16, 135 (3.3) 122 -> 124, 247 (6.1) 185 -> 186, 360 (8.8) 230 -> 237.
+// A step from host memory goes up and home by a kernel each as long as it moves no more than this (queries, output, keys and values) and its
+// attention is one part.  Window of six frames, eight processes a side in turn, us a call as the shortest and the middle one of their medians: the runtime's copies
+// on two streams against the kernels.  24 / 8 heads, 30 tokens (0.5 MB both ways) 69 / 74 -> 56 / 58, 135 (2.2) 101 / 155 -> 93 / 100, 247 (4.0) 130 / 206
+// -> 133 / 137, 360 (5.9) 168 / 279 -> 175 / 177; 8 / 8, 682 (5.6) 167 / 265 -> 170 / 171, 988 (8.1) 217 / 310 -> 224 / 225; 32 / 16, 135 (3.3) 158 / 202 -> 117 / 121,
+// 247 (6.1) 171 / 208 -> 176 / 177, 360 (8.8) 219 / 259 -> 232 / 233.  What the copies take depends on the process: in its best case up to 5 % less than the
+// kernels from 4 MB on, mostly a good deal more, by less the larger the step (a third below 6 MB, a tenth at 9).  What the kernels take does not.
 constexpr size_t SMALL_STEP = 6 << 20;
 
 // Runs of 16-byte chunks between pinned host memory and the device in one launch.  Bound by the link: 50 GB/s from and to pinned memory
