@@ -31,8 +31,9 @@
 // 1,024 at 16 a clock, twice).
 // That form -> this one, a call: the step at 12 frames 81.8 -> 78.8 us, at 47 157.8 -> 150.2, of 4,032-token frames 635 -> 588; the
 // whole cache of 47 frames 618 -> 568 (1.15 PFLOP/s without the rotary pre-pass), five passes over 7,184 keys 486 -> 452; since the
-// bounded wait lost its loop of questions 77.2, 148.5, 586, 569 and 450; with the merge in this kernel, both sides in turn on one box, the step at
-// 12 frames 75.5 -> 74.5, at 47 149.0 -> 147.0, of 4,032-token frames 588 -> 579, five passes 452 -> 441, the whole cache 569 -> 565.
+// bounded wait lost its loop of questions 77.2, 148.5, 586, 569 and 450; with the merge in this kernel and the way out for a part that
+// does not come, both sides in turn on one box, the step at 12 frames 75.5 -> 74.9, at 47 149.0 -> 147.3, of 4,032-token frames 589 -> 582, five passes
+// 452 -> 445, the whole cache level.
 // Every wait is bounded: a wait that runs out records PC_ERR_TIMEOUT and raises a CTA-wide abort flag; every later wait whose
 // phase is not complete gives up within some ten microseconds, and the CTA still drains its multiply-adds and copies, frees TMEM and exits.
 #include <algorithm>

@@ -15,7 +15,7 @@
 //                  x 5,168 keys 70.7 us against 43.7, 9,200 72.9 / 70.5, 12,980 106.3 / 95.6; 16 / 16, 300 x 1,200 10.1 / 9.9;
 //                  8 / 8, 1,500 x 4,000, a unit per CTA either way, 21.8 / 22.1.)  The step's
 //                  normalisers go into an eight-slot ring beside it, fetched by the warp that issues the copies (laid out by a kernel of its own for a bulk
-//                  copy first: guided steps of 28 to 294 tokens 4 to 10 % longer, of 1,008 0.7 %).  S^T = K Q^T (keys on the TMEM lanes,
+//                  copy first: guided steps of 28 to 294 tokens 2 to 10 % longer, of 1,008 0.8 % at 12 frames).  S^T = K Q^T (keys on the TMEM lanes,
 //                  queries on the columns) goes to one of two TMEM buffers per key tile.  Sixteen warps turn scores
 //                  into sums: per key tile and column half one warp per TMEM lane quadrant, one key per thread, 64
 //                  columns per step: 2^(s + (-lse2)) added up in registers.  Four such warps share each scheduler, so

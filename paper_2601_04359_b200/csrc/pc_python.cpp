@@ -2,7 +2,7 @@
 //
 // The calls of a frame step are short on the GPU for small frames, so the time that the host takes to issue them decides:
 // building the same structs through ctypes took 51 us of host time for a frame step (6.4 us per cache, 9.6 us for the plan,
-// 2.3 us per array pointer), more than the step's six launches.  Host time of a
+// 2.3 us per array pointer), more than the launches of the step.  Host time of a
 // pass, ctypes against this file: frame step 51 -> 27 us (fp32 62 -> 24, with a shorter launch list), attention over a cache
 // 19.8 -> 10.6, mask, score, pack and attend 82 -> 36; the small bf16 step 53.8 -> 37.5 us a pass.
 // Tensors are read through their Python methods (data_ptr, is_contiguous, shape), so nothing here depends on torch's C++ ABI.
